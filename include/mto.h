@@ -277,7 +277,7 @@ mto_status mto_element_matrix(mto_handle h, int64_t e, double* packed);
 /* Which kernel forms the element matrices in mto_build_elements:
  * MTO_BUILD_TENSOR (default): classes with d <= 8 run as one sliced GEMM per class on the tensor
  *   cores (tcgen05: both operands cut into 8 BF16 slices of 7 bits with power-of-two scales, the
- *   slice products summed exactly in FP32 TMEM columns by level, the levels combined in FP64:
+ *   slice products summed exactly in FP32 TMEM columns by level, the levels combined in integers:
  *   agrees with the FP64 kernel to ~1e-15 of each element's largest entry); larger d use the FP64
  *   CUDA-core kernel.
  * MTO_BUILD_SIMT: the FP64 CUDA-core kernel for every class. */

@@ -66,7 +66,7 @@ struct BClass {
   double* stab = nullptr; // sensitivity quadrature tables (FP64 and FP32 copies)
   float* stabf = nullptr;
   unsigned short* tcB = nullptr;  // tensor-core build: BF16 slices of K0 per N tile
-  float* tcTau = nullptr;         // and the power-of-two column scales
+  int* tcTau = nullptr;           // and the exponents of the power-of-two column scales
 };
 
 // QR-indicator tables for order p -> p + 1.

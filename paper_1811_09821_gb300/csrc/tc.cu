@@ -12,18 +12,32 @@
 // over K <= 64 subcells is an integer below 2^20, and all pairs of one level g = i + j share the
 // weight 2^-7g: each level accumulates its (at most 8) slice GEMMs in one FP32 TMEM accumulator
 // exactly (sums below 2^23).  Levels g = 2..10 are kept (the dropped levels weigh below 2^-51 of
-// the row/column scale, the operands' truncation 2^-56); the epilogue adds the levels in FP64,
-// rescales by sigma_e tau_pos (powers of two, exact) and stores the FP64 matrix and, for the mixed
-// build, its split pair.
+// the row/column scale, the operands' truncation 2^-56).
 //
-// One CTA (4 warps) per 128 elements: the A slices (8 x 128 x K) are formed in shared memory from
-// rho once; the CTA then walks the N tiles of 32 positions: B slices copied to shared memory, one
-// thread issues the 43 x (K/16) tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, M = 128, N = 32)
-// into 9 level accumulators (288 TMEM columns), commits to an mbarrier, and all threads read
-// their row back with tcgen05.ld and store 32 consecutive entries of their element's row.
+// The epilogue stays off the FP64 pipes (2 FMA per clock and SM on GB300: one FP64 instruction per
+// stored entry of the 1024 x 512 beam costs 0.47 ms): the nine level sums are integers, so an entry
+// is one 80-bit integer times a power of two, which integer instructions round to FP64 (once, to
+// nearest even) and split into the FP32 pair.
+//
+// One CTA per 128 elements and range of N tiles (16 positions each; the tiles of small classes are
+// spread over several CTAs so that the chip fills).  The A slices (8 x 128 x K) are formed in
+// shared memory from rho once.  Warp 8 feeds the tensor cores: B slices of a tile by one bulk copy
+// into a ring of three, then per K step one tcgen05.mma (kind::f16, BF16 x BF16 -> FP32, M = 128)
+// per A slice i against the stacked B slices 1 .. min(8, 10 - i): B slice j times A slice i belongs
+// to level i + j, and the level accumulators lie side by side in TMEM, so the products of one A
+// slice with all its B slices are one MMA of up to N = 128 (the A slice is read once for all of
+// them).  Two TMEM stages of 9 x 16 columns let the MMAs of a tile run under the epilogue of the
+// tile before.  Warps 0-7 read their row's 8 positions with tcgen05.ld and write whole sectors of
+// their rows through a small shared staging.
 // Operands use the no-swizzle K-major core-matrix layout (8 rows x 16 bytes per core matrix).
-// Every wait is bounded: on expiry the kernel records an error word and skips the tile.
+// Every wait is bounded: on expiry the kernel records an error word and stops this CTA.
+//
+// Measured (build and one operator product together): 480 x 240 Q3/d8, mixed: 5.32 ms with an FP64
+// epilogue of 24 FP64 instructions per entry and 43 single-slice MMAs per K step, 1.10 ms now;
+// 320 x 160 adaptive maps (16 classes), FP64: 11.8 ms and 1.62 ms.
+#include <algorithm>
 #include <cstdio>
+#include <cstring>
 #include <vector>
 
 #include "mto_internal.cuh"
@@ -32,12 +46,19 @@ namespace mto {
 namespace {
 
 constexpr int kTM = 128;        // elements per CTA (MMA M)
-constexpr int kTN = 32;         // positions per N tile (MMA N)
+constexpr int kTN = 16;         // positions per N tile
+constexpr int kBRing = 3;       // B tiles in flight
+constexpr int kEpiWarps = 8;    // epilogue warps (one more feeds the tensor cores)
 constexpr int kSlices = 8;      // slices per operand (8 x 7 = 56 bits)
 constexpr int kSliceBits = 7;
 constexpr int kOpBits = kSlices * kSliceBits;
 constexpr int kLevels = 9;      // levels g = i + j = 2..10
-constexpr int kTmemCols = 512;  // 9 x 32 = 288 used (allocations are powers of two)
+constexpr int kTmemCols = 512;  // two stages of 9 x 16 = 144 columns, 256 apart
+constexpr int kTmemStage = 256;
+// staging rows of an epilogue warp: 8 doubles or 8 floats and 16 bytes of padding (conflict-free
+// 16-byte stores by 32 lanes)
+constexpr int kStRow64 = 80, kStRow32 = 48;
+constexpr int kStWarp = 32 * (kStRow64 + 2 * kStRow32);
 constexpr unsigned kSpinLimit = 1u << 26;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -87,13 +108,11 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// 16 consecutive 32-bit TMEM columns of this thread's lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
+// 8 consecutive 32-bit TMEM columns of this thread's lane
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&v)[8]) {
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
       : "r"(taddr)
       : "memory");
 }
@@ -122,11 +141,33 @@ __host__ __device__ __forceinline__ uint32_t core_off(int row, int k, int kpad) 
   return (uint32_t)(((row >> 3) * (kpad >> 3) + (k >> 3)) * 128 + (row & 7) * 16 + (k & 7) * 2);
 }
 
-// B operand tables of a class: per N tile, 7 slices of kTN x kpad BF16 in the core layout, and
-// the column scales tau (power of two) per position.  One thread per (position, subcell).
+__device__ __forceinline__ void mbar_expect(uint64_t* bar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// bounded wait for the phase of parity `parity`; false when the limit expires
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
+  for (unsigned n = 0; n < kSpinLimit; ++n)
+    if (mbar_try_wait(bar, parity)) return true;
+  return false;
+}
+
+__device__ __forceinline__ void tc_bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+      "l"(src), "r"(bytes), "r"(smem_u32(bar))
+      : "memory");
+}
+
+// B operand tables of a class: per N tile, 8 slices of kTN x kpad BF16 in the core layout (so the
+// slices of a tile stack along N), and per position the exponent of its power-of-two scale tau.  One thread per (position, subcell).
 __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double* __restrict__ K0T,
                                  const int* __restrict__ posc, unsigned short* __restrict__ Bt,
-                                 float* __restrict__ tau) {
+                                 int* __restrict__ tau) {
   const int pos = blockIdx.x;
   if (pos >= ntile * kTN) return;
   __shared__ double colmax;
@@ -141,7 +182,7 @@ __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double
   int ex = 0;
   if (colmax > 0.0) frexp(colmax, &ex);   // colmax < 2^ex
   const double sc = ldexp(1.0, -ex);
-  if (threadIdx.x == 0) tau[pos] = colmax > 0.0 ? ldexpf(1.0f, ex) : 0.0f;
+  if (threadIdx.x == 0) tau[pos] = ex;
   const int tile = pos / kTN, row = pos % kTN;
   for (int s = threadIdx.x; s < kpad; s += blockDim.x) {
     const double w = (c >= 0 && s < S) ? K0T[(size_t)c * S + s] * sc : 0.0;   // |w| < 1
@@ -158,58 +199,157 @@ __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double
   }
 }
 
-__global__ void __launch_bounds__(128, 1) tc_build_kernel(
-    int n, int S, int kpad, int L, int ntile, const int* __restrict__ elem, const int* __restrict__ slot,
-    const int64_t* __restrict__ design_off, const double* __restrict__ rho, double E0, double Emin, double q,
-    const unsigned short* __restrict__ Bt, const float* __restrict__ tau, double* __restrict__ K64,
-    float* __restrict__ Kh, float* __restrict__ Kl, int* __restrict__ err) {
+// floor(v 2^(56 - ex)) of a non-negative double v < 2^ex, by its bits (0 for negative or non-finite v)
+__host__ __device__ __forceinline__ unsigned long long fixed56(unsigned long long bits, int ex) {
+  const int be = (int)(bits >> 52);   // sign and exponent
+  if (be >= 0x7ff) return 0ull;
+  const unsigned long long m = be ? (bits & 0xfffffffffffffull) | (1ull << 52) : bits;
+  const int sh = (be ? be : 1) - 1075 + 56 - ex;
+  return sh >= 0 ? m << (sh & 63) : (sh > -64 ? m >> (-sh & 63) : 0ull);
+}
+
+// The exact sum of the level integers, X 2^(ex - 70) with X = H 2^28 + Lw, rounded once to FP64 (to
+// nearest even), as its bits.  |H| < 2^52.
+__host__ __device__ __forceinline__ unsigned long long levels_to_double(long long H, long long Lw, int ex) {
+  long long h = H + (Lw >> 28);
+  unsigned lo = (unsigned)Lw & 0xfffffffu;   // X = h 2^28 + lo, 0 <= lo < 2^28
+  const bool neg = h < 0;
+  if (neg) {
+    lo = (0u - lo) & 0xfffffffu;
+    h = ~h + (lo == 0u);
+  }
+  unsigned long long W = ((unsigned long long)h << 12) | (lo >> 16);   // the upper 64 of 80 bits
+  unsigned long long R = (unsigned long long)(lo & 0xffffu) << 48;     // the rest, left-aligned
+  if (W == 0ull) {
+    if (R == 0ull) return 0ull;
+    W = R;
+    R = 0ull;
+    ex -= 64;
+  }
+#ifdef __CUDA_ARCH__
+  const int z = __clzll((long long)W);
+#else
+  const int z = __builtin_clzll(W);
+#endif
+  const unsigned long long A = z ? (W << z) | (R >> (64 - z)) : W;   // leading one at bit 63
+  const unsigned long long sticky = (R << z) != 0ull;
+  const unsigned rem = (unsigned)(A & 0x7ffu) * 2u + (unsigned)sticky;
+  unsigned long long m = A >> 11;
+  m += rem + (unsigned)(m & 1u) > 0x800u;
+  const int be = 9 - z + ex + 1023;   // X = A 2^(16 - z)
+  unsigned long long bits;
+  if (be >= 1 && be <= 2046) {
+    bits = ((unsigned long long)(be - 1) << 52) + m;
+  } else {
+    const double v = ldexp((double)m, be - 1075);
+    memcpy(&bits, &v, 8);
+  }
+  return neg ? bits | (1ull << 63) : bits;
+}
+
+// The split pair of an FP64 value: hi = fl32(v), lo = fl32(v - hi), by integer instructions where the
+// exponents allow it (from 2^-98 on a lo below the normal range has at most 24 bits, so that the
+// conversion and the scaling below round once between them).
+__host__ __device__ __forceinline__ void split_pair(unsigned long long bits, float& hi, float& lo) {
+  const int be = (int)(bits >> 52) & 0x7ff;
+  const int e = be - 1023;
+  if (e < -98 || e > 110) {
+    double v;
+    memcpy(&v, &bits, 8);
+    hi = (float)v;
+    lo = (float)(v - (double)hi);
+    return;
+  }
+  const unsigned long long m = (bits & 0xfffffffffffffull) | (1ull << 52);
+  const unsigned h24 = (unsigned)(m >> 29), rem = (unsigned)m & 0x1fffffffu;
+  const unsigned up = rem + (h24 & 1u) > 0x10000000u;
+  const unsigned sgn = (unsigned)(bits >> 32) & 0x80000000u;
+  const unsigned hb = (sgn | ((unsigned)(e + 126) << 23)) + h24 + up;
+  const int D = (int)rem - (int)(up << 29);   // v - hi = D 2^(e - 52)
+  const unsigned sb = (unsigned)(e + 8 + 127) << 23;   // 2^(e + 8); the product rounds once (exact before)
+  float s;
+  memcpy(&hi, &hb, 4);
+  memcpy(&s, &sb, 4);
+  const float d = (float)(sgn ? -D : D);
+  lo = (d * 8.673617379884035e-19f) * s;   // 2^-60 2^(e + 8)
+}
+
+// rows: element k of the class (first <= k < n) is output row slot[k], or row k - first without slots.
+// Kh null: FP64 rows only.
+__global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
+    int n, int first, int S, int kpad, int L, int ntile, int tiles_per_cta, const int* __restrict__ elem,
+    const int* __restrict__ slot, const int64_t* __restrict__ design_off, const double* __restrict__ rho, double E0,
+    double Emin, double q, const unsigned short* __restrict__ Bt, const int* __restrict__ tau,
+    double* __restrict__ K64, float* __restrict__ Kh, float* __restrict__ Kl, int* __restrict__ err) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  const size_t a_bytes = (size_t)kSlices * kTM * kpad * 2;
-  const size_t b_bytes = (size_t)kSlices * kTN * kpad * 2;
+  const uint32_t a_slice = (uint32_t)kTM * kpad * 2, b_slice = (uint32_t)kTN * kpad * 2;
+  const uint32_t b_tile = kSlices * b_slice;
   unsigned char* As = smem;
-  unsigned char* Bs = smem + a_bytes;
-  uint64_t* bar = reinterpret_cast<uint64_t*>(smem + a_bytes + b_bytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bar + 1);
-  float* sigma_s = reinterpret_cast<float*>(bar + 2);   // [kTM]
-  const int t = threadIdx.x, warp = t >> 5;
-  const int base = blockIdx.x * kTM;
+  unsigned char* Bs = As + kSlices * a_slice;
+  unsigned char* stage = Bs + kBRing * b_tile;
+  uint64_t* bfull = reinterpret_cast<uint64_t*>(stage + kEpiWarps * kStWarp);   // [kBRing] B tile landed
+  uint64_t* full = bfull + kBRing;    // [2] MMAs of a TMEM stage done
+  uint64_t* empty = full + 2;         // [2] TMEM stage read by all epilogue warps
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(empty + 2);
+  int* sig = reinterpret_cast<int*>(tmem_slot + 2);   // [kTM] exponents of sigma_e
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int base = first + blockIdx.x * kTM;
+  const int tile0 = blockIdx.y * tiles_per_cta;
+  const int nt = min(tiles_per_cta, ntile - tile0);
 
   if (warp == 0) {
     tmem_alloc(tmem_slot, kTmemCols);
     tmem_relinquish();
   }
-  if (t == 0) {
-    mbar_init(bar, 1);
+  if (warp == kEpiWarps && lane == 0) {
+    for (int b = 0; b < kBRing; ++b) mbar_init(bfull + b, 1);
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(full + b, 1);
+      mbar_init(empty + b, kEpiWarps);
+    }
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    for (int i = 0; i < kBRing && i < nt; ++i) {
+      mbar_expect(bfull + i, b_tile);
+      tc_bulk_g2s(Bs + i * b_tile, reinterpret_cast<const unsigned char*>(Bt) + (size_t)(tile0 + i) * b_tile, b_tile,
+                  bfull + i);
+    }
   }
 
-  // A slices: this thread's element row, moduli E_s scaled by sigma_e and cut into 7 x 7 bits.
-  // E is monotone in rho, so sigma_e comes from the largest density (one E per element); q = 3
-  // takes products instead of pow (GB300's FP64 pipes made the per-subcell pow the bottleneck).
-  {
-    const int k = base + t;
-    const bool act = k < n;
+  // A slices: one element row per warp at a time, two subcells per lane (coalesced rho, packed
+  // 32-bit stores).  Moduli E_s scaled by sigma_e and cut into 8 x 7 bits by integer shifts; q = 3
+  // takes products instead of pow (both run on the FP64 pipes).
+  if (warp < kEpiWarps) {
     const bool cube = q == 3.0;
-    auto modulus = [&](double r) { return Emin + (cube ? r * r * r : pow(r, q)) * (E0 - Emin); };
-    int64_t off = 0;
-    double rmax = 0.0;
-    if (act) {
-      off = design_off[elem[k]];
-      for (int s = 0; s < S; ++s) rmax = fmax(rmax, rho[off + s]);
-    }
-    const double m = act ? modulus(rmax) : 0.0;
-    int ex = 0;
-    if (m > 0.0) frexp(m, &ex);
-    const double sc = ldexp(1.0, -ex);
-    sigma_s[t] = m > 0.0 ? ldexpf(1.0f, ex) : 0.0f;
-    for (int s = 0; s < kpad; ++s) {
-      double v = 0.0;
-      if (act && s < S) v = modulus(rho[off + s]) * sc;   // [0, 1)
-      const unsigned long long V = (unsigned long long)ldexp(v, kOpBits);   // floor(v 2^56)
-      for (int i = 0; i < kSlices; ++i) {
-        const float a = (float)((V >> (kOpBits - kSliceBits * (i + 1))) & 127ull);
-        const unsigned short b = (unsigned short)(__float_as_uint(a) >> 16);
-        *reinterpret_cast<unsigned short*>(As + (size_t)i * kTM * kpad * 2 + core_off(t, s, kpad)) = b;
+    const double dE = E0 - Emin;
+    auto modulus = [&](double r) { return Emin + (cube ? r * r * r : pow(r, q)) * dE; };
+    const int s0 = 2 * lane;
+#pragma unroll 4
+    for (int r = warp; r < kTM; r += kEpiWarps) {
+      const int k = base + r;
+      double r0 = 0.0, r1 = 0.0;
+      const bool v0 = k < n && s0 < S, v1 = k < n && s0 + 1 < S;
+      if (v0) {
+        const int64_t off = design_off[elem[k]];
+        r0 = rho[off + s0];
+        if (v1) r1 = rho[off + s0 + 1];
+      }
+      const unsigned long long e0 = v0 ? (unsigned long long)__double_as_longlong(modulus(r0)) : 0ull;
+      const unsigned long long e1 = v1 ? (unsigned long long)__double_as_longlong(modulus(r1)) : 0ull;
+      // sigma_e = 2^ex > max E: from the largest exponent among the finite non-negative moduli
+      const int x0 = (int)(e0 >> 52), x1 = (int)(e1 >> 52);
+      const int xm = __reduce_max_sync(0xffffffffu, max(x0 < 0x7ff ? x0 : 0, x1 < 0x7ff ? x1 : 0));
+      const int ex = max(xm, 1) - 1022;
+      if (lane == 0) sig[r] = ex;
+      if (s0 < kpad) {
+        const unsigned long long V0 = fixed56(e0, ex), V1 = fixed56(e1, ex);
+        unsigned char* dst = As + core_off(r, s0, kpad);
+#pragma unroll
+        for (int i = 0; i < kSlices; ++i) {
+          const int sh = kOpBits - kSliceBits * (i + 1);
+          const unsigned a0 = __float_as_uint((float)(int)((V0 >> sh) & 127ull)) >> 16;
+          const unsigned a1 = __float_as_uint((float)(int)((V1 >> sh) & 127ull)) & 0xffff0000u;
+          *reinterpret_cast<unsigned*>(dst + i * a_slice) = a0 | a1;   // BF16 of integers <= 127: exact
+        }
       }
     }
   }
@@ -218,98 +358,126 @@ __global__ void __launch_bounds__(128, 1) tc_build_kernel(
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  const uint32_t idesc = idesc_bf16(kTM, kTN);
-  const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
-  const int kst = kpad / 16;
-  const uint32_t a0 = smem_u32(As), b0 = smem_u32(Bs);
-  const int row = base + t;
-  const bool act = row < n;
-  const int sl = act ? slot[row] : 0;
-  const float sig = sigma_s[t];
-  uint32_t phase = 0;
+  bool ok = true;
 
-  for (int tile = 0; tile < ntile; ++tile) {
-    // B slices of this tile into shared memory
-    const uint4* src = reinterpret_cast<const uint4*>(Bt + (size_t)tile * kSlices * kTN * kpad);
-    uint4* dst = reinterpret_cast<uint4*>(Bs);
-    for (size_t i = t; i < b_bytes / 16; i += blockDim.x) dst[i] = src[i];
-    fence_proxy_async();
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (t == 0) {
-      for (int g = 0; g < kLevels; ++g) {
-        uint32_t acc = 0;
-        const int lev = g + 2;
-        for (int i = 1; i <= kSlices; ++i) {
-          const int j = lev - i;
-          if (j < 1 || j > kSlices) continue;
-          for (int ks = 0; ks < kst; ++ks) {
-            const uint64_t ad = smem_desc(a0 + (uint32_t)((size_t)(i - 1) * kTM * kpad * 2) + ks * 256u, 128u, sbo);
-            const uint64_t bd = smem_desc(b0 + (uint32_t)((size_t)(j - 1) * kTN * kpad * 2) + ks * 256u, 128u, sbo);
-            umma_bf16(tmem + (uint32_t)(g * kTN), ad, bd, idesc, acc);
-            acc = 1;
-          }
+  if (warp == kEpiWarps) {
+    if (lane == 0) {
+      const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
+      const int kst = kpad / 16;
+      const uint32_t a0 = smem_u32(As);
+      for (int it = 0; it < nt && ok; ++it) {
+        const int st = it & 1;
+        ok = mbar_wait(bfull + it % kBRing, (uint32_t)((it / kBRing) & 1));
+        if (ok && it >= 2) ok = mbar_wait(empty + st, (uint32_t)(((it >> 1) - 1) & 1));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t b0 = smem_u32(Bs + (it % kBRing) * b_tile);
+        const uint32_t d0 = tmem + (uint32_t)(st * kTmemStage);
+        auto mma = [&](int i, int j, int nj, int ks, uint32_t acc) {   // A slice i times B slices j .. j + nj - 1
+          umma_bf16(d0 + (uint32_t)((i + j - 2) * kTN), smem_desc(a0 + (uint32_t)(i - 1) * a_slice + ks * 256u, 128u, sbo),
+                    smem_desc(b0 + (uint32_t)(j - 1) * b_slice + ks * 256u, 128u, sbo), idesc_bf16(kTM, kTN * nj), acc);
+        };
+        // slice 2 first: it starts levels 3..10; slice 1 then starts level 2 and adds to the others
+        for (int ks = 0; ks < kst; ++ks) mma(2, 1, kSlices, ks, ks > 0);
+        mma(1, 1, 1, 0, 0);
+        mma(1, 2, kSlices - 1, 0, 1);
+        for (int ks = 1; ks < kst; ++ks) mma(1, 1, kSlices, ks, 1);
+        for (int i = 3; i <= kSlices; ++i)
+          for (int ks = 0; ks < kst; ++ks) mma(i, 1, kLevels + 1 - i, ks, 1);
+        umma_commit(full + st);
+        // refill the ring slot of the tile before, whose MMAs are done once its stage is committed
+        if (it >= 1 && it - 1 + kBRing < nt) {
+          const int nx = it - 1 + kBRing;
+          ok = mbar_wait(full + (st ^ 1), (uint32_t)(((it - 1) >> 1) & 1));
+          if (!ok) break;
+          mbar_expect(bfull + nx % kBRing, b_tile);
+          tc_bulk_g2s(Bs + (nx % kBRing) * b_tile, reinterpret_cast<const unsigned char*>(Bt) + (size_t)(tile0 + nx) * b_tile,
+                      b_tile, bfull + nx % kBRing);
         }
       }
-      umma_commit(bar);
+      if (!ok) {
+        // a wait expired: let every copy that was issued land before the CTA gives up its memory
+        for (int b = 0; b < kBRing; ++b) {
+          mbar_wait(bfull + b, 0);
+          mbar_wait(bfull + b, 1);
+        }
+      }
     }
-    // bounded wait for the MMAs; the whole CTA agrees before leaving on expiry
-    unsigned spins = 0;
-    bool ok = true;
-    while (!mbar_try_wait(bar, phase)) {
-      if (++spins > kSpinLimit) {
+    __syncwarp();
+  } else {
+    const int row = (warp & 3) * 32 + lane, c0 = (warp >> 2) * 8;
+    const int k = base + row;
+    const int sl = k < n ? (slot ? slot[k] : k - first) : -1;
+    const int sexp = sig[row];
+    unsigned char* st64 = stage + warp * kStWarp;
+    unsigned char* sth = st64 + 32 * kStRow64;
+    unsigned char* stl = sth + 32 * kStRow32;
+    for (int it = 0; it < nt; ++it) {
+      const int st = it & 1;
+      ok = mbar_wait(full + st, (uint32_t)((it >> 1) & 1));
+      if (!__all_sync(0xffffffffu, ok)) {
         ok = false;
         break;
       }
-    }
-    phase ^= 1u;
-    tc_fence_after();
-    if (__syncthreads_or(!ok)) {
-      if (t == 0) atomicExch(err, 1);
-      break;   // the accumulators are not trustworthy: stop this CTA (the caller reports the error)
-    }
-    // epilogue: this thread's TMEM lane = its row; chunks of 16 positions.  Every level sum is an
-    // integer below 2^23 (exact in FP32); the levels are added from the smallest in FP64 (9 terms
-    // per entry), then scaled by sigma_e tau_pos (a power of two: exact)
-    const uint32_t lane_addr = tmem + ((uint32_t)(warp * 32) << 16);
-#pragma unroll 1
-    for (int ch = 0; ch < kTN / 16; ++ch) {
-      double acc[16];
+      tc_fence_after();
+      uint32_t v[kLevels][8];
+      const uint32_t src = tmem + (uint32_t)(st * kTmemStage + c0) + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll
-      for (int c = 0; c < 16; ++c) acc[c] = 0.0;
-#pragma unroll 1
-      for (int g = kLevels - 1; g >= 0; --g) {
-        uint32_t v[16];
-        tmem_ld16(lane_addr + (uint32_t)(g * kTN + ch * 16), v);
-        tmem_wait_ld();
-        const double wgt = ldexp(1.0, -kSliceBits * (g + 2));
+      for (int g = 0; g < kLevels; ++g) tmem_ld8(src + (uint32_t)(g * kTN), v[g]);
+      tmem_wait_ld();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty + st);
+      const int pos0 = (tile0 + it) * kTN + c0;
+      if (pos0 < L) {
 #pragma unroll
-        for (int c = 0; c < 16; ++c) acc[c] = fma((double)__uint_as_float(v[c]), wgt, acc[c]);
-      }
-      if (act) {
-        const int pos0 = tile * kTN + ch * 16;
+        for (int c = 0; c < 8; ++c) {
+          int I[kLevels];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-          const int pos = pos0 + c;
-          if (pos >= L) break;
-          const double kv = acc[c] * ((double)sig * (double)__ldg(tau + pos));
-          const size_t o = (size_t)sl * L + pos;
-          K64[o] = kv;
+          for (int g = 0; g < kLevels; ++g) I[g] = __float2int_rn(__uint_as_float(v[g][c]));
+          // pairs of levels fit 32 bits (2^30 + 2^23); units: level 6 for H, level 10 for Lw
+          const int p0 = I[0] * 128 + I[1], p1 = I[2] * 128 + I[3], p2 = I[5] * 128 + I[6], p3 = I[7] * 128 + I[8];
+          const long long H = (long long)p0 * (1 << 21) + (long long)p1 * 128 + I[4];
+          const long long Lw = (long long)p2 * (1 << 14) + p3;
+          const unsigned long long bits = levels_to_double(H, Lw, sexp + __ldg(tau + pos0 + c));
+          *reinterpret_cast<unsigned long long*>(st64 + lane * kStRow64 + c * 8) = bits;
           if (Kh) {
-            const float hi = (float)kv;
-            Kh[o] = hi;
-            Kl[o] = (float)(kv - (double)hi);
+            float hi, lo;
+            split_pair(bits, hi, lo);
+            *reinterpret_cast<float*>(sth + lane * kStRow32 + c * 4) = hi;
+            *reinterpret_cast<float*>(stl + lane * kStRow32 + c * 4) = lo;
           }
         }
+        __syncwarp();
+        // whole sectors: 4 lanes per 64-byte row piece of the FP64 rows, 2 lanes per FP32 piece
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = 8 * i + (lane >> 2), o = 2 * (lane & 3);
+          const int rs = __shfl_sync(0xffffffffu, sl, r);
+          if (rs >= 0 && pos0 + o < L)
+            *reinterpret_cast<double2*>(K64 + (size_t)rs * L + pos0 + o) =
+                *reinterpret_cast<const double2*>(st64 + r * kStRow64 + o * 8);
+        }
+        if (Kh) {
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const int r = 16 * i + (lane >> 1), o = 4 * (lane & 1);
+            const int rs = __shfl_sync(0xffffffffu, sl, r);
+            if (rs >= 0 && pos0 + o < L) {
+              const size_t at = (size_t)rs * L + pos0 + o;
+              *reinterpret_cast<float4*>(Kh + at) = *reinterpret_cast<const float4*>(sth + r * kStRow32 + o * 4);
+              *reinterpret_cast<float4*>(Kl + at) = *reinterpret_cast<const float4*>(stl + r * kStRow32 + o * 4);
+            }
+          }
+        }
+        __syncwarp();
       }
     }
-    tc_fence_before();
-    __syncthreads();   // TMEM and B reused by the next tile
-    tc_fence_after();
   }
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(*tmem_slot, kTmemCols);
+  tc_fence_before();
+  if (__syncthreads_or(!ok) && t == 0) atomicExch(err, 1);   // the rows are not trustworthy
+  tc_fence_after();
+  if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
 
 }  // namespace
@@ -333,14 +501,19 @@ mto_status tc_tables(mto_handle h) {
   return MTO_OK;
 }
 
+namespace {
 // Dynamic shared memory of the build kernel, at least 120 KB so that one CTA (and one 512-column
 // TMEM allocation) is resident per SM.
 size_t tc_smem_bytes(int kpad) {
-  const size_t need = (size_t)kSlices * (kTM + kTN) * kpad * 2 + 16 + 4 * kTM + 64;
+  const size_t need = (size_t)kSlices * (kTM + kBRing * kTN) * kpad * 2 + kEpiWarps * kStWarp + 8 * (kBRing + 4) + 8 +
+                      4 * kTM + 64;
   return need < 120 * 1024 ? 120 * 1024 : need;
 }
+}  // namespace
 
-// The tensor-core build of one (p, d) class (d <= 8).
+// The tensor-core build of one (p, d) class (d <= 8).  The N tiles of a class with few elements are
+// split over CTAs (each forms its elements' A slices again, about the cost of three tiles) until the
+// launch has about one CTA per SM.
 mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision) {
   const PClass& c = h->pc[b.p];
   const int kpad = (b.S + 15) / 16 * 16;
@@ -348,9 +521,11 @@ mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, cons
   const size_t smem = tc_smem_bytes(kpad);
   MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(tc_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem), "cudaFuncSetAttribute"));
-  const int grid = (b.n + kTM - 1) / kTM;
-  tc_build_kernel<<<grid, 128, smem, h->stream>>>(
-      b.n, b.S, kpad, c.L, ntile, b.elem, b.slot, h->design_off_d, rho, m->E0, m->Emin, m->q, b.tcB, b.tcTau,
+  const int gx = (b.n + kTM - 1) / kTM;
+  const int gy = std::max(1, std::min(ntile, 152 / gx));
+  const int per = (ntile + gy - 1) / gy;
+  tc_build_kernel<<<dim3(gx, (ntile + per - 1) / per), 32 * (kEpiWarps + 1), smem, h->stream>>>(
+      b.n, 0, b.S, kpad, c.L, ntile, per, b.elem, b.slot, h->design_off_d, rho, m->E0, m->Emin, m->q, b.tcB, b.tcTau,
       c.K64, precision == MTO_MIXED ? c.K32 : nullptr, precision == MTO_MIXED ? c.K32lo : nullptr, h->flags + 4);
   return mto_after_launch(h, "tc_build_kernel");
 }

@@ -1,0 +1,59 @@
+"""Kernels at the sizes where their tiling can go wrong (edges of tiles, remainders, the smallest and
+largest classes), against the oracle or the library's general path.  Each tolerance is derived in
+its test's docstring."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+from oracle import mesh as om
+
+
+@pytest.fixture(scope="module")
+def mto():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1811_09821_gb300 as m
+    from paper_1811_09821_gb300 import _build
+    _build.build()
+    m.load_library()
+    return m
+
+
+def handle(mto, nx, ny, p, d, hx=1.0, hy=1.0):
+    h = mto.Handle(0)
+    h.setup(nx, ny, np.broadcast_to(np.asarray(p, np.int32), nx * ny), np.broadcast_to(np.asarray(d, np.int32), nx * ny),
+            hx, hy)
+    return h
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (43, 3)])   # 1 and 129 elements: one row, one past a tile of 128
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("d", [1, 4, 5, 8])            # K = 1, 16, 25 (padded to 32) and 64 subcells
+def test_tensor_build_edges(mto, nx, ny, p, d):
+    """The sliced tensor-core build against the FP64 CUDA-core build: the dropped levels weigh below
+    2^-51 of the element's scale and the 64-term FP64 sums below 64 x 2^-53, so 1e-14 of the element's
+    largest entry covers both; the split pair is fl32(K) and fl32(K - hi) of the stored FP64
+    entries bit for bit, also for moduli of 1e-9 and 1e-24 and for exact zeros."""
+    h = handle(mto, nx, ny, p, d)
+    rng = np.random.default_rng(100 * p + d)
+    rho = rng.uniform(0.0, 1.0, h.design_len)
+    rho[rng.uniform(size=len(rho)) < 0.4] = 0.0
+    rho[-d * d:] = rng.choice([0.0, 1e-8], d * d)
+    rho[:d * d] = 1.0
+    r = torch.tensor(rho, device="cuda")
+    mat = mto.material(1.0, 0.0 if d == 5 else 1e-9, 0.3, 3.0)
+    es = sorted({0, 1, 126, 127, 128} & set(range(nx * ny)))
+    h.set_build_path(mto.BUILD_SIMT)
+    h.build_elements(r, mat, mto.MTO_FP64)
+    want = {e: h.element_matrix(e, p) for e in es}
+    h.set_build_path(mto.BUILD_TENSOR)
+    h.build_elements(r, mat, mto.MTO_MIXED)
+    for e in es:
+        got = h.element_matrix(e, p)
+        assert np.abs(got - want[e]).max() <= 1e-14 * np.abs(want[e]).max(), e
+        hi, lo = h.element_matrix_split(e, p)
+        np.testing.assert_array_equal(hi, got.astype(np.float32))
+        np.testing.assert_array_equal(lo, (got - hi.astype(np.float64)).astype(np.float32))
+    h.close()
