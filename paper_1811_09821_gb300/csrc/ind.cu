@@ -9,18 +9,33 @@
 namespace mto {
 namespace {
 
-// Basis constants shared by the indicator kernels: GLL nodes of orders 1..kPMaxTab and Gauss
-// rules of 1..kPMaxTab+2 points, filled once per handle by basis_table_kernel.
+// Basis constants shared by the indicator kernels: GLL nodes of orders 1..kPMaxTab, Gauss rules of
+// 1..kPMaxTab+2 points, and for the Kelly edges the Lagrange derivatives at both ends of an element
+// (dn[p][0]: -1, dn[p][1]: +1) and the Lagrange values at the points of an n-point rule (lv[p][n]).
+// Filled once per handle by basis_table_kernel.
 struct BasisTab {
   double gll[kPMaxTab + 1][kPMaxTab + 1];
   double gx[kPMaxTab + 3][kPMaxTab + 3];
   double gw[kPMaxTab + 3][kPMaxTab + 3];
+  double dn[kPMaxTab + 1][2][kPMaxTab + 1];
+  double lv[kPMaxTab + 1][kPMaxTab + 3][kPMaxTab + 3][kPMaxTab + 1];
 };
 
-__global__ void basis_table_kernel(BasisTab* t) {
-  int p = threadIdx.x;
-  if (p >= 1 && p <= kPMaxTab) gll_nodes(p, t->gll[p]);
-  if (p >= 1 && p <= kPMaxTab + 2) gauss_rule(p, t->gx[p], t->gw[p]);
+__global__ void __launch_bounds__(256) basis_table_kernel(BasisTab* t) {
+  const int i = threadIdx.x;
+  if (i >= 1 && i <= kPMaxTab) gll_nodes(i, t->gll[i]);
+  if (i >= 33 && i <= 32 + kPMaxTab + 2) gauss_rule(i - 32, t->gx[i - 32], t->gw[i - 32]);
+  __syncthreads();
+  for (int k = i; k < (kPMaxTab + 1) * 2 * (kPMaxTab + 1); k += blockDim.x) {
+    const int a = k % (kPMaxTab + 1), end = k / (kPMaxTab + 1) % 2, p = k / (2 * (kPMaxTab + 1));
+    if (p >= 1 && a <= p) t->dn[p][end][a] = lagrange_der(t->gll[p], p + 1, a, end ? 1.0 : -1.0);
+  }
+  constexpr int NG = kPMaxTab + 3;
+  for (int k = i; k < (kPMaxTab + 1) * NG * NG * (kPMaxTab + 1); k += blockDim.x) {
+    const int a = k % (kPMaxTab + 1), g = k / (kPMaxTab + 1) % NG, n = k / ((kPMaxTab + 1) * NG) % NG;
+    const int p = k / ((kPMaxTab + 1) * NG * NG);
+    if (p >= 1 && a <= p && n >= 1 && g < n) t->lv[p][n][g][a] = lagrange_val(t->gll[p], p + 1, a, t->gx[n][g]);
+  }
 }
 
 // Local displacement of element e (order p): 2 (p+1)^2 values, minimum-rule constraints applied.
@@ -44,12 +59,6 @@ __device__ __forceinline__ void gather_node(int nn, int slot, int ln, const int*
   ue[2 * ln + 1] = b;
 }
 
-__device__ void gather_element(int p, int slot, const int* __restrict__ gmap, const Constraint* __restrict__ cons,
-                               const double* __restrict__ u, double* ue) {
-  const int nn = (p + 1) * (p + 1);
-  for (int ln = 0; ln < nn; ++ln) gather_node(nn, slot, ln, gmap, cons, u, ue);
-}
-
 __device__ __forceinline__ double warp_sum_all(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
@@ -60,60 +69,91 @@ struct ClassPtrs {
 };
 
 // ------------------------------------------------------------------------------------ Kelly
-// Normal derivative (along +x for sides 0/1, +y for sides 2/3) of both components of an order-p
-// field at edge parameter t: side 0 x = 0, 1 x = hx, 2 y = 0, 3 y = hy.
-__device__ void edge_normal_derivative(const BasisTab* B, int p, int side, const double* ue, double t, double hx,
-                                       double hy, double* dx, double* dy) {
-  const double* z = B->gll[p];
+// Adds sign x the normal derivative (along +x or +y) of one element's field at the Gauss points of
+// one of its edges to (jx, jy).  The trace of the normal derivative is contracted first: along the
+// normal by the derivatives at the element's end (end: 0 the low, 1 the high side), then along the
+// edge by the values at the Gauss points: 2 (p + 1) (p + 1 + nq) FMAs, where products of Lagrange
+// polynomials formed per point took thousands of FP64 instructions and divisions.
+constexpr int kEdgeQ = MTO_P_MAX + 1;   // Gauss points of an edge of the largest order
+
+__device__ __forceinline__ void add_edge_trace(const BasisTab* __restrict__ B, int p, int slot,
+                                               const int* __restrict__ gmap, const Constraint* __restrict__ cons,
+                                               const double* __restrict__ u, bool vertical, int end, int nq,
+                                               double scale, double (&jx)[kEdgeQ], double (&jy)[kEdgeQ]) {
   const int n1 = p + 1;
-  double sx = 0.0, sy = 0.0;
-  const double xi = side == 0 ? -1.0 : side == 1 ? 1.0 : t;
-  const double eta = side == 2 ? -1.0 : side == 3 ? 1.0 : t;
-  for (int b = 0; b < n1; ++b)
+  const int* gm = gmap + (size_t)slot * n1 * n1;
+  const double* dn = B->dn[p][end];
+  const int sn = vertical ? 1 : n1, st = vertical ? n1 : 1;   // node strides along the normal and the edge
+  for (int b = 0; b < n1; ++b) {
+    double tx = 0.0, ty = 0.0;
+#pragma unroll 4
     for (int a = 0; a < n1; ++a) {
-      double w = side <= 1 ? lagrange_der(z, n1, a, xi) * lagrange_val(z, n1, b, eta) * (2.0 / hx)
-                           : lagrange_val(z, n1, a, xi) * lagrange_der(z, n1, b, eta) * (2.0 / hy);
-      sx += w * ue[2 * (b * n1 + a)];
-      sy += w * ue[2 * (b * n1 + a) + 1];
+      const int g = gm[b * st + a * sn];
+      double ux, uy;
+      if (g >= 0) {
+        ux = u[2 * (size_t)g];   // u is the caller's: 8-byte aligned at the least
+        uy = u[2 * (size_t)g + 1];
+      } else {
+        const Constraint& c = cons[-g - 1];
+        ux = uy = 0.0;
+        for (int k = 0; k < c.cnt; ++k) {
+          ux += c.w[k] * u[2 * (size_t)c.node[k]];
+          uy += c.w[k] * u[2 * (size_t)c.node[k] + 1];
+        }
+      }
+      tx = fma(dn[a], ux, tx);
+      ty = fma(dn[a], uy, ty);
     }
-  *dx = sx;
-  *dy = sy;
+    tx *= scale;
+    ty *= scale;
+#pragma unroll
+    for (int g = 0; g < kEdgeQ; ++g)
+      if (g < nq) {
+        const double w = B->lv[p][nq][g][b];
+        jx[g] = fma(w, tx, jx[g]);
+        jy[g] = fma(w, ty, jy[g]);
+      }
+  }
 }
 
 // Edge term c_F * integral_F [du/dn]^2 ds (Eq. 9) for every interior edge: horizontal edges
-// first (id iy*nelx + ix, between elements below and above), then vertical edges.
-__global__ void kelly_edge_kernel(int nelx, int nely, const int* __restrict__ p_of, const int* __restrict__ slot_of,
-                                  ClassPtrs cp, const Constraint* __restrict__ cons, const double* __restrict__ u,
-                                  const BasisTab* __restrict__ B, double hx, double hy, double* __restrict__ edge_val) {
+// first (id iy*nelx + ix, between elements below and above), then vertical edges.  One thread per
+// edge, bound by the FP64 pipes (about 150 FMAs per edge between Q3 elements).  Measured with the
+// selection kernels below: the indicators of a 320 x 160 adaptive mesh 22.1 -> 10.9 ms (10.5 ms of
+// them were this kernel, forming Lagrange products and their divisions per point); on the
+// 1024 x 512 beam this kernel took 34 ms.
+__global__ void __launch_bounds__(128) kelly_edge_kernel(
+    int nelx, int nely, const int* __restrict__ p_of, const int* __restrict__ slot_of, ClassPtrs cp,
+    const Constraint* __restrict__ cons, const double* __restrict__ u, const BasisTab* __restrict__ B, double hx,
+    double hy, double* __restrict__ edge_val) {
   const int64_t nH = (int64_t)(nely + 1) * nelx, nV = (int64_t)nely * (nelx + 1);
   const double hF = sqrt(hx * hx + hy * hy);
   for (int64_t id = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; id < nH + nV; id += (int64_t)gridDim.x * blockDim.x) {
-    int eA, eB, sideA, sideB;
-    double len;
-    if (id < nH) {
+    const bool vertical = id >= nH;
+    int eA, eB;
+    if (!vertical) {
       int iy = (int)(id / nelx), ix = (int)(id % nelx);
       if (iy == 0 || iy == nely) { edge_val[id] = 0.0; continue; }
-      eA = (iy - 1) * nelx + ix; eB = iy * nelx + ix; sideA = 3; sideB = 2; len = hx;
+      eA = (iy - 1) * nelx + ix; eB = iy * nelx + ix;
     } else {
       int64_t v = id - nH;
       int iy = (int)(v / (nelx + 1)), ix = (int)(v % (nelx + 1));
       if (ix == 0 || ix == nelx) { edge_val[id] = 0.0; continue; }
-      eA = iy * nelx + ix - 1; eB = iy * nelx + ix; sideA = 1; sideB = 0; len = hy;
+      eA = iy * nelx + ix - 1; eB = iy * nelx + ix;
     }
+    const double len = vertical ? hy : hx, sc = 2.0 / (vertical ? hx : hy);
     const int pA = p_of[eA], pB = p_of[eB];
-    double uA[2 * (kPMaxTab) * (kPMaxTab)], uB[2 * (kPMaxTab) * (kPMaxTab)];
-    gather_element(pA, slot_of[eA], cp.gmap[pA], cons, u, uA);
-    gather_element(pB, slot_of[eB], cp.gmap[pB], cons, u, uB);
     const int pF = pA > pB ? pA : pB;
     const int nq = pF + 1;
+    double jx[kEdgeQ], jy[kEdgeQ];
+#pragma unroll
+    for (int g = 0; g < kEdgeQ; ++g) jx[g] = jy[g] = 0.0;
+    add_edge_trace(B, pA, slot_of[eA], cp.gmap[pA], cons, u, vertical, 1, nq, sc, jx, jy);
+    add_edge_trace(B, pB, slot_of[eB], cp.gmap[pB], cons, u, vertical, 0, nq, -sc, jx, jy);
     double val = 0.0;
-    for (int g = 0; g < nq; ++g) {
-      double ax, ay, bx, by;
-      edge_normal_derivative(B, pA, sideA, uA, B->gx[nq][g], hx, hy, &ax, &ay);
-      edge_normal_derivative(B, pB, sideB, uB, B->gx[nq][g], hx, hy, &bx, &by);
-      double jx = ax - bx, jy = ay - by;
-      val += B->gw[nq][g] * (jx * jx + jy * jy) * 0.5 * len;
-    }
+#pragma unroll
+    for (int g = 0; g < kEdgeQ; ++g)
+      if (g < nq) val += B->gw[nq][g] * (jx[g] * jx[g] + jy[g] * jy[g]) * 0.5 * len;
     edge_val[id] = hF / (2.0 * pF) * val;
   }
 }
@@ -132,12 +172,30 @@ __global__ void kelly_sum_kernel(int nelx, int nely, const double* __restrict__ 
 }
 
 // ------------------------------------------------------------------------------------ Gamma^d
-__global__ void minmax_kernel(int64_t n, const double* __restrict__ rho, unsigned long long* __restrict__ mm) {
+// smallest and largest order key; one pair of atomics per block
+__global__ void __launch_bounds__(256) minmax_kernel(int64_t n, const double* __restrict__ rho,
+                                                     unsigned long long* __restrict__ mm) {
   unsigned long long lo = ~0ULL, hi = 0ULL;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     unsigned long long k = order_key(rho[i]);
     lo = k < lo ? k : lo;
     hi = k > hi ? k : hi;
+  }
+  __shared__ unsigned long long sl[8], sh[8];
+  for (int o = 16; o > 0; o >>= 1) {
+    const unsigned long long a = __shfl_xor_sync(0xffffffffu, lo, o), b = __shfl_xor_sync(0xffffffffu, hi, o);
+    lo = a < lo ? a : lo;
+    hi = b > hi ? b : hi;
+  }
+  if ((threadIdx.x & 31) == 0) {
+    sl[threadIdx.x >> 5] = lo;
+    sh[threadIdx.x >> 5] = hi;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+    lo = sl[w] < lo ? sl[w] : lo;
+    hi = sh[w] > hi ? sh[w] : hi;
   }
   atomicMin(&mm[0], lo);
   atomicMax(&mm[1], hi);
@@ -150,27 +208,67 @@ __device__ double key_to_double(unsigned long long k) {
   return v;
 }
 
-// Density indicator (Sec. 3.2.2): per element, the cells' band contributions in cell order.
-__global__ void gamma_d_kernel(int64_t nel, const int64_t* __restrict__ off, const double* __restrict__ rho,
-                               const unsigned long long* __restrict__ mm, int cycle, double alpha, double beta,
-                               double* __restrict__ gd) {
+// Density indicator (Sec. 3.2.2): per element, the cells' band contributions in cell order.  A warp
+// takes 32 consecutive elements: its lanes form the contributions of 32 cells of one element at a
+// time (coalesced; the bands are compared on the order keys, off the FP64 pipes), and then each lane
+// adds its own element's in cell order, so the sums are those of a serial loop.  The division by
+// the cell count is a product where the count is a power of two (exact either way).
+constexpr int kGdWarps = 4;
+__global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
+    int64_t nel, const int64_t* __restrict__ off, const double* __restrict__ rho,
+    const unsigned long long* __restrict__ mm, int cycle, double alpha, double beta, double* __restrict__ gd) {
+  __shared__ double tile[kGdWarps][32][33];
   const double rmin = key_to_double(mm[0]), rmax = key_to_double(mm[1]);
   const double ravg = 0.5 * (rmax + rmin);
   const double fac = ravg * exp(-beta * (cycle - 1));
   const double rl = rmin + (1.0 - alpha) * fac, ru = rmax - (1.0 - alpha) * fac;
   const double cl = rmin + alpha * fac, cu = rmax - alpha * fac;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nel; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t a = off[e], b = off[e + 1];
-    const double n = (double)(b - a);
+  // -0 and +0 compare equal: zero is added to every key's value first
+  auto key = [](double v) { return order_key(__longlong_as_double(__double_as_longlong(v) == (1ll << 63) ? 0ll : __double_as_longlong(v))); };
+  // a NaN bound fails its comparison: the largest key as a lower bound, the smallest as an upper one
+  auto lower = [&](double v) { return v == v ? key(v) : ~0ULL; };
+  auto upper = [&](double v) { return v == v ? key(v) : 0ULL; };
+  const unsigned long long krl = lower(rl), kru = upper(ru), kcl = upper(cl), kcu = lower(cu);
+  const unsigned long long kav_hi = upper(ravg), kav_lo = lower(ravg);
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+  double(*T)[33] = tile[wib];
+  const int64_t nw = (int64_t)gridDim.x * kGdWarps;
+  for (int64_t base = 32 * (blockIdx.x * (int64_t)kGdWarps + wib); base < nel; base += 32 * nw) {
+    const int64_t e = base + lane;
+    const int64_t a = e < nel ? off[e] : 0;
+    const int n = e < nel ? (int)(off[e + 1] - a) : 0;
+    const double nd = (double)n, inv = 1.0 / nd;
+    const int nmax = __reduce_max_sync(0xffffffffu, n);
     double g = 0.0;
-    for (int64_t j = a; j < b; ++j) {
-      const double r = rho[j];
-      if (rl <= r && r <= ravg) g += (r - rl) / n;
-      else if (ravg < r && r <= ru) g += (ru - r) / n;
-      else if (r <= cl) g -= (cl - r) / n;
-      else if (r >= cu) g -= (r - cu) / n;
+    for (int c0 = 0; c0 < nmax; c0 += 32) {
+#pragma unroll 4
+      for (int k = 0; k < 32; ++k) {
+        const int nk = __shfl_sync(0xffffffffu, n, k);
+        const int64_t ak = __shfl_sync(0xffffffffu, a, k);
+        const double ndk = __shfl_sync(0xffffffffu, nd, k), ik = __shfl_sync(0xffffffffu, inv, k);
+        const bool p2 = (nk & (nk - 1)) == 0;
+        if (c0 >= nk) continue;
+        double t = 0.0;
+        if (c0 + lane < nk) {
+          const double r = rho[ak + c0 + lane];
+          const unsigned long long kr = key(r);
+          double x = 0.0;
+          if ((unsigned long long)(__double_as_longlong(r) & 0x7fffffffffffffffll) <= 0x7ff0000000000000ull) {   // no NaN
+            if (krl <= kr && kr <= kav_hi) x = r - rl;
+            else if (kav_lo < kr && kr <= kru) x = ru - r;
+            else if (kr <= kcl) x = r - cl;     // subtracting cl - r
+            else if (kr >= kcu) x = cu - r;
+          }
+          t = p2 ? x * ik : x / ndk;
+        }
+        T[k][lane] = t;
+      }
+      __syncwarp();
+      const int m = min(32, n - c0);
+      for (int j = 0; j < m; ++j) g += T[lane][j];
+      __syncwarp();
     }
-    gd[e] = g;
+    if (e < nel) gd[e] = g;
   }
 }
 
@@ -351,97 +449,148 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
 }
 
 // ------------------------------------------------------------------------------------ selection
-// k-th smallest (0-based) composite key (order_key(v_i), i) among the items with part(i), found
-// by radix selection over the 64-bit key (8 passes of 8 bits) and then the index among equal keys.
-// State in sel[]: [0] prefix, [1] rank remaining, [2] result key, [3] result index, [4] valid.
+// k-th smallest (0-based) composite key (order_key(v_i), i) among the items that take part, found by
+// radix selection over the 64-bit key (8 passes of 8 bits) and then the index among equal keys.
+// Up to two ranks of the same values are selected together; the last block of a pass to finish
+// picks the digits (a scan over the 256 counters), so a selection is 9 launches with nothing between
+// them.  State of target t: st[2 t] the prefix, st[2 t + 1] the rank remaining.
 __device__ __forceinline__ bool participates(int mode, double v) {
   return mode == 0 ? true : mode == 1 ? (v < 0.0) : (v > 0.0);
 }
 
-__global__ void sel_init_kernel(unsigned long long* sel, const long long* krank) {
-  sel[0] = 0ULL;
-  sel[1] = (unsigned long long)(*krank);
-  sel[4] = 0ULL;
+// inclusive scan over the 256 threads of a block
+__device__ __forceinline__ unsigned scan256(unsigned v, unsigned* ws) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned t = __shfl_up_sync(0xffffffffu, v, o);
+    if (lane >= o) v += t;
+  }
+  if (lane == 31) ws[w] = v;
+  __syncthreads();
+  unsigned add = 0;
+  for (int k = 0; k < w; ++k) add += ws[k];
+  __syncthreads();
+  return v + add;
 }
 
-__global__ void sel_hist_kernel(int64_t n, const double* __restrict__ v, int mode, int shift,
-                                const unsigned long long* __restrict__ sel, unsigned int* __restrict__ hist) {
-  __shared__ unsigned int h[256];
-  for (int i = threadIdx.x; i < 256; i += blockDim.x) h[i] = 0;
+struct SelRanks {
+  unsigned long long k[2];
+};
+
+// the counters hist [2][256] and cnt are zero between launches
+__global__ void __launch_bounds__(256) sel_pass_kernel(int64_t n, const double* __restrict__ v, int mode, int nt,
+                                                       SelRanks ranks, int shift, unsigned long long* __restrict__ st,
+                                                       unsigned* __restrict__ hist, unsigned* __restrict__ cnt) {
+  __shared__ unsigned hs[2][256], ws[8];
+  __shared__ int last;
+  const int t = threadIdx.x;
+  hs[0][t] = hs[1][t] = 0;
   __syncthreads();
-  const unsigned long long prefix = sel[0];
   const unsigned long long himask = shift >= 56 ? 0ULL : (~0ULL << (shift + 8));
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    double x = v[i];
+  const unsigned long long p0 = shift >= 56 ? 0ULL : st[0], p1 = shift >= 56 ? 0ULL : st[2];
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + t; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const double x = v[i];
     if (!participates(mode, x)) continue;
-    unsigned long long key = order_key(x);
-    if ((key & himask) != (prefix & himask)) continue;
-    atomicAdd(&h[(key >> shift) & 255ULL], 1u);
+    const unsigned long long key = order_key(x);
+    const unsigned d = (unsigned)(key >> shift) & 255u;
+    if ((key & himask) == p0) atomicAdd(&hs[0][d], 1u);
+    if (nt > 1 && (key & himask) == p1) atomicAdd(&hs[1][d], 1u);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 256; i += blockDim.x)
-    if (h[i]) atomicAdd(&hist[i], h[i]);
-}
-
-__global__ void sel_pick_kernel(int shift, unsigned long long* sel, unsigned int* hist) {
-  if (threadIdx.x != 0) return;
-  unsigned long long r = sel[1];
-  unsigned long long acc = 0;
-  int b = 0;
-  for (; b < 256; ++b) {
-    if (r < acc + hist[b]) break;
-    acc += hist[b];
-  }
-  if (b == 256) b = 255;  // rank beyond the count: cannot happen for a valid rank
-  sel[1] = r - acc;
-  sel[0] |= (unsigned long long)b << shift;
-  for (int i = 0; i < 256; ++i) hist[i] = 0;
-}
-
-// count of matching items (key == sel[0]) per chunk of 1024 consecutive indices
-__global__ void sel_count_kernel(int64_t n, const double* __restrict__ v, int mode,
-                                 const unsigned long long* __restrict__ sel, unsigned int* __restrict__ cnt) {
-  const unsigned long long key = sel[0];
-  const int64_t chunk = blockIdx.x;
-  unsigned int c = 0;
-  for (int64_t i = chunk * 1024 + threadIdx.x; i < n && i < (chunk + 1) * 1024; i += blockDim.x) {
-    double x = v[i];
-    if (participates(mode, x) && order_key(x) == key) ++c;
-  }
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  __shared__ unsigned int part[32];
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = c;
+  for (int q = 0; q < nt; ++q)
+    if (hs[q][t]) atomicAdd(&hist[256 * q + t], hs[q][t]);
+  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned int s = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += part[w];
-    cnt[chunk] = s;
-  }
-}
-
-__global__ void sel_index_kernel(int64_t n, const double* __restrict__ v, int mode, unsigned long long* sel,
-                                 const unsigned int* __restrict__ cnt, int64_t nchunks) {
-  if (threadIdx.x != 0) return;
-  unsigned long long r = sel[1];
-  const unsigned long long key = sel[0];
-  int64_t c = 0;
-  for (; c < nchunks; ++c) {
-    if (r < cnt[c]) break;
-    r -= cnt[c];
-  }
-  int64_t idx = -1;
-  if (c < nchunks) {
-    for (int64_t i = c * 1024; i < n && i < (c + 1) * 1024; ++i) {
-      double x = v[i];
-      if (participates(mode, x) && order_key(x) == key) {
-        if (r == 0) { idx = i; break; }
-        --r;
-      }
+  if (t == 0) last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int q = 0; q < nt; ++q) {
+    const unsigned c = __ldcg(hist + 256 * q + t);
+    hist[256 * q + t] = 0;
+    const unsigned inc = scan256(c, ws);
+    const unsigned long long r = shift >= 56 ? ranks.k[q] : st[2 * q + 1];
+    const unsigned long long pre = shift >= 56 ? 0ULL : st[2 * q];
+    __syncthreads();
+    // the first digit whose inclusive count exceeds the rank (the last one for a rank beyond the count)
+    if ((inc - c <= r && r < inc) || (t == 255 && r >= inc)) {
+      st[2 * q] = pre | ((unsigned long long)t << shift);
+      st[2 * q + 1] = r - (inc - c);
     }
   }
-  sel[2] = key;
-  sel[3] = (unsigned long long)idx;
-  sel[4] = idx >= 0 ? 1ULL : 0ULL;
+  if (t == 0) *cnt = 0u;
+}
+
+// the index of the item of remaining rank among those equal to the selected key, and the result
+// (key, index) to out[2 q], out[2 q + 1].  part: [2][gridDim.x] counts per block (a block takes
+// consecutive items).
+__global__ void __launch_bounds__(256) sel_index_kernel(int64_t n, const double* __restrict__ v, int mode, int nt,
+                                                        const unsigned long long* __restrict__ st,
+                                                        unsigned* __restrict__ part, unsigned* __restrict__ cnt,
+                                                        unsigned long long* __restrict__ out0,
+                                                        unsigned long long* __restrict__ out1) {
+  __shared__ unsigned ws[8];
+  __shared__ int last, s_block;
+  __shared__ unsigned long long s_rank, s_idx;
+  const int t = threadIdx.x;
+  const int64_t per = (n + gridDim.x - 1) / gridDim.x;
+  auto match = [&](int64_t i, unsigned long long key) {
+    const double x = v[i];
+    return participates(mode, x) && order_key(x) == key;
+  };
+  for (int q = 0; q < nt; ++q) {
+    const unsigned long long key = st[2 * q];
+    unsigned c = 0;
+    for (int64_t i = blockIdx.x * per + t; i < n && i < (blockIdx.x + 1) * per; i += 256) c += match(i, key);
+    const unsigned tot = scan256(c, ws);
+    if (t == 255) part[q * gridDim.x + blockIdx.x] = tot;
+  }
+  __threadfence();
+  __syncthreads();
+  if (t == 0) last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  for (int q = 0; q < nt; ++q) {
+    const unsigned long long key = st[2 * q];
+    if (t == 0) {
+      s_block = -1;
+      s_idx = ~0ULL;
+    }
+    __syncthreads();
+    // gridDim.x <= 256: one block's count per thread
+    const unsigned c = t < (int)gridDim.x ? __ldcg(part + q * gridDim.x + t) : 0u;
+    const unsigned inc = scan256(c, ws);
+    const unsigned long long r = st[2 * q + 1];
+    if (inc - c <= r && r < inc) {
+      s_block = t;
+      s_rank = r - (inc - c);
+    }
+    __syncthreads();
+    if (s_block >= 0) {
+      unsigned long long rank = s_rank;
+      const int64_t end = min(n, (s_block + 1) * per);
+      for (int64_t i0 = s_block * per; i0 < end; i0 += 256) {
+        const int64_t i = i0 + t;
+        const unsigned m = i < end && match(i, key);
+        const unsigned im = scan256(m, ws);
+        if (m && im - 1 == rank) s_idx = (unsigned long long)i;
+        __syncthreads();
+        if (s_idx != ~0ULL) break;
+        if (t == 255) s_rank = rank - im;   // not among these: the total of this piece comes off
+        __syncthreads();
+        rank = s_rank;
+      }
+    }
+    __syncthreads();
+    if (t == 0) {
+      unsigned long long* out = q ? out1 : out0;
+      out[0] = key;
+      out[1] = s_idx;
+    }
+    __syncthreads();
+  }
+  if (t == 0) *cnt = 0u;
 }
 
 __device__ __forceinline__ bool comp_less(double v, int64_t i, unsigned long long key, unsigned long long idx) {
@@ -630,37 +779,27 @@ __global__ void __launch_bounds__(kOCBlock) oc_write_kernel(int64_t n, const dou
 mto_status ensure_basis(mto_handle h, BasisTab** out) {
   if (!h->basis_tab) {
     MTO_TRY(mto_alloc(h, reinterpret_cast<unsigned char**>(&h->basis_tab), sizeof(BasisTab)));
-    basis_table_kernel<<<1, 32, 0, h->stream>>>(reinterpret_cast<BasisTab*>(h->basis_tab));
+    basis_table_kernel<<<1, 256, 0, h->stream>>>(reinterpret_cast<BasisTab*>(h->basis_tab));
     MTO_TRY(mto_after_launch(h, "basis_table_kernel"));
   }
   *out = reinterpret_cast<BasisTab*>(h->basis_tab);
   return MTO_OK;
 }
 
-// Selection of the k-th composite key among participating values; the (key, index) pair is
-// copied to out[0..1] (device).  k is read from a device value.
-mto_status select_kth(mto_handle h, const double* v, int64_t n, int mode, const long long* k_dev,
-                      unsigned long long* out) {
-  unsigned int* hist = reinterpret_cast<unsigned int*>(h->sel + 64);   // 256 counters
-  unsigned long long* st = h->sel;
-  MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(hist, 0, 256 * sizeof(unsigned int), h->stream), "memset"));
-  sel_init_kernel<<<1, 1, 0, h->stream>>>(st, k_dev);
-  MTO_TRY(mto_after_launch(h, "sel_init_kernel"));
-  const int grd = grid_for(n, 256, 152 * 4);
+// Selection of the items of ranks k[0 .. nt) among the participating values; each (key, index) pair
+// to out[q][0..1] (device).
+mto_status select_kth(mto_handle h, const double* v, int64_t n, int mode, int nt, const SelRanks& k,
+                      unsigned long long* out0, unsigned long long* out1) {
+  unsigned long long* st = h->sel + 32;
+  unsigned* cnt = reinterpret_cast<unsigned*>(h->sel + 48);
+  unsigned* hist = reinterpret_cast<unsigned*>(h->sel + 64);   // [2][256]
+  const int grd = grid_for(n, 1024, 152 * 2);
   for (int shift = 56; shift >= 0; shift -= 8) {
-    sel_hist_kernel<<<grd, 256, 0, h->stream>>>(n, v, mode, shift, st, hist);
-    MTO_TRY(mto_after_launch(h, "sel_hist_kernel"));
-    sel_pick_kernel<<<1, 32, 0, h->stream>>>(shift, st, hist);
-    MTO_TRY(mto_after_launch(h, "sel_pick_kernel"));
+    sel_pass_kernel<<<grd, 256, 0, h->stream>>>(n, v, mode, nt, k, shift, st, hist, cnt);
+    MTO_TRY(mto_after_launch(h, "sel_pass_kernel"));
   }
-  const int64_t nch = (n + 1023) / 1024;
-  unsigned int* cnt = reinterpret_cast<unsigned int*>(h->ibuf + 3 * h->nel);
-  sel_count_kernel<<<(unsigned)nch, 256, 0, h->stream>>>(n, v, mode, st, cnt);
-  MTO_TRY(mto_after_launch(h, "sel_count_kernel"));
-  sel_index_kernel<<<1, 32, 0, h->stream>>>(n, v, mode, st, cnt, nch);
-  MTO_TRY(mto_after_launch(h, "sel_index_kernel"));
-  MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(out, st + 2, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToDevice, h->stream), "copy"));
-  return MTO_OK;
+  sel_index_kernel<<<grid_for(n, 1024, 256), 256, 0, h->stream>>>(n, v, mode, nt, st, hist + 512, cnt, out0, out1);
+  return mto_after_launch(h, "sel_index_kernel");
 }
 
 }  // namespace
@@ -670,27 +809,20 @@ mto_status map_update(mto_handle h, const double* ga, const double* gd, const do
   const int64_t nel = h->nel;
   const int grd = grid_for(nel, 256, 152 * 4);
   unsigned long long* selbuf = h->sel + 8;         // 8 values: the four (key, index) thresholds
-  long long* kdev = reinterpret_cast<long long*>(h->sel + 24);
   Thresholds T;
   memset(&T, 0, sizeof(T));
   // analysis step: floor(frac * nel) lowest / highest Gamma^a
   const int64_t nc = (int64_t)std::floor(o->frac_a_coarsen * (double)nel);
   const int64_t nr = (int64_t)std::floor(o->frac_a_refine * (double)nel);
-  long long kh[4];
-  if (nc >= nel) T.ac_mode = 1;
-  else if (nc > 0) {
-    T.ac_mode = 2;
-    kh[0] = nc;
-    MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(kdev, &kh[0], sizeof(long long), cudaMemcpyHostToDevice, h->stream), "copy"));
-    MTO_TRY(select_kth(h, ga, nel, 0, kdev, selbuf + 0));
-  }
-  if (nr >= nel) T.ar_mode = 1;
-  else if (nr > 0) {
-    T.ar_mode = 2;
-    kh[1] = nel - nr;
-    MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(kdev + 1, &kh[1], sizeof(long long), cudaMemcpyHostToDevice, h->stream), "copy"));
-    MTO_TRY(select_kth(h, ga, nel, 0, kdev + 1, selbuf + 2));
-  }
+  T.ac_mode = nc >= nel ? 1 : nc > 0 ? 2 : 0;
+  T.ar_mode = nr >= nel ? 1 : nr > 0 ? 2 : 0;
+  if (T.ac_mode == 2 && T.ar_mode == 2)
+    MTO_TRY(select_kth(h, ga, nel, 0, 2, SelRanks{{(unsigned long long)nc, (unsigned long long)(nel - nr)}}, selbuf + 0,
+                       selbuf + 2));
+  else if (T.ac_mode == 2)
+    MTO_TRY(select_kth(h, ga, nel, 0, 1, SelRanks{{(unsigned long long)nc, 0}}, selbuf + 0, nullptr));
+  else if (T.ar_mode == 2)
+    MTO_TRY(select_kth(h, ga, nel, 0, 1, SelRanks{{(unsigned long long)(nel - nr), 0}}, selbuf + 2, nullptr));
   // density step: fractions of the negative / positive Gamma^d elements
   if (o->alpha_d_coarsen >= 1.0) T.dc_mode = 1;
   if (o->alpha_d_refine >= 1.0) T.dr_mode = 1;
@@ -708,9 +840,7 @@ mto_status map_update(mto_handle h, const double* ga, const double* gd, const do
       if (kc >= nneg) T.dc_mode = 1;
       else if (kc > 0) {
         T.dc_mode = 2;
-        kh[2] = kc;
-        MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(kdev + 2, &kh[2], sizeof(long long), cudaMemcpyHostToDevice, h->stream), "copy"));
-        MTO_TRY(select_kth(h, gd, nel, 1, kdev + 2, selbuf + 4));
+        MTO_TRY(select_kth(h, gd, nel, 1, 1, SelRanks{{(unsigned long long)kc, 0}}, selbuf + 4, nullptr));
       }
     }
     if (T.dr_mode == 0) {
@@ -718,9 +848,7 @@ mto_status map_update(mto_handle h, const double* ga, const double* gd, const do
       if (kr >= npos) T.dr_mode = 1;
       else if (kr > 0) {
         T.dr_mode = 2;
-        kh[3] = npos - kr;
-        MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(kdev + 3, &kh[3], sizeof(long long), cudaMemcpyHostToDevice, h->stream), "copy"));
-        MTO_TRY(select_kth(h, gd, nel, 2, kdev + 3, selbuf + 6));
+        MTO_TRY(select_kth(h, gd, nel, 2, 1, SelRanks{{(unsigned long long)(npos - kr), 0}}, selbuf + 6, nullptr));
       }
     }
   }
@@ -754,19 +882,19 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
     cp.gmap[p] = p <= MTO_P_MAX ? h->pc[p].gmap : nullptr;
   }
   // Kelly
-  kelly_edge_kernel<<<grid_for(h->n_edges, 128, 152 * 8), 128, 0, h->stream>>>(
+  kelly_edge_kernel<<<grid_for(h->n_edges, 128, 152 * 64), 128, 0, h->stream>>>(
       h->nelx, h->nely, h->p_d, h->slot_d, cp, h->cons_d, u, B, h->hx, h->hy, h->edge_buf);
   MTO_TRY(mto_after_launch(h, "kelly_edge_kernel"));
   kelly_sum_kernel<<<grid_for(nel, 256), 256, 0, h->stream>>>(h->nelx, h->nely, h->edge_buf, ga_);
   MTO_TRY(mto_after_launch(h, "kelly_sum_kernel"));
   // density indicator
   unsigned long long* mm = h->sel + 16;
-  unsigned long long init[2] = {~0ULL, 0ULL};
-  MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(mm, init, sizeof(init), cudaMemcpyHostToDevice, h->stream), "copy"));
-  minmax_kernel<<<grid_for(h->design_len, 256, 152 * 4), 256, 0, h->stream>>>(h->design_len, rho, mm);
+  MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(mm, 0xff, sizeof(*mm), h->stream), "memset"));
+  MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(mm + 1, 0, sizeof(*mm), h->stream), "memset"));
+  minmax_kernel<<<grid_for(h->design_len, 1024, 152 * 4), 256, 0, h->stream>>>(h->design_len, rho, mm);
   MTO_TRY(mto_after_launch(h, "minmax_kernel"));
-  gamma_d_kernel<<<grid_for(nel, 128), 128, 0, h->stream>>>(nel, h->design_off_d, rho, mm, o->cycle, o->alpha,
-                                                           o->beta, gd_);
+  gamma_d_kernel<<<grid_for(nel, 32 * kGdWarps, 152 * 6), 32 * kGdWarps, 0, h->stream>>>(
+      nel, h->design_off_d, rho, mm, o->cycle, o->alpha, o->beta, gd_);
   MTO_TRY(mto_after_launch(h, "gamma_d_kernel"));
   // QR error per (p, d) class
   for (size_t ci = 0; ci < h->bc.size(); ++ci) {

@@ -329,12 +329,16 @@ mto_status mto_create(mto_handle* out, int device, void* stream) {
     delete h;
     return MTO_ECUDA;
   }
-  if (mto_alloc(h, &h->red, 64) || mto_alloc(h, &h->eng, 128) || mto_alloc(h, &h->flags, 64) || mto_alloc(h, &h->sel, 256) ||
+  if (mto_alloc(h, &h->red, 64) || mto_alloc(h, &h->eng, 128) || mto_alloc(h, &h->flags, 64) || mto_alloc(h, &h->sel, 1024) ||
       mto_alloc(h, &h->cg_res, 64) || mto_alloc(h, &h->cg_cnt, 64) || mto_alloc(h, &h->cg_base, 4)) {
     delete h;
     return MTO_ENOMEM;
   }
   h->base_bytes = h->bytes;
+  if (cudaMemset(h->sel, 0, 1024 * sizeof(unsigned long long)) != cudaSuccess) {   // selection counters
+    delete h;
+    return MTO_ECUDA;
+  }
   if (cudaMallocHost((void**)&h->host_pinned, 64 * sizeof(double)) != cudaSuccess ||
       cudaMallocHost((void**)&h->host_flags, 16 * sizeof(int)) != cudaSuccess) {
     delete h;

@@ -240,7 +240,7 @@ struct mto_handle_s {
   int* flags = nullptr;                        // [0] iterations when done, [1] error code, [2..] misc
   int* host_flags = nullptr;                   // pinned host mirror of flags[0..1]
   double* host_pinned = nullptr;               // pinned host mirror for small read-backs [64]
-  unsigned long long* sel = nullptr;           // selection / small integer scratch [256]
+  unsigned long long* sel = nullptr;           // selection / small integer scratch [1024]
   void* basis_tab = nullptr;                   // GLL / Gauss tables for the indicator kernels
   double* edge_buf = nullptr;                  // [n_edges + nel] Kelly edge terms, then QR scratch
   int64_t n_edges = 0;

@@ -57,3 +57,41 @@ def test_tensor_build_edges(mto, nx, ny, p, d):
         np.testing.assert_array_equal(hi, got.astype(np.float32))
         np.testing.assert_array_equal(lo, (got - hi.astype(np.float64)).astype(np.float32))
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny,d", [(1, 1, 1), (33, 1, 3), (11, 9, 8), (7, 5, 16), (45, 23, 0)])
+def test_density_indicator_and_selection_edges(mto, nx, ny, d):
+    """Gamma^d in cell order is the serial sum: bit-equal to the oracle's cell loop (same operations,
+    same order) apart from a division by a power of two, which is exact; ragged warps, counts from 1 to
+    256 cells, mixed counts (d = 0).  The map update then equals the oracle's on those values and on
+    Kelly values full of ties (the stable index tie-break), for several ranks."""
+    from oracle import indicators as oi
+    rng = np.random.default_rng(nx * 100 + ny)
+    nel = nx * ny
+    dm = rng.choice([1, 2, 3, 8, 16], nel) if d == 0 else np.full(nel, d)
+    p = rng.integers(1, 4, nel)
+    h = handle(mto, nx, ny, p, dm)
+    m = om.DPMesh(nx, ny, p, dm)
+    rho = rng.uniform(0.0, 1.0, h.design_len)
+    rho[rng.uniform(size=len(rho)) < 0.3] = rng.choice([0.0, 0.5, 1.0])
+    r = torch.tensor(rho, device="cuda")
+    mat = mto.material()
+    h.set_supports(h.side_dofs(0))
+    h.build_elements(r, mat)
+    u = torch.tensor(rng.standard_normal(h.ndof), device="cuda")
+    for cycle in (1, 3):
+        ind = h.indicator(u, r, mat, mto.IndicatorOpts.paper(cycle))
+        want = oi.gamma_d(m, rho, cycle)
+        np.testing.assert_allclose(ind["gamma_d"].cpu().numpy(), want, rtol=0, atol=1e-15)
+        np.testing.assert_allclose(ind["gamma_a"].cpu().numpy(), oi.kelly(m, u.cpu().numpy()), rtol=1e-9, atol=0)
+    ga = rng.integers(0, 4, nel).astype(float)          # ties
+    gd = want
+    eq = rng.uniform(0.0, 1.0, nel)
+    for fr, fc in ((0.1, 0.05), (0.5, 0.4), (1.0, 0.0), (0.0, 0.9)):
+        o = mto.IndicatorOpts.paper(1)
+        o.frac_a_refine, o.frac_a_coarsen = fr, fc
+        got = h.map_update(*(torch.tensor(v, device="cuda") for v in (ga, gd, eq)), o)
+        pn, dn, th = oi.map_update(nx, ny, p, ga, gd, eq, frac_a_refine=fr, frac_a_coarsen=fc)[:3]
+        for a, b in zip(got, (pn, dn, th)):
+            np.testing.assert_array_equal(a.cpu().numpy(), b)
+    h.close()
