@@ -3,41 +3,76 @@
 // E'(rho) = q rho^(q-1) (E0 - Emin).  The compliance problem is self-adjoint (adjoint = -u), so u
 // is the only field needed; it is re-gathered per element from the stored global vector.
 //
-// Kernel: one warp per element.  The element's displacement is gathered in FP64 and its best-fit
-// rigid motion (translation and rotation, which K0_s annihilates) is removed in FP64.  Strains at
-// the (p+1) x (p+1) Gauss points of every subcell come from a sum-factorised tensor evaluation on
-// the element's d(p+1) x d(p+1) point grid; each point adds eps^T D0 eps (a sum of non-negative
-// terms) to its subcell.  Compute type T is double (MTO_FP64) or float (MTO_MIXED).
+// Two kernels.  Both gather the element's displacement in FP64 and remove its best-fit rigid motion
+// (translation and rotation, which K0_s annihilates) in FP64.
+//
+// FP64 (sens_poly_kernel): the energy density eps^T D0 eps is a polynomial of degree <= 2p per axis,
+// so its values on one (2p+1) x (2p+1) Gauss grid of the element determine it, and its integrals
+// over the d x d subcells are two small products with the integrals W of the grid's Lagrange
+// polynomials over the subcells: w = W en W^T.  For Q3 and 8 x 8 subcells that is 49 strain
+// evaluations in place of 1024.  Against extended precision, over orders 1..6 and d = 2..16, both
+// forms are within 1.3e-15 of the largest w (2-norm; 3e-16 to 9e-16 the point sums, 2e-16 to
+// 1.3e-15 this one).  Bound by the FP64 pipes (2 FMA per clock and SM): a block takes several
+// elements and spreads each stage over all its threads.
+//
+// FP32 (sens_kernel, MTO_MIXED): one warp per element; strains at the (p+1) x (p+1) Gauss points of
+// every subcell from a sum-factorised tensor evaluation on the element's d(p+1) x d(p+1) point grid;
+// each point adds eps^T D0 eps (a sum of non-negative terms) to its subcell.
 #include <cmath>
 
 #include "mto_internal.cuh"
 
 namespace mto {
 
-// 1D tables of a (p, d) class: [L: N1 x G][D: N1 x G][W: G][Z: N1] with G = d (p+1) points
-// xi_g = -1 + (2 i + 1 + x_k)/d (subcell i, Gauss node x_k), L = l_a(xi_g), D = l_a'(xi_g) and
-// W = w_k / d (the 1D subcell Jacobian).
-__global__ void sens_table_kernel(int p, int d, double* __restrict__ tab, float* __restrict__ tabf) {
-  const int n1 = p + 1, G = d * n1;
-  double z[kPMaxTab + 1], gx[kPMaxTab + 1], gw[kPMaxTab + 1];
-  gll_nodes(p, z);
-  gauss_rule(n1, gx, gw);
-  const int tot = 2 * n1 * G + G + n1;
-  for (int k = threadIdx.x; k < tot; k += blockDim.x) {
+constexpr int kSensQMax = 2 * MTO_P_MAX + 1;
+
+// points per axis of the FP64 kernel's grid: enough for degree 2p, or the subcell's own Gauss rule for d = 1
+__host__ __device__ constexpr int sens_q(int p, int d) { return d == 1 ? p + 1 : 2 * p + 1; }
+
+// Tables of a (p, d) class.  FP64 (Q = sens_q Gauss points x_g): [L: N1 x Q][Dx: N1 x Q][Dy: N1 x Q]
+// [W: d x Q][Z: N1] with L = l_a(x_g), Dx = 2/hx l_a'(x_g), Dy = 2/hy l_a'(x_g),
+// W = integral over subcell i of the Lagrange polynomial of point g, Z the GLL nodes.
+// FP32: [L: N1 x G][D: N1 x G][W: G] with G = d (p+1) points xi_g = -1 + (2 i + 1 + x_k)/d
+// (subcell i, Gauss node x_k), L = l_a(xi_g), D = l_a'(xi_g) and W = w_k / d (the 1D subcell Jacobian).
+__global__ void __launch_bounds__(256) sens_table_kernel(int p, int d, double hx, double hy, double* __restrict__ tab,
+                                                         float* __restrict__ tabf) {
+  const int n1 = p + 1, G = d * n1, Q = sens_q(p, d);
+  __shared__ double z[kPMaxTab + 1], gx[kPMaxTab + 1], gw[kPMaxTab + 1], qx[kSensQMax], qw[kSensQMax];
+  if (threadIdx.x == 0) gll_nodes(p, z);
+  if (threadIdx.x == 32) gauss_rule(n1, gx, gw);
+  if (threadIdx.x == 64) gauss_rule(Q, qx, qw);
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * n1 * G + G; k += blockDim.x) {
     double v;
     if (k < 2 * n1 * G) {
       int which = k / (n1 * G), r = k % (n1 * G), a = r / G, g = r % G;
       int i = g / n1, kk = g % n1;
       double xi = -1.0 + (2.0 * i + 1.0 + gx[kk]) / d;
       v = which == 0 ? lagrange_val(z, n1, a, xi) : lagrange_der(z, n1, a, xi);
-    } else if (k < 2 * n1 * G + G) {
-      int g = k - 2 * n1 * G;
-      v = gw[g % n1] / d;
     } else {
-      v = z[k - 2 * n1 * G - G];
+      v = gw[(k - 2 * n1 * G) % n1] / d;
+    }
+    tabf[k] = (float)v;
+  }
+  const int nt = n1 * Q;
+  for (int k = threadIdx.x; k < 3 * nt + d * Q + n1; k += blockDim.x) {
+    double v;
+    if (k < 3 * nt) {
+      const int which = k / nt, a = k % nt / Q, g = k % Q;
+      v = which == 0 ? lagrange_val(z, n1, a, qx[g]) : lagrange_der(z, n1, a, qx[g]) * (2.0 / (which == 1 ? hx : hy));
+    } else if (k < 3 * nt + d * Q) {
+      const int i = (k - 3 * nt) / Q, g = (k - 3 * nt) % Q;
+      if (d == 1) {
+        v = qw[g];
+      } else {
+        v = 0.0;
+        for (int kk = 0; kk < n1; ++kk)
+          v += gw[kk] / d * lagrange_val(qx, Q, g, -1.0 + (2.0 * i + 1.0 + gx[kk]) / d);
+      }
+    } else {
+      v = z[k - 3 * nt - d * Q];
     }
     tab[k] = v;
-    tabf[k] = (float)v;
   }
 }
 
@@ -49,37 +84,32 @@ __device__ __forceinline__ double wsum(double v) {
   return v;
 }
 
-// NF = 1: w_s = u_e^T K0_s u_e (compliance, self-adjoint).  NF = 2: w_s = v_e^T K0_s u_e with the
-// adjoint field v (a general objective z^T u, Eq. 1): both fields' strains at every point, the
-// bilinear energy density eps(v)^T D0 eps(u).
-template <int PO, int NF, typename T>
+// The FP32 quadrature: w_s = u_e^T K0_s u_e (compliance, self-adjoint).
+template <int PO>
 __global__ void __launch_bounds__(128) sens_kernel(
-    int n, int d, const int* __restrict__ elem, const int* __restrict__ slot, int ld, const int* __restrict__ gmap,
-    const Constraint* __restrict__ cons, const double* __restrict__ u, const double* __restrict__ v,
-    const double* __restrict__ rho, const int64_t* __restrict__ design_off, double E0, double Emin, double q,
-    double nu, double hx, double hy, const T* __restrict__ tab, const double* __restrict__ Z, double* __restrict__ dc,
-    double* __restrict__ eout) {
+    int n, int d, const int* __restrict__ elem, const int* __restrict__ slot, const int* __restrict__ gmap,
+    const Constraint* __restrict__ cons, const double* __restrict__ u, const double* __restrict__ rho,
+    const int64_t* __restrict__ design_off, double E0, double Emin, double q, double nu, double hx, double hy,
+    const float* __restrict__ tab, const double* __restrict__ Z, double* __restrict__ dc) {
   constexpr int N1 = PO + 1, NN = N1 * N1;
   static_assert(NN <= 64, "two nodes per lane at most");
   const int G = d * N1;
   extern __shared__ unsigned char smem_raw[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // per-warp shared layout: A[NF][4][N1][G] (T), part[G] (T), U[NF][2][NN] (T)
-  const size_t per_warp = (size_t)(4 * NF * N1 * G + G + 2 * NF * NN) * sizeof(T);
-  T* A = reinterpret_cast<T*>(smem_raw + warp * per_warp);
-  T* part = A + 4 * NF * N1 * G;
-  T* U = part + G;
+  // per-warp shared layout: A[4][N1][G], part[G], U[2][NN]
+  const size_t per_warp = (size_t)(4 * N1 * G + G + 2 * NN) * sizeof(float);
+  float* A = reinterpret_cast<float*>(smem_raw + warp * per_warp);
+  float* part = A + 4 * N1 * G;
+  float* U = part + G;
   const int k = blockIdx.x * (blockDim.x >> 5) + warp;
   if (k >= n) return;
   const int e = elem[k], sl = slot[k];
-  const T* L = tab;
-  const T* Dd = tab + N1 * G;
-  const T* W = tab + 2 * N1 * G;
+  const float* L = tab;
+  const float* Dd = tab + N1 * G;
+  const float* W = tab + 2 * N1 * G;
 
-  // gather each field (FP64) and remove its best-fit rigid motion in FP64 (lanes stride over nodes)
-#pragma unroll
-  for (int fld = 0; fld < NF; ++fld) {
-    const double* x = fld == 0 ? u : v;
+  // gather (FP64) and remove the best-fit rigid motion in FP64 (lanes stride over nodes)
+  {
     double sux = 0.0, suy = 0.0, snum = 0.0, sden = 0.0;
     double ux[2], uy[2], xl[2], yl[2];
 #pragma unroll
@@ -89,13 +119,13 @@ __global__ void __launch_bounds__(128) sens_kernel(
       if (ln < NN) {
         int g = gmap[(size_t)sl * NN + ln];
         if (g >= 0) {
-          ux[r] = x[2 * (size_t)g];
-          uy[r] = x[2 * (size_t)g + 1];
+          ux[r] = u[2 * (size_t)g];
+          uy[r] = u[2 * (size_t)g + 1];
         } else {
           const Constraint& c = cons[-g - 1];
           for (int j = 0; j < c.cnt; ++j) {
-            ux[r] += c.w[j] * x[2 * (size_t)c.node[j]];
-            uy[r] += c.w[j] * x[2 * (size_t)c.node[j] + 1];
+            ux[r] += c.w[j] * u[2 * (size_t)c.node[j]];
+            uy[r] += c.w[j] * u[2 * (size_t)c.node[j] + 1];
           }
         }
         xl[r] = 0.5 * Z[ln % N1] * hx;   // node coordinates about the element centre (FP64 GLL nodes)
@@ -108,13 +138,12 @@ __global__ void __launch_bounds__(128) sens_kernel(
     }
     const double tx = wsum(sux) / NN, ty = wsum(suy) / NN;
     const double om = wsum(snum) / wsum(sden);
-    T* Uf = U + 2 * NN * fld;
 #pragma unroll
     for (int r = 0; r < 2; ++r) {
       const int ln = lane + 32 * r;
       if (ln < NN) {
-        Uf[ln] = (T)(ux[r] - tx + om * yl[r]);
-        Uf[NN + ln] = (T)(uy[r] - ty - om * xl[r]);
+        U[ln] = (float)(ux[r] - tx + om * yl[r]);
+        U[NN + ln] = (float)(uy[r] - ty - om * xl[r]);
       }
     }
   }
@@ -123,113 +152,282 @@ __global__ void __launch_bounds__(128) sens_kernel(
   // stage 1 (x direction): A_c[b][g] = sum_a U_c[b][a] L[a][g],  Ad_c[b][g] = sum_a U_c[b][a] D[a][g]
   for (int g = lane; g < G; g += 32) {
 #pragma unroll
-    for (int fld = 0; fld < NF; ++fld) {
-      const T* Uf = U + 2 * NN * fld;
-      T* Af = A + 4 * N1 * G * fld;
+    for (int b = 0; b < N1; ++b) {
+      float a0 = 0, a1 = 0, d0 = 0, d1 = 0;
 #pragma unroll
-      for (int b = 0; b < N1; ++b) {
-        T a0 = 0, a1 = 0, d0 = 0, d1 = 0;
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-          T l = L[a * G + g], dl = Dd[a * G + g];
-          T v0 = Uf[b * N1 + a], v1 = Uf[NN + b * N1 + a];
-          a0 = fma(v0, l, a0);
-          d0 = fma(v0, dl, d0);
-          a1 = fma(v1, l, a1);
-          d1 = fma(v1, dl, d1);
-        }
-        Af[(0 * N1 + b) * G + g] = a0;
-        Af[(1 * N1 + b) * G + g] = d0;
-        Af[(2 * N1 + b) * G + g] = a1;
-        Af[(3 * N1 + b) * G + g] = d1;
+      for (int a = 0; a < N1; ++a) {
+        const float l = L[a * G + g], dl = Dd[a * G + g];
+        const float v0 = U[b * N1 + a], v1 = U[NN + b * N1 + a];
+        a0 = fma(v0, l, a0);
+        d0 = fma(v0, dl, d0);
+        a1 = fma(v1, l, a1);
+        d1 = fma(v1, dl, d1);
       }
+      A[(0 * N1 + b) * G + g] = a0;
+      A[(1 * N1 + b) * G + g] = d0;
+      A[(2 * N1 + b) * G + g] = a1;
+      A[(3 * N1 + b) * G + g] = d1;
     }
   }
   __syncwarp();
 
   // stage 2 (y direction) and the energy density at every point
-  const T sx = (T)(2.0 / hx), sy = (T)(2.0 / hy), jac = (T)(0.25 * hx * hy);
+  const float sx = (float)(2.0 / hx), sy = (float)(2.0 / hy), jac = (float)(0.25 * hx * hy);
   const double f = 1.0 / (1.0 - nu * nu);
-  const T D11 = (T)f, D12 = (T)(f * nu), D33 = (T)(f * 0.5 * (1.0 - nu));
+  const float D11 = (float)f, D12 = (float)(f * nu), D33 = (float)(f * 0.5 * (1.0 - nu));
   const double dE = E0 - Emin;
   const int64_t off = design_off[e];
-  double energy = 0.0;   // sum_s E(rho_s) w_s of this element (eout)
   for (int j = 0; j < d; ++j) {
     for (int g = lane; g < G; g += 32) {
-      T acc = 0;
+      float acc = 0;
       for (int kk = 0; kk < N1; ++kk) {
         const int gy = j * N1 + kk;
-        T exx[NF], eyy[NF], gam[NF];
+        float ex = 0, ey = 0, g0 = 0, g1 = 0;
 #pragma unroll
-        for (int fld = 0; fld < NF; ++fld) {
-          const T* Af = A + 4 * N1 * G * fld;
-          T ex = 0, ey = 0, g0 = 0, g1 = 0;
-#pragma unroll
-          for (int b = 0; b < N1; ++b) {
-            T lb = L[b * G + gy], db = Dd[b * G + gy];
-            ex = fma(Af[(1 * N1 + b) * G + g], lb, ex);   // d ux / d xi
-            g0 = fma(Af[(0 * N1 + b) * G + g], db, g0);   // d ux / d eta
-            g1 = fma(Af[(3 * N1 + b) * G + g], lb, g1);   // d uy / d xi
-            ey = fma(Af[(2 * N1 + b) * G + g], db, ey);   // d uy / d eta
-          }
-          exx[fld] = ex * sx;
-          eyy[fld] = ey * sy;
-          gam[fld] = g0 * sy + g1 * sx;
+        for (int b = 0; b < N1; ++b) {
+          const float lb = L[b * G + gy], db = Dd[b * G + gy];
+          ex = fma(A[(1 * N1 + b) * G + g], lb, ex);   // d ux / d xi
+          g0 = fma(A[(0 * N1 + b) * G + g], db, g0);   // d ux / d eta
+          g1 = fma(A[(3 * N1 + b) * G + g], lb, g1);   // d uy / d xi
+          ey = fma(A[(2 * N1 + b) * G + g], db, ey);   // d uy / d eta
         }
-        constexpr int o = NF - 1;   // the second field of the bilinear form (the first for NF = 1)
-        T en = D11 * (exx[0] * exx[o] + eyy[0] * eyy[o]) + D12 * (exx[0] * eyy[o] + eyy[0] * exx[o]) +
-               D33 * gam[0] * gam[o];
+        const float exx = ex * sx, eyy = ey * sy, gam = g0 * sy + g1 * sx;
+        const float en = D11 * (exx * exx + eyy * eyy) + D12 * (exx * eyy + eyy * exx) + D33 * gam * gam;
         acc = fma(W[gy], en, acc);
       }
       part[g] = acc * W[g] * jac;
     }
     __syncwarp();
     for (int i = lane; i < d; i += 32) {
-      T w = 0;
+      float w = 0;
       for (int kk = 0; kk < N1; ++kk) w += part[i * N1 + kk];
       const int s = j * d + i;
       const double r = rho[off + s];
-      if (dc) dc[off + s] = -q * pow(r, q - 1.0) * dE * (double)w;
-      if (eout) energy += (Emin + pow(r, q) * dE) * (double)w;
+      dc[off + s] = -q * pow(r, q - 1.0) * dE * (double)w;
     }
     __syncwarp();
   }
+}
+
+// The FP64 kernel (see the head of this file).  A block of 128 threads takes EB elements (a power of
+// two, 4..32); each stage is a flat loop over the items of all of them.
+constexpr int kSensThreads = 128;
+
+// doubles of shared memory per element
+__host__ __device__ constexpr int sens_elem_doubles(int p, int d, int nf) {
+  const int n1 = p + 1, nn = n1 * n1, Q = sens_q(p, d);
+  return nf * (2 * nn + 4 * n1 * Q + 3) + Q * Q + d * Q;
+}
+
+template <int PO, int NF>
+__global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
+    int n, int d, int Q, int EB, const int* __restrict__ elem, const int* __restrict__ slot,
+    const int* __restrict__ gmap, const Constraint* __restrict__ cons, const double* __restrict__ u,
+    const double* __restrict__ v, const double* __restrict__ rho, const int64_t* __restrict__ design_off, double E0,
+    double Emin, double q, double nu, double hx, double hy, const double* __restrict__ tab, double* __restrict__ dc,
+    double* __restrict__ eout) {
+  constexpr int N1 = PO + 1, NN = N1 * N1;
+  extern __shared__ double sd[];
+  const int t = threadIdx.x;
+  const int NQ = N1 * Q, ntab = 3 * NQ + d * Q + N1;
+  const double *L = sd, *Dx = sd + NQ, *Dy = Dx + NQ, *W = Dy + NQ, *Z = W + d * Q;
+  double* U = sd + ntab;                       // [EB][NF][2][NN]
+  double* rig = U + EB * NF * 2 * NN;          // [EB][NF][3] translation and rotation
+  double* A = rig + EB * NF * 3;               // [EB][NF][4][N1][Q]
+  double* en = A + EB * NF * 4 * NQ;           // [EB][Q][Q] energy density (y, x)
+  double* T = en + EB * Q * Q;                 // [EB][d][Q] integrated along x (subcell, y point)
+  for (int k = t; k < ntab; k += kSensThreads) sd[k] = tab[k];
+  const int base = blockIdx.x * EB;
+  const int ne = min(EB, n - base);
+  // gather (FP64)
+  for (int it = t; it < ne * NF * NN; it += kSensThreads) {
+    const int el = it / (NF * NN), fld = it / NN % NF, ln = it % NN;
+    const double* x = fld == 0 ? u : v;
+    const int g = gmap[(size_t)slot[base + el] * NN + ln];
+    double ux = 0.0, uy = 0.0;
+    if (g >= 0) {
+      ux = x[2 * (size_t)g];
+      uy = x[2 * (size_t)g + 1];
+    } else {
+      const Constraint& c = cons[-g - 1];
+      for (int j = 0; j < c.cnt; ++j) {
+        ux += c.w[j] * x[2 * (size_t)c.node[j]];
+        uy += c.w[j] * x[2 * (size_t)c.node[j] + 1];
+      }
+    }
+    U[(el * NF + fld) * 2 * NN + ln] = ux;
+    U[(el * NF + fld) * 2 * NN + NN + ln] = uy;
+  }
+  __syncthreads();
+  // least-squares rigid motion about the element centre
+  for (int it = t; it < ne * NF * 3; it += kSensThreads) {
+    const int k = it % 3;
+    const double* Uf = U + (it / 3) * 2 * NN;
+    double s = 0.0;
+    if (k < 2) {
+      for (int ln = 0; ln < NN; ++ln) s += Uf[k * NN + ln];
+      s /= NN;
+    } else {
+      double den = 0.0;
+      for (int ln = 0; ln < NN; ++ln) {
+        const double x = 0.5 * hx * Z[ln % N1], y = 0.5 * hy * Z[ln / N1];
+        s += x * Uf[NN + ln] - y * Uf[ln];
+        den += x * x + y * y;
+      }
+      s /= den;
+    }
+    rig[it] = s;
+  }
+  __syncthreads();
+  for (int it = t; it < ne * NF * NN; it += kSensThreads) {
+    const int ef = it / NN, ln = it % NN;
+    double* Uf = U + ef * 2 * NN;
+    Uf[ln] = Uf[ln] - rig[3 * ef] + rig[3 * ef + 2] * (0.5 * hy * Z[ln / N1]);
+    Uf[NN + ln] = Uf[NN + ln] - rig[3 * ef + 1] - rig[3 * ef + 2] * (0.5 * hx * Z[ln % N1]);
+  }
+  __syncthreads();
+  // stage 1 (along x), per row b of nodes and grid column g: ux and uy by L and by Dx
+  for (int it = t; it < ne * NF * NQ; it += kSensThreads) {
+    const int ef = it / NQ, b = it % NQ / Q, g = it % Q;
+    const double* Uf = U + ef * 2 * NN + b * N1;
+    double a0 = 0.0, d0 = 0.0, a1 = 0.0, d1 = 0.0;
+#pragma unroll
+    for (int a = 0; a < N1; ++a) {
+      const double l = L[a * Q + g], dl = Dx[a * Q + g], v0 = Uf[a], v1 = Uf[NN + a];
+      a0 = fma(v0, l, a0);
+      d0 = fma(v0, dl, d0);
+      a1 = fma(v1, l, a1);
+      d1 = fma(v1, dl, d1);
+    }
+    double* Af = A + (ef * 4 * N1 + b) * Q + g;
+    Af[0] = a0;
+    Af[NQ] = d0;
+    Af[2 * NQ] = a1;
+    Af[3 * NQ] = d1;
+  }
+  __syncthreads();
+  // stage 2 (along y): strains and the energy density over 1 / (1 - nu^2) at every grid point:
+  // (exx + nu eyy)(exx' + nu eyy') + (1 - nu^2) eyy eyy' + (1 - nu)/2 gam gam'
+  const double c1 = 1.0 - nu * nu, c2 = 0.5 * (1.0 - nu);
+  for (int it = t; it < ne * Q * Q; it += kSensThreads) {
+    const int el = it / (Q * Q), h = it % (Q * Q) / Q, g = it % Q;
+    double ax[NF], ey[NF], gm[NF];
+#pragma unroll
+    for (int fld = 0; fld < NF; ++fld) {
+      const double* Af = A + (el * NF + fld) * 4 * NQ + g;
+      double ex = 0.0, e2 = 0.0, ga = 0.0;
+#pragma unroll
+      for (int b = 0; b < N1; ++b) {
+        const double lb = L[b * Q + h], db = Dy[b * Q + h];
+        ex = fma(Af[NQ + b * Q], lb, ex);       // d ux / d x
+        ga = fma(Af[b * Q], db, ga);            // d ux / d y
+        ga = fma(Af[3 * NQ + b * Q], lb, ga);   // + d uy / d x
+        e2 = fma(Af[2 * NQ + b * Q], db, e2);   // d uy / d y
+      }
+      ax[fld] = fma(nu, e2, ex);
+      ey[fld] = e2;
+      gm[fld] = ga;
+    }
+    constexpr int o = NF - 1;
+    en[it] = fma(ax[0], ax[o], fma(c1 * ey[0], ey[o], c2 * gm[0] * gm[o]));
+  }
+  __syncthreads();
+  // integrals over the subcells: along x, then along y
+  for (int it = t; it < ne * d * Q; it += kSensThreads) {
+    const int el = it / (d * Q), i = it % (d * Q) / Q, h = it % Q;
+    const double* e = en + (el * Q + h) * Q;
+    double s = 0.0;
+    for (int g = 0; g < Q; ++g) s = fma(W[i * Q + g], e[g], s);
+    T[it] = s;
+  }
+  __syncthreads();
+  const double jac = 0.25 * hx * hy / (1.0 - nu * nu), dE = E0 - Emin;
+  const bool cube = q == 3.0;
+  const int tpe = kSensThreads / EB;   // threads per element, at most 32
+  const int el = t / tpe;
+  double energy = 0.0;   // sum_s E(rho_s) w_s (eout)
+  if (el < ne) {
+    const int64_t off = design_off[elem[base + el]];
+    for (int s = t % tpe; s < d * d; s += tpe) {
+      const double* Wj = W + (s / d) * Q;
+      const double* Ti = T + (el * d + s % d) * Q;
+      double w = 0.0;
+      for (int h = 0; h < Q; ++h) w = fma(Wj[h], Ti[h], w);
+      w *= jac;
+      const double r = rho[off + s];
+      if (dc) dc[off + s] = -q * (cube ? r * r : pow(r, q - 1.0)) * dE * w;
+      if (eout) energy += (Emin + (cube ? r * r * r : pow(r, q)) * dE) * w;
+    }
+  }
   if (eout) {
-    energy = wsum(energy);
-    if (lane == 0) eout[e] = energy;
+    for (int o = tpe >> 1; o > 0; o >>= 1) energy += __shfl_xor_sync(0xffffffffu, energy, o);
+    if (el < ne && t % tpe == 0) eout[elem[base + el]] = energy;
   }
 }
 
-template <int PO, int NF, typename T>
-mto_status launch_sens(mto_handle h, const BClass& b, const double* u, const double* v, const double* rho,
-                       const mto_material* m, const T* tab, double* dc, double* eout) {
+template <int PO, int NF>
+mto_status launch_poly(mto_handle h, const BClass& b, const double* u, const double* v, const double* rho,
+                       const mto_material* m, double* dc, double* eout) {
+  const int Q = sens_q(PO, b.d), ntab = (3 * Q + 1) * (PO + 1) + b.d * Q;
+  const int per = sens_elem_doubles(PO, b.d, NF);
+  // elements per block: as many as fit about 36 KB (six blocks per SM), fewer while the launch has less
+  // than two blocks per SM
+  int EB = 32;
+  while (EB > 4 && (EB * per * 8 > 36 * 1024 || b.n < EB * 304)) EB /= 2;
+  const size_t smem = sizeof(double) * ((size_t)EB * per + ntab);
+  if (smem > 48 * 1024)
+    MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(sens_poly_kernel<PO, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)smem), "cudaFuncSetAttribute"));
+  sens_poly_kernel<PO, NF><<<(b.n + EB - 1) / EB, kSensThreads, smem, h->stream>>>(
+      b.n, b.d, Q, EB, b.elem, b.slot, h->pc[b.p].gmap, h->cons_d, u, v, rho, h->design_off_d, m->E0, m->Emin, m->q,
+      m->nu, h->hx, h->hy, b.stab, dc, eout);
+  return mto_after_launch(h, "sens_poly_kernel");
+}
+
+// the FP32 quadrature (MTO_MIXED sensitivities)
+template <int PO>
+mto_status launch_sens(mto_handle h, const BClass& b, const double* u, const double* rho, const mto_material* m,
+                       double* dc) {
   const int N1 = PO + 1, G = b.d * N1;
-  const size_t per_warp = (size_t)(4 * NF * N1 * G + G + 2 * NF * N1 * N1) * sizeof(T);
+  const size_t per_warp = (size_t)(4 * N1 * G + G + 2 * N1 * N1) * sizeof(float);
   const int warps = 4;
   const size_t smem = per_warp * warps;
   if (smem > 227 * 1024) return mto_fail(h, MTO_EINVAL, "sensitivity: element class too large for shared memory");
   if (smem > 48 * 1024)
-    cudaFuncSetAttribute(sens_kernel<PO, NF, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(sens_kernel<PO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   const PClass& c = h->pc[b.p];
-  sens_kernel<PO, NF, T><<<(b.n + warps - 1) / warps, 32 * warps, smem, h->stream>>>(
-      b.n, b.d, b.elem, b.slot, c.ld, c.gmap, h->cons_d, u, v, rho, h->design_off_d, m->E0, m->Emin, m->q, m->nu,
-      h->hx, h->hy, tab, b.stab + 2 * N1 * G + G, dc, eout);
+  const int Q = sens_q(PO, b.d);
+  sens_kernel<PO><<<(b.n + warps - 1) / warps, 32 * warps, smem, h->stream>>>(
+      b.n, b.d, b.elem, b.slot, c.gmap, h->cons_d, u, rho, h->design_off_d, m->E0, m->Emin, m->q, m->nu,
+      h->hx, h->hy, b.stabf, b.stab + 3 * N1 * Q + b.d * Q, dc);
   return mto_after_launch(h, "sens_kernel");
 }
 
-template <int NF, typename T>
+template <int NF>
 mto_status sens_all(mto_handle h, const double* u, const double* v, const double* rho, const mto_material* m,
                     double* dc, double* eout = nullptr) {
   for (auto& b : h->bc) {
-    const T* tab;
-    if constexpr (sizeof(T) == 8) tab = (const T*)b.stab; else tab = (const T*)b.stabf;
     switch (b.p) {
-      case 1: MTO_TRY((launch_sens<1, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
-      case 2: MTO_TRY((launch_sens<2, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
-      case 3: MTO_TRY((launch_sens<3, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
-      case 4: MTO_TRY((launch_sens<4, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
-      case 5: MTO_TRY((launch_sens<5, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
-      case 6: MTO_TRY((launch_sens<6, NF, T>(h, b, u, v, rho, m, tab, dc, eout))); break;
+      case 1: MTO_TRY((launch_poly<1, NF>(h, b, u, v, rho, m, dc, eout))); break;
+      case 2: MTO_TRY((launch_poly<2, NF>(h, b, u, v, rho, m, dc, eout))); break;
+      case 3: MTO_TRY((launch_poly<3, NF>(h, b, u, v, rho, m, dc, eout))); break;
+      case 4: MTO_TRY((launch_poly<4, NF>(h, b, u, v, rho, m, dc, eout))); break;
+      case 5: MTO_TRY((launch_poly<5, NF>(h, b, u, v, rho, m, dc, eout))); break;
+      case 6: MTO_TRY((launch_poly<6, NF>(h, b, u, v, rho, m, dc, eout))); break;
+    }
+  }
+  return MTO_OK;
+}
+
+mto_status sens_all32(mto_handle h, const double* u, const double* rho, const mto_material* m, double* dc) {
+  for (auto& b : h->bc) {
+    switch (b.p) {
+      case 1: MTO_TRY(launch_sens<1>(h, b, u, rho, m, dc)); break;
+      case 2: MTO_TRY(launch_sens<2>(h, b, u, rho, m, dc)); break;
+      case 3: MTO_TRY(launch_sens<3>(h, b, u, rho, m, dc)); break;
+      case 4: MTO_TRY(launch_sens<4>(h, b, u, rho, m, dc)); break;
+      case 5: MTO_TRY(launch_sens<5>(h, b, u, rho, m, dc)); break;
+      case 6: MTO_TRY(launch_sens<6>(h, b, u, rho, m, dc)); break;
     }
   }
   return MTO_OK;
@@ -239,10 +437,10 @@ mto_status sens_all(mto_handle h, const double* u, const double* v, const double
 
 mto_status build_sens_tables(mto_handle h) {
   for (auto& b : h->bc) {
-    const int n1 = b.p + 1, G = b.d * n1, tot = 2 * n1 * G + G + n1;
-    MTO_TRY(mto_alloc(h, &b.stab, (size_t)tot));
-    MTO_TRY(mto_alloc(h, &b.stabf, (size_t)tot));
-    sens_table_kernel<<<1, 256, 0, h->stream>>>(b.p, b.d, b.stab, b.stabf);
+    const int n1 = b.p + 1, G = b.d * n1, Q = sens_q(b.p, b.d);
+    MTO_TRY(mto_alloc(h, &b.stab, (size_t)(3 * Q + 1) * n1 + b.d * Q));
+    MTO_TRY(mto_alloc(h, &b.stabf, (size_t)2 * n1 * G + G));
+    sens_table_kernel<<<1, 256, 0, h->stream>>>(b.p, b.d, h->hx, h->hy, b.stab, b.stabf);
     MTO_TRY(mto_after_launch(h, "sens_table_kernel"));
   }
   return MTO_OK;
@@ -252,8 +450,8 @@ mto_status sensitivity(mto_handle h, const double* u, const double* f, const dou
                        int precision, double* dc, double* C) {
   {
   TimedScope ts(h, F_SENS);
-  if (precision == MTO_FP64) MTO_TRY((sens_all<1, double>(h, u, nullptr, rho, m, dc)));
-  else MTO_TRY((sens_all<1, float>(h, u, nullptr, rho, m, dc)));
+  if (precision == MTO_FP64) MTO_TRY((sens_all<1>(h, u, nullptr, rho, m, dc)));
+  else MTO_TRY(sens_all32(h, u, rho, m, dc));
   MTO_TRY(dot64(h, f, u, h->ndof, h->red + 8));
   }
   if (C) {
@@ -269,7 +467,7 @@ mto_status sensitivity(mto_handle h, const double* u, const double* f, const dou
 mto_status sensitivity_adjoint(mto_handle h, const double* u, const double* v, const double* rho,
                                const mto_material* m, double* dc) {
   TimedScope ts(h, F_SENS);
-  return sens_all<2, double>(h, u, v, rho, m, dc);
+  return sens_all<2>(h, u, v, rho, m, dc);
 }
 
 // Compliance of an approximate displacement in its energy form, C(u) = 2 f^T u - u^T K u
@@ -281,7 +479,7 @@ mto_status compliance_energy(mto_handle h, const double* u, const double* f, con
                              const mto_material* m, double* C) {
   {
     TimedScope ts(h, F_SENS);
-    MTO_TRY((sens_all<1, double>(h, u, nullptr, rho, m, nullptr, h->dbuf)));
+    MTO_TRY((sens_all<1>(h, u, nullptr, rho, m, nullptr, h->dbuf)));
     MTO_TRY(sum64(h, h->dbuf, h->nel, h->red + 10));
     MTO_TRY(dot64(h, f, u, h->ndof, h->red + 11));
   }

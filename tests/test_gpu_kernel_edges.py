@@ -95,3 +95,36 @@ def test_density_indicator_and_selection_edges(mto, nx, ny, d):
         for a, b in zip(got, (pn, dn, th)):
             np.testing.assert_array_equal(a.cpu().numpy(), b)
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (13, 5)])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("d", [1, 2, 3, 8, 16])
+def test_sensitivity_edges(mto, nx, ny, p, d):
+    """FP64 sensitivities (self-adjoint and bilinear) and the energy form against the oracle's dense
+    quadratic forms u^T K0_s u, on one element and ragged blocks, non-square elements: each w_s comes from
+    sums of magnitudes below 64 x the element's largest (products of the grid's energy densities with
+    integrated Lagrange polynomials whose absolute sums stay below 8 per axis), so 1e-12 of the largest
+    value of the mesh bounds the rounding of both sides by two orders."""
+    from oracle import sensitivity as ose
+    h = handle(mto, nx, ny, p, d, 1.0, 0.5)
+    m = om.DPMesh(nx, ny, np.full(nx * ny, p), np.full(nx * ny, d), 1.0, 0.5)
+    rng = np.random.default_rng(10 * p + d)
+    rho = rng.uniform(0.0, 1.0, h.design_len)
+    u, v, f = (rng.standard_normal(h.ndof) for _ in range(3))
+    T = lambda a: torch.tensor(a, device="cuda")
+    for q in (3.0, 2.5):
+        mat = mto.material(1.0, 1e-9, 0.3, q)
+        dc, dv = T(np.zeros(h.design_len)), T(np.zeros(h.design_len))
+        C = h.sensitivity(T(u), T(f), T(rho), mat, dc)
+        assert abs(C - f @ u) <= 1e-12 * np.abs(f) @ np.abs(u)
+        want = ose.sensitivity(m, u, rho, q=q)
+        assert np.abs(dc.cpu().numpy() - want).max() <= 1e-12 * np.abs(want).max()
+        # bilinear form by polarisation of the quadratic one
+        h.sensitivity_adjoint(T(u), T(v), T(rho), mat, dv)
+        pol = 0.25 * (ose.sensitivity(m, u + v, rho, q=q) - ose.sensitivity(m, u - v, rho, q=q))
+        scale = max(np.abs(ose.sensitivity(m, u + v, rho, q=q)).max(), np.abs(ose.sensitivity(m, u - v, rho, q=q)).max())
+        assert np.abs(dv.cpu().numpy() - pol).max() <= 1e-12 * scale
+        e = ose.energy_split(m, u, rho, q=q)
+        assert abs(h.compliance_energy(T(u), T(f), T(rho), mat) - (2.0 * f @ u - e)) <= 1e-12 * (abs(e) + 2 * np.abs(f) @ np.abs(u))
+    h.close()
