@@ -203,6 +203,8 @@ void release_mesh(mto_handle h) {
   free_dev(h, h->spring_k_d);
   h->n_springs = 0;
   free_dev(h, h->filt_W);
+  free_dev(h, h->filt_H);
+  free_dev(h, h->filt_ext);
   free_dev(h, h->oc_t);
   h->bytes = h->base_bytes;
 }

@@ -177,7 +177,9 @@ struct mto_handle_s {
   int* slot_d = nullptr;                       // [nel] slot of each element within its order class
   int64_t* fixed_d = nullptr;                  // [n_fixed] supported DOFs
   int64_t n_fixed = 0;
-  double* filt_W = nullptr;                    // [design_len] density-filter weight sums (adjoint)
+  double* filt_W = nullptr;                    // [design_len] density filter: x / W of the adjoint
+  double* filt_H = nullptr;                    // its weight tables per design count, and
+  int* filt_ext = nullptr;                     // their row extents
   double* oc_t = nullptr;                      // [4][design_len] OC: rho_j B_j^eta and the area-scaled T, L, H
   int64_t* spring_dof_d = nullptr;             // [n_springs] DOFs with a spring to ground (K + k e e^T)
   double* spring_k_d = nullptr;                // [n_springs] their stiffness

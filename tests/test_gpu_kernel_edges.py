@@ -128,3 +128,34 @@ def test_sensitivity_edges(mto, nx, ny, p, d):
         e = ose.energy_split(m, u, rho, q=q)
         assert abs(h.compliance_energy(T(u), T(f), T(rho), mat) - (2.0 * f @ u - e)) <= 1e-12 * (abs(e) + 2 * np.abs(f) @ np.abs(u))
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (12, 7), (3, 11)])
+@pytest.mark.parametrize("d", [1, 3, 5, 8, 16, 0, -1])   # 0, -1: mixed counts (two maps)
+@pytest.mark.parametrize("R,hy", [(0.05, 1.0), (0.3, 1.0), (1.0, 0.5), (1.9, 0.5), (4.0, 1.0)])
+def test_filter_edges(mto, nx, ny, d, R, hy):
+    """The filter's fine-grid stencil (one design count) and its mixed path against the oracle's sparse
+    rows: stencils inside, across and wider than the mesh, non-square elements, radii from below one
+    subcell to the largest of four elements.  The oracle's subcell centres are rounded at up to 12
+    elements (12 x 2^-53), a distance to 8 of those units, a weight of mean R / 3 to 24 / R of them: 4e-14 /
+    min(R, 1) covers both sides' rounding with the sums."""
+    from oracle import filter as ofl
+    if R > 4.0 * min(1.0, hy) or (R > 2.0 and nx > 3 and d in (16, -1)):   # the latter: 10^8 pairs in the oracle
+        R = 2.0
+    rng = np.random.default_rng(3 + nx)
+    nel = nx * ny
+    dm = np.full(nel, d) if d > 0 else rng.choice([1, 2, 4, 8] if d == 0 else [1, 3, 7, 16], nel)
+    h = handle(mto, nx, ny, 1, dm, 1.0, hy)
+    m = om.DPMesh(nx, ny, np.full(nel, 1), dm, 1.0, hy)
+    x, g = rng.uniform(size=m.design_len), rng.standard_normal(m.design_len)
+    xt, gt = torch.tensor(x, device="cuda"), torch.tensor(g, device="cuda")
+    out = torch.empty_like(xt)
+    tol = 4e-14 / min(R, 1.0)
+    for _ in range(2):
+        h.filter(xt, out, R)
+        want = ofl.density_filter(m, x, R)
+        assert np.abs(out.cpu().numpy() - want).max() <= tol * np.abs(want).max()
+        h.filter_adjoint(gt, out, R)
+        want = ofl.density_filter_adjoint(m, g, R)
+        assert np.abs(out.cpu().numpy() - want).max() <= tol * np.abs(want).max()
+    h.close()
