@@ -1447,13 +1447,6 @@ mto_status apply_block32(mto_handle h, const float* x, float* y, const int* done
   return apply_all<float>(h, 1, x, y, -1, done, none, nullptr, true);
 }
 
-mto_status apply_q1(mto_handle h, const MGLevel& l, const double* x, double* y, const int* done) {
-  ConvTest none{};
-  ebe_kernel<1, false, double><<<ebe_blocks_p<1>(l.nel), 256, 0, h->stream>>>(
-      l.K, nullptr, nullptr, 40, l.nel, l.gmap, nullptr, x, y, Red{nullptr, nullptr, nullptr}, done, none);
-  return mto_after_launch(h, "ebe_kernel");
-}
-
 __global__ void __launch_bounds__(256) vsum_kernel(int64_t n, const double* __restrict__ a, double* __restrict__ part) {
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) s += a[i];

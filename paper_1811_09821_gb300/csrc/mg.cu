@@ -339,61 +339,340 @@ __global__ void mg_invd_kernel(int64_t n, const double* __restrict__ mask, doubl
   }
 }
 
-// coarsest level: dense assembly, supported rows/columns replaced by identity, in-place
-// Gauss-Jordan inversion (SPD: no pivoting) in one block
-__global__ void mg_dense_assemble_kernel(int nel, int N, const int* __restrict__ gmap, const double* __restrict__ K,
-                                         double* __restrict__ A) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nel) return;
-  for (int i = 0; i < 8; ++i) {
-    const int gi = 2 * gmap[4 * e + (i >> 1)] + (i & 1);
-    for (int j = 0; j < 8; ++j) {
-      const int gj = 2 * gmap[4 * e + (j >> 1)] + (j & 1);
-      atomicAdd(A + (size_t)gi * N + gj, K[(size_t)e * 40 + circ_pos(i, j, 8)]);
+// ---------------------------------------------------------------- coarsest level: dense inverse
+// The coarsest operator couples neighbouring vertices only, so with the DOFs ordered by grid lines
+// across the shorter side (m <= 64 DOFs a line, nl lines) it is block tridiagonal with blocks D_l and
+// couplings of six entries a row.  Its inverse X comes from one block elimination from both ends to
+// the middle line k (par(l): the next line towards k, C_l = A_{l, par(l)}):
+//   chains   S_l = D_l - C^T S^-1 C of the line before, G_l = S_l^-1: two blocks, one for each side
+//            (N / 2 pivots one after the other), and the middle line from both;
+//   columns  of one line c: y_par = -C^T G y from c to k, x_k = G_k y_k, and back
+//            x_l = G_l y_l - G_l C_l x_par; every column on its own.  The rows on the way from c to k and,
+//            for the lines before k, those beyond k: every pair of lines once, mirrored.
+// One factorisation serves every block: on designs with nearly loose pieces (contrast 1e9) the
+// softest pivots carry few digits, and blocks from two different eliminations (a diagonal from
+// S_l + S'_l - D_l, say) no longer fit together to a positive definite matrix.
+// About N^2 m FMAs in three launches; the Gauss-Jordan steps over the dense matrix that this replaces,
+// N launches of N^2 FMAs, took 35.7 ms for N = 1722 (40 x 20), 14.1 ms for N = 1122 (32 x 16) and
+// 3.1 ms for N = 462 (20 x 10).  Supported DOFs have identity rows and columns.
+constexpr int kLineMax = 64;      // 2 (min(nx, ny) + 1) <= 64 for at most 2048 DOFs
+constexpr int kInvWarps = 8;      // warps holding the matrix of an inversion, two more form the multipliers
+constexpr int kInvThreads = 32 * (kInvWarps + 2);
+constexpr int kInvEntries = (kLineMax * (kLineMax + 1) / 2 + 32 * kInvWarps - 1) / (32 * kInvWarps);
+
+struct StripGeom {
+  int nx, ny;    // elements of the level
+  int along_x;   // lines run along y and follow one another along x (else the other way round)
+  int m, nl;
+  __host__ __device__ int vertex(int line, int pos) const {
+    return along_x ? pos * (nx + 1) + line : line * (nx + 1) + pos;
+  }
+};
+
+// 1 / d of a positive double: Newton's iteration x <- x + x (1 - d x) on the mantissa, from its FP32
+// reciprocal (2^-23, squared twice)
+__device__ __forceinline__ double newton_rcp(double d) {
+  const long long b = __double_as_longlong(d);
+  const int be = (int)(b >> 52);
+  if (be < 8 || be > 2038) return 1.0 / d;
+  const double md = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
+  double r = (double)(1.0f / __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff)));
+  r = fma(r, fma(-md, r, 1.0), r);
+  r = fma(r, fma(-md, r, 1.0), r);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)(be - 1023) << 52));
+}
+
+// In-place symmetric inversion (Gauss-Jordan sweeps, SPD: no pivoting) of an m x m matrix held as its
+// packed lower triangle over the threads of kInvWarps warps: entry e of thread t is (ij[e] >> 8,
+// ij[e] & 255), ij < 0 beyond the end.  On return a = -inverse.  While those warps apply a pivot to
+// the matrix, two helper warps already form the reciprocal and the multipliers of the next one.
+// cb, ub: [2][kLineMax] shared.  Returns false (in every thread) at a pivot that is not positive.
+__device__ bool sym_invert(int m, double (&a)[kInvEntries], const int (&ij)[kInvEntries], double (*cb)[kLineMax],
+                           double (*ub)[kLineMax], double* inv) {
+  const int t = threadIdx.x;
+  const bool helper = t >= 32 * kInvWarps;
+  const int ht = t - 32 * kInvWarps;
+  bool ok = true;
+  auto publish = [&](int k) {   // column k of the current matrix
+#pragma unroll
+    for (int e = 0; e < kInvEntries; ++e) {
+      if (ij[e] < 0) continue;
+      const int i = ij[e] >> 8, j = ij[e] & 255;
+      if (j == k) cb[k & 1][i] = a[e];
+      else if (i == k) cb[k & 1][j] = a[e];
     }
+  };
+  auto multipliers = [&](int k) {
+    const double d = cb[k & 1][k];
+    const double r = newton_rcp(d);
+    if (ht == 0) inv[k & 1] = r;
+    if (ht < m) ub[k & 1][ht] = cb[k & 1][ht] * r;
+  };
+  if (!helper) publish(0);
+  __syncthreads();
+  if (helper) multipliers(0);
+  __syncthreads();
+  for (int k = 0; k < m; ++k) {
+    const double* c = cb[k & 1];
+    const double* u = ub[k & 1];
+    ok = ok && c[k] > 0.0;
+    auto update = [&](int e, int i, int j) {
+      if (j == k) a[e] = i == k ? -inv[k & 1] : u[i];
+      else if (i == k) a[e] = u[j];
+      else a[e] = fma(-u[i], c[j], a[e]);
+    };
+    if (!helper && k + 1 < m) {   // the next pivot's column first
+#pragma unroll
+      for (int e = 0; e < kInvEntries; ++e) {
+        if (ij[e] < 0) continue;
+        const int i = ij[e] >> 8, j = ij[e] & 255;
+        if (i == k + 1 || j == k + 1) {
+          update(e, i, j);
+          cb[(k + 1) & 1][j == k + 1 ? i : j] = a[e];
+        }
+      }
+    }
+    __syncthreads();
+    if (helper) {
+      if (k + 1 < m) multipliers(k + 1);
+    } else {
+#pragma unroll
+      for (int e = 0; e < kInvEntries; ++e) {
+        if (ij[e] < 0) continue;
+        const int i = ij[e] >> 8, j = ij[e] & 255;
+        if (k + 1 >= m || (i != k + 1 && j != k + 1)) update(e, i, j);
+      }
+    }
+    __syncthreads();
+  }
+  return ok;
+}
+
+__device__ void packed_owner(int m, int (&ij)[kInvEntries]) {
+  const int t = threadIdx.x;
+#pragma unroll
+  for (int e = 0; e < kInvEntries; ++e) {
+    const int idx = t + 32 * kInvWarps * e;
+    ij[e] = -1;
+    if (t >= 32 * kInvWarps || idx >= m * (m + 1) / 2) continue;
+    int i = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
+    while (i * (i + 1) / 2 > idx) --i;
+    while ((i + 1) * (i + 2) / 2 <= idx) ++i;
+    ij[e] = i << 8 | (idx - i * (i + 1) / 2);
   }
 }
 
-__global__ void mg_dense_fix_kernel(int N, const double* __restrict__ mask, double* __restrict__ A) {
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)N * N;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t / N), j = (int)(t % N);
-    if (mask[i] == 0.0 || mask[j] == 0.0) A[t] = (i == j) ? 1.0 : 0.0;
+// entry (pos a, comp ca) x (pos b, comp cb) of the coupling between `line` and `line + step`
+// (step 0: within the line) with the supported DOFs' rows and columns replaced by the identity's
+__device__ __forceinline__ double strip_entry(const StripGeom& g, const double* __restrict__ S,
+                                              const double* __restrict__ mask, int line, int step, int i, int j) {
+  const int a = i >> 1, b = j >> 1, dp = b - a;
+  if (dp < -1 || dp > 1) return 0.0;
+  const int64_t v = g.vertex(line, a), w = g.vertex(line + step, b), nv = (int64_t)(g.nx + 1) * (g.ny + 1);
+  if (mask[2 * v + (i & 1)] == 0.0 || mask[2 * w + (j & 1)] == 0.0) return (step == 0 && i == j) ? 1.0 : 0.0;
+  const int o = g.along_x ? 3 * (dp + 1) + step + 1 : 3 * (step + 1) + dp + 1;
+  return S[(o * 4 + 2 * (i & 1) + (j & 1)) * nv + v];
+}
+
+// The elimination.  middle = 0: block 0 the lines 0 .. k - 1, block 1 the lines nl - 1 .. k + 1;
+// middle = 1: the line k.  The inverse of line l's Schur complement goes to Gc + l m^2 (full).
+__global__ void __launch_bounds__(kInvThreads) mg_strip_chain_kernel(StripGeom g, int middle,
+                                                                     const double* __restrict__ S,
+                                                                     const double* __restrict__ mask, double* Gc,
+                                                                     int* __restrict__ err) {
+  extern __shared__ double shm[];
+  const int m = g.m, ld = m + 1, t = threadIdx.x, kmid = g.nl / 2;
+  double* G = shm;               // [m][ld] inverse of the line before
+  double* F = G + m * ld;        // [m][ld] C^T G
+  double* E = F + m * ld;        // [m][6] C^T: this line's rows
+  __shared__ double cb[2][kLineMax], ub[2][kLineMax], inv[2];
+  double a[kInvEntries];
+  int ij[kInvEntries];
+  packed_owner(m, ij);
+  bool ok = true;
+  // a -= C^T G C for the line l + step, whose inverse is in G
+  auto subtract = [&](int l, int step) {
+    for (int k = t; k < 6 * m; k += kInvThreads) {
+      const int i = k / 6, j = 2 * (i >> 1) - 2 + k % 6;   // the DOFs of positions a - 1 .. a + 1
+      E[k] = (j >= 0 && j < m) ? strip_entry(g, S, mask, l, step, i, j) : 0.0;
+    }
+    __syncthreads();
+    for (int k = t; k < m * m; k += kInvThreads) {
+      const int i = k / m, j = k % m, j0 = 2 * (i >> 1) - 2;
+      double f = 0.0;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const int r = j0 + c;
+        if (r >= 0 && r < m) f = fma(E[6 * i + c], G[r * ld + j], f);
+      }
+      F[i * ld + j] = f;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < kInvEntries; ++e) {
+      if (ij[e] < 0) continue;
+      const int i = ij[e] >> 8, j = ij[e] & 255, j0 = 2 * (j >> 1) - 2;
+#pragma unroll
+      for (int c = 0; c < 6; ++c) {
+        const int r = j0 + c;
+        if (r >= 0 && r < m) a[e] = fma(-F[i * ld + r], E[6 * j + c], a[e]);
+      }
+    }
+    __syncthreads();
+  };
+  const int dir = blockIdx.x == 0 ? 1 : -1;
+  const int n = middle ? 1 : (dir > 0 ? kmid : g.nl - 1 - kmid);
+  for (int s = 0; s < n; ++s) {
+    const int l = middle ? kmid : (dir > 0 ? s : g.nl - 1 - s);
+#pragma unroll
+    for (int e = 0; e < kInvEntries; ++e) a[e] = ij[e] < 0 ? 0.0 : strip_entry(g, S, mask, l, 0, ij[e] >> 8, ij[e] & 255);
+    if (middle) {
+      for (int step = -1; step <= 1; step += 2) {
+        if (l + step < 0 || l + step >= g.nl) continue;
+        const double* src = Gc + (size_t)(l + step) * m * m;
+        for (int k = t; k < m * m; k += kInvThreads) G[k / m * ld + k % m] = src[k];
+        subtract(l, step);
+      }
+    } else if (s > 0) {
+      subtract(l, -dir);
+    }
+    ok = sym_invert(m, a, ij, cb, ub, inv) && ok;
+#pragma unroll
+    for (int e = 0; e < kInvEntries; ++e) {
+      if (ij[e] < 0) continue;
+      const int i = ij[e] >> 8, j = ij[e] & 255;
+      G[i * ld + j] = G[j * ld + i] = -a[e];
+      Gc[(size_t)l * m * m + i * m + j] = -a[e];
+      Gc[(size_t)l * m * m + j * m + i] = -a[e];
+    }
+    __syncthreads();
+  }
+  if (!ok && t == 0) *err = MTO_ENAN;
+}
+
+// the columns of the inverse, a few of one line per block (the longest ways, from the first lines, first)
+constexpr int kStripCols = 4;
+constexpr int kStripThreads = 192;
+__global__ void __launch_bounds__(kStripThreads) mg_strip_columns_kernel(StripGeom g, const double* __restrict__ S,
+                                                                         const double* __restrict__ mask,
+                                                                         const double* __restrict__ Gc,
+                                                                         double* __restrict__ X) {
+  extern __shared__ double shm[];
+  const int m = g.m, t = threadIdx.x, kmid = g.nl / 2;
+  const size_t N = (size_t)m * g.nl;
+  double* Y = shm;                    // [m][kStripCols]
+  double* T = Y + m * kStripCols;     // [m][kStripCols]
+  double* E = T + m * kStripCols;     // [m][6]
+  const int per = (m + kStripCols - 1) / kStripCols;
+  const int c = blockIdx.x / per, q0 = blockIdx.x % per * kStripCols;
+  const int nq = min(kStripCols, m - q0);
+  const size_t col0 = (size_t)c * m + q0;
+  // E = the couplings of line l's rows to line l + step
+  auto coupling = [&](int l, int step) {
+    for (int k = t; k < 6 * m; k += kStripThreads) {
+      const int r = k / 6, j = 2 * (r >> 1) - 2 + k % 6;
+      E[k] = (j >= 0 && j < m) ? strip_entry(g, S, mask, l, step, r, j) : 0.0;
+    }
+  };
+  // dst = sgn E src (sparse)
+  auto sparse = [&](double* dst, const double* src, double sgn) {
+    for (int k = t; k < m * kStripCols; k += kStripThreads) {
+      const int r = k / kStripCols, q = k % kStripCols, j0 = 2 * (r >> 1) - 2;
+      double v = 0.0;
+#pragma unroll
+      for (int cc = 0; cc < 6; ++cc) {
+        const int j = j0 + cc;
+        if (j >= 0 && j < m) v = fma(E[6 * r + cc], src[j * kStripCols + q], v);
+      }
+      dst[k] = sgn * v;
+    }
+  };
+  // dst = G_l src (+ X's rows of line l where add), and written to those rows (mirrored where final)
+  auto dense = [&](int l, double* dst, const double* src, bool add, bool final) {
+    const double* G = Gc + (size_t)l * m * m;
+    for (int k = t; k < m * kStripCols; k += kStripThreads) {
+      const int r = k / kStripCols, q = k % kStripCols;
+      double v0 = 0.0, v1 = 0.0;
+#pragma unroll 4
+      for (int j = 0; j < m; j += 2) {   // m is even; G symmetric
+        v0 = fma(G[(size_t)j * m + r], src[j * kStripCols + q], v0);
+        v1 = fma(G[(size_t)(j + 1) * m + r], src[(j + 1) * kStripCols + q], v1);
+      }
+      double v = v0 + v1;
+      if (q < nq) {
+        const size_t gi = (size_t)l * m + r, gj = col0 + q;
+        if (add) v += X[gi * N + gj];
+        X[gi * N + gj] = v;
+        if (final && l != c) X[gj * N + gi] = v;
+      }
+      dst[k] = v;
+    }
+  };
+  const int dir = c < kmid ? 1 : -1;   // towards the middle
+  for (int k = t; k < m * kStripCols; k += kStripThreads) Y[k] = (k / kStripCols == q0 + k % kStripCols) ? 1.0 : 0.0;
+  __syncthreads();
+  // z_l = G_l y_l kept in X's rows of line l, y_par = -C_l^T z_l
+  for (int l = c; l != kmid; l += dir) {
+    dense(l, T, Y, false, false);
+    coupling(l + dir, -dir);
+    __syncthreads();
+    sparse(Y, T, -1.0);
+    __syncthreads();
+  }
+  dense(kmid, T, Y, false, true);
+  __syncthreads();
+  for (int k = t; k < m * kStripCols; k += kStripThreads) Y[k] = T[k];   // x_k
+  // back to c: x_l = z_l - G_l C_l x_par
+  for (int l = kmid - dir; dir > 0 ? l >= c : l <= c; l -= dir) {
+    coupling(l, dir);
+    __syncthreads();
+    sparse(E + 6 * m, T, -1.0);
+    __syncthreads();
+    dense(l, T, E + 6 * m, true, true);
+    __syncthreads();
+  }
+  if (c >= kmid) return;
+  // the lines beyond the middle: x_l = -G_l C_l x_par
+  for (int l = kmid + 1; l < g.nl; ++l) {
+    coupling(l, -1);
+    __syncthreads();
+    sparse(T, Y, -1.0);
+    __syncthreads();
+    dense(l, Y, T, false, true);
+    __syncthreads();
   }
 }
 
-// One Gauss-Jordan step of the in-place inversion (SPD: no pivoting), from buffer A into B so that
-// every entry is computed from the previous step's values; N launches invert the matrix.
-__global__ void __launch_bounds__(256) mg_gj_step_kernel(int N, int k, const double* __restrict__ A,
-                                                         double* __restrict__ B, int* __restrict__ err) {
-  const double piv = A[(size_t)k * N + k];
-  if (!(piv > 0.0)) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) *err = MTO_ENAN;
-  }
-  const double inv = 1.0 / piv;
-  for (int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; t < (int64_t)N * N;
-       t += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(t / N), j = (int)(t - (int64_t)i * N);
-    double v;
-    if (i == k) v = (j == k) ? inv : A[(size_t)k * N + j] * inv;
-    else if (j == k) v = -A[(size_t)i * N + k] * inv;
-    else v = fma(-A[(size_t)i * N + k] * inv, A[(size_t)k * N + j], A[t]);
-    B[t] = v;
-  }
-}
-
-// x = Ainv b (one warp per row; FP64 inverse and sums, vectors of the cycle's type)
+// x = Ainv b (one warp per row of the line order; FP64 inverse and sums, vectors of the cycle's type)
 template <typename V>
-__global__ void __launch_bounds__(256) mg_coarse_solve_kernel(int N, const double* __restrict__ Ainv,
+__global__ void __launch_bounds__(256) mg_coarse_solve_kernel(StripGeom g, const double* __restrict__ Ainv,
                                                               const V* __restrict__ b, V* __restrict__ x,
                                                               const int* __restrict__ done) {
   if (done && *done) return;
+  extern __shared__ double bs[];   // b in line order
+  const int N = g.m * g.nl;
+  for (int j = threadIdx.x; j < N; j += blockDim.x) {
+    const int line = j / g.m, i = j - line * g.m;
+    bs[j] = (double)b[2 * g.vertex(line, i >> 1) + (i & 1)];
+  }
+  __syncthreads();
   const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, l = threadIdx.x & 31;
   if (w >= N) return;
-  double s = 0.0;
-  for (int j = l; j < N; j += 32) s = fma(Ainv[(size_t)w * N + j], (double)b[j], s);
-  s = warp_sum(s);
-  if (l == 0) x[w] = (V)s;
+  const double* row = Ainv + (size_t)w * N;
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+  int j = l;
+  for (; j + 96 < N; j += 128) {
+    s0 = fma(row[j], bs[j], s0);
+    s1 = fma(row[j + 32], bs[j + 32], s1);
+    s2 = fma(row[j + 64], bs[j + 64], s2);
+    s3 = fma(row[j + 96], bs[j + 96], s3);
+  }
+  for (; j < N; j += 32) s0 = fma(row[j], bs[j], s0);
+  const double s = warp_sum((s0 + s1) + (s2 + s3));
+  if (l == 0) {
+    const int line = w / g.m, i = w - line * g.m;
+    x[2 * g.vertex(line, i >> 1) + (i & 1)] = (V)s;
+  }
 }
 
 // ---------------------------------------------------------------- smoothing and transfers
@@ -669,6 +948,16 @@ __global__ void mg_cheb_coef_kernel(int nlev, const double* __restrict__ lmax, d
 
 int vec_grid(int64_t n) { return grid_for(n, 256, kMGBlocks); }
 
+StripGeom strip_geom(const MGLevel& L) {
+  StripGeom g;
+  g.nx = L.nx;
+  g.ny = L.ny;
+  g.along_x = L.nx >= L.ny;
+  g.m = 2 * (std::min(L.nx, L.ny) + 1);
+  g.nl = std::max(L.nx, L.ny) + 1;
+  return g;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------- host side
@@ -688,7 +977,7 @@ void mg_release(mto_handle h) {
   h->mg_pidx = nullptr;
   h->mg_pw = h->mg_rw = h->mg_btab = h->mg_v0 = h->mg_q0 = h->mg_d0 = h->mg_Ainv = h->mg_lmax = nullptr;
   h->mg_f32 = nullptr;
-  h->mg_Awork = h->mg_Acur = nullptr;
+  h->mg_Awork = nullptr;
   h->mg_coef = nullptr;
   h->mg_part = h->mg_res = nullptr;
   h->mg_rptr = h->mg_rnode = nullptr;
@@ -732,10 +1021,8 @@ mto_status mg_setup(mto_handle h) {
     MTO_TRY(mto_alloc(h, &L.gmap, gm.size()));
     MTO_TRY(mto_cuda_check(h, cudaMemcpy(L.gmap, gm.data(), gm.size() * sizeof(int), cudaMemcpyHostToDevice), "upload"));
     MTO_TRY(mto_alloc(h, &L.K, (size_t)40 * L.nel));
-    if (l + 1 < dims.size()) {   // smoothed levels
-      MTO_TRY(mto_alloc(h, &L.S, (size_t)36 * L.nv));
-      MTO_TRY(mto_alloc(h, &L.S32, (size_t)36 * L.nv));
-    }
+    MTO_TRY(mto_alloc(h, &L.S, (size_t)36 * L.nv));
+    MTO_TRY(mto_alloc(h, &L.S32, (size_t)36 * L.nv));
     for (double** v : {&L.mask, &L.invd, &L.x, &L.xa, &L.b, &L.q, &L.d}) MTO_TRY(mto_alloc(h, v, L.n));
     for (float** v : {&L.invd32, &L.mask32}) MTO_TRY(mto_alloc(h, v, L.n));
     MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(L.q, 0, L.n * sizeof(double), h->stream), "memset"));
@@ -817,7 +1104,8 @@ mto_status mg_setup(mto_handle h) {
   MTO_TRY(mto_alloc(h, &h->mg_f32, (size_t)6 * h->ndof));
   MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->mg_q0, 0, h->ndof * sizeof(double), h->stream), "memset"));
   MTO_TRY(mto_alloc(h, &h->mg_Ainv, (size_t)ncoarse * ncoarse));
-  MTO_TRY(mto_alloc(h, &h->mg_Awork, (size_t)ncoarse * ncoarse));
+  const StripGeom sg = strip_geom(h->mg.back());
+  MTO_TRY(mto_alloc(h, &h->mg_Awork, (size_t)ncoarse * sg.m));   // the lines' inverses
   MTO_TRY(mto_alloc(h, &h->mg_lmax, h->mg.size() + 1));
   MTO_TRY(mto_alloc(h, &h->mg_coef, (h->mg.size() + 1) * kMaxDegree));
   MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->mg_lmax, 0, (h->mg.size() + 1) * sizeof(double), h->stream), "memset"));
@@ -859,11 +1147,10 @@ mto_status mg_set_masks(mto_handle h) {
 
 namespace {
 
-// y = A x on Q1 level l (written, not accumulated): the vertex stencil where it exists, in FP32
+// y = A x on Q1 level l (written, not accumulated) by the vertex stencil, in FP32
 // when the cycle runs on FP32 copies (FP32 vectors in the cycle, FP64 ones in the power
-// iteration), else in FP64; the coarsest level (no stencil) by its element matrices
+// iteration), else in FP64
 mto_status mg_level_apply(mto_handle h, const MGLevel& l, const double* x, double* y, const int* done) {
-  if (!l.S) return apply_q1(h, l, x, y, done);
   if (mg_fp32_cycle(h))
     mg_stencil_apply_kernel<float, double><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S32, x, y, done);
   else
@@ -871,7 +1158,6 @@ mto_status mg_level_apply(mto_handle h, const MGLevel& l, const double* x, doubl
   return mto_after_launch(h, "mg_stencil_apply_kernel");
 }
 mto_status mg_level_apply(mto_handle h, const MGLevel& l, const float* x, float* y, const int* done) {
-  if (!l.S32) return mto_fail(h, MTO_EINVAL, "mg: no stencil on this level");
   mg_stencil_apply_kernel<float, float><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S32, x, y, done);
   return mto_after_launch(h, "mg_stencil_apply_kernel");
 }
@@ -987,10 +1273,8 @@ mto_status mg_build(mto_handle h) {
     MTO_TRY(mto_after_launch(h, "mg_galerkin_h_kernel"));
   }
   for (auto& L : h->mg) {
-    if (L.S) {
-      mg_stencil_kernel<<<vec_grid(L.nv), 256, 0, h->stream>>>(L.nx, L.ny, L.K, L.S, L.S32);
-      MTO_TRY(mto_after_launch(h, "mg_stencil_kernel"));
-    }
+    mg_stencil_kernel<<<vec_grid(L.nv), 256, 0, h->stream>>>(L.nx, L.ny, L.K, L.S, L.S32);
+    MTO_TRY(mto_after_launch(h, "mg_stencil_kernel"));
     MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(L.invd, 0, L.n * sizeof(double), h->stream), "memset"));
     mg_diag_kernel<<<(L.nel + 127) / 128, 128, 0, h->stream>>>(L.nel, L.gmap, L.K, L.invd);
     MTO_TRY(mto_after_launch(h, "mg_diag_kernel"));
@@ -999,22 +1283,23 @@ mto_status mg_build(mto_handle h) {
     MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(L.q, 0, L.n * sizeof(double), h->stream), "memset"));
   }
   // coarsest: dense inverse
-  const MGLevel& C = h->mg.back();
-  const int N = (int)C.n;
-  MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->mg_Ainv, 0, sizeof(double) * N * N, h->stream), "memset"));
-  mg_dense_assemble_kernel<<<(C.nel + 127) / 128, 128, 0, h->stream>>>(C.nel, N, C.gmap, C.K, h->mg_Ainv);
-  MTO_TRY(mto_after_launch(h, "mg_dense_assemble_kernel"));
-  mg_dense_fix_kernel<<<vec_grid((int64_t)N * N), 256, 0, h->stream>>>(N, C.mask, h->mg_Ainv);
-  MTO_TRY(mto_after_launch(h, "mg_dense_fix_kernel"));
-  MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->flags + 6, 0, sizeof(int), h->stream), "memset"));
   {
-    double* bufs[2] = {h->mg_Ainv, h->mg_Awork};
-    const int grd = vec_grid((int64_t)N * N);
-    for (int k = 0; k < N; ++k) {
-      mg_gj_step_kernel<<<grd, 256, 0, h->stream>>>(N, k, bufs[k & 1], bufs[(k + 1) & 1], h->flags + 6);
-      MTO_TRY(mto_after_launch(h, "mg_gj_step_kernel"));
+    const MGLevel& C = h->mg.back();
+    const StripGeom g = strip_geom(C);
+    double* Gc = h->mg_Awork;
+    MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->flags + 6, 0, sizeof(int), h->stream), "memset"));
+    const size_t smem = sizeof(double) * (2 * g.m * (g.m + 1) + 6 * g.m);
+    if (smem > 48 * 1024)
+      MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(mg_strip_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                     (int)smem), "cudaFuncSetAttribute"));
+    for (int middle = 0; middle < 2; ++middle) {
+      mg_strip_chain_kernel<<<middle ? 1 : 2, kInvThreads, smem, h->stream>>>(g, middle, C.S, C.mask, Gc, h->flags + 6);
+      MTO_TRY(mto_after_launch(h, "mg_strip_chain_kernel"));
     }
-    h->mg_Acur = bufs[N & 1];
+    const int per = (g.m + kStripCols - 1) / kStripCols;
+    mg_strip_columns_kernel<<<g.nl * per, kStripThreads, sizeof(double) * g.m * (3 * kStripCols + 6), h->stream>>>(
+        g, C.S, C.mask, Gc, h->mg_Ainv);
+    MTO_TRY(mto_after_launch(h, "mg_strip_columns_kernel"));
   }
   }
   // element-block smoothing of the fine level: the blocks (K_e + Delta_e)^-1 of the element-block
@@ -1162,8 +1447,8 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, const
     TimedScope ts(h, F_PRECOND);
     const MGLevel& C = h->mg.back();
     const LevelV<V> cv = level_vecs<V>(C);
-    mg_coarse_solve_kernel<V><<<(int)((C.n * 32 + 255) / 256), 256, 0, h->stream>>>((int)C.n, h->mg_Acur, cv.b,
-                                                                                      cv.x, done);
+    mg_coarse_solve_kernel<V><<<(int)((C.n * 32 + 255) / 256), 256, sizeof(double) * C.n, h->stream>>>(
+        strip_geom(C), h->mg_Ainv, cv.b, cv.x, done);
     MTO_TRY(mto_after_launch(h, "mg_coarse_solve_kernel"));
   }
   // up

@@ -219,9 +219,8 @@ struct mto_handle_s {
   double* mg_btab = nullptr;                   // bilinear weights at the GLL nodes, per order
   int mg_boff[mto::kPMaxTab + 2] = {0};
   double *mg_v0 = nullptr, *mg_q0 = nullptr, *mg_d0 = nullptr;   // [ndof] fine-level scratch
-  double* mg_Ainv = nullptr;                   // coarsest level: two [N][N] buffers of the
-  double* mg_Awork = nullptr;                  // Gauss-Jordan steps ...
-  double* mg_Acur = nullptr;                   // ... and the one holding the inverse
+  double* mg_Ainv = nullptr;                   // coarsest level: its inverse [N][N] in line order,
+  double* mg_Awork = nullptr;                  // and the blocks of its elimination
   double* mg_lmax = nullptr;                   // [levels] Chebyshev upper bounds
   double2* mg_coef = nullptr;                  // [levels][16] Chebyshev step coefficients (c1, c2)
   double* mg_part = nullptr;                   // reduction partials
@@ -461,7 +460,6 @@ mto_status apply_block(mto_handle h, const double* x, double* y, const int* done
 // the same on FP32 vectors with the leading part (the FP32 multigrid cycle)
 mto_status apply_fine32(mto_handle h, const float* x, float* y, const int* done);
 mto_status apply_block32(mto_handle h, const float* x, float* y, const int* done);
-mto_status apply_q1(mto_handle h, const MGLevel& l, const double* x, double* y, const int* done);
 mto_status solve(mto_handle h, const double* f, double* u, const mto_solve_opts* o, int32_t* iters,
                  double* relres);
 mto_status solve_batched(mto_handle* hs, int n, const double* const* f, double* const* u, const mto_solve_opts* o,

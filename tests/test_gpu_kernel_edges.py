@@ -159,3 +159,34 @@ def test_filter_edges(mto, nx, ny, d, R, hy):
         want = ofl.density_filter_adjoint(m, g, R)
         assert np.abs(out.cpu().numpy() - want).max() <= tol * np.abs(want).max()
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (1, 9), (9, 1), (2, 1), (31, 31), (500, 1), (3, 200), (5, 4), (40, 23)])
+def test_coarsest_inverse_edges(mto, nx, ny):
+    """On a Q1 mesh of at most 2048 vertex DOFs the coarsest level is the operator itself, so a V-cycle
+    with its exact inverse solves the system and the FP64 PCG takes a few iterations (the FP32 cycle's
+    vectors are not checked here: they leave kappa 2^-24 a cycle).  The solution is checked by
+    its backward error, which does not depend on the conditioning (a slender cantilever's error in u is
+    kappa eps on either side, kappa ~ 1e11 for 500 x 1): every free row's residual with the oracle's K within
+    the asked 1e-11 of |f| and 64 eps of that row of |K||u| (18 products and the rounding of K and u).  Lines
+    along either axis, one element, two lines, 64 DOFs a line, supported DOFs."""
+    from oracle import solve as osv
+    rng = np.random.default_rng(nx + 7 * ny)
+    h = handle(mto, nx, ny, 1, 2)
+    m = om.DPMesh(nx, ny, np.full(nx * ny, 1), np.full(nx * ny, 2))
+    rho = rng.uniform(0.1, 1.0, h.design_len)
+    fixed, f = mto.load_case(h, "cantilever")
+    h.set_supports(fixed)
+    K = osv.assemble(m, osv.element_matrices(m, rho, 1.0, 1e-9, 0.3, 3.0))
+    free = np.setdiff1d(np.arange(h.ndof), fixed)
+    fn = f.cpu().numpy()
+    h.build_elements(torch.tensor(rho, device="cuda"), mto.material(), mto.MTO_FP64)
+    u = torch.zeros(h.ndof, dtype=torch.float64, device="cuda")
+    it, _ = h.solve(f, u, precision=mto.MTO_FP64, rtol=1e-11, precond=mto.PREC_MG, check_every=2, max_iter=200,
+                    max_outer=4, raise_on_noconv=False)
+    assert it <= 8, it
+    un = u.cpu().numpy()
+    assert np.all(un[fixed] == 0.0)
+    r = np.abs(fn - K @ un)[free]
+    assert np.all(r <= 1e-11 * np.linalg.norm(fn) + 64 * 2.0 ** -52 * (abs(K) @ np.abs(un))[free]), r.max()
+    h.close()
