@@ -453,6 +453,12 @@ mto_status build_tables(mto_handle h) {
     MTO_TRY(mto_alloc(h, &q.R, (size_t)(p + 2) * (p + 2) * (p + 1) * (p + 1)));
     qr_table_kernel<<<1, 64, 0, h->stream>>>(p, h->hx, h->hy, q.R);
     MTO_TRY(mto_after_launch(h, "qr_table_kernel"));
+    const int n1 = 2 * (p + 2) * (p + 2);
+    std::vector<int> pos(qr_row_len(p + 1), -1);
+    for (int i = 0; i < n1; ++i)
+      for (int j = 0; j <= i; ++j) pos[i * (i + 1) / 2 + j] = packed_index(n1, j, i);
+    MTO_TRY(mto_alloc(h, &q.pos, pos.size()));
+    MTO_TRY(mto_cuda_check(h, cudaMemcpy(q.pos, pos.data(), pos.size() * sizeof(int), cudaMemcpyHostToDevice), "upload"));
   }
   return MTO_OK;
 }

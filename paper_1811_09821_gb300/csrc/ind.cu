@@ -1,6 +1,7 @@
 // Step (d): the composite refinement indicator and the dp map update (Sec. 3.2, 3.3), and the
 // optimality-criteria design update.  All FP64: the integer maps must match the oracle exactly,
 // so every floating-point decision is taken in double with a fixed reduction order.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -273,42 +274,66 @@ __global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
 }
 
 // ------------------------------------------------------------------------------------ QR error
-// One warp per element of a (p, d) class (Eq. 14).  Shared layout (doubles): A[P1] (the order p+1
+// One warp per element of a (p, d) class (Eq. 14).  Shared layout (doubles): A[L1] (the order p+1
 // matrix, lower triangle packed by rows, A_ij at i (i + 1) / 2 + j, factorised in place as
-// L D L^T), f[n0], f1[n1], u1[n1], E[S], ue[n0], rd[n1] (reciprocal pivots), cl[n1] (the pivot
-// column before scaling), pr[3 n1] (the pinned rows of the unmodified matrix), with
-// n0 = 2 (p+1)^2, n1 = 2 (p+2)^2, P1 = n1 (n1 + 1) / 2.  The footprint sets how many elements an
-// SM works on at once, and the kernel is bound by GB300's FP64 pipes, so it keeps one triangle.
+// L D L^T), f[n0], f1[n1], u1[n1], ue[n0], rd[n1] (reciprocal pivots), cl[n1] (the pivot
+// column before scaling), pr[3 n1] (the pinned rows of the unmodified matrix) and, without rows, E[S],
+// with n0 = 2 (p+1)^2, n1 = 2 (p+2)^2, L1 = n1 (n1 + 1) / 2 rounded up.
+// K^(p+1) = sum_s E_s K0_s comes as rows formed on the tensor cores (tc_rows, d <= 8), or is summed
+// here from the table (rows null).  The kernel is bound by the FP64 pipes (2 FMA per clock and SM),
+// where those sums were 81.6 k of 115 k FMAs of a Q3/d8 element (170.5 ms on the 1024 x 512 beam).
+// Indicators of a 320 x 160 adaptive mesh with the sums here 10.9 ms, with rows 6.9 ms.
 // eps is invariant to rigid motions of u^(p), which are removed first (FP64) so that the element
 // energies carry no cancellation.
-__global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* __restrict__ elem,
-                                                const int* __restrict__ slot, int L, const int2* __restrict__ dpos,
-                                                const int* __restrict__ gmap,
+
+// 1 / d: Newton's iteration x <- x + x (1 - d x) on the mantissa from its FP32 reciprocal; plain
+// division at the ends of the exponent range, for negative values, infinities and NaN
+__device__ __forceinline__ double qr_rcp(double d) {
+  const long long b = __double_as_longlong(d);
+  const int be = (int)(b >> 52);
+  if (be < 8 || be > 2038) return 1.0 / d;
+  const double md = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
+  double r = (double)(1.0f / __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff)));
+  r = fma(r, fma(-md, r, 1.0), r);
+  r = fma(r, fma(-md, r, 1.0), r);
+  return __longlong_as_double(__double_as_longlong(r) - ((long long)(be - 1023) << 52));
+}
+
+__global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, const int* __restrict__ elem,
+                                                const int* __restrict__ slot, int L, const int* __restrict__ gmap,
                                                 const Constraint* __restrict__ cons, const double* __restrict__ K64,
-                                                const float* __restrict__ Kh, const float* __restrict__ Kl,
-                                                const double* __restrict__ K0T1, const double* __restrict__ R,
-                                                const double* __restrict__ u, const double* __restrict__ rho,
-                                                const int64_t* __restrict__ off, double E0, double Emin, double q,
-                                                const BasisTab* __restrict__ B, double hx, double hy,
-                                                double* __restrict__ eps) {
-  extern __shared__ double sh[];
+                                                const double* __restrict__ rows, const double* __restrict__ K0T1,
+                                                const double* __restrict__ R, const double* __restrict__ u,
+                                                const double* __restrict__ rho, const int64_t* __restrict__ off,
+                                                double E0, double Emin, double q, const BasisTab* __restrict__ B,
+                                                double hx, double hy, double* __restrict__ eps) {
+  extern __shared__ __align__(16) double sh[];
   const int lane = threadIdx.x;
-  const int k = blockIdx.x;
+  const int k = first + blockIdx.x;
   if (k >= n) return;
   const int e = elem[k], sl = slot[k];
   const int n1d = p + 1;
   const int na = (p + 1) * (p + 1), nb = (p + 2) * (p + 2);
   const int n0 = 2 * na, n1 = 2 * nb, S = d * d;
-  const int P1 = packed_size(n1);
+  const int P1 = packed_size(n1), L1 = qr_row_len(p + 1);
   double* A = sh;
-  double* f = A + P1;
+  double* f = A + L1;
   double* f1 = f + n0;
   double* u1 = f1 + n1;
-  double* E = u1 + n1;
-  double* ue = E + S;
+  double* ue = u1 + n1;
   double* rd = ue + n0;
   double* cl = rd + n1;
   double* pr = cl + n1;
+  double* E = pr + 3 * n1;
+  if (rows) {
+    const double2* src = reinterpret_cast<const double2*>(rows + (size_t)blockIdx.x * L1);
+    for (int c = lane; c < L1 / 2; c += 32) reinterpret_cast<double2*>(A)[c] = src[c];
+  } else {
+    for (int s = lane; s < S; s += 32) {
+      double r = rho[off[e] + s];
+      E[s] = Emin + (q == 3.0 ? r * r * r : pow(r, q)) * (E0 - Emin);
+    }
+  }
   // gather u_e (lanes over nodes), then remove its least-squares rigid motion about the element
   // centre (translations and rotation; node sums over the warp)
   for (int ln = lane; ln < na; ln += 32) gather_node(na, sl, ln, gmap, cons, u, ue);
@@ -332,18 +357,17 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
       ue[2 * ln + 1] = ue[2 * ln + 1] - ty - om * x;
     }
   }
-  for (int s = lane; s < S; s += 32) {
-    double r = rho[off[e] + s];
-    E[s] = Emin + pow(r, q) * (E0 - Emin);
-  }
   __syncwarp();
-  // f = K_e u_e (order p, FP64 element matrix of the build) and J^(p) = u^T f / 2
+  // f = K_e u_e (order p, FP64 element matrix of the build: row i of the circulant-diagonal layout from
+  // D_k[i] and D_k[i - k]) and J^(p) = u^T f / 2
   double jp = 0.0;
+  const double* Ke = K64 + (size_t)sl * L;
   for (int i = lane; i < n0; i += 32) {
     double s = 0.0;
-    for (int j = 0; j < n0; ++j) {
-      int a = i < j ? i : j, b = i < j ? j : i;
-      s += k_entry(K64, Kh, Kl, L, sl, dpos[packed_index(n0, a, b)].x) * ue[j];
+    for (int kk = 0; 2 * kk <= n0; ++kk) {
+      const int j = i + kk < n0 ? i + kk : i + kk - n0, jm = i >= kk ? i - kk : i - kk + n0;
+      s += Ke[kk * n0 + i] * ue[j];
+      if (kk > 0 && 2 * kk < n0) s += Ke[kk * n0 + jm] * ue[jm];
     }
     f[i] = s;
     jp += ue[i] * s;
@@ -358,15 +382,17 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
     for (int kk = 0; kk < na; ++kk) s += R[jn * na + kk] * f[2 * kk + c];
     f1[i] = s;
   }
-  // K^(p+1) = sum_s E_s K0_s^(p+1) (table rows by upper packed index (i <= j)) into the lower triangle
-  for (int c = lane; c < P1; c += 32) {
-    double s = 0.0;
-    const double* kc = K0T1 + (size_t)c * S;
-    for (int t = 0; t < S; ++t) s = fma(E[t], kc[t], s);
-    int i = 0, rem = c;
-    while (rem >= n1 - i) { rem -= n1 - i; ++i; }
-    const int j = i + rem;
-    A[j * (j + 1) / 2 + i] = s;
+  if (!rows) {
+    // K^(p+1) (table rows by upper packed index (i <= j)) into the lower triangle
+    for (int c = lane; c < P1; c += 32) {
+      double s = 0.0;
+      const double* kc = K0T1 + (size_t)c * S;
+      for (int t = 0; t < S; ++t) s = fma(E[t], kc[t], s);
+      int i = 0, rem = c;
+      while (rem >= n1 - i) { rem -= n1 - i; ++i; }
+      const int j = i + rem;
+      A[j * (j + 1) / 2 + i] = s;
+    }
   }
   __syncwarp();
   // pinned DOFs of the (p+1) element: u_x, u_y at the bottom-left vertex, u_y at the bottom-right
@@ -387,21 +413,23 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
   }
   __syncwarp();
   // identity rows and columns on the pinned DOFs
-  for (int c = lane; c < P1; c += 32) {
-    int i = (int)((sqrtf(8.0f * (float)c + 1.0f) - 1.0f) * 0.5f);
-    while (i * (i + 1) / 2 > c) --i;
-    while ((i + 1) * (i + 2) / 2 <= c) ++i;
-    const int j = c - i * (i + 1) / 2;
-    const bool pin = i == fx[0] || i == fx[1] || i == fx[2] || j == fx[0] || j == fx[1] || j == fx[2];
-    if (pin) A[c] = (i == j) ? 1.0 : 0.0;
-  }
+  for (int k = 0; k < 3; ++k)
+    for (int i = lane; i < n1; i += 32) {
+      const int a = i > fx[k] ? i : fx[k], b = i > fx[k] ? fx[k] : i;
+      A[a * (a + 1) / 2 + b] = i == fx[k] ? 1.0 : 0.0;
+    }
   __syncwarp();
   // A = L D L^T (right-looking).  Column c: the pivot's reciprocal into rd[c], the column kept
   // unscaled in cl and scaled into L; the trailing update A_ij -= L_ic cl_j (c < j <= i) runs over
   // the m (m + 1) / 2 pairs of the trailing block spread evenly over the lanes: pair
-  // t = s (s + 1) / 2 + r (0 <= r <= s < m) is row n1 - 1 - r, column n1 - 1 - s.
+  // t = s (s + 1) / 2 + r (0 <= r <= s < m) is row n1 - 1 - r, column n1 - 1 - s.  A pinned column is
+  // the identity's: nothing to update.
   for (int c = 0; c < n1; ++c) {
-    const double inv = 1.0 / A[c * (c + 1) / 2 + c];
+    if (c == fx[0] || c == fx[1] || c == fx[2]) {
+      if (lane == 0) rd[c] = 1.0;
+      continue;
+    }
+    const double inv = qr_rcp(A[c * (c + 1) / 2 + c]);
     for (int i = c + 1 + lane; i < n1; i += 32) {
       const double a = A[i * (i + 1) / 2 + c];
       cl[i] = a;
@@ -422,8 +450,9 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
     __syncwarp();
   }
   // L y = b, y <- D^-1 y, L^T x = y, column by column (each solved entry updates the rest over the
-  // lanes)
+  // lanes; a pinned column has nothing to give)
   for (int j = 0; j < n1; ++j) {
+    if (j == fx[0] || j == fx[1] || j == fx[2]) continue;
     const double yj = u1[j];
     for (int i = j + 1 + lane; i < n1; i += 32) u1[i] -= A[i * (i + 1) / 2 + j] * yj;
     __syncwarp();
@@ -431,6 +460,7 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, const int* 
   for (int i = lane; i < n1; i += 32) u1[i] *= rd[i];
   __syncwarp();
   for (int j = n1 - 1; j >= 0; --j) {
+    if (j == fx[0] || j == fx[1] || j == fx[2]) continue;
     const double xj = u1[j];
     for (int i = lane; i < j; i += 32) u1[i] -= A[j * (j + 1) / 2 + i] * xj;
     __syncwarp();
@@ -896,19 +926,40 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
   gamma_d_kernel<<<grid_for(nel, 32 * kGdWarps, 152 * 6), 32 * kGdWarps, 0, h->stream>>>(
       nel, h->design_off_d, rho, mm, o->cycle, o->alpha, o->beta, gd_);
   MTO_TRY(mto_after_launch(h, "gamma_d_kernel"));
-  // QR error per (p, d) class
+  // QR error per (p, d) class, in chunks of elements whose rows fit 448 MB, full waves of the row
+  // kernel (128 elements per SM) where a chunk is that large (38,912 elements of Q3)
   for (size_t ci = 0; ci < h->bc.size(); ++ci) {
     const BClass& b = h->bc[ci];
     const BClass& b1 = h->bc_qr[ci];
     const PClass& c = h->pc[b.p];
-    const int n0 = 2 * (b.p + 1) * (b.p + 1), n1 = 2 * (b.p + 2) * (b.p + 2);
-    size_t smem = sizeof(double) * ((size_t)packed_size(n1) + n0 + n1 + n1 + b.S + n0 + n1 + n1 + 3 * n1);
+    const int n0 = 2 * (b.p + 1) * (b.p + 1), n1 = 2 * (b.p + 2) * (b.p + 2), L1 = qr_row_len(b.p + 1);
+    const bool tc = h->build_path == MTO_BUILD_TENSOR && b1.tcB;
+    const size_t smem = sizeof(double) * ((size_t)L1 + 2 * n0 + 7 * n1 + (tc ? 0 : b.S));
     if (smem > 48 * 1024) cudaFuncSetAttribute(qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    qr_kernel<<<b.n, 32, smem, h->stream>>>(b.p, b.d, b.n, b.elem, b.slot, c.L, c.dpos, c.gmap, h->cons_d,
-                                            c.K64, c.K32, c.K32lo, b1.K0T,
-                                            h->qr[b.p].R, u, rho, h->design_off_d, m->E0, m->Emin, m->q, B, h->hx,
-                                            h->hy, eq_);
-    MTO_TRY(mto_after_launch(h, "qr_kernel"));
+    int chunk = b.n;
+    if (tc) {
+      const int wave = 152 * 128;
+      const int most = (int)(((size_t)448 << 20) / (sizeof(double) * L1));
+      chunk = std::min(b.n, most >= wave ? most / wave * wave : most / 128 * 128);
+      if ((size_t)chunk * L1 > h->qr_cap) {
+        if (h->qr_rows) {
+          MTO_TRY(mto_cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+          cudaFree(h->qr_rows);
+          h->bytes -= (int64_t)(h->qr_cap * sizeof(double));
+          h->qr_cap = 0;
+        }
+        MTO_TRY(mto_alloc(h, &h->qr_rows, (size_t)chunk * L1));
+        h->qr_cap = (size_t)chunk * L1;
+      }
+    }
+    for (int first = 0; first < b.n; first += chunk) {
+      const int cn = std::min(chunk, b.n - first);
+      if (tc) MTO_TRY(tc_rows(h, b, b1, L1, first, cn, nullptr, rho, m, h->qr_rows, nullptr, nullptr));
+      qr_kernel<<<cn, 32, smem, h->stream>>>(b.p, b.d, b.n, first, b.elem, b.slot, c.L, c.gmap, h->cons_d, c.K64,
+                                             tc ? h->qr_rows : nullptr, b1.K0T, h->qr[b.p].R, u, rho,
+                                             h->design_off_d, m->E0, m->Emin, m->q, B, h->hx, h->hy, eq_);
+      MTO_TRY(mto_after_launch(h, "qr_kernel"));
+    }
   }
   if (!pn && !dn && !th) return MTO_OK;
   if (!pn || !dn || !th) return mto_fail(h, MTO_EINVAL, "mto_indicator: p_new, d_new and theta go together");

@@ -180,6 +180,7 @@ void release_mesh(mto_handle h) {
   }
   for (auto& q : h->qr) {
     free_dev(h, q.R);
+    free_dev(h, q.pos);
     q = QRTab();
   }
   free_dev(h, h->slot_d);
@@ -206,6 +207,8 @@ void release_mesh(mto_handle h) {
   free_dev(h, h->filt_H);
   free_dev(h, h->filt_ext);
   free_dev(h, h->oc_t);
+  free_dev(h, h->qr_rows);
+  h->qr_cap = 0;
   h->bytes = h->base_bytes;
 }
 

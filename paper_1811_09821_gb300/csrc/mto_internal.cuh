@@ -73,7 +73,11 @@ struct BClass {
 struct QRTab {
   int p = 0;
   double* R = nullptr;   // [(p+2)^2][(p+1)^2] scalar load transfer M^(p+1,p) M^(p)^-1
+  int* pos = nullptr;    // [qr_row_len(p + 1)] upper packed entry at each place of the lower packed row, or -1
 };
+
+// Row length of the QR indicator's order-p matrices: the packed lower triangle, padded to whole 32 bytes.
+__host__ __device__ constexpr int qr_row_len(int p) { return round_up(packed_size(2 * (p + 1) * (p + 1)), 4); }
 
 // Kernel families timed with CUDA events when timing is enabled (see mto_timing_enable).
 enum Family { F_APPLY32 = 0, F_APPLY64 = 1, F_BUILD = 2, F_SENS = 3, F_INDICATOR = 4, F_VECTOR = 5,
@@ -180,6 +184,8 @@ struct mto_handle_s {
   double* filt_W = nullptr;                    // [design_len] density filter: x / W of the adjoint
   double* filt_H = nullptr;                    // its weight tables per design count, and
   int* filt_ext = nullptr;                     // their row extents
+  double* qr_rows = nullptr;                   // QR indicator: a chunk of elements' order p + 1 matrices
+  size_t qr_cap = 0;                           // and its doubles
   double* oc_t = nullptr;                      // [4][design_len] OC: rho_j B_j^eta and the area-scaled T, L, H
   int64_t* spring_dof_d = nullptr;             // [n_springs] DOFs with a spring to ground (K + k e e^T)
   double* spring_k_d = nullptr;                // [n_springs] their stiffness
@@ -448,6 +454,8 @@ void mg_release(mto_handle h);
 // tc.cu
 mto_status tc_tables(mto_handle h);
 mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision);
+mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int first, int n, const int* slot,
+                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl);
 int ebe_blocks(int p, int n);                                           // grid of one operator launch
 // apply.cu
 mto_status apply64(mto_handle h, const double* x, double* y);        // y += K x (FP64 vectors)

@@ -172,11 +172,12 @@ __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double
   if (pos >= ntile * kTN) return;
   __shared__ double colmax;
   const int c = pos < L ? posc[pos] : -1;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 32) {
     double m = 0.0;
     if (c >= 0)
-      for (int s = 0; s < S; ++s) m = fmax(m, fabs(K0T[(size_t)c * S + s]));
-    colmax = m;
+      for (int s = threadIdx.x; s < S; s += 32) m = fmax(m, fabs(K0T[(size_t)c * S + s]));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) colmax = m;
   }
   __syncthreads();
   int ex = 0;
@@ -482,21 +483,23 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
 
 }  // namespace
 
-// Per (p, d) class with d <= 8: B slice tables (once per nu) for the tensor-core build.
+// Per (p, d) class with d <= 8: B slice tables (once per nu) for the tensor-core build, and for the
+// QR indicator's order p + 1 matrices (in its packed row order).
 mto_status tc_tables(mto_handle h) {
-  for (auto& b : h->bc) {
-    if (b.S > 64) continue;
-    const PClass& c = h->pc[b.p];
-    const int kpad = (b.S + 15) / 16 * 16;
-    const int ntile = (c.L + kTN - 1) / kTN;
-    if (!b.tcB) {
-      MTO_TRY(mto_alloc(h, &b.tcB, (size_t)ntile * kSlices * kTN * kpad));
-      MTO_TRY(mto_alloc(h, &b.tcTau, (size_t)ntile * kTN));
-      MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(b.tcB, 0, sizeof(unsigned short) * ntile * kSlices * kTN * kpad,
-                                                h->stream), "memset"));
+  for (int qr = 0; qr < 2; ++qr) {
+    for (auto& b : qr ? h->bc_qr : h->bc) {
+      if (b.S > 64) continue;
+      const int L = qr ? qr_row_len(b.p) : h->pc[b.p].L;
+      const int* pos = qr ? h->qr[b.p - 1].pos : h->pc[b.p].posc;
+      const int kpad = (b.S + 15) / 16 * 16;
+      const int ntile = (L + kTN - 1) / kTN;
+      if (!b.tcB) {
+        MTO_TRY(mto_alloc(h, &b.tcB, (size_t)ntile * kSlices * kTN * kpad));
+        MTO_TRY(mto_alloc(h, &b.tcTau, (size_t)ntile * kTN));
+      }
+      tc_btable_kernel<<<ntile * kTN, 64, 0, h->stream>>>(b.S, kpad, L, ntile, b.K0T, pos, b.tcB, b.tcTau);
+      MTO_TRY(mto_after_launch(h, "tc_btable_kernel"));
     }
-    tc_btable_kernel<<<ntile * kTN, 64, 0, h->stream>>>(b.S, kpad, c.L, ntile, b.K0T, c.posc, b.tcB, b.tcTau);
-    MTO_TRY(mto_after_launch(h, "tc_btable_kernel"));
   }
   return MTO_OK;
 }
@@ -511,23 +514,31 @@ size_t tc_smem_bytes(int kpad) {
 }
 }  // namespace
 
-// The tensor-core build of one (p, d) class (d <= 8).  The N tiles of a class with few elements are
-// split over CTAs (each forms its elements' A slices again, about the cost of three tiles) until the
-// launch has about one CTA per SM.
-mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision) {
-  const PClass& c = h->pc[b.p];
+// Rows sum_s E(rho_s) K0_s of elements first .. first + n - 1 of a class (its elements and counts from
+// `b`, the tables from `tab`): to row slot[k] of K64 (and the pair), or to row k - first without slots.
+// The N tiles of few elements are split over CTAs (each forms its elements' A slices again, about the
+// cost of three tiles) until the launch has about one CTA per SM.
+mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int first, int n, const int* slot,
+                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl) {
   const int kpad = (b.S + 15) / 16 * 16;
-  const int ntile = (c.L + kTN - 1) / kTN;
+  const int ntile = (L + kTN - 1) / kTN;
   const size_t smem = tc_smem_bytes(kpad);
   MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(tc_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                  (int)smem), "cudaFuncSetAttribute"));
-  const int gx = (b.n + kTM - 1) / kTM;
+  const int gx = (n + kTM - 1) / kTM;
   const int gy = std::max(1, std::min(ntile, 152 / gx));
   const int per = (ntile + gy - 1) / gy;
   tc_build_kernel<<<dim3(gx, (ntile + per - 1) / per), 32 * (kEpiWarps + 1), smem, h->stream>>>(
-      b.n, 0, b.S, kpad, c.L, ntile, per, b.elem, b.slot, h->design_off_d, rho, m->E0, m->Emin, m->q, b.tcB, b.tcTau,
-      c.K64, precision == MTO_MIXED ? c.K32 : nullptr, precision == MTO_MIXED ? c.K32lo : nullptr, h->flags + 4);
+      first + n, first, b.S, kpad, L, ntile, per, b.elem, slot, h->design_off_d, rho, m->E0, m->Emin, m->q, tab.tcB,
+      tab.tcTau, K64, Kh, Kl, h->flags + 4);
   return mto_after_launch(h, "tc_build_kernel");
+}
+
+// The tensor-core build of one (p, d) class (d <= 8).
+mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision) {
+  const PClass& c = h->pc[b.p];
+  const bool mixed = precision == MTO_MIXED;
+  return tc_rows(h, b, b, c.L, 0, b.n, b.slot, rho, m, c.K64, mixed ? c.K32 : nullptr, mixed ? c.K32lo : nullptr);
 }
 
 }  // namespace mto

@@ -190,3 +190,31 @@ def test_coarsest_inverse_edges(mto, nx, ny):
     r = np.abs(fn - K @ un)[free]
     assert np.all(r <= 1e-11 * np.linalg.norm(fn) + 64 * 2.0 ** -52 * (abs(K) @ np.abs(un))[free]), r.max()
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny", [(1, 1), (43, 3)])
+@pytest.mark.parametrize("p", [1, 2, 3, 4, 5, 6])
+@pytest.mark.parametrize("d", [1, 3, 8, 9])   # the last: more than 64 subcells, summed in the kernel
+def test_qr_error_edges(mto, nx, ny, p, d):
+    """The QR indicator with order p + 1 matrices formed on the tensor cores (one element, one past a
+    tile of 128) and summed in the kernel, against the oracle's dense Cholesky: eps = 1 - J_p / J_(p+1) is
+    determined to kappa eps of the pinned element problem, kappa < 1e7 for densities of 0.3 to 1 (modulus
+    contrast 40), so 1e-8; the two paths agree with each other to the same bound."""
+    from oracle import indicators as oi
+    h = handle(mto, nx, ny, p, d)
+    m = om.DPMesh(nx, ny, np.full(nx * ny, p), np.full(nx * ny, d))
+    rng = np.random.default_rng(p * 31 + d)
+    rho = rng.uniform(0.3, 1.0, h.design_len)
+    u = rng.standard_normal(h.ndof)
+    T = lambda a: torch.tensor(a, device="cuda")
+    mat = mto.material()
+    h.set_supports(h.side_dofs(0))
+    h.build_elements(T(rho), mat)
+    got = h.indicator(T(u), T(rho), mat, maps=False)["eps_qr"].cpu().numpy()
+    h.set_build_path(mto.BUILD_SIMT)
+    ref = h.indicator(T(u), T(rho), mat, maps=False)["eps_qr"].cpu().numpy()
+    assert np.abs(got - ref).max() <= 1e-8
+    for e in sorted({0, 1, 127, 128} & set(range(nx * ny))):
+        want = oi.qr_error_element(p, d, rho[m.design_off[e]:m.design_off[e + 1]], m.gather(e, u), 1.0, 1e-9, 0.3, 3.0)
+        assert abs(got[e] - want) <= 1e-8, (e, got[e], want)
+    h.close()
