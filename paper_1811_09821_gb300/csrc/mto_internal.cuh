@@ -187,6 +187,7 @@ struct mto_handle_s {
   double* qr_rows = nullptr;                   // QR indicator: a chunk of elements' order p + 1 matrices
   size_t qr_cap = 0;                           // and its doubles
   double* oc_t = nullptr;                      // [4][design_len] OC: rho_j B_j^eta and the area-scaled T, L, H
+  unsigned char* oc_work = nullptr;            // OC: bisection state, block partials and segment lengths
   int64_t* spring_dof_d = nullptr;             // [n_springs] DOFs with a spring to ground (K + k e e^T)
   double* spring_k_d = nullptr;                // [n_springs] their stiffness
   int n_springs = 0;

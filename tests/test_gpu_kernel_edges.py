@@ -218,3 +218,45 @@ def test_qr_error_edges(mto, nx, ny, p, d):
         want = oi.qr_error_element(p, d, rho[m.design_off[e]:m.design_off[e + 1]], m.gather(e, u), 1.0, 1e-9, 0.3, 3.0)
         assert abs(got[e] - want) <= 1e-8, (e, got[e], want)
     h.close()
+
+
+@pytest.mark.parametrize("nx,ny,d", [(1, 1, 1), (2, 1, 3), (16, 16, 4), (32, 33, 2), (150, 70, 8), (61, 47, 0)])
+@pytest.mark.parametrize("kind", ["late", "uniform", "flat", "void", "unreachable"])
+def test_oc_update_edges(mto, nx, ny, d, kind):
+    """The OC update that settles values as its interval shrinks (and the one-block path of small designs)
+    against the oracle's plain bisection over every value: the same midpoints and the same tests, so
+    lambda agrees to the interval's relative width 1e-10 (the volumes' rounding can turn a test only where
+    they differ from the target by less than n 2^-53) and the design to 1e-9.  Designs: sensitivities over
+    many decades, one value everywhere, steps (many equal breakpoints), no sensitivity at all (the
+    interval halves towards 0), and a volume no design within the move limit reaches."""
+    from oracle import oc as ooc
+    rng = np.random.default_rng(nx + d)
+    nel = nx * ny
+    dm = np.full(nel, d) if d else rng.choice([1, 2, 4, 8, 5], nel)
+    h = handle(mto, nx, ny, 1, dm, 1.0, 0.5 if d == 2 else 1.0)
+    n = h.design_len
+    rho = rng.uniform(0.0, 1.0, n)
+    dc = -np.exp(3.0 * rng.standard_normal(n)) * rho ** 2
+    vol = 0.9 * rho.mean() + 0.05
+    if kind == "uniform":
+        rho[:], dc[:], vol = 0.4, -2.0, 0.4
+    if kind == "flat":
+        rho, dc = np.round(rho, 1), np.round(dc) - 1.0   # (all zero is "void": the oracle cannot take it)
+    if kind == "void":
+        dc[:] = 0.0
+    if kind == "unreachable":
+        vol = 1.0
+    m = om.DPMesh(nx, ny, np.full(nel, 1), dm, h.hx, h.hy)
+    dv = ooc.subcell_areas(m)
+    for eta in (0.5, 0.7):
+        out = torch.zeros(n, dtype=torch.float64, device="cuda")
+        lam = h.oc_update(torch.tensor(rho, device="cuda"), torch.tensor(dc, device="cuda"), vol, out, eta=eta)
+        if kind in ("void", "unreachable"):   # the oracle's loop has no limit of steps there: its design in closed form
+            lo, hi = np.maximum(0.0, rho - 0.2), np.minimum(1.0, rho + 0.2)
+            want = lo if kind == "void" else np.where(dc < 0.0, hi, lo)
+            assert 0.0 < lam < 1e-28
+        else:
+            want, wl = ooc.oc_update(rho, dc, dv, vol * nel * h.hx * h.hy, eta=eta)
+            assert abs(lam - wl) <= 4e-10 * wl
+        np.testing.assert_allclose(out.cpu().numpy(), want, rtol=1e-9, atol=1e-12)
+    h.close()
