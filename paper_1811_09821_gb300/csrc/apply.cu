@@ -5,6 +5,7 @@
 //
 // Operator layout: one element per group of W lanes (one warp for Q3), element matrices in the
 // circulant-diagonal layout of mto_internal.cuh; see ebe_kernel.
+#include <algorithm>
 #include <array>
 #include <chrono>
 #include <cmath>
@@ -142,6 +143,43 @@ __device__ __forceinline__ void reduce_out(double v, const Red& rd) {
   }
 }
 
+// Up to three reductions of one launch behind a single counter (the first's): one atomic per block instead
+// of one per value, whose serialised round trips were most of the vector kernels' time on small systems.
+template <int K>
+__device__ __forceinline__ void reduce_out_n(const double (&v)[K], const Red (&rd)[K]) {
+  __shared__ double ws[K][32];
+  __shared__ int last;
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int k = 0; k < K; ++k) {
+    const double s = warp_sum(v[k]);
+    if (l == 0) ws[k][w] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double s = 0.0;
+      for (int i = 0; i < nw; ++i) s += ws[k][i];
+      rd[k].part[blockIdx.x] = s;
+    }
+    __threadfence();
+    last = atomicAdd(rd[0].cnt, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last) {
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      double s = 0.0;
+      for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(rd[k].part + i);
+      s = block_sum(s);
+      if (threadIdx.x == 0) *rd[k].res = s;
+    }
+    if (threadIdx.x == 0) *rd[0].cnt = 0u;
+  }
+}
+
 // sum of a few launch results, same order in every thread
 __device__ __forceinline__ double sum_res(const double* __restrict__ res, int n) {
   double s = 0.0;
@@ -247,7 +285,6 @@ __global__ void __launch_bounds__(256) ebe_kernel(const double* __restrict__ K64
 #pragma unroll
     for (int k = 0; k < ND; ++k) {
       const bool pair = k > 0 && 2 * k != NE;   // the entry also serves row i + k
-      double tdv[M];
       float tph[M], tpe[M];
 #pragma unroll
       for (int m = 0; m < M; ++m) {
@@ -260,7 +297,6 @@ __global__ void __launch_bounds__(256) ebe_kernel(const double* __restrict__ K64
           const double a = vi ? __ldg(K64 + rowb + k * NE + i) : 0.0;
           const double xj = shfl_sel<M>(xd, src, reg);
           acc[m] = fma(a, xj, acc[m]);
-          tdv[m] = a * xd[m];
         } else {
           const float ah = vi ? __ldg(Kh + rowb + k * NE + i) : 0.0f;
           const float al = (vi && Kl) ? __ldg(Kl + rowb + k * NE + i) : 0.0f;
@@ -280,7 +316,11 @@ __global__ void __launch_bounds__(256) ebe_kernel(const double* __restrict__ K64
           if (s < 0) s += NE;
           const int src = gb + (s & 31), reg = (s >> 5) < M ? (s >> 5) : 0;
           if (!kDF) {
-            acc[m] += shfl_sel<M>(tdv, src, reg);
+            // K[s][r] x_s with the entry read again (a cache hit) and x_s by shuffle: one FP64
+            // instruction, where handing over the product takes two and the FP64 pipes are the bound
+            const double xs = shfl_sel<M>(xd, src, reg);
+            const double a = (act && r < NE) ? __ldg(K64 + rowb + k * NE + s) : 0.0;
+            acc[m] = fma(a, xs, acc[m]);
           } else {
             const float pp = shfl_sel<M>(tph, src, reg);
             const float pe = shfl_sel<M>(tpe, src, reg);
@@ -610,13 +650,17 @@ size_t tma_smem_bytes(int L, int G, int nm, int stages) {
 
 }  // namespace
 
+// Threads per block of an element-operator launch of `warps` warps: two warps while that leaves at most
+// one wave of blocks, so that the warps of small classes spread over the SMs, else eight.
+static int ebe_threads(int warps) { return warps <= 2 * 152 * 8 ? 64 : 256; }
+
 // Blocks of one element-operator launch for an order class (fixed per class size).
 template <int PO>
 int ebe_blocks_p(int n) {
   constexpr int NE = 2 * (PO + 1) * (PO + 1);
   constexpr int G = WarpShape<NE>::G;
   const int warps = (n + G - 1) / G;
-  return grid_for((int64_t)warps * 32, 256, 152 * 8);
+  return grid_for((int64_t)warps * 32, ebe_threads(warps), 152 * 8);
 }
 
 int ebe_blocks(int p, int n) {
@@ -713,20 +757,22 @@ void launch_ebe(mto_handle h, const PClass& c, const double* M64, const float* M
         }
         return;
       }
-      // persistent: two blocks of 8 warps per SM (the register budget of the pipelined rows)
-      int blocks = (warps + 7) / 8;
-      if (blocks > 152 * 2) blocks = 152 * 2;
+      // persistent: two blocks of 8 warps per SM (the register budget of the pipelined rows); small
+      // classes in blocks of two warps, spread over the SMs
+      const int th = warps <= 152 * 8 ? 64 : 256;
+      int blocks = (warps + th / 32 - 1) / (th / 32);
+      if (th == 256 && blocks > 152 * 2) blocks = 152 * 2;
       if (lo)
-        ebe_df_pipe_kernel<PO, true, TX><<<blocks, 256, 0, h->stream>>>(Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x, y,
-                                                                         red, done);
+        ebe_df_pipe_kernel<PO, true, TX><<<blocks, th, 0, h->stream>>>(Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x, y, red,
+                                                                        done);
       else
-        ebe_df_pipe_kernel<PO, false, TX><<<blocks, 256, 0, h->stream>>>(Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x, y,
-                                                                          red, done);
+        ebe_df_pipe_kernel<PO, false, TX><<<blocks, th, 0, h->stream>>>(Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x, y, red,
+                                                                         done);
       return;
     }
   }
-  ebe_kernel<PO, kDF, TX><<<ebe_blocks_p<PO>(c.n), 256, 0, h->stream>>>(M64, Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x,
-                                                                        y, red, done, cv);
+  ebe_kernel<PO, kDF, TX><<<ebe_blocks_p<PO>(c.n), ebe_threads((c.n + WarpShape<NE>::G - 1) / WarpShape<NE>::G), 0,
+                            h->stream>>>(M64, Mh, Ml, c.L, c.n, c.gmap, h->cons_d, x, y, red, done, cv);
 }
 
 // y += S x for the springs to ground (distinct DOFs; launched after the element classes on the same
@@ -816,9 +862,9 @@ mto_status apply_all(mto_handle h, int which, const T* x, T* y, int slot, const 
 
 // ---------------------------------------------------------------------------------- CG
 // Preconditioned CG (Hestenes-Stiefel form).  Per iteration: the operator launch q = K p, which
-// also yields p^T K p; a fused vector kernel (alpha, x, r, q = 0, Jacobi z and r^T z, r^T r,
+// also yields p^T K p; a fused vector kernel (alpha, x, r, Jacobi z and r^T z, r^T r,
 // r^T D^-1 r); the element-block preconditioner z = M^-1 r (Schwarz only, also yielding r^T z);
-// and the direction kernel (convergence test, beta, p = z + beta p).  The curvature p^T K p is
+// and the direction kernel (convergence test, beta, p = z + beta p, q = 0).  The curvature p^T K p is
 // accumulated directly (never formed by subtraction), which matters at the 1e9 stiffness contrast
 // of these problems.  Every reduction is finished by the last block of its launch in a fixed order
 // (deterministic); consumers add the few launch results of a slot in class order.  Slots alternate
@@ -830,7 +876,7 @@ __global__ void __launch_bounds__(256) cg_vector_kernel(
     int64_t n, T* __restrict__ x, T* __restrict__ r, const T* __restrict__ p, T* __restrict__ q, T* __restrict__ z,
     const T* __restrict__ invd, const double* __restrict__ gin, int ng, const double* __restrict__ pin, int np,
     Red gout, Red rrout, Red rdout, const int* __restrict__ base, int local, int* __restrict__ done,
-    int* __restrict__ err, double* __restrict__ eng) {
+    int* __restrict__ err, double* __restrict__ eng, float* __restrict__ r32) {
   if (*done) return;
   // the step length once per block (an FP64 division per thread costs more than the vector pass
   // on GB300's FP64 pipes)
@@ -863,29 +909,36 @@ __global__ void __launch_bounds__(256) cg_vector_kernel(
   double g = 0.0, rr = 0.0, rd = 0.0;
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
     const T inv = invd[j];
-    const T qj = q[j];   // q is cleared by the next launch (zero_kernel): see there
-    if (!kJacobi) z[j] = (T)0;
+    const T qj = q[j];   // q is cleared by the direction kernel: see there
+    if (!kJacobi && z) z[j] = (T)0;
     if (inv != (T)0) {
       x[j] = fma(a, p[j], x[j]);
       const T rj = fma(-a, qj, r[j]);
       r[j] = rj;
+      if (r32) r32[j] = (float)rj;
       const double rjd = (double)rj;
       if (kJacobi) g += rjd * rjd * (double)inv;
       rr += rjd * rjd;
       rd += rjd * rjd * (double)inv;
     }
   }
-  if (kJacobi) reduce_out(g, gout);
-  reduce_out(rr, rrout);
-  reduce_out(rd, rdout);
+  if constexpr (kJacobi) {
+    const double v[3] = {g, rr, rd};
+    const Red o[3] = {gout, rrout, rdout};
+    reduce_out_n<3>(v, o);
+  } else {
+    const double v[2] = {rr, rd};
+    const Red o[2] = {rrout, rdout};
+    reduce_out_n<2>(v, o);
+  }
 }
 
 // convergence test on the new residual, then beta = (r^T z)_new / (r^T z)_old and p = z + beta p
 // (Jacobi: z = D^-1 r on the fly)
 template <typename T, bool kJacobi>
 __global__ void __launch_bounds__(256) cg_direction_kernel(
-    int64_t n, const T* __restrict__ r, const T* __restrict__ z, T* __restrict__ p, const T* __restrict__ invd,
-    const double* __restrict__ gnew, const double* __restrict__ gold, int ng, ConvTest cv) {
+    int64_t n, const T* __restrict__ r, const T* __restrict__ z, T* __restrict__ p, T* __restrict__ q,
+    const T* __restrict__ invd, const double* __restrict__ gnew, const double* __restrict__ gold, int ng, ConvTest cv) {
   if (*cv.done) return;
   __shared__ double s_beta;
   __shared__ int s_stop;
@@ -930,6 +983,7 @@ __global__ void __launch_bounds__(256) cg_direction_kernel(
     // interpolate, supported ones included: z is masked to the free DOFs here
     const T zj = kJacobi ? invd[j] * r[j] : (invd[j] != (T)0 ? z[j] : (T)0);
     p[j] = fma(b, p[j], zj);
+    q[j] = (T)0;   // the next operator launch adds into it
   }
 }
 
@@ -953,17 +1007,9 @@ __global__ void __launch_bounds__(256) cg_init_kernel(int64_t n, const T* __rest
   if (kJacobi) reduce_out(g, gout);
 }
 
-// v = 0.  Measured on GB300: a vector kernel that reads an array and then stores zeros into it
-// streams at ~1.6 TB/s (9.4M doubles, 5 reads and 3 writes), the same kernel without that store at
-// ~4.9 TB/s and a kernel of plain stores at ~5.9 TB/s, so the accumulators that the next operator
-// launch adds into are cleared by this separate launch instead of by the kernel that consumed them.
-template <typename T>
-__global__ void __launch_bounds__(256) zero_kernel(int64_t n, T* __restrict__ v, const int* __restrict__ done) {
-  if (done && *done) return;
-  for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-    v[j] = (T)0;
-}
-
+// Accumulators are cleared by a kernel that does not read them.  Measured on GB300: a vector kernel that
+// reads an array and then stores zeros into it streams at ~1.6 TB/s (9.4M doubles, 5 reads and 3
+// writes), the same kernel without that store at ~4.9 TB/s and a kernel of plain stores at ~5.9 TB/s.
 // b = a on free DOFs (invd != 0), 0 on supported ones
 template <typename T>
 __global__ void __launch_bounds__(256) masked_copy_kernel(int64_t n, const T* __restrict__ a, T* __restrict__ b,
@@ -1066,6 +1112,17 @@ __global__ void sum1_kernel(const double* __restrict__ part, int nb, double* __r
 // SM, so that enough loads are in flight to stream the vectors at HBM speed (with 4 blocks per SM
 // the grid-stride loops ran latency-bound at about a sixth of it)
 constexpr int kVecBlocks = 152 * 8;
+}  // namespace
+
+// Blocks of 256 threads of a vector kernel over n entries: one entry per thread up to one block per SM, then
+// four per thread, up to one full wave.  Every block costs the reductions one atomic on one address:
+// with the full wave for any n the vector update of 14 k DOFs took 17 us.
+int vec_blocks(int64_t n) {
+  const int64_t b1 = (n + 255) / 256, b4 = (n + 1023) / 1024;
+  return (int)std::max<int64_t>(1, b1 <= 152 ? b1 : std::min<int64_t>(std::max<int64_t>(b4, 152), kVecBlocks));
+}
+
+namespace {
 
 template <typename T>
 struct CGVecs {
@@ -1087,20 +1144,21 @@ CGVecs<float> cg_vecs<float>(mto_handle h, float* x, float* r) {
 // result j of reduction slot k
 inline const double* res_slot(mto_handle h, int k) { return h->cg_res + 8 * k; }
 
-// The preconditioner step z = M^-1 r with r^T z into reduction slot `slot` (element-block Schwarz:
+// The preconditioner step (rounded: the FP32 cycle finds r already rounded) z = M^-1 r with r^T z into reduction slot `slot` (element-block Schwarz:
 // one result per class launch; multigrid: one).
 template <typename T>
-mto_status precond_step(mto_handle h, const CGVecs<T>& v, int pc, int deg, int slot, const int* done);
+mto_status precond_step(mto_handle h, const CGVecs<T>& v, int pc, int deg, int slot, const int* done,
+                        bool rounded = false);
 template <>
-mto_status precond_step<double>(mto_handle h, const CGVecs<double>& v, int pc, int deg, int slot,
-                                const int* done) {
+mto_status precond_step<double>(mto_handle h, const CGVecs<double>& v, int pc, int deg, int slot, const int* done,
+                                bool rounded) {
   ConvTest none{};
   if (pc == MTO_PREC_SCHWARZ) return apply_all<double>(h, 1, v.r, v.z, slot, done, none);
   const Red rd = red_slot(h, slot, 0);   // r^T z from the cycle's last smoothing step
-  return mg_vcycle(h, v.r, v.z, deg, done, rd.part, rd.cnt, rd.res);
+  return mg_vcycle(h, v.r, v.z, deg, done, rd.part, rd.cnt, rd.res, rounded);
 }
 template <>
-mto_status precond_step<float>(mto_handle h, const CGVecs<float>& v, int pc, int deg, int slot, const int* done) {
+mto_status precond_step<float>(mto_handle h, const CGVecs<float>& v, int pc, int deg, int slot, const int* done, bool) {
   ConvTest none{};
   if (pc == MTO_PREC_SCHWARZ) return apply_all<float>(h, 1, v.r, v.z, slot, done, none);
   return mto_fail(h, MTO_EINVAL, "the multigrid preconditioner needs FP64 vectors (precision MTO_FP64)");
@@ -1125,23 +1183,24 @@ mto_status cg_iteration(mto_handle h, const CGVecs<T>& v, int pc, int deg, int n
   MTO_TRY(sa);
   {
     TimedScope ts(h, F_VECTOR);
+    // the element-block preconditioner adds into z; the FP32 cycle starts from a rounded copy of r
+    T* zz = pc == MTO_PREC_SCHWARZ ? v.z : nullptr;
+    float* r32 = sizeof(T) == 8 && pc == MTO_PREC_MG ? mg_residual32(h) : nullptr;
     if (!jac)
-      cg_vector_kernel<T, false><<<kVecBlocks, 256, 0, h->stream>>>(
-          n, v.x, v.r, v.p, v.q, v.z, v.invd, res_slot(h, kGam + par), ng, res_slot(h, kDel + par), nop,
+      cg_vector_kernel<T, false><<<vec_blocks(n), 256, 0, h->stream>>>(
+          n, v.x, v.r, v.p, v.q, zz, v.invd, res_slot(h, kGam + par), ng, res_slot(h, kDel + par), nop,
           red_slot(h, -1, 0), red_slot(h, kRR + nxt, 0), red_slot(h, kRD + nxt, 0), h->cg_base, local, h->flags,
-          h->flags + 1, eng);
+          h->flags + 1, eng, r32);
     else
-      cg_vector_kernel<T, true><<<kVecBlocks, 256, 0, h->stream>>>(
-          n, v.x, v.r, v.p, v.q, v.z, v.invd, res_slot(h, kGam + par), ng, res_slot(h, kDel + par), nop,
+      cg_vector_kernel<T, true><<<vec_blocks(n), 256, 0, h->stream>>>(
+          n, v.x, v.r, v.p, v.q, nullptr, v.invd, res_slot(h, kGam + par), ng, res_slot(h, kDel + par), nop,
           red_slot(h, kGam + nxt, 0), red_slot(h, kRR + nxt, 0), red_slot(h, kRD + nxt, 0), h->cg_base, local,
-          h->flags, h->flags + 1, eng);
+          h->flags, h->flags + 1, eng, nullptr);
     MTO_TRY(mto_after_launch(h, "cg_vector_kernel"));
-    zero_kernel<T><<<kVecBlocks, 256, 0, h->stream>>>(n, v.q, h->flags);
-    MTO_TRY(mto_after_launch(h, "zero_kernel"));
   }
   if (!jac) {
     h->timing.sample_lead = local == 0;   // sampled timing: the cycle's leading-part launches too
-    const mto_status sp = precond_step<T>(h, v, pc, deg, kGam + nxt, h->flags);
+    const mto_status sp = precond_step<T>(h, v, pc, deg, kGam + nxt, h->flags, true);
     h->timing.sample_lead = false;
     MTO_TRY(sp);
   }
@@ -1150,11 +1209,11 @@ mto_status cg_iteration(mto_handle h, const CGVecs<T>& v, int pc, int deg, int n
     ConvTest cv{res_slot(h, nrm == 1 ? kRD + nxt : kRR + nxt), 1, ref, tol2, h->cg_base, local, h->flags, h->flags + 1,
                 eng};
     if (!jac)
-      cg_direction_kernel<T, false><<<kVecBlocks, 256, 0, h->stream>>>(
-          n, v.r, v.z, v.p, v.invd, res_slot(h, kGam + nxt), res_slot(h, kGam + par), ng, cv);
+      cg_direction_kernel<T, false><<<vec_blocks(n), 256, 0, h->stream>>>(
+          n, v.r, v.z, v.p, v.q, v.invd, res_slot(h, kGam + nxt), res_slot(h, kGam + par), ng, cv);
     else
-      cg_direction_kernel<T, true><<<kVecBlocks, 256, 0, h->stream>>>(
-          n, v.r, v.z, v.p, v.invd, res_slot(h, kGam + nxt), res_slot(h, kGam + par), ng, cv);
+      cg_direction_kernel<T, true><<<vec_blocks(n), 256, 0, h->stream>>>(
+          n, v.r, v.z, v.p, v.q, v.invd, res_slot(h, kGam + nxt), res_slot(h, kGam + par), ng, cv);
     MTO_TRY(mto_after_launch(h, "cg_direction_kernel"));
   }
   return MTO_OK;
@@ -1207,9 +1266,9 @@ mto_status cg_prepare(mto_handle h, CGRun<T>& run, T* x, T* r, int pc, int deg, 
   {
     TimedScope ts(h, F_VECTOR);
     if (schwarz)
-      cg_init_kernel<T, false><<<kVecBlocks, 256, 0, h->stream>>>(n, v.r, v.p, v.q, v.z, v.invd, red_slot(h, -1, 0));
+      cg_init_kernel<T, false><<<vec_blocks(n), 256, 0, h->stream>>>(n, v.r, v.p, v.q, v.z, v.invd, red_slot(h, -1, 0));
     else
-      cg_init_kernel<T, true><<<kVecBlocks, 256, 0, h->stream>>>(n, v.r, v.p, v.q, v.z, v.invd,
+      cg_init_kernel<T, true><<<vec_blocks(n), 256, 0, h->stream>>>(n, v.r, v.p, v.q, v.z, v.invd,
                                                                  red_slot(h, kGam, 0));
     MTO_TRY(mto_after_launch(h, "cg_init_kernel"));
   }
@@ -1220,7 +1279,7 @@ mto_status cg_prepare(mto_handle h, CGRun<T>& run, T* x, T* r, int pc, int deg, 
   if (schwarz) {
     MTO_TRY(precond_step<T>(h, v, pc, deg, kGam, nullptr));
     TimedScope ts(h, F_VECTOR);
-    masked_copy_kernel<T><<<kVecBlocks, 256, 0, h->stream>>>(n, v.z, v.p, v.invd);
+    masked_copy_kernel<T><<<vec_blocks(n), 256, 0, h->stream>>>(n, v.z, v.p, v.invd);
     MTO_TRY(mto_after_launch(h, "masked_copy_kernel"));
   }
   if (!h->use_graphs) return MTO_OK;
@@ -1308,9 +1367,9 @@ mto_status residual_enqueue(mto_handle h, const double* f, const double* u) {
   MTO_TRY(apply_all<double>(h, 0, u, h->s64, -1, nullptr, none));
   {
     TimedScope ts(h, F_VECTOR);
-    residual_kernel<<<kVecBlocks, 256, 0, h->stream>>>(h->ndof, f, h->s64, h->invd64, h->r64, h->cg_part);
+    residual_kernel<<<vec_blocks(h->ndof), 256, 0, h->stream>>>(h->ndof, f, h->s64, h->invd64, h->r64, h->cg_part);
     MTO_TRY(mto_after_launch(h, "residual_kernel"));
-    sum4_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, kVecBlocks, h->red);
+    sum4_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, vec_blocks(h->ndof), h->red);
     MTO_TRY(mto_after_launch(h, "sum4_kernel"));
   }
   return mto_cuda_check(h, cudaMemcpyAsync(h->host_pinned, h->red, 4 * sizeof(double), cudaMemcpyDeviceToHost,
@@ -1461,16 +1520,16 @@ __global__ void __launch_bounds__(256) vsum_kernel(int64_t n, const double* __re
 }
 
 mto_status sum64(mto_handle h, const double* a, int64_t n, double* out_dev) {
-  vsum_kernel<<<kVecBlocks, 256, 0, h->stream>>>(n, a, h->cg_part);
+  vsum_kernel<<<vec_blocks(n), 256, 0, h->stream>>>(n, a, h->cg_part);
   MTO_TRY(mto_after_launch(h, "vsum_kernel"));
-  sum1_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, kVecBlocks, out_dev);
+  sum1_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, vec_blocks(n), out_dev);
   return mto_after_launch(h, "sum1_kernel");
 }
 
 mto_status dot64(mto_handle h, const double* a, const double* b, int64_t n, double* out_dev) {
-  dot_kernel<<<kVecBlocks, 256, 0, h->stream>>>(n, a, b, h->cg_part);
+  dot_kernel<<<vec_blocks(n), 256, 0, h->stream>>>(n, a, b, h->cg_part);
   MTO_TRY(mto_after_launch(h, "dot_kernel"));
-  sum1_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, kVecBlocks, out_dev);
+  sum1_kernel<<<1, 256, 0, h->stream>>>(h->cg_part, vec_blocks(n), out_dev);
   return mto_after_launch(h, "sum1_kernel");
 }
 

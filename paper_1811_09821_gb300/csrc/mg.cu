@@ -679,19 +679,21 @@ __global__ void __launch_bounds__(256) mg_coarse_solve_kernel(StripGeom g, const
 // The cycle's vectors are of type V: double, or float for the cycle on FP32 copies (mixed builds,
 // mg_operator LEAD), where the level kernels then also compute in FP32.
 //
-// One Chebyshev step on level vectors: r = D^-1 (b - q) (q = A x, then cleared), step 0:
+// One Chebyshev step on level vectors: r = D^-1 (b - q) (q = A x, null: 0), step 0:
 // d = r / theta, step s > 0: d = rho_s rho_{s-1} d + (2 rho_s / delta) r; x = d (xzero) or x += d.
+// `clear`, an accumulator that this kernel does not read, is zeroed for the next operator launch (a kernel
+// that stores zeros into an array it reads streams at a third of the rate).
 // With dpart set, also b^T x of the updated x (the PCG's r^T z after the cycle's last step),
 // reduced by the last block to finish in index order into *dres.  With zout set (the FP32
 // cycle's last step), the updated x goes to the FP64 output zout instead of x and the reduction
 // takes its b from bout (FP64).
 template <typename V>
-__global__ void __launch_bounds__(256) mg_cheb_kernel(int64_t n, const V* __restrict__ b, V* __restrict__ q,
-                                                      const V* __restrict__ invd, V* __restrict__ x,
+__global__ void __launch_bounds__(256) mg_cheb_kernel(int64_t n, const V* __restrict__ b, const V* __restrict__ q,
+                                                      V* __restrict__ clear, const V* __restrict__ invd, V* __restrict__ x,
                                                       V* __restrict__ d, const double2* __restrict__ coef,
                                                       int step, int xzero, const int* __restrict__ done,
                                                       double* __restrict__ dpart, unsigned* __restrict__ dcnt,
-                                                      double* __restrict__ dres, int given, int zq,
+                                                      double* __restrict__ dres, int given,
                                                       double* __restrict__ zout, const double* __restrict__ bout) {
   if (done && *done) return;
   const double2 cc = coef[step];   // (c1, c2), precomputed per level
@@ -701,8 +703,8 @@ __global__ void __launch_bounds__(256) mg_cheb_kernel(int64_t n, const V* __rest
     const V bi = b[i];
     // given: q already holds the preconditioned residual (element-block smoothing), else the
     // Jacobi-scaled residual is formed here from q = A x
-    const V r = given ? (invd[i] != V(0) ? q[i] : V(0)) : invd[i] * (bi - q[i]);
-    if (zq) q[i] = V(0);   // else a separate launch clears q (see mg_zero_kernel)
+    const V r = given ? (invd[i] != V(0) ? q[i] : V(0)) : invd[i] * (q ? bi - q[i] : bi);
+    if (clear) clear[i] = V(0);
     const V dn = step > 0 ? fma(c1, d[i], c2 * r) : c2 * r;   // c1 = 0 at step 0
     d[i] = dn;
     const V xn = xzero ? dn : x[i] + dn;
@@ -735,24 +737,18 @@ __global__ void __launch_bounds__(256) mg_cheb_kernel(int64_t n, const V* __rest
   }
 }
 
-// element-block smoothing: w = b - q on free DOFs (0 on supports); q is cleared by the next launch
+// element-block smoothing: w = b - q on free DOFs (0 on supports; q null: 0); `clear`, the accumulator of
+// the block launch that follows, is zeroed
 template <typename V>
 __global__ void __launch_bounds__(256) mg_block_resid_kernel(int64_t n, const V* __restrict__ b,
-                                                             const V* __restrict__ q, const V* __restrict__ invd,
-                                                             V* __restrict__ w, const int* __restrict__ done) {
+                                                             const V* __restrict__ q, V* __restrict__ clear,
+                                                             const V* __restrict__ invd, V* __restrict__ w,
+                                                             const int* __restrict__ done) {
   if (done && *done) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    w[i] = invd[i] != V(0) ? (b ? b[i] : V(0)) - q[i] : V(0);
-}
-
-// v = 0 as its own launch: on GB300 a kernel that reads an array and stores zeros into it streams
-// at about a third of the rate of the same kernel without that store (see zero_kernel in apply.cu),
-// so the large accumulators are cleared separately
-template <typename V>
-__global__ void __launch_bounds__(256) mg_zero_kernel(int64_t n, V* __restrict__ v, const int* __restrict__ done) {
-  if (done && *done) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = V(0);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    w[i] = invd[i] != V(0) ? (b ? b[i] : V(0)) - (q ? q[i] : V(0)) : V(0);
+    if (clear) clear[i] = V(0);
+  }
 }
 
 // the FP32 cycle's entry: b32 = r (rounded), its level-0 vectors' FP32 copy of the inverse diagonal
@@ -768,12 +764,8 @@ __global__ void __launch_bounds__(256) mg_round_kernel(int64_t n, const double* 
     b[i] = (float)a[i];
 }
 
-// accumulators of at least this many entries are cleared by mg_zero_kernel (smaller ones, which stay
-// in L2, by the consuming kernel itself)
-constexpr int64_t kSeparateZero = 1 << 20;
-
 // level 0 -> 1: b1 = P^T r by the vertex-wise transposed table, the residual r = b - q formed on
-// the fly on free DOFs (q = A x stays; the prolongation clears it)
+// the fly on free DOFs (q = A x)
 template <typename V>
 __global__ void __launch_bounds__(256) mg_restrict0_kernel(int64_t nv, const int* __restrict__ ptr,
                                                            const int* __restrict__ node, const double* __restrict__ w,
@@ -794,7 +786,7 @@ __global__ void __launch_bounds__(256) mg_restrict0_kernel(int64_t nv, const int
   }
 }
 
-// level 1 -> 0: x += P x1 on free DOFs; q (A x of the pre-smoothed x) cleared
+// level 1 -> 0: x += P x1 on free DOFs; q, an accumulator not read here, cleared
 template <typename V>
 __global__ void __launch_bounds__(256) mg_prolong0_kernel(int64_t nn, const int* __restrict__ idx,
                                                           const double* __restrict__ w, const V* __restrict__ x1,
@@ -884,17 +876,20 @@ __global__ void mg_pow_init_kernel(int64_t n, const double* __restrict__ invd, d
   }
 }
 
-// w = D^-1 q (q cleared), ||w||^2 reduced by the last block into *res
-__global__ void __launch_bounds__(256) mg_pow_step_kernel(int64_t n, double* __restrict__ q,
-                                                          const double* __restrict__ invd, double* __restrict__ w,
-                                                          double* __restrict__ part, unsigned* __restrict__ cnt,
-                                                          double* __restrict__ res, int given) {
+// ||w||^2 of w = D^-1 q (given: q on the free DOFs) reduced by the last block into *res; w is formed again
+// where it is used (mg_pow_norm_kernel)
+__device__ __forceinline__ double pow_entry(const double* q, const double* invd, int64_t i, int given) {
+  return given ? (invd[i] != 0.0 ? q[i] : 0.0) : invd[i] * q[i];
+}
+
+__global__ void __launch_bounds__(256) mg_pow_step_kernel(int64_t n, const double* __restrict__ q,
+                                                          const double* __restrict__ invd, double* __restrict__ part,
+                                                          unsigned* __restrict__ cnt, double* __restrict__ res,
+                                                          int given) {
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const double wi = given ? (invd[i] != 0.0 ? q[i] : 0.0) : invd[i] * q[i];
-    q[i] = 0.0;
-    w[i] = wi;
-    s += wi * wi;
+    const double wi = pow_entry(q, invd, i, given);
+    s = fma(wi, wi, s);
   }
   __shared__ int last;
   s = block_sum(s);
@@ -916,12 +911,19 @@ __global__ void __launch_bounds__(256) mg_pow_step_kernel(int64_t n, double* __r
   }
 }
 
-// v = w / ||w||
-__global__ void mg_pow_norm_kernel(int64_t n, const double* __restrict__ w, const double* __restrict__ res,
-                                   double* __restrict__ v) {
-  const double sc = 1.0 / sqrt(__ldcg(res));
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    v[i] = w[i] * sc;
+// v = w / ||w||, and `clear`, an accumulator that this kernel does not read, zeroed
+__global__ void __launch_bounds__(256) mg_pow_norm_kernel(int64_t n, const double* __restrict__ q,
+                                                          const double* __restrict__ invd,
+                                                          const double* __restrict__ res, double* __restrict__ v,
+                                                          double* __restrict__ clear, int given) {
+  __shared__ double s_sc;
+  if (threadIdx.x == 0) s_sc = 1.0 / sqrt(__ldcg(res));
+  __syncthreads();
+  const double sc = s_sc;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    v[i] = pow_entry(q, invd, i, given) * sc;
+    if (clear) clear[i] = 0.0;
+  }
 }
 
 __global__ void mg_pow_final_kernel(const double* __restrict__ res, double* __restrict__ lmax) {
@@ -969,13 +971,13 @@ void mg_release(mto_handle h) {
       cudaFree(p);
   h->mg.clear();
   for (void* p : {(void*)h->mg_pidx, (void*)h->mg_pw, (void*)h->mg_rptr, (void*)h->mg_rnode, (void*)h->mg_rw,
-                  (void*)h->mg_btab, (void*)h->mg_v0, (void*)h->mg_q0, (void*)h->mg_d0, (void*)h->mg_f32,
+                  (void*)h->mg_btab, (void*)h->mg_v0, (void*)h->mg_q0, (void*)h->mg_d0, (void*)h->mg_w0, (void*)h->mg_f32,
                   (void*)h->mg_Ainv,
                   (void*)h->mg_Awork,
                   (void*)h->mg_lmax, (void*)h->mg_coef, (void*)h->mg_part, (void*)h->mg_cnt, (void*)h->mg_res})
     cudaFree(p);
   h->mg_pidx = nullptr;
-  h->mg_pw = h->mg_rw = h->mg_btab = h->mg_v0 = h->mg_q0 = h->mg_d0 = h->mg_Ainv = h->mg_lmax = nullptr;
+  h->mg_pw = h->mg_rw = h->mg_btab = h->mg_v0 = h->mg_q0 = h->mg_d0 = h->mg_w0 = h->mg_Ainv = h->mg_lmax = nullptr;
   h->mg_f32 = nullptr;
   h->mg_Awork = nullptr;
   h->mg_coef = nullptr;
@@ -1100,8 +1102,8 @@ mto_status mg_setup(mto_handle h) {
   MTO_TRY(mto_cuda_check(h, cudaMemcpy(h->mg_rnode, rnode.data(), rnode.size() * sizeof(int), cudaMemcpyHostToDevice), "upload"));
   MTO_TRY(mto_cuda_check(h, cudaMemcpy(h->mg_rw, rw.data(), rw.size() * sizeof(double), cudaMemcpyHostToDevice), "upload"));
 
-  for (double** v : {&h->mg_v0, &h->mg_q0, &h->mg_d0}) MTO_TRY(mto_alloc(h, v, h->ndof));
-  MTO_TRY(mto_alloc(h, &h->mg_f32, (size_t)6 * h->ndof));
+  for (double** v : {&h->mg_v0, &h->mg_q0, &h->mg_d0, &h->mg_w0}) MTO_TRY(mto_alloc(h, v, h->ndof));
+  MTO_TRY(mto_alloc(h, &h->mg_f32, (size_t)7 * h->ndof));
   MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->mg_q0, 0, h->ndof * sizeof(double), h->stream), "memset"));
   MTO_TRY(mto_alloc(h, &h->mg_Ainv, (size_t)ncoarse * ncoarse));
   const StripGeom sg = strip_geom(h->mg.back());
@@ -1188,21 +1190,23 @@ mto_status mg_power(mto_handle h, int level, double* lmax_out) {
   mg_pow_init_kernel<<<grd, 256, 0, h->stream>>>(n, invd, v, q);
   MTO_TRY(mto_after_launch(h, "mg_pow_init_kernel"));
   const bool block = fine && h->mg_block;   // lmax of M^-1 A, M^-1 the element-block inverse
+  // the fine operator adds into q: the kernel that normalises clears the accumulator it does not read
+  double* other = w;
   for (int it = 0; it < kPowerIts; ++it) {
     if (fine) MTO_TRY(apply_fine(h, v, q, nullptr, h->mg_lead));
     else MTO_TRY(mg_level_apply(h, h->mg[level], v, q, nullptr));
     if (block) {
-      mg_block_resid_kernel<double><<<grd, 256, 0, h->stream>>>(n, nullptr, q, invd, w, nullptr);   // w = -A v
+      mg_block_resid_kernel<double><<<grd, 256, 0, h->stream>>>(n, nullptr, q, h->mg_w0, invd, w, nullptr);   // w = -A v
       MTO_TRY(mto_after_launch(h, "mg_block_resid_kernel"));
-      mg_zero_kernel<double><<<grd, 256, 0, h->stream>>>(n, q, nullptr);
-      MTO_TRY(mto_after_launch(h, "mg_zero_kernel"));
-      MTO_TRY(apply_block(h, w, q, nullptr, h->mg_lead));
+      MTO_TRY(apply_block(h, w, h->mg_w0, nullptr, h->mg_lead));
     }
-    mg_pow_step_kernel<<<grd, 256, 0, h->stream>>>(n, q, invd, w, h->mg_part, h->mg_cnt, h->mg_res, block);
+    const double* y = block ? h->mg_w0 : q;
+    mg_pow_step_kernel<<<vec_blocks(n), 256, 0, h->stream>>>(n, y, invd, h->mg_part, h->mg_cnt, h->mg_res, block);
     MTO_TRY(mto_after_launch(h, "mg_pow_step_kernel"));
     if (it + 1 < kPowerIts) {
-      mg_pow_norm_kernel<<<grd, 256, 0, h->stream>>>(n, w, h->mg_res, v);
+      mg_pow_norm_kernel<<<grd, 256, 0, h->stream>>>(n, y, invd, h->mg_res, v, block ? q : (fine ? other : nullptr), block);
       MTO_TRY(mto_after_launch(h, "mg_pow_norm_kernel"));
+      if (fine && !block) std::swap(q, other);
     }
   }
   mg_pow_final_kernel<<<1, 32, 0, h->stream>>>(h->mg_res, lmax_out);
@@ -1363,18 +1367,23 @@ mto_status fine_apply(mto_handle h, const float* x, float* y, const int* done, b
   return block ? apply_block32(h, x, y, done) : apply_fine32(h, x, y, done);
 }
 
-// One V-cycle in vector type V.  Level-0 vectors: b (the residual), x (the output), q (A x, kept
-// zero between uses), d (Chebyshev direction), v (element-block scratch), invd.  With dot_part
+// One V-cycle in vector type V.  Level-0 vectors: b (the residual), x (the output), q (A x, zero between
+// cycles), d (Chebyshev direction), v (element-block residual, or the second accumulator of Jacobi
+// smoothing), w (the blocks' accumulator), invd.  With dot_part
 // set, the last smoothing step also reduces b^T x into *dot_res; with zout set (the FP32 cycle),
 // that step writes x to zout in FP64 and takes the reduction's b from bout.
 template <typename V>
-mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, const V* invd0, int degree,
+mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, V* w0, const V* invd0, int degree,
                     const int* done, double* dot_part, unsigned* dot_cnt, double* dot_res, double* zout,
                     const double* bout) {
   const int nl = (int)h->mg.size();
   const bool lead = h->mg_lead;
-  auto smooth = [&](int lev, const V* b, V* x, V* q, V* d, const V* invd, int64_t n, bool pre,
-                    bool last) -> mto_status {
+  // Accumulators of the level-0 operator: `acc` is zero before every operator launch; the kernel that
+  // consumes it clears `other` and the two change places (an even number of times per cycle, so a
+  // captured cycle starts with the same one).  Block smoothing keeps the operator in acc and the blocks
+  // in w0, each cleared by the kernel that consumes the other.
+  V *acc = q0, *other = v0;
+  auto smooth = [&](int lev, const V* b, V* x, V* d, const V* invd, int64_t n, bool pre, bool last) -> mto_status {
     const int k = lev < 0 ? degree : (h->mg_q1deg > 0 ? h->mg_q1deg : kCoarseDegree);
     const double2* cf = h->mg_coef + (size_t)(lev + 1) * kMaxDegree;
     const int grd = vec_grid(n);
@@ -1396,39 +1405,37 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, const
     const bool block = h->mg_block;   // element-block (additive Schwarz) smoothing of level 0
     for (int s = 0; s < k; ++s) {
       const bool skip_apply = pre && s == 0;   // x = 0: A x = 0
-      if (!skip_apply) MTO_TRY(fine_apply(h, x, q, done, lead, false));
-      if (block) {   // q <- M^-1 (b - A x)
+      if (!skip_apply) MTO_TRY(fine_apply(h, x, acc, done, lead, false));
+      const V* q = skip_apply ? nullptr : acc;
+      V* clear = skip_apply ? nullptr : other;
+      if (block) {   // w <- M^-1 (b - A x)
         {
           TimedScope ts(h, F_PRECOND);
-          mg_block_resid_kernel<V><<<grd, 256, 0, h->stream>>>(n, b, q, invd, v0, done);
+          mg_block_resid_kernel<V><<<grd, 256, 0, h->stream>>>(n, b, q, w0, invd, v0, done);
           MTO_TRY(mto_after_launch(h, "mg_block_resid_kernel"));
-          mg_zero_kernel<V><<<grd, 256, 0, h->stream>>>(n, q, done);
-          MTO_TRY(mto_after_launch(h, "mg_zero_kernel"));
         }
-        MTO_TRY(fine_apply(h, v0, q, done, lead, true));
+        MTO_TRY(fine_apply(h, v0, w0, done, lead, true));
+        q = w0;
+        clear = skip_apply ? nullptr : acc;
       }
       TimedScope ts(h, F_PRECOND);
       const bool fin = last && s == k - 1;
-      const bool sep = n >= kSeparateZero;
-      mg_cheb_kernel<V><<<grd, 256, 0, h->stream>>>(n, b, q, invd, x, d, cf, s, pre && s == 0, done,
-                                                     fin ? dot_part : nullptr, dot_cnt, dot_res, block, !sep,
-                                                     fin ? zout : nullptr, bout);
+      mg_cheb_kernel<V><<<fin ? vec_blocks(n) : grd, 256, 0, h->stream>>>(
+          n, b, q, clear, invd, x, d, cf, s, pre && s == 0, done, fin ? dot_part : nullptr, dot_cnt, dot_res, block,
+          fin ? zout : nullptr, bout);
       MTO_TRY(mto_after_launch(h, "mg_cheb_kernel"));
-      if (sep) {
-        mg_zero_kernel<V><<<grd, 256, 0, h->stream>>>(n, q, done);
-        MTO_TRY(mto_after_launch(h, "mg_zero_kernel"));
-      }
+      if (!block && !skip_apply) std::swap(acc, other);
     }
     return MTO_OK;
   };
   // level 0 pre-smoothing and residual
-  MTO_TRY(smooth(-1, b0, x0, q0, d0, invd0, h->ndof, true, false));
-  MTO_TRY(fine_apply(h, x0, q0, done, lead, false));
+  MTO_TRY(smooth(-1, b0, x0, d0, invd0, h->ndof, true, false));
+  MTO_TRY(fine_apply(h, x0, acc, done, lead, false));
   {
     TimedScope ts(h, F_PRECOND);
     const LevelV<V> L1 = level_vecs<V>(h->mg[0]);
     mg_restrict0_kernel<V><<<vec_grid(h->mg[0].nv), 256, 0, h->stream>>>(
-        h->mg[0].nv, h->mg_rptr, h->mg_rnode, h->mg_rw, b0, q0, invd0, L1.mask, L1.b, done);
+        h->mg[0].nv, h->mg_rptr, h->mg_rnode, h->mg_rw, b0, acc, invd0, L1.mask, L1.b, done);
     MTO_TRY(mto_after_launch(h, "mg_restrict0_kernel"));
   }
   // Q1 levels down
@@ -1436,7 +1443,7 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, const
     const MGLevel& L = h->mg[l];
     const MGLevel& C = h->mg[l + 1];
     const LevelV<V> lv = level_vecs<V>(L), cv = level_vecs<V>(C);
-    MTO_TRY(smooth(l, lv.b, lv.x, lv.q, lv.d, lv.invd, L.n, true, false));
+    MTO_TRY(smooth(l, lv.b, lv.x, lv.d, lv.invd, L.n, true, false));
     TimedScope ts(h, F_PRECOND);
     MTO_TRY(mg_level_apply(h, L, lv.x, lv.q, done));
     mg_restrict_h_kernel<V><<<vec_grid(C.nv), 256, 0, h->stream>>>(C.nx, C.ny, L.nx, L.ny, lv.b, lv.q, lv.invd,
@@ -1462,39 +1469,43 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, const
                                                                      done);
       MTO_TRY(mto_after_launch(h, "mg_prolong_h_kernel"));
     }
-    MTO_TRY(smooth(l, lv.b, lv.x, lv.q, lv.d, lv.invd, L.n, false, false));
+    MTO_TRY(smooth(l, lv.b, lv.x, lv.d, lv.invd, L.n, false, false));
   }
   {
     TimedScope ts(h, F_PRECOND);
     const LevelV<V> L1 = level_vecs<V>(h->mg[0]);
     mg_prolong0_kernel<V><<<vec_grid(h->n_nodes), 256, 0, h->stream>>>(h->n_nodes, h->mg_pidx, h->mg_pw, L1.x,
-                                                                        invd0, x0, q0, done);
+                                                                        invd0, x0, h->mg_block ? acc : other, done);
     MTO_TRY(mto_after_launch(h, "mg_prolong0_kernel"));
+    if (!h->mg_block) std::swap(acc, other);
   }
-  return smooth(-1, b0, x0, q0, d0, invd0, h->ndof, false, true);
+  return smooth(-1, b0, x0, d0, invd0, h->ndof, false, true);
 }
 
 }  // namespace
 
-// z = M^-1 r: one V-cycle, with r^T z into *dot_res when dot_part is set (block partials in
+// the FP32 cycle's rounded residual, for the PCG kernel that updates r (null when the cycle is in FP64)
+float* mg_residual32(mto_handle h) { return mg_fp32_cycle(h) ? h->mg_f32 : nullptr; }
+
+// z = M^-1 r (rounded: r is already rounded into the FP32 cycle's b): one V-cycle, with r^T z into *dot_res when dot_part is set (block partials in
 // dot_part, counter dot_cnt).  FP64 cycle: level-0 vectors b = r, x = z, q = mg_q0, d = mg_d0,
 // v = mg_v0.  FP32 cycle (the cycle on FP32 copies of a mixed build): r rounded into its own FP32
 // level-0 vectors, z and r^T z written in FP64 by the last smoothing step.
 mto_status mg_vcycle(mto_handle h, const double* r, double* z, int degree, const int* done, double* dot_part,
-                     unsigned* dot_cnt, double* dot_res) {
+                     unsigned* dot_cnt, double* dot_res, bool rounded) {
   if (mg_fp32_cycle(h)) {
     const int64_t n = h->ndof;
     float* F = h->mg_f32;
     float *b = F, *x = F + n, *q = F + 2 * n, *d = F + 3 * n, *v = F + 4 * n;
     const float* invd = F + 5 * n;
-    {
+    if (!rounded) {
       TimedScope ts(h, F_PRECOND);
       mg_demote_kernel<<<vec_grid(n), 256, 0, h->stream>>>(n, r, b, done);
       MTO_TRY(mto_after_launch(h, "mg_demote_kernel"));
     }
-    return mg_cycle<float>(h, b, x, q, d, v, invd, degree, done, dot_part, dot_cnt, dot_res, z, r);
+    return mg_cycle<float>(h, b, x, q, d, v, F + 6 * n, invd, degree, done, dot_part, dot_cnt, dot_res, z, r);
   }
-  return mg_cycle<double>(h, r, z, h->mg_q0, h->mg_d0, h->mg_v0, h->invd64, degree, done, dot_part, dot_cnt,
+  return mg_cycle<double>(h, r, z, h->mg_q0, h->mg_d0, h->mg_v0, h->mg_w0, h->invd64, degree, done, dot_part, dot_cnt,
                           dot_res, nullptr, r);
 }
 

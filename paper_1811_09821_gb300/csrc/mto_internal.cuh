@@ -225,7 +225,7 @@ struct mto_handle_s {
   double* mg_rw = nullptr;
   double* mg_btab = nullptr;                   // bilinear weights at the GLL nodes, per order
   int mg_boff[mto::kPMaxTab + 2] = {0};
-  double *mg_v0 = nullptr, *mg_q0 = nullptr, *mg_d0 = nullptr;   // [ndof] fine-level scratch
+  double *mg_v0 = nullptr, *mg_q0 = nullptr, *mg_d0 = nullptr, *mg_w0 = nullptr;   // [ndof] fine-level scratch
   double* mg_Ainv = nullptr;                   // coarsest level: its inverse [N][N] in line order,
   double* mg_Awork = nullptr;                  // and the blocks of its elimination
   double* mg_lmax = nullptr;                   // [levels] Chebyshev upper bounds
@@ -239,7 +239,7 @@ struct mto_handle_s {
   double mg_ratio = 0.0;                       // MTO_MG_RATIO: Chebyshev interval lmax / ratio .. lmax (0: 100)
   int mg_q1deg = 0;                            // MTO_MG_Q1DEG: smoothing degree on the Q1 levels (0: 4)
   bool mg_lead = true;   // mg_operator: the cycle of a mixed build on FP32 copies with FP32 vectors
-  float* mg_f32 = nullptr;   // [6][ndof] the FP32 cycle's level-0 vectors b, x, q, d, v and invd
+  float* mg_f32 = nullptr;   // [7][ndof] the FP32 cycle's level-0 vectors b, x, q, d, v, invd and w
   int mg_smoother = 0;                         // fine-level smoothing: MTO_SMOOTH_JACOBI or MTO_SMOOTH_BLOCK
   bool mg_block = false;                       // element-block smoothing in use (set by mg_build)
   std::vector<mto::GraphEntry*> graphs;
@@ -450,7 +450,8 @@ mto_status mg_set_masks(mto_handle h);                                  // suppo
 mto_status mg_build(mto_handle h);                                      // Galerkin operators, bounds
 mto_status mg_select_smoother(mto_handle h, int smoother);              // MTO_SMOOTH_* for next solves
 mto_status mg_vcycle(mto_handle h, const double* r, double* z, int degree, const int* done, double* dot_part,
-                     unsigned* dot_cnt, double* dot_res);
+                     unsigned* dot_cnt, double* dot_res, bool rounded);
+float* mg_residual32(mto_handle h);                                     // the FP32 cycle's copy of r (else null)
 void mg_release(mto_handle h);
 // tc.cu
 mto_status tc_tables(mto_handle h);
@@ -489,6 +490,7 @@ mto_status map_update(mto_handle h, const double* ga, const double* gd, const do
                       const mto_indicator_opts* o, int32_t* pn, int32_t* dn, int8_t* th);
 mto_status oc_update(mto_handle h, const double* rho, const double* dc, double volfrac, double move,
                      double eta, double* rho_new, double* lambda);
+int vec_blocks(int64_t n);                                            // grid of a vector kernel of 256 threads
 // reductions shared by several units
 mto_status dot64(mto_handle h, const double* a, const double* b, int64_t n, double* out_dev);
 mto_status sum64(mto_handle h, const double* a, int64_t n, double* out_dev);
