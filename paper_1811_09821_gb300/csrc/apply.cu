@@ -1573,6 +1573,7 @@ mto_status solve(mto_handle h, const double* f, double* u, const mto_solve_opts*
     // FP64 residual with the FP64 element matrices
     h->inner_split = false;
     MTO_TRY(true_residual(h, f, u, nrm, &rr, &ff));
+    MTO_TRY(mg_build_check(h));
     if (h->solve_log)
       std::fprintf(stderr, "mto_solve: step %d inner_iters %d relres %.3e split %d wall_ms %.1f\n", outer, last_it,
                    ff > 0 ? std::sqrt(rr / ff) : 0.0, (int)split,
@@ -1692,6 +1693,13 @@ mto_status job_on_residual(BatchJob& j) {
   mto_handle h = j.h;
   const mto_solve_opts* o = j.o;
   residual_take(h, j.nrm, &j.rr, &j.ff);
+  {
+    const mto_status sb = mg_build_check(h);
+    if (sb != MTO_OK) {
+      job_finish(j, sb);
+      return MTO_OK;
+    }
+  }
   if (o->precision == MTO_MIXED && j.rr_prev > 0.0 && std::sqrt(j.rr / j.rr_prev) > 10.0 * j.asked) j.split = false;
   j.rr_prev = j.rr;
   if (!std::isfinite(j.rr)) {

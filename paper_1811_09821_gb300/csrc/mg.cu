@@ -358,7 +358,8 @@ __global__ void mg_invd_kernel(int64_t n, const double* __restrict__ mask, doubl
 constexpr int kLineMax = 64;      // 2 (min(nx, ny) + 1) <= 64 for at most 2048 DOFs
 constexpr int kInvWarps = 8;      // warps holding the matrix of an inversion, two more form the multipliers
 constexpr int kInvThreads = 32 * (kInvWarps + 2);
-constexpr int kInvEntries = (kLineMax * (kLineMax + 1) / 2 + 32 * kInvWarps - 1) / (32 * kInvWarps);
+// packed entries per thread for m DOFs a line (the kernels are instantiated for 1, 2, 4, 6 and 9)
+constexpr int inv_entries(int m) { return (m * (m + 1) / 2 + 32 * kInvWarps - 1) / (32 * kInvWarps); }
 
 struct StripGeom {
   int nx, ny;    // elements of the level
@@ -384,31 +385,27 @@ __device__ __forceinline__ double newton_rcp(double d) {
 
 // In-place symmetric inversion (Gauss-Jordan sweeps, SPD: no pivoting) of an m x m matrix held as its
 // packed lower triangle over the threads of kInvWarps warps: entry e of thread t is (ij[e] >> 8,
-// ij[e] & 255), ij < 0 beyond the end.  On return a = -inverse.  While those warps apply a pivot to
-// the matrix, two helper warps already form the reciprocal and the multipliers of the next one.
+// ij[e] & 255), ij < 0 beyond the end.  On return a = -inverse.  Two helper warps form each pivot's
+// reciprocal and multipliers.
 // cb, ub: [2][kLineMax] shared.  Returns false (in every thread) at a pivot that is not positive.
-__device__ bool sym_invert(int m, double (&a)[kInvEntries], const int (&ij)[kInvEntries], double (*cb)[kLineMax],
-                           double (*ub)[kLineMax], double* inv) {
+template <int E>
+__device__ __forceinline__ bool sym_invert(int m, double (&a)[E], const int (&ij)[E], double (*cb)[kLineMax],
+                                           double (*ub)[kLineMax], double* inv) {
   const int t = threadIdx.x;
   const bool helper = t >= 32 * kInvWarps;
   const int ht = t - 32 * kInvWarps;
   bool ok = true;
-  auto publish = [&](int k) {   // column k of the current matrix
-#pragma unroll
-    for (int e = 0; e < kInvEntries; ++e) {
-      if (ij[e] < 0) continue;
-      const int i = ij[e] >> 8, j = ij[e] & 255;
-      if (j == k) cb[k & 1][i] = a[e];
-      else if (i == k) cb[k & 1][j] = a[e];
-    }
-  };
   auto multipliers = [&](int k) {
-    const double d = cb[k & 1][k];
-    const double r = newton_rcp(d);
+    const double ck = ht < m ? cb[k & 1][ht] : 0.0;
+    const double r = newton_rcp(cb[k & 1][k]);
     if (ht == 0) inv[k & 1] = r;
-    if (ht < m) ub[k & 1][ht] = cb[k & 1][ht] * r;
+    if (ht < m) ub[k & 1][ht] = ck * r;
   };
-  if (!helper) publish(0);
+  if (!helper) {
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+      if (ij[e] >= 0 && (ij[e] & 255) == 0) cb[0][ij[e] >> 8] = a[e];
+  }
   __syncthreads();
   if (helper) multipliers(0);
   __syncthreads();
@@ -416,44 +413,38 @@ __device__ bool sym_invert(int m, double (&a)[kInvEntries], const int (&ij)[kInv
     const double* c = cb[k & 1];
     const double* u = ub[k & 1];
     ok = ok && c[k] > 0.0;
-    auto update = [&](int e, int i, int j) {
-      if (j == k) a[e] = i == k ? -inv[k & 1] : u[i];
-      else if (i == k) a[e] = u[j];
-      else a[e] = fma(-u[i], c[j], a[e]);
-    };
-    if (!helper && k + 1 < m) {   // the next pivot's column first
+    const int nk = k + 1;
+    if (!helper) {
+      // every entry in one go, without branches; those of the next pivot's column (row) are published
+      const double piv = inv[k & 1];
 #pragma unroll
-      for (int e = 0; e < kInvEntries; ++e) {
-        if (ij[e] < 0) continue;
-        const int i = ij[e] >> 8, j = ij[e] & 255;
-        if (i == k + 1 || j == k + 1) {
-          update(e, i, j);
-          cb[(k + 1) & 1][j == k + 1 ? i : j] = a[e];
-        }
+      for (int e = 0; e < E; ++e) {
+        const int i = (ij[e] >> 8) & 255, j = ij[e] & 255;   // entries beyond the end compute and keep nothing
+        const double ui = u[i], uj = u[j], cj = c[j];
+        double v = fma(-ui, cj, a[e]);
+        v = j == k ? ui : v;
+        v = i == k ? uj : v;
+        v = (i == k && j == k) ? -piv : v;
+        a[e] = v;
+        if (ij[e] >= 0 && (i == nk || j == nk)) cb[nk & 1][j == nk ? i : j] = v;
       }
     }
-    __syncthreads();
-    if (helper) {
-      if (k + 1 < m) multipliers(k + 1);
-    } else {
-#pragma unroll
-      for (int e = 0; e < kInvEntries; ++e) {
-        if (ij[e] < 0) continue;
-        const int i = ij[e] >> 8, j = ij[e] & 255;
-        if (k + 1 >= m || (i != k + 1 && j != k + 1)) update(e, i, j);
-      }
+    if (nk < m) {
+      __syncthreads();
+      if (helper) multipliers(nk);
     }
     __syncthreads();
   }
   return ok;
 }
 
-__device__ void packed_owner(int m, int (&ij)[kInvEntries]) {
+template <int E>
+__device__ __forceinline__ void packed_owner(int m, int (&ij)[E]) {
   const int t = threadIdx.x;
 #pragma unroll
-  for (int e = 0; e < kInvEntries; ++e) {
+  for (int e = 0; e < E; ++e) {
     const int idx = t + 32 * kInvWarps * e;
-    ij[e] = -1;
+    ij[e] = -65536;   // negative, and (0, 0) by its low bits
     if (t >= 32 * kInvWarps || idx >= m * (m + 1) / 2) continue;
     int i = (int)((sqrtf(8.0f * (float)idx + 1.0f) - 1.0f) * 0.5f);
     while (i * (i + 1) / 2 > idx) --i;
@@ -476,6 +467,7 @@ __device__ __forceinline__ double strip_entry(const StripGeom& g, const double* 
 
 // The elimination.  middle = 0: block 0 the lines 0 .. k - 1, block 1 the lines nl - 1 .. k + 1;
 // middle = 1: the line k.  The inverse of line l's Schur complement goes to Gc + l m^2 (full).
+template <int E>
 __global__ void __launch_bounds__(kInvThreads) mg_strip_chain_kernel(StripGeom g, int middle,
                                                                      const double* __restrict__ S,
                                                                      const double* __restrict__ mask, double* Gc,
@@ -484,61 +476,79 @@ __global__ void __launch_bounds__(kInvThreads) mg_strip_chain_kernel(StripGeom g
   const int m = g.m, ld = m + 1, t = threadIdx.x, kmid = g.nl / 2;
   double* G = shm;               // [m][ld] inverse of the line before
   double* F = G + m * ld;        // [m][ld] C^T G
-  double* E = F + m * ld;        // [m][6] C^T: this line's rows
+  double* C = F + m * ld;        // [m][6] C^T: this line's rows
   __shared__ double cb[2][kLineMax], ub[2][kLineMax], inv[2];
-  double a[kInvEntries];
-  int ij[kInvEntries];
-  packed_owner(m, ij);
+  double a[E], an[E];
+  int ij[E];
+  packed_owner<E>(m, ij);
+  constexpr int kC = (6 * kLineMax + kInvThreads - 1) / kInvThreads;   // couplings per thread
+  double cn[kC];
   bool ok = true;
-  // a -= C^T G C for the line l + step, whose inverse is in G
-  auto subtract = [&](int l, int step) {
-    for (int k = t; k < 6 * m; k += kInvThreads) {
-      const int i = k / 6, j = 2 * (i >> 1) - 2 + k % 6;   // the DOFs of positions a - 1 .. a + 1
-      E[k] = (j >= 0 && j < m) ? strip_entry(g, S, mask, l, step, i, j) : 0.0;
+  auto load_diag = [&](int l, double (&d)[E]) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) d[e] = ij[e] < 0 ? 0.0 : strip_entry(g, S, mask, l, 0, ij[e] >> 8, ij[e] & 255);
+  };
+  auto load_coupling = [&](int l, int step, double (&d)[kC]) {
+#pragma unroll
+    for (int q = 0; q < kC; ++q) {
+      const int k = t + kInvThreads * q, i = k / 6, j = 2 * (i >> 1) - 2 + k % 6;   // positions a - 1 .. a + 1
+      d[q] = (k < 6 * m && j >= 0 && j < m) ? strip_entry(g, S, mask, l, step, i, j) : 0.0;
     }
+  };
+  // a -= C^T G C for a line whose inverse is in G and whose couplings are given
+  auto subtract = [&](const double (&d)[kC]) {
+#pragma unroll
+    for (int q = 0; q < kC; ++q)
+      if (t + kInvThreads * q < 6 * m) C[t + kInvThreads * q] = d[q];
     __syncthreads();
     for (int k = t; k < m * m; k += kInvThreads) {
       const int i = k / m, j = k % m, j0 = 2 * (i >> 1) - 2;
       double f = 0.0;
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        const int r = j0 + c;
-        if (r >= 0 && r < m) f = fma(E[6 * i + c], G[r * ld + j], f);
+        const int r = min(max(j0 + c, 0), m - 1);   // the couplings beyond the ends are zero
+        f = fma(C[6 * i + c], G[r * ld + j], f);
       }
       F[i * ld + j] = f;
     }
     __syncthreads();
 #pragma unroll
-    for (int e = 0; e < kInvEntries; ++e) {
+    for (int e = 0; e < E; ++e) {
       if (ij[e] < 0) continue;
       const int i = ij[e] >> 8, j = ij[e] & 255, j0 = 2 * (j >> 1) - 2;
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        const int r = j0 + c;
-        if (r >= 0 && r < m) a[e] = fma(-F[i * ld + r], E[6 * j + c], a[e]);
+        const int r = min(max(j0 + c, 0), m - 1);
+        a[e] = fma(-F[i * ld + r], C[6 * j + c], a[e]);
       }
     }
     __syncthreads();
   };
   const int dir = blockIdx.x == 0 ? 1 : -1;
   const int n = middle ? 1 : (dir > 0 ? kmid : g.nl - 1 - kmid);
+  if (n > 0) load_diag(middle ? kmid : (dir > 0 ? 0 : g.nl - 1), an);
   for (int s = 0; s < n; ++s) {
     const int l = middle ? kmid : (dir > 0 ? s : g.nl - 1 - s);
 #pragma unroll
-    for (int e = 0; e < kInvEntries; ++e) a[e] = ij[e] < 0 ? 0.0 : strip_entry(g, S, mask, l, 0, ij[e] >> 8, ij[e] & 255);
+    for (int e = 0; e < E; ++e) a[e] = an[e];
     if (middle) {
       for (int step = -1; step <= 1; step += 2) {
         if (l + step < 0 || l + step >= g.nl) continue;
         const double* src = Gc + (size_t)(l + step) * m * m;
+        load_coupling(l, step, cn);
         for (int k = t; k < m * m; k += kInvThreads) G[k / m * ld + k % m] = src[k];
-        subtract(l, step);
+        subtract(cn);
       }
     } else if (s > 0) {
-      subtract(l, -dir);
+      subtract(cn);
     }
-    ok = sym_invert(m, a, ij, cb, ub, inv) && ok;
+    if (s + 1 < n) {   // the next line's entries, in flight during the inversion
+      load_diag(l + dir, an);
+      load_coupling(l + dir, -dir, cn);
+    }
+    ok = sym_invert<E>(m, a, ij, cb, ub, inv) && ok;
 #pragma unroll
-    for (int e = 0; e < kInvEntries; ++e) {
+    for (int e = 0; e < E; ++e) {
       if (ij[e] < 0) continue;
       const int i = ij[e] >> 8, j = ij[e] & 255;
       G[i * ld + j] = G[j * ld + i] = -a[e];
@@ -984,7 +994,7 @@ void mg_release(mto_handle h) {
   h->mg_part = h->mg_res = nullptr;
   h->mg_rptr = h->mg_rnode = nullptr;
   h->mg_cnt = nullptr;
-  h->mg_ok = h->mg_valid = false;
+  h->mg_ok = h->mg_valid = h->mg_unchecked = false;
 }
 
 // Level sizes, vertex maps and the level-0 <-> level-1 transfer tables (host, once per mesh).
@@ -1293,13 +1303,22 @@ mto_status mg_build(mto_handle h) {
     double* Gc = h->mg_Awork;
     MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->flags + 6, 0, sizeof(int), h->stream), "memset"));
     const size_t smem = sizeof(double) * (2 * g.m * (g.m + 1) + 6 * g.m);
-    if (smem > 48 * 1024)
-      MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(mg_strip_chain_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     (int)smem), "cudaFuncSetAttribute"));
-    for (int middle = 0; middle < 2; ++middle) {
-      mg_strip_chain_kernel<<<middle ? 1 : 2, kInvThreads, smem, h->stream>>>(g, middle, C.S, C.mask, Gc, h->flags + 6);
-      MTO_TRY(mto_after_launch(h, "mg_strip_chain_kernel"));
-    }
+    auto chain = [&](auto kernel) -> mto_status {
+      if (smem > 48 * 1024)
+        MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
+                               "cudaFuncSetAttribute"));
+      for (int middle = 0; middle < 2; ++middle) {
+        kernel<<<middle ? 1 : 2, kInvThreads, smem, h->stream>>>(g, middle, C.S, C.mask, Gc, h->flags + 6);
+        MTO_TRY(mto_after_launch(h, "mg_strip_chain_kernel"));
+      }
+      return MTO_OK;
+    };
+    const int ne = inv_entries(g.m);
+    if (ne <= 1) MTO_TRY(chain(mg_strip_chain_kernel<1>));
+    else if (ne <= 2) MTO_TRY(chain(mg_strip_chain_kernel<2>));
+    else if (ne <= 4) MTO_TRY(chain(mg_strip_chain_kernel<4>));
+    else if (ne <= 6) MTO_TRY(chain(mg_strip_chain_kernel<6>));
+    else MTO_TRY(chain(mg_strip_chain_kernel<9>));
     const int per = (g.m + kStripCols - 1) / kStripCols;
     mg_strip_columns_kernel<<<g.nl * per, kStripThreads, sizeof(double) * g.m * (3 * kStripCols + 6), h->stream>>>(
         g, C.S, C.mask, Gc, h->mg_Ainv);
@@ -1329,14 +1348,23 @@ mto_status mg_build(mto_handle h) {
   MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->mg_f32, 0, 5 * h->ndof * sizeof(float), h->stream), "memset"));
   mg_round_kernel<<<vec_grid(h->ndof), 256, 0, h->stream>>>(h->ndof, h->invd64, h->mg_f32 + 5 * h->ndof);
   MTO_TRY(mto_after_launch(h, "mg_round_kernel"));
-  int err = 0;
+  // the coarsest operator's definiteness is read back with the caller's next synchronisation
+  // (mg_build_check), so that the builds of a batch run side by side
+  h->host_flags[8] = 0;
   MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(h->host_flags + 8, h->flags + 6, sizeof(int), cudaMemcpyDeviceToHost,
                                             h->stream), "copy"));
-  MTO_TRY(mto_cuda_check(h, cudaStreamSynchronize(h->stream), "mg_build"));
-  err = h->host_flags[8];
-  if (err) return mto_fail(h, MTO_ENAN, "mg_build: coarsest operator not positive definite");
+  h->mg_unchecked = true;
   h->mg_valid = true;
   return MTO_OK;
+}
+
+// after a synchronisation that follows mg_build: its verdict, once
+mto_status mg_build_check(mto_handle h) {
+  if (!h->mg_unchecked) return MTO_OK;
+  h->mg_unchecked = false;
+  if (!h->host_flags[8]) return MTO_OK;
+  h->mg_valid = false;
+  return mto_fail(h, MTO_ENAN, "mg_build: coarsest operator not positive definite");
 }
 
 namespace {

@@ -217,6 +217,7 @@ struct mto_handle_s {
   // multigrid preconditioner: levels 1.. (Q1), fine-level transfer tables and work vectors
   std::vector<mto::MGLevel> mg;
   bool mg_ok = false, mg_valid = false;
+  bool mg_unchecked = false;                   // the last mg_build's verdict has not been read yet
   std::string mg_why;                          // why no hierarchy exists (mesh does not coarsen)
   int* mg_pidx = nullptr;                      // [n_nodes][4] Q1 vertices of each fine node
   double* mg_pw = nullptr;                     // [n_nodes][4] their bilinear weights
@@ -452,6 +453,7 @@ mto_status mg_select_smoother(mto_handle h, int smoother);              // MTO_S
 mto_status mg_vcycle(mto_handle h, const double* r, double* z, int degree, const int* done, double* dot_part,
                      unsigned* dot_cnt, double* dot_res, bool rounded);
 float* mg_residual32(mto_handle h);                                     // the FP32 cycle's copy of r (else null)
+mto_status mg_build_check(mto_handle h);                                // its verdict, after a synchronisation
 void mg_release(mto_handle h);
 // tc.cu
 mto_status tc_tables(mto_handle h);
