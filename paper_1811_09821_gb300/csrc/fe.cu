@@ -9,11 +9,30 @@
 namespace mto {
 namespace {
 
+// Values and derivatives of a (p, d) class's Lagrange polynomials at the (p+1)-point Gauss rule of every
+// subcell interval: T = [values | derivatives][d][n1 points][n1], then the n1 weights.
+__global__ void __launch_bounds__(256) k0_point_kernel(int p, int d, double* __restrict__ T) {
+  __shared__ double z[kPMaxTab + 1], gx[kPMaxTab + 1], gw[kPMaxTab + 1];
+  const int n1 = p + 1, nv = d * n1 * n1;
+  if (threadIdx.x == 0) gll_nodes(p, z);
+  if (threadIdx.x == 32) gauss_rule(n1, gx, gw);
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * nv; k += blockDim.x) {
+    const int r = k % nv, i = r / (n1 * n1), g = r / n1 % n1, a = r % n1;
+    const double xi = -1.0 + (2.0 * i + 1.0 + gx[g]) / d;
+    T[k] = k < nv ? lagrange_val(z, n1, a, xi) : lagrange_der(z, n1, a, xi);
+  }
+  for (int k = threadIdx.x; k < n1; k += blockDim.x) T[2 * nv + k] = gw[k];
+}
+
 // K0T[c][s] = integral over subcell s of (B^T D0 B)_{ij}, c = packed (i, j), unit modulus.
 // The (p+1) x (p+1) Gauss rule mapped to the subcell is exact (the integrand has degree <= 2p per
-// axis on an affine square).  One thread per (c, s).
-__global__ void k0_kernel(int p, int d, double nu, double hx, double hy, double* __restrict__ K0T) {
-  const int S = d * d, n1 = p + 1, ne = 2 * n1 * n1, P = packed_size(ne);
+// axis on an affine square).  One thread per (c, s), the 1D values from k0_point_kernel (each thread
+// forming its nodes, rule and polynomials took most of a first build: 80 ms of the 32 tables of an
+// adaptive 320 x 160 mesh).
+__global__ void __launch_bounds__(256) k0_kernel(int p, int d, double nu, double hx, double hy,
+                                                 const double* __restrict__ T, double* __restrict__ K0T) {
+  const int S = d * d, n1 = p + 1, ne = 2 * n1 * n1, P = packed_size(ne), nv = d * n1 * n1;
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= P * S) return;
   int c = idx / S, s = idx - c * S;
@@ -23,24 +42,22 @@ __global__ void k0_kernel(int p, int d, double nu, double hx, double hy, double*
     ++i;
   }
   int j = i + rem;
-  double z[kPMaxTab + 1], gx[kPMaxTab + 1], gw[kPMaxTab + 1];
-  gll_nodes(p, z);
-  gauss_rule(n1, gx, gw);
   const double f = 1.0 / (1.0 - nu * nu);
   const double D11 = f, D12 = f * nu, D33 = f * 0.5 * (1.0 - nu);
   const int si = s % d, sj = s / d;
   const int ni = i >> 1, ci = i & 1, nj = j >> 1, cj = j & 1;
   const int ai = ni % n1, bi = ni / n1, aj = nj % n1, bj = nj / n1;
+  const double* gw = T + 2 * nv;
   double sum = 0.0;
   for (int qy = 0; qy < n1; ++qy) {
-    double eta = -1.0 + (2.0 * sj + 1.0 + gx[qy]) / d;
+    const double *vy = T + (sj * n1 + qy) * n1, *dy = vy + nv;
     for (int qx = 0; qx < n1; ++qx) {
-      double xi = -1.0 + (2.0 * si + 1.0 + gx[qx]) / d;
+      const double *vx = T + (si * n1 + qx) * n1, *dx = vx + nv;
       double wq = gw[qx] * gw[qy] * (hx / (2.0 * d)) * (hy / (2.0 * d));
-      double Nxi = lagrange_der(z, n1, ai, xi) * lagrange_val(z, n1, bi, eta) * (2.0 / hx);
-      double Nyi = lagrange_val(z, n1, ai, xi) * lagrange_der(z, n1, bi, eta) * (2.0 / hy);
-      double Nxj = lagrange_der(z, n1, aj, xi) * lagrange_val(z, n1, bj, eta) * (2.0 / hx);
-      double Nyj = lagrange_val(z, n1, aj, xi) * lagrange_der(z, n1, bj, eta) * (2.0 / hy);
+      double Nxi = dx[ai] * vy[bi] * (2.0 / hx);
+      double Nyi = vx[ai] * dy[bi] * (2.0 / hy);
+      double Nxj = dx[aj] * vy[bj] * (2.0 / hx);
+      double Nyj = vx[aj] * dy[bj] * (2.0 / hy);
       // B columns: u_x -> (Nx, 0, Ny), u_y -> (0, Ny, Nx)
       double bi0 = ci == 0 ? Nxi : 0.0, bi1 = ci == 0 ? 0.0 : Nyi, bi2 = ci == 0 ? Nyi : Nxi;
       double bj0 = cj == 0 ? Nxj : 0.0, bj1 = cj == 0 ? 0.0 : Nyj, bj2 = cj == 0 ? Nyj : Nxj;
@@ -53,66 +70,62 @@ __global__ void k0_kernel(int p, int d, double nu, double hx, double hy, double*
 
 // Scalar load-transfer table of the QR indicator for order p -> p + 1:
 // R = M^(p+1,p) M^(p)^-1, M^(p)_{kl} = int N_k^p N_l^p, M^(p+1,p)_{jk} = int N_j^(p+1) N_k^p,
-// integrated exactly by a (p+2)-point Gauss rule per axis.  Thread 0 forms and factors M^(p)
-// (Cholesky) in shared memory; thread t solves for row t of R.
-__global__ void qr_table_kernel(int p, double hx, double hy, double* __restrict__ R) {
-  constexpr int NA = (kPMaxTab) * (kPMaxTab);        // max (p+1)^2 for p <= MTO_P_MAX
-  constexpr int NB = (kPMaxTab + 1) * (kPMaxTab + 1);
-  __shared__ double M[NA * NA];
-  __shared__ double Mb[NB * NA];
-  const int n1 = p + 1, n2 = p + 2, na = n1 * n1, nb = n2 * n2;
-  if (threadIdx.x == 0) {
-    double z1[kPMaxTab + 1], z2[kPMaxTab + 1], gx[kPMaxTab + 2], gw[kPMaxTab + 2];
-    gll_nodes(p, z1);
-    gll_nodes(p + 1, z2);
-    int nq = p + 2;
-    gauss_rule(nq, gx, gw);
-    for (int k = 0; k < na * na; ++k) M[k] = 0.0;
-    for (int k = 0; k < nb * na; ++k) Mb[k] = 0.0;
-    const double jac = 0.25 * hx * hy;
-    for (int qy = 0; qy < nq; ++qy)
-      for (int qx = 0; qx < nq; ++qx) {
-        double w = gw[qx] * gw[qy] * jac;
-        double N1[NA], N2[NB];
-        for (int b = 0; b < n1; ++b)
-          for (int a = 0; a < n1; ++a)
-            N1[b * n1 + a] = lagrange_val(z1, n1, a, gx[qx]) * lagrange_val(z1, n1, b, gx[qy]);
-        for (int b = 0; b < n2; ++b)
-          for (int a = 0; a < n2; ++a)
-            N2[b * n2 + a] = lagrange_val(z2, n2, a, gx[qx]) * lagrange_val(z2, n2, b, gx[qy]);
-        for (int k = 0; k < na; ++k)
-          for (int l = 0; l < na; ++l) M[k * na + l] += w * N1[k] * N1[l];
-        for (int j = 0; j < nb; ++j)
-          for (int k = 0; k < na; ++k) Mb[j * na + k] += w * N2[j] * N1[k];
-      }
-    // Cholesky M = L L^T in place (lower triangle)
-    for (int k = 0; k < na; ++k) {
-      double s = M[k * na + k];
-      for (int m = 0; m < k; ++m) s -= M[k * na + m] * M[k * na + m];
+// integrated exactly by a (p+2)-point Gauss rule per axis.  The nodal basis is a tensor product, so R is
+// the tensor square of the 1D table (and independent of the element's size): thread t solves for row t
+// of the 1D one by Cholesky.
+__global__ void __launch_bounds__(256) qr_table_kernel(int p, double* __restrict__ R) {
+  constexpr int NA = kPMaxTab, NB = kPMaxTab + 1;   // p + 1 and p + 2 for p <= MTO_P_MAX
+  __shared__ double M[NA * NA], Mb[NB * NA], R1[NB * NA];
+  __shared__ double z1[NB], z2[NB], gx[NB + 1], gw[NB + 1], v1[NB + 1][NA], v2[NB + 1][NB];
+  const int n1 = p + 1, n2 = p + 2, t = threadIdx.x;
+  if (t == 0) gll_nodes(p, z1);
+  if (t == 32) gll_nodes(p + 1, z2);
+  if (t == 64) gauss_rule(n2, gx, gw);
+  __syncthreads();
+  for (int k = t; k < n2 * n1; k += blockDim.x) v1[k / n1][k % n1] = lagrange_val(z1, n1, k % n1, gx[k / n1]);
+  for (int k = t; k < n2 * n2; k += blockDim.x) v2[k / n2][k % n2] = lagrange_val(z2, n2, k % n2, gx[k / n2]);
+  __syncthreads();
+  for (int k = t; k < (n1 + n2) * n1; k += blockDim.x) {
+    const int r = k / n1, c = k % n1;
+    double s = 0.0;
+    for (int g = 0; g < n2; ++g) s = fma(gw[g], (r < n1 ? v1[g][r] : v2[g][r - n1]) * v1[g][c], s);
+    if (r < n1) M[r * n1 + c] = s;
+    else Mb[(r - n1) * n1 + c] = s;
+  }
+  __syncthreads();
+  if (t == 0) {   // Cholesky M = L L^T in place (lower triangle)
+    for (int k = 0; k < n1; ++k) {
+      double s = M[k * n1 + k];
+      for (int m = 0; m < k; ++m) s -= M[k * n1 + m] * M[k * n1 + m];
       s = sqrt(s);
-      M[k * na + k] = s;
-      for (int i = k + 1; i < na; ++i) {
-        double t = M[i * na + k];
-        for (int m = 0; m < k; ++m) t -= M[i * na + m] * M[k * na + m];
-        M[i * na + k] = t / s;
+      M[k * n1 + k] = s;
+      for (int i = k + 1; i < n1; ++i) {
+        double q = M[i * n1 + k];
+        for (int m = 0; m < k; ++m) q -= M[i * n1 + m] * M[k * n1 + m];
+        M[i * n1 + k] = q / s;
       }
     }
   }
   __syncthreads();
-  // row j of R solves M r = (row j of Mb)^T  (M symmetric)
-  for (int j = threadIdx.x; j < nb; j += blockDim.x) {
+  if (t < n2) {   // row t of R1 solves M r = (row t of Mb)^T  (M symmetric)
     double y[NA];
-    for (int k = 0; k < na; ++k) {
-      double t = Mb[j * na + k];
-      for (int m = 0; m < k; ++m) t -= M[k * na + m] * y[m];
-      y[k] = t / M[k * na + k];
+    for (int k = 0; k < n1; ++k) {
+      double q = Mb[t * n1 + k];
+      for (int m = 0; m < k; ++m) q -= M[k * n1 + m] * y[m];
+      y[k] = q / M[k * n1 + k];
     }
-    for (int k = na - 1; k >= 0; --k) {
-      double t = y[k];
-      for (int m = k + 1; m < na; ++m) t -= M[m * na + k] * y[m];
-      y[k] = t / M[k * na + k];
+    for (int k = n1 - 1; k >= 0; --k) {
+      double q = y[k];
+      for (int m = k + 1; m < n1; ++m) q -= M[m * n1 + k] * y[m];
+      y[k] = q / M[k * n1 + k];
     }
-    for (int k = 0; k < na; ++k) R[j * na + k] = y[k];
+    for (int k = 0; k < n1; ++k) R1[t * n1 + k] = y[k];
+  }
+  __syncthreads();
+  const int na = n1 * n1, nb = n2 * n2;
+  for (int k = t; k < nb * na; k += blockDim.x) {
+    const int j = k / na, i = k % na;
+    R[k] = R1[(j / n2) * n1 + i / n1] * R1[(j % n2) * n1 + i % n1];
   }
 }
 
@@ -451,7 +464,7 @@ mto_status build_tables(mto_handle h) {
     QRTab& q = h->qr[p];
     q.p = p;
     MTO_TRY(mto_alloc(h, &q.R, (size_t)(p + 2) * (p + 2) * (p + 1) * (p + 1)));
-    qr_table_kernel<<<1, 64, 0, h->stream>>>(p, h->hx, h->hy, q.R);
+    qr_table_kernel<<<1, 256, 0, h->stream>>>(p, q.R);
     MTO_TRY(mto_after_launch(h, "qr_table_kernel"));
     const int n1 = 2 * (p + 2) * (p + 2);
     std::vector<int> pos(qr_row_len(p + 1), -1);
@@ -468,10 +481,14 @@ mto_status build_elements(mto_handle h, const double* rho, const mto_material* m
   // the subcell tables depend only on nu (and the mesh): computed on the first build and again
   // whenever nu changes
   if (!(h->k0_nu == m->nu)) {
+    if (!h->k0_work) MTO_TRY(mto_alloc(h, &h->k0_work, (size_t)3 * MTO_D_MAX * (kPMaxTab + 1) * (kPMaxTab + 1)));
     for (auto* v : {&h->bc, &h->bc_qr})
       for (auto& b : *v) {
-        int n = b.P * b.S;
-        k0_kernel<<<(n + 127) / 128, 128, 0, h->stream>>>(b.p, b.d, m->nu, h->hx, h->hy, b.K0T);
+        // the 1D values in the handle's work vector (one table after the other on the stream)
+        const int n = b.P * b.S;
+        k0_point_kernel<<<1, 256, 0, h->stream>>>(b.p, b.d, h->k0_work);
+        MTO_TRY(mto_after_launch(h, "k0_point_kernel"));
+        k0_kernel<<<(n + 255) / 256, 256, 0, h->stream>>>(b.p, b.d, m->nu, h->hx, h->hy, h->k0_work, b.K0T);
         MTO_TRY(mto_after_launch(h, "k0_kernel"));
       }
     MTO_TRY(tc_tables(h));

@@ -208,6 +208,7 @@ void release_mesh(mto_handle h) {
   free_dev(h, h->filt_ext);
   free_dev(h, h->oc_t);
   free_dev(h, h->oc_work);
+  free_dev(h, h->k0_work);
   free_dev(h, h->qr_rows);
   h->qr_cap = 0;
   h->bytes = h->base_bytes;

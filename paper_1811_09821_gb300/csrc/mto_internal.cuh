@@ -167,6 +167,7 @@ struct mto_handle_s {
   bool have_setup = false, have_supports = false;
   int built_precision = -1;
   double k0_nu = -2.0;                         // nu of the current subcell tables
+  double* k0_work = nullptr;                   // the 1D values of the table being formed
 
   // device tables
   int* p_d = nullptr;
