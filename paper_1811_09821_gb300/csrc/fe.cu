@@ -272,90 +272,91 @@ void launch_diag(mto_handle h, const PClass& c, double* diag) {
 // holds the element's near-null modes exactly (those of solid/void elements, whose stiffness can
 // be 1e-10 of the element's largest, which point Jacobi cannot see).  Supported DOFs are
 // decoupled (unit row and column): B_e maps their zero residual to zero.  One warp per element:
-// FP64 in-place Gauss-Jordan inversion of the SPD block in shared memory, symmetrised, written in
-// the circulant-diagonal layout (FP64, or the split-precision pair).
+// FP64 in-place inversion of the SPD block (symmetric Gauss-Jordan sweeps, no pivoting) in shared
+// memory, written in the circulant-diagonal layout (FP64, or the split-precision pair).  Bound by the
+// FP64 pipes, so only one triangle is kept and swept (n^2 / 2 FMAs a pivot): the 1024 x 512 beam's blocks
+// took 38 ms with the whole matrix.
 template <int PO>
-__global__ void schwarz_kernel(int n, int L, const int2* __restrict__ dpos, const int* __restrict__ gmap,
-                               const Constraint* __restrict__ cons,
-                               const double* __restrict__ K64, const float* __restrict__ Kh,
-                               const float* __restrict__ Kl, const double* __restrict__ diag,
+__global__ void schwarz_kernel(int n, int L, const int* __restrict__ gmap, const Constraint* __restrict__ cons,
+                               const double* __restrict__ K64, const double* __restrict__ diag,
                                const double* __restrict__ invd, double* __restrict__ B64, float* __restrict__ Bh,
                                float* __restrict__ Bl) {
-  constexpr int N1 = PO + 1, NN = N1 * N1, NE = 2 * NN, LDA = NE + 1, P = NE * (NE + 1) / 2;
+  constexpr int N1 = PO + 1, NN = N1 * N1, NE = 2 * NN, P = NE * (NE + 1) / 2;
   extern __shared__ double sm[];
   const int wpb = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double* A = sm + (size_t)warp * NE * LDA;
-  int* fx = reinterpret_cast<int*>(sm + (size_t)wpb * NE * LDA) + warp * NE;
+  double* A = sm + (size_t)warp * (P + 2 * NE);   // packed lower triangle: A_ij at i (i + 1) / 2 + j
+  double* c = A + P;                              // the pivot's column and its multipliers
+  double* u = c + NE;
+  int* fx = reinterpret_cast<int*>(sm + (size_t)wpb * (P + 2 * NE)) + warp * NE;
+  unsigned short* ij = reinterpret_cast<unsigned short*>(reinterpret_cast<int*>(sm + (size_t)wpb * (P + 2 * NE)) + wpb * NE);
+  for (int i = threadIdx.x; i < NE; i += blockDim.x)
+    for (int j = 0; j <= i; ++j) ij[i * (i + 1) / 2 + j] = (unsigned short)(i << 8 | j);
+  __syncthreads();
+  // packed place of position `pos` of a circulant-diagonal row
+  auto place = [](int pos) {
+    const int k = pos / NE, r = pos - k * NE;
+    int q = r + k;
+    if (q >= NE) q -= NE;
+    return r > q ? r * (r + 1) / 2 + q : q * (q + 1) / 2 + r;
+  };
   for (int e = blockIdx.x * wpb + warp; e < n; e += gridDim.x * wpb) {
-    for (int idx = lane; idx < NE * NE; idx += 32) {
-      const int i = idx / NE, j = idx - (idx / NE) * NE;
-      const int a = i < j ? i : j, b = i < j ? j : i;
-      A[i * LDA + j] = k_entry(K64, Kh, Kl, L, e, dpos[packed_index(NE, a, b)].x);
-    }
+    const double* row = K64 + (size_t)e * L;
+    for (int pos = lane; pos < L; pos += 32) A[place(pos)] = row[pos];
     __syncwarp();
     for (int i = lane; i < NE; i += 32) {
       const int g = gmap[(size_t)e * NN + (i >> 1)];
+      double* Aii = A + i * (i + 1) / 2 + i;
       int fixed = 0;
       if (g >= 0) {
         const size_t gd = 2 * (size_t)g + (i & 1);
         if (invd[gd] == 0.0) fixed = 1;
-        else A[i * LDA + i] += fmax(diag[gd] - A[i * LDA + i], 0.0);
+        else *Aii += fmax(diag[gd] - *Aii, 0.0);
       } else {
         // a hanging local DOF interpolates free global DOFs: it takes their weighted diagonal
-        const Constraint& c = cons[-g - 1];
+        const Constraint& cn = cons[-g - 1];
         double dh = 0.0;
-        for (int k = 0; k < c.cnt; ++k) {
-          const size_t gd = 2 * (size_t)c.node[k] + (i & 1);
-          if (invd[gd] != 0.0) dh += c.w[k] * c.w[k] * diag[gd];
+        for (int k = 0; k < cn.cnt; ++k) {
+          const size_t gd = 2 * (size_t)cn.node[k] + (i & 1);
+          if (invd[gd] != 0.0) dh += cn.w[k] * cn.w[k] * diag[gd];
         }
-        A[i * LDA + i] += fmax(dh - A[i * LDA + i], 0.0);
+        *Aii += fmax(dh - *Aii, 0.0);
       }
       fx[i] = fixed;
     }
     __syncwarp();
-    for (int i = lane; i < NE; i += 32)
-      for (int j = 0; j < NE; ++j)
-        if (fx[i] || fx[j]) A[i * LDA + j] = (i == j) ? 1.0 : 0.0;
+    for (int t = lane; t < P; t += 32) {
+      const int i = ij[t] >> 8, j = ij[t] & 255;
+      if (fx[i] || fx[j]) A[t] = (i == j) ? 1.0 : 0.0;
+    }
     __syncwarp();
-    // in-place Gauss-Jordan inversion (SPD: no pivoting)
     for (int k = 0; k < NE; ++k) {
-      const double pinv = 1.0 / A[k * LDA + k];
-      __syncwarp();
-      for (int j = lane; j < NE; j += 32)
-        if (j != k) A[k * LDA + j] *= pinv;
-      __syncwarp();
-      for (int i = lane; i < NE; i += 32) {
-        if (i == k) continue;
-        const double f = A[i * LDA + k];
-        for (int j = 0; j < NE; ++j)
-          if (j != k) A[i * LDA + j] -= f * A[k * LDA + j];
-        A[i * LDA + k] = -f * pinv;
+      const double inv = newton_rcp(A[k * (k + 1) / 2 + k]);
+      for (int j = lane; j < NE; j += 32) {
+        const double v = j > k ? A[j * (j + 1) / 2 + k] : A[k * (k + 1) / 2 + j];
+        c[j] = v;
+        u[j] = v * inv;
       }
       __syncwarp();
-      if (lane == 0) A[k * LDA + k] = pinv;
+#pragma unroll 4
+      for (int t = lane; t < P; t += 32) {
+        const int i = ij[t] >> 8, j = ij[t] & 255;
+        double v = fma(-u[i], c[j], A[t]);
+        v = j == k ? u[i] : v;
+        v = i == k ? u[j] : v;
+        v = (i == k && j == k) ? -inv : v;
+        A[t] = v;
+      }
       __syncwarp();
     }
-    for (int c = lane; c < P; c += 32) {
-      int i = 0, rem = c;
-      while (rem >= NE - i) {
-        rem -= NE - i;
-        ++i;
-      }
-      const int j = i + rem;
-      const double v = 0.5 * (A[i * LDA + j] + A[j * LDA + i]);
-      const int2 ps = dpos[c];
-      const size_t o1 = (size_t)e * L + ps.x, o2 = (size_t)e * L + ps.y;
+    for (int pos = lane; pos < L; pos += 32) {   // A = -inverse
+      const double v = -A[place(pos)];
+      const size_t o = (size_t)e * L + pos;
       if (B64) {
-        B64[o1] = v;
-        if (ps.y >= 0) B64[o2] = v;
+        B64[o] = v;
       } else {
-        const float hi = (float)v, lo = (float)(v - (double)hi);
-        Bh[o1] = hi;
-        Bl[o1] = lo;
-        if (ps.y >= 0) {
-          Bh[o2] = hi;
-          Bl[o2] = lo;
-        }
+        const float hi = (float)v;
+        Bh[o] = hi;
+        Bl[o] = (float)(v - (double)hi);
       }
     }
     __syncwarp();
@@ -364,17 +365,16 @@ __global__ void schwarz_kernel(int n, int L, const int2* __restrict__ dpos, cons
 
 template <int PO>
 mto_status launch_schwarz(mto_handle h, PClass& c) {
-  constexpr int NE = 2 * (PO + 1) * (PO + 1);
+  constexpr int NE = 2 * (PO + 1) * (PO + 1), P = NE * (NE + 1) / 2;
   const int wpb = NE <= 32 ? 8 : (NE <= 50 ? 4 : 2);
-  const size_t smem = (size_t)wpb * NE * (NE + 1) * sizeof(double) + (size_t)wpb * NE * sizeof(int);
+  const size_t smem = (size_t)wpb * (P + 2 * NE) * sizeof(double) + (size_t)wpb * NE * sizeof(int) + 2 * P + 16;
   if (smem > 48 * 1024)
     MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(schwarz_kernel<PO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)smem), "cudaFuncSetAttribute"));
   const bool df = h->built_precision == MTO_MIXED;
   const int blocks = grid_for(c.n, wpb, 152 * 8);
-  schwarz_kernel<PO><<<blocks, 32 * wpb, smem, h->stream>>>(c.n, c.L, c.dpos, c.gmap, h->cons_d, c.K64, c.K32,
-                                                            c.K32lo, h->diag64, h->invd64, df ? nullptr : c.B64,
-                                                            c.B32, c.B32lo);
+  schwarz_kernel<PO><<<blocks, 32 * wpb, smem, h->stream>>>(c.n, c.L, c.gmap, h->cons_d, c.K64, h->diag64, h->invd64,
+                                                            df ? nullptr : c.B64, c.B32, c.B32lo);
   return mto_after_launch(h, "schwarz_kernel");
 }
 

@@ -285,20 +285,6 @@ __global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
 // Indicators of a 320 x 160 adaptive mesh with the sums here 10.9 ms, with rows 6.9 ms.
 // eps is invariant to rigid motions of u^(p), which are removed first (FP64) so that the element
 // energies carry no cancellation.
-
-// 1 / d: Newton's iteration x <- x + x (1 - d x) on the mantissa from its FP32 reciprocal; plain
-// division at the ends of the exponent range, for negative values, infinities and NaN
-__device__ __forceinline__ double qr_rcp(double d) {
-  const long long b = __double_as_longlong(d);
-  const int be = (int)(b >> 52);
-  if (be < 8 || be > 2038) return 1.0 / d;
-  const double md = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
-  double r = (double)(1.0f / __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff)));
-  r = fma(r, fma(-md, r, 1.0), r);
-  r = fma(r, fma(-md, r, 1.0), r);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)(be - 1023) << 52));
-}
-
 __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, const int* __restrict__ elem,
                                                 const int* __restrict__ slot, int L, const int* __restrict__ gmap,
                                                 const Constraint* __restrict__ cons, const double* __restrict__ K64,
@@ -429,7 +415,7 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, 
       if (lane == 0) rd[c] = 1.0;
       continue;
     }
-    const double inv = qr_rcp(A[c * (c + 1) / 2 + c]);
+    const double inv = newton_rcp(A[c * (c + 1) / 2 + c]);
     for (int i = c + 1 + lane; i < n1; i += 32) {
       const double a = A[i * (i + 1) / 2 + c];
       cl[i] = a;

@@ -370,19 +370,6 @@ struct StripGeom {
   }
 };
 
-// 1 / d of a positive double: Newton's iteration x <- x + x (1 - d x) on the mantissa, from its FP32
-// reciprocal (2^-23, squared twice)
-__device__ __forceinline__ double newton_rcp(double d) {
-  const long long b = __double_as_longlong(d);
-  const int be = (int)(b >> 52);
-  if (be < 8 || be > 2038) return 1.0 / d;
-  const double md = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
-  double r = (double)(1.0f / __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff)));
-  r = fma(r, fma(-md, r, 1.0), r);
-  r = fma(r, fma(-md, r, 1.0), r);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)(be - 1023) << 52));
-}
-
 // In-place symmetric inversion (Gauss-Jordan sweeps, SPD: no pivoting) of an m x m matrix held as its
 // packed lower triangle over the threads of kInvWarps warps: entry e of thread t is (ij[e] >> 8,
 // ij[e] & 255), ij < 0 beyond the end.  On return a = -inverse.  Two helper warps form each pivot's
