@@ -269,17 +269,34 @@ __global__ void __launch_bounds__(256) mg_stencil_apply_kernel(int nx, int ny, c
   }
 }
 
+// Bilinear interpolation of a coarse level's vertex values at fine vertex (i, j) (both components)
+template <typename V>
+__device__ __forceinline__ void coarse_value(const V* __restrict__ xc, int nxc, int i, int j, V& s0, V& s1) {
+  const int i0 = i >> 1, j0 = j >> 1, ni = i & 1, nj = j & 1;
+  const V w = (ni ? V(0.5) : V(1)) * (nj ? V(0.5) : V(1));
+  s0 = s1 = V(0);
+  for (int b = 0; b <= nj; ++b)
+    for (int a = 0; a <= ni; ++a) {
+      const size_t c = 2 * ((size_t)(j0 + b) * (nxc + 1) + i0 + a);
+      s0 = fma(w, xc[c], s0);
+      s1 = fma(w, xc[c + 1], s1);
+    }
+}
+
 // One Chebyshev step on a Q1 level with q = A x formed in place by the vertex stencil (the apply and
 // the update of mg_cheb_kernel in one pass): reads x from xin, writes the updated x to xout (the
 // level's two x buffers alternate, so no vertex reads a neighbour's new value), d in place.
-// xzero: x = 0 before the step (A x = 0, xin not read).  Stencil and arithmetic as in
-// mg_stencil_apply_kernel.
-template <typename TS, typename V>
+// kCorrect: x is xin plus the coarse level's correction xc (nxc elements wide), interpolated on the free
+// DOFs as it is read, which saves the launch that would write it (the small levels are bound by their
+// launches).  Stencil and arithmetic as in mg_stencil_apply_kernel.
+template <typename TS, typename V, bool kCorrect>
 __global__ void __launch_bounds__(256) mg_stencil_cheb_kernel(int nx, int ny, const TS* __restrict__ S,
                                                               const V* __restrict__ xin, V* __restrict__ xout,
                                                               const V* __restrict__ b, const V* __restrict__ invd,
                                                               V* __restrict__ d, const double2* __restrict__ coef,
-                                                              int step, int xzero, const int* __restrict__ done) {
+                                                              int step, const V* __restrict__ xc, int nxc,
+                                                              const V* __restrict__ mask,
+                                                              const int* __restrict__ done) {
   if (done && *done) return;
   const double2 cc = coef[step];
   const V c1 = (V)cc.x, c2 = (V)cc.y;
@@ -287,21 +304,31 @@ __global__ void __launch_bounds__(256) mg_stencil_cheb_kernel(int nx, int ny, co
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
     const int i = (int)(v % (nx + 1)), j = (int)(v / (nx + 1));
     TS y0 = 0, y1 = 0;
-    if (!xzero) {
+    V xv[2] = {V(0), V(0)};
 #pragma unroll
-      for (int dj = -1; dj <= 1; ++dj) {
+    for (int dj = -1; dj <= 1; ++dj) {
 #pragma unroll
-        for (int di = -1; di <= 1; ++di) {
-          const int ii = i + di, jj = j + dj;
-          if (ii < 0 || ii > nx || jj < 0 || jj > ny) continue;
-          const int o = 3 * (dj + 1) + di + 1;
-          const size_t w = 2 * ((size_t)jj * (nx + 1) + ii);
-          const TS x0 = (TS)xin[w], x1 = (TS)xin[w + 1];
-          y0 = fma(S[(size_t)(o * 4 + 0) * nv + v], x0, y0);
-          y0 = fma(S[(size_t)(o * 4 + 1) * nv + v], x1, y0);
-          y1 = fma(S[(size_t)(o * 4 + 2) * nv + v], x0, y1);
-          y1 = fma(S[(size_t)(o * 4 + 3) * nv + v], x1, y1);
+      for (int di = -1; di <= 1; ++di) {
+        const int ii = i + di, jj = j + dj;
+        if (ii < 0 || ii > nx || jj < 0 || jj > ny) continue;
+        const int o = 3 * (dj + 1) + di + 1;
+        const size_t w = 2 * ((size_t)jj * (nx + 1) + ii);
+        V a0 = xin[w], a1 = xin[w + 1];
+        if (kCorrect) {
+          V s0, s1;
+          coarse_value(xc, nxc, ii, jj, s0, s1);
+          a0 += mask[w] * s0;
+          a1 += mask[w + 1] * s1;
         }
+        if (di == 0 && dj == 0) {
+          xv[0] = a0;
+          xv[1] = a1;
+        }
+        const TS x0 = (TS)a0, x1 = (TS)a1;
+        y0 = fma(S[(size_t)(o * 4 + 0) * nv + v], x0, y0);
+        y0 = fma(S[(size_t)(o * 4 + 1) * nv + v], x1, y0);
+        y1 = fma(S[(size_t)(o * 4 + 2) * nv + v], x0, y1);
+        y1 = fma(S[(size_t)(o * 4 + 3) * nv + v], x1, y1);
       }
     }
 #pragma unroll
@@ -310,17 +337,85 @@ __global__ void __launch_bounds__(256) mg_stencil_cheb_kernel(int nx, int ny, co
       const V r = invd[k] * (b[k] - (V)(c ? y1 : y0));
       const V dn = step > 0 ? fma(c1, d[k], c2 * r) : c2 * r;
       d[k] = dn;
-      xout[k] = (xzero ? V(0) : xin[k]) + dn;
+      xout[k] = xv[c] + dn;
     }
   }
 }
 
+// The first smoothing step of a level from x = 0, d = x = invd b / theta, taken where b is formed.
+// x null: the coarsest level, solved directly.
 template <typename V>
-__global__ void __launch_bounds__(256) mg_copy_kernel(int64_t n, const V* __restrict__ a, V* __restrict__ b,
-                                                      const int* __restrict__ done) {
+struct FirstStep {
+  const V* invd;
+  V *d, *x;
+  const double2* coef;
+  __device__ __forceinline__ void take(size_t k, V b) const {
+    if (!x) return;
+    const V dn = (V)coef[0].y * (invd[k] * b);
+    d[k] = dn;
+    x[k] = dn;
+  }
+};
+
+// level l -> l+1: the residual b - A x by the stencil on a tile of fine vertices in shared memory, full
+// weighting (the transpose of bilinear interpolation) on the free DOFs, and the coarse level's first step.
+// One launch of the four that the residual, the restriction, the first step and (above) the correction
+// took: 160 x 80 solve 74.3 -> 71.1 ms.  Tiles of 8 x 4: with 16 x 8 the middle levels have too few blocks
+// (the same solve 6 % slower than unfused).
+constexpr int kRX = 8, kRY = 4;   // coarse vertices per block
+constexpr int kRThreads = 160;    // 17 x 9 fine vertices
+template <typename TS, typename V>
+__global__ void __launch_bounds__(kRThreads) mg_resid_restrict_kernel(int nx, int ny, const TS* __restrict__ S,
+                                                                const V* __restrict__ x, const V* __restrict__ b,
+                                                                const V* __restrict__ invd, int nxc, int nyc,
+                                                                const V* __restrict__ maskc, V* __restrict__ bc,
+                                                                FirstStep<V> fs, const int* __restrict__ done) {
   if (done && *done) return;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-    b[i] = a[i];
+  constexpr int FX = 2 * kRX + 1, FY = 2 * kRY + 1;
+  __shared__ V r[2][FY][FX + 1];
+  const int I0 = blockIdx.x * kRX, J0 = blockIdx.y * kRY;
+  const int64_t nv = (int64_t)(nx + 1) * (ny + 1);
+  for (int k = threadIdx.x; k < FX * FY; k += kRThreads) {
+    const int fi = k % FX, fj = k / FX, i = 2 * I0 - 1 + fi, j = 2 * J0 - 1 + fj;
+    V r0 = V(0), r1 = V(0);
+    if (i >= 0 && i <= nx && j >= 0 && j <= ny) {
+      const int64_t v = (int64_t)j * (nx + 1) + i;
+      TS y0 = 0, y1 = 0;
+#pragma unroll
+      for (int dj = -1; dj <= 1; ++dj) {
+#pragma unroll
+        for (int di = -1; di <= 1; ++di) {
+          const int ii = i + di, jj = j + dj;
+          if (ii < 0 || ii > nx || jj < 0 || jj > ny) continue;
+          const int o = 3 * (dj + 1) + di + 1;
+          const size_t w = 2 * ((size_t)jj * (nx + 1) + ii);
+          const TS x0 = (TS)x[w], x1 = (TS)x[w + 1];
+          y0 = fma(S[(size_t)(o * 4 + 0) * nv + v], x0, y0);
+          y0 = fma(S[(size_t)(o * 4 + 1) * nv + v], x1, y0);
+          y1 = fma(S[(size_t)(o * 4 + 2) * nv + v], x0, y1);
+          y1 = fma(S[(size_t)(o * 4 + 3) * nv + v], x1, y1);
+        }
+      }
+      if (invd[2 * v] != V(0)) r0 = b[2 * v] - (V)y0;
+      if (invd[2 * v + 1] != V(0)) r1 = b[2 * v + 1] - (V)y1;
+    }
+    r[0][fj][fi] = r0;
+    r[1][fj][fi] = r1;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < 2 * kRX * kRY; k += kRThreads) {
+    const int c = k & 1, ci = (k >> 1) % kRX, cj = (k >> 1) / kRX, I = I0 + ci, J = J0 + cj;
+    if (I > nxc || J > nyc) continue;
+    V s = V(0);
+#pragma unroll
+    for (int dy = 0; dy < 3; ++dy)
+#pragma unroll
+      for (int dx = 0; dx < 3; ++dx) s = fma((dx == 1 ? V(1) : V(0.5)) * (dy == 1 ? V(1) : V(0.5)), r[c][2 * cj + dy][2 * ci + dx], s);
+    const size_t at = 2 * ((size_t)J * (nxc + 1) + I) + c;
+    const V bv = maskc[at] * s;
+    bc[at] = bv;
+    fs.take(at, bv);
+  }
 }
 
 // assembled diagonal of a Q1 level (atomics), then the masked inverse
@@ -768,7 +863,8 @@ __global__ void __launch_bounds__(256) mg_restrict0_kernel(int64_t nv, const int
                                                            const int* __restrict__ node, const double* __restrict__ w,
                                                            const V* __restrict__ b, const V* __restrict__ q,
                                                            const V* __restrict__ invd, const V* __restrict__ mask,
-                                                           V* __restrict__ b1, const int* __restrict__ done) {
+                                                           V* __restrict__ b1, FirstStep<V> fs,
+                                                           const int* __restrict__ done) {
   if (done && *done) return;
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nv; v += (int64_t)gridDim.x * blockDim.x) {
     V s0 = V(0), s1 = V(0);
@@ -778,8 +874,12 @@ __global__ void __launch_bounds__(256) mg_restrict0_kernel(int64_t nv, const int
       if (invd[g] != V(0)) s0 = fma(wk, b[g] - q[g], s0);
       if (invd[g + 1] != V(0)) s1 = fma(wk, b[g + 1] - q[g + 1], s1);
     }
-    b1[2 * v] = mask[2 * v] * s0;
-    b1[2 * v + 1] = mask[2 * v + 1] * s1;
+    s0 *= mask[2 * v];
+    s1 *= mask[2 * v + 1];
+    b1[2 * v] = s0;
+    b1[2 * v + 1] = s1;
+    fs.take(2 * v, s0);
+    fs.take(2 * v + 1, s1);
   }
 }
 
@@ -803,63 +903,6 @@ __global__ void __launch_bounds__(256) mg_prolong0_kernel(int64_t nn, const int*
     if (invd[2 * g + 1] != V(0)) x[2 * g + 1] += s1;
     q[2 * g] = V(0);
     q[2 * g + 1] = V(0);
-  }
-}
-
-// level l -> l+1 on vertex grids (full weighting: the transpose of bilinear interpolation) of the
-// residual r = b - q formed on the fly on free DOFs (q stays; the prolongation clears it)
-template <typename V>
-__global__ void __launch_bounds__(256) mg_restrict_h_kernel(int nxc, int nyc, int nxf, int nyf,
-                                                            const V* __restrict__ b, const V* __restrict__ q,
-                                                            const V* __restrict__ invd, const V* __restrict__ mask,
-                                                            V* __restrict__ bc, const int* __restrict__ done) {
-  if (done && *done) return;
-  const int64_t nvc = (int64_t)(nxc + 1) * (nyc + 1);
-  for (int64_t Vx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; Vx < nvc; Vx += (int64_t)gridDim.x * blockDim.x) {
-    const int I = (int)(Vx % (nxc + 1)), J = (int)(Vx / (nxc + 1));
-    V s0 = V(0), s1 = V(0);
-    for (int dy = -1; dy <= 1; ++dy) {
-      const int j = 2 * J + dy;
-      if (j < 0 || j > nyf) continue;
-      const V wy = dy == 0 ? V(1) : V(0.5);
-      for (int dx = -1; dx <= 1; ++dx) {
-        const int i = 2 * I + dx;
-        if (i < 0 || i > nxf) continue;
-        const V wgt = wy * (dx == 0 ? V(1) : V(0.5));
-        const size_t f = 2 * ((size_t)j * (nxf + 1) + i);
-        if (invd[f] != V(0)) s0 = fma(wgt, b[f] - q[f], s0);
-        if (invd[f + 1] != V(0)) s1 = fma(wgt, b[f + 1] - q[f + 1], s1);
-      }
-    }
-    bc[2 * Vx] = mask[2 * Vx] * s0;
-    bc[2 * Vx + 1] = mask[2 * Vx + 1] * s1;
-  }
-}
-
-// level l+1 -> l: x += bilinear interpolation of the coarse correction (free DOFs); q cleared
-template <typename V>
-__global__ void __launch_bounds__(256) mg_prolong_h_kernel(int nxc, int nxf, int nyf, const V* __restrict__ xc,
-                                                           const V* __restrict__ mask, V* __restrict__ xf,
-                                                           V* __restrict__ q, const int* __restrict__ done) {
-  if (done && *done) return;
-  const int64_t nvf = (int64_t)(nxf + 1) * (nyf + 1);
-  for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < nvf; v += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(v % (nxf + 1)), j = (int)(v / (nxf + 1));
-    const int i0 = i >> 1, i1 = (i + 1) >> 1, j0 = j >> 1, j1 = (j + 1) >> 1;
-    const V wi = (i & 1) ? V(0.5) : V(1), wj = (j & 1) ? V(0.5) : V(1);
-    V s0 = V(0), s1 = V(0);
-    const int is[2] = {i0, i1}, js[2] = {j0, j1};
-    const int ni = (i & 1) ? 2 : 1, nj = (j & 1) ? 2 : 1;
-    for (int b = 0; b < nj; ++b)
-      for (int a = 0; a < ni; ++a) {
-        const size_t c = 2 * ((size_t)js[b] * (nxc + 1) + is[a]);
-        s0 = fma(wi * wj, xc[c], s0);
-        s1 = fma(wi * wj, xc[c + 1], s1);
-      }
-    xf[2 * v] += mask[2 * v] * s0;
-    xf[2 * v + 1] += mask[2 * v + 1] * s1;
-    q[2 * v] = V(0);
-    q[2 * v + 1] = V(0);
   }
 }
 
@@ -1156,22 +1199,22 @@ mto_status mg_level_apply(mto_handle h, const MGLevel& l, const double* x, doubl
     mg_stencil_apply_kernel<double, double><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S, x, y, done);
   return mto_after_launch(h, "mg_stencil_apply_kernel");
 }
-mto_status mg_level_apply(mto_handle h, const MGLevel& l, const float* x, float* y, const int* done) {
-  mg_stencil_apply_kernel<float, float><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S32, x, y, done);
-  return mto_after_launch(h, "mg_stencil_apply_kernel");
-}
+// one fused Chebyshev step on a smoothed Q1 level (FP64 stencil in the FP64 cycle, FP32 in the FP32 one), with
+// the correction xc of the coarse level `C` added to xin where given
+const double* level_stencil(const MGLevel& l, const double*) { return l.S; }
+const float* level_stencil(const MGLevel& l, const float*) { return l.S32; }
 
-// one fused Chebyshev step on a smoothed Q1 level (FP64 stencil in the FP64 cycle, FP32 in the FP32 one)
-mto_status mg_level_cheb(mto_handle h, const MGLevel& l, const double* xin, double* xout, const double* b,
-                         const double* invd, double* d, const double2* cf, int step, bool xzero, const int* done) {
-  mg_stencil_cheb_kernel<double, double><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S, xin, xout, b, invd,
-                                                                                d, cf, step, xzero, done);
-  return mto_after_launch(h, "mg_stencil_cheb_kernel");
-}
-mto_status mg_level_cheb(mto_handle h, const MGLevel& l, const float* xin, float* xout, const float* b,
-                         const float* invd, float* d, const double2* cf, int step, bool xzero, const int* done) {
-  mg_stencil_cheb_kernel<float, float><<<vec_grid(l.nv), 256, 0, h->stream>>>(l.nx, l.ny, l.S32, xin, xout, b, invd,
-                                                                              d, cf, step, xzero, done);
+template <typename V>
+mto_status mg_level_cheb(mto_handle h, const MGLevel& l, const V* xin, V* xout, const V* b, const V* invd, V* d,
+                         const double2* cf, int step, const V* xc, const MGLevel* C, const V* mask, const int* done) {
+  const V* S = level_stencil(l, (const V*)nullptr);
+  const int grd = vec_grid(l.nv);
+  if (xc)
+    mg_stencil_cheb_kernel<V, V, true><<<grd, 256, 0, h->stream>>>(l.nx, l.ny, S, xin, xout, b, invd, d, cf, step, xc,
+                                                                   C->nx, mask, done);
+  else
+    mg_stencil_cheb_kernel<V, V, false><<<grd, 256, 0, h->stream>>>(l.nx, l.ny, S, xin, xout, b, invd, d, cf, step,
+                                                                    nullptr, 0, nullptr, done);
   return mto_after_launch(h, "mg_stencil_cheb_kernel");
 }
 
@@ -1398,25 +1441,10 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, V* w0
   // captured cycle starts with the same one).  Block smoothing keeps the operator in acc and the blocks
   // in w0, each cleared by the kernel that consumes the other.
   V *acc = q0, *other = v0;
-  auto smooth = [&](int lev, const V* b, V* x, V* d, const V* invd, int64_t n, bool pre, bool last) -> mto_status {
-    const int k = lev < 0 ? degree : (h->mg_q1deg > 0 ? h->mg_q1deg : kCoarseDegree);
-    const double2* cf = h->mg_coef + (size_t)(lev + 1) * kMaxDegree;
+  auto smooth0 = [&](const V* b, V* x, V* d, const V* invd, int64_t n, bool pre, bool last) -> mto_status {
+    const int k = degree;
+    const double2* cf = h->mg_coef;
     const int grd = vec_grid(n);
-    if (lev >= 0) {   // Q1 level: one fused stencil + Chebyshev launch per step, x ping-ponged
-      const MGLevel& L = h->mg[lev];
-      V* cur = x;
-      V* nxt = level_vecs<V>(L).xa;
-      TimedScope ts(h, F_PRECOND);
-      for (int s = 0; s < k; ++s) {
-        MTO_TRY(mg_level_cheb(h, L, cur, nxt, b, invd, d, cf, s, pre && s == 0, done));
-        std::swap(cur, nxt);
-      }
-      if (cur != x) {   // odd degree: the result is in the other buffer
-        mg_copy_kernel<V><<<grd, 256, 0, h->stream>>>(n, cur, x, done);
-        MTO_TRY(mto_after_launch(h, "mg_copy_kernel"));
-      }
-      return MTO_OK;
-    }
     const bool block = h->mg_block;   // element-block (additive Schwarz) smoothing of level 0
     for (int s = 0; s < k; ++s) {
       const bool skip_apply = pre && s == 0;   // x = 0: A x = 0
@@ -1444,57 +1472,59 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, V* w0
     return MTO_OK;
   };
   // level 0 pre-smoothing and residual
-  MTO_TRY(smooth(-1, b0, x0, d0, invd0, h->ndof, true, false));
+  MTO_TRY(smooth0(b0, x0, d0, invd0, h->ndof, true, false));
   MTO_TRY(fine_apply(h, x0, acc, done, lead, false));
-  {
-    TimedScope ts(h, F_PRECOND);
-    const LevelV<V> L1 = level_vecs<V>(h->mg[0]);
-    mg_restrict0_kernel<V><<<vec_grid(h->mg[0].nv), 256, 0, h->stream>>>(
-        h->mg[0].nv, h->mg_rptr, h->mg_rnode, h->mg_rw, b0, acc, invd0, L1.mask, L1.b, done);
-    MTO_TRY(mto_after_launch(h, "mg_restrict0_kernel"));
+  // Q1 levels: x alternates between the level's two buffers, cur[l] holds the current one.  The kernel that
+  // forms a level's right-hand side takes its first step into xa.
+  const int kq = h->mg_q1deg > 0 ? h->mg_q1deg : kCoarseDegree;
+  std::vector<LevelV<V>> lv;
+  std::vector<V*> cur(nl), nxt(nl);
+  for (int l = 0; l < nl; ++l) {
+    lv.push_back(level_vecs<V>(h->mg[l]));
+    cur[l] = l + 1 < nl ? lv[l].xa : lv[l].x;
+    nxt[l] = lv[l].x;
   }
-  // Q1 levels down
-  for (int l = 0; l < nl - 1; ++l) {
-    const MGLevel& L = h->mg[l];
-    const MGLevel& C = h->mg[l + 1];
-    const LevelV<V> lv = level_vecs<V>(L), cv = level_vecs<V>(C);
-    MTO_TRY(smooth(l, lv.b, lv.x, lv.d, lv.invd, L.n, true, false));
-    TimedScope ts(h, F_PRECOND);
-    MTO_TRY(mg_level_apply(h, L, lv.x, lv.q, done));
-    mg_restrict_h_kernel<V><<<vec_grid(C.nv), 256, 0, h->stream>>>(C.nx, C.ny, L.nx, L.ny, lv.b, lv.q, lv.invd,
-                                                                   cv.mask, cv.b, done);
-    MTO_TRY(mto_after_launch(h, "mg_restrict_h_kernel"));
-  }
-  {
-    TimedScope ts(h, F_PRECOND);
-    const MGLevel& C = h->mg.back();
-    const LevelV<V> cv = level_vecs<V>(C);
-    mg_coarse_solve_kernel<V><<<(int)((C.n * 32 + 255) / 256), 256, sizeof(double) * C.n, h->stream>>>(
-        strip_geom(C), h->mg_Ainv, cv.b, cv.x, done);
-    MTO_TRY(mto_after_launch(h, "mg_coarse_solve_kernel"));
-  }
-  // up
-  for (int l = nl - 2; l >= 0; --l) {
-    const MGLevel& L = h->mg[l];
-    const MGLevel& C = h->mg[l + 1];
-    const LevelV<V> lv = level_vecs<V>(L), cv = level_vecs<V>(C);
-    {
-      TimedScope ts(h, F_PRECOND);
-      mg_prolong_h_kernel<V><<<vec_grid(L.nv), 256, 0, h->stream>>>(C.nx, L.nx, L.ny, cv.x, lv.mask, lv.x, lv.q,
-                                                                     done);
-      MTO_TRY(mto_after_launch(h, "mg_prolong_h_kernel"));
+  auto first_step = [&](int l) {
+    const bool smoothed = l + 1 < nl;
+    return FirstStep<V>{lv[l].invd, lv[l].d, smoothed ? lv[l].xa : nullptr, h->mg_coef + (size_t)(l + 1) * kMaxDegree};
+  };
+  auto smooth = [&](int l, int from, const V* xc) -> mto_status {   // steps from .. kq - 1, the first with xc
+    const double2* cf = h->mg_coef + (size_t)(l + 1) * kMaxDegree;
+    for (int s = from; s < kq; ++s) {
+      MTO_TRY(mg_level_cheb<V>(h, h->mg[l], cur[l], nxt[l], lv[l].b, lv[l].invd, lv[l].d, cf, s, s == from ? xc : nullptr,
+                               xc ? &h->mg[l + 1] : nullptr, lv[l].mask, done));
+      std::swap(cur[l], nxt[l]);
     }
-    MTO_TRY(smooth(l, lv.b, lv.x, lv.d, lv.invd, L.n, false, false));
-  }
+    return MTO_OK;
+  };
   {
     TimedScope ts(h, F_PRECOND);
-    const LevelV<V> L1 = level_vecs<V>(h->mg[0]);
-    mg_prolong0_kernel<V><<<vec_grid(h->n_nodes), 256, 0, h->stream>>>(h->n_nodes, h->mg_pidx, h->mg_pw, L1.x,
-                                                                        invd0, x0, h->mg_block ? acc : other, done);
+    mg_restrict0_kernel<V><<<vec_grid(h->mg[0].nv), 256, 0, h->stream>>>(
+        h->mg[0].nv, h->mg_rptr, h->mg_rnode, h->mg_rw, b0, acc, invd0, lv[0].mask, lv[0].b, first_step(0), done);
+    MTO_TRY(mto_after_launch(h, "mg_restrict0_kernel"));
+    // down
+    for (int l = 0; l < nl - 1; ++l) {
+      const MGLevel& L = h->mg[l];
+      const MGLevel& C = h->mg[l + 1];
+      MTO_TRY(smooth(l, 1, nullptr));
+      const dim3 grid((C.nx + kRX) / kRX, (C.ny + kRY) / kRY);
+      mg_resid_restrict_kernel<V, V><<<grid, kRThreads, 0, h->stream>>>(L.nx, L.ny, level_stencil(L, (const V*)nullptr), cur[l],
+                                                                  lv[l].b, lv[l].invd, C.nx, C.ny, lv[l + 1].mask,
+                                                                  lv[l + 1].b, first_step(l + 1), done);
+      MTO_TRY(mto_after_launch(h, "mg_resid_restrict_kernel"));
+    }
+    const MGLevel& C = h->mg.back();
+    mg_coarse_solve_kernel<V><<<(int)((C.n * 32 + 255) / 256), 256, sizeof(double) * C.n, h->stream>>>(
+        strip_geom(C), h->mg_Ainv, lv[nl - 1].b, lv[nl - 1].x, done);
+    MTO_TRY(mto_after_launch(h, "mg_coarse_solve_kernel"));
+    // up
+    for (int l = nl - 2; l >= 0; --l) MTO_TRY(smooth(l, 0, cur[l + 1]));
+    mg_prolong0_kernel<V><<<vec_grid(h->n_nodes), 256, 0, h->stream>>>(h->n_nodes, h->mg_pidx, h->mg_pw, cur[0], invd0,
+                                                                        x0, h->mg_block ? acc : other, done);
     MTO_TRY(mto_after_launch(h, "mg_prolong0_kernel"));
     if (!h->mg_block) std::swap(acc, other);
   }
-  return smooth(-1, b0, x0, d0, invd0, h->ndof, false, true);
+  return smooth0(b0, x0, d0, invd0, h->ndof, false, true);
 }
 
 }  // namespace
