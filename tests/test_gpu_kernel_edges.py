@@ -260,3 +260,38 @@ def test_oc_update_edges(mto, nx, ny, d, kind):
             assert abs(lam - wl) <= 4e-10 * wl
         np.testing.assert_allclose(out.cpu().numpy(), want, rtol=1e-9, atol=1e-12)
     h.close()
+
+
+@pytest.mark.parametrize("orders", [(1, 1), (1, 2), (2, 3), (1, 4), (4, 5), (3, 6), (1, 2, 3, 4, 5, 6)])
+@pytest.mark.parametrize("nx,ny", [(2, 1), (7, 5)])
+def test_assembled_diagonal_edges(mto, nx, ny, orders):
+    """The assembled diagonal D, read through the scaled norm of the start vector's residual
+    (sqrt(r^T D^-1 r / f^T D^-1 f), accepted before the first iteration), against D_i = e_i^T K e_i of the
+    FP64 operator, on meshes with and without hanging nodes.  Both sum the same up to a few hundred FP64
+    products of entries and weights of order 1 (void at 0.3^3 of solid), so 1e-13 each, and r = f - K u
+    of random vectors has no cancellation: 1e-10."""
+    rng = np.random.default_rng(nx * 100 + sum(orders))
+    p = rng.permutation(np.resize(np.asarray(orders, np.int32), nx * ny))
+    h = handle(mto, nx, ny, p, 3)
+    T = lambda a: torch.tensor(a, device="cuda")
+    fixed = np.asarray(h.side_dofs(0))
+    h.set_supports(h.side_dofs(0))
+    h.build_elements(T(rng.uniform(0.3, 1.0, h.design_len)), mto.material())
+    free = np.setdiff1d(np.arange(h.ndof), fixed)
+    D = np.zeros(h.ndof)
+    x, y = torch.zeros(h.ndof, dtype=torch.float64, device="cuda"), torch.empty(h.ndof, dtype=torch.float64, device="cuda")
+    for i in free:
+        x.zero_()
+        x[i] = 1.0
+        h.apply(x, y)
+        D[i] = y[i].item()
+    f, u = np.zeros(h.ndof), np.zeros(h.ndof)
+    f[free], u[free] = rng.standard_normal(free.size), rng.standard_normal(free.size)
+    uT = T(u)
+    h.apply(uT, y)
+    r = f - y.cpu().numpy()
+    want = np.sqrt((r[free] ** 2 / D[free]).sum() / (f[free] ** 2 / D[free]).sum())
+    it, got = h.solve(T(f), uT, rtol=1e6, warm_start=True, norm=mto.NORM_JACOBI, precond=mto.PREC_JACOBI)
+    assert it == 0
+    assert abs(got - want) <= 1e-10 * want
+    h.close()
