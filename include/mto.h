@@ -99,7 +99,9 @@ typedef struct {
  *              they are extrapolated from the sums of the last two windows of 32 gains (S_last,
  *              S_prev: error ~ S_last / (1 - S_last / S_prev)) and the stop is taken when that is
  *              below rtol / 4 times the compliance estimate (a margin for uneven decay).  rtol is then a relative compliance
- *              error (not squared); *relres still reports the l2 residual.
+ *              error (not squared); *relres still reports the l2 residual.  A step with
+ *              r^T z < 0 (a preconditioner that is not definite) counts as an infinite gain: no stop
+ *              is taken while one of the two windows holds it.
  *              Needs FP64 vectors (MTO_FP64 or MTO_MIXED).  At 10^7 DOFs and stiffness contrasts
  *              of 1e9 the l2 residual of an FP64 evaluation floors near 1e-7, so l2 tolerances
  *              below that cannot be met there, while compliance accuracy can.  A correction solve
