@@ -6,9 +6,9 @@
 // The element matrices need FP64 accuracy (on the binary designs a relative error of 1e-13 in K_e
 // moves the compliance by ~1e-6), so the products cannot be plain BF16 products.  The GEMM is made
 // exact by slicing (an Ozaki-type error-free splitting): each element's moduli row is scaled by a
-// power of two sigma_e (max E <= sigma_e) and each K0 column by a power of two tau_pos, and both
+// power of two sigma_e (max |E| <= sigma_e) and each K0 column by a power of two tau_pos, and both
 // are cut into 8 slices of 7 bits (56 bits), E/sigma = sum_i a_i 2^-7i and K0/tau = sum_j b_j 2^-7j
-// with integer a_i in [0, 127], b_j in [-127, 127] (exact in BF16).  Every slice product a_i . b_j
+// with integer a_i, b_j in [-127, 127] (exact in BF16).  Every slice product a_i . b_j
 // over K <= 64 subcells is an integer below 2^20, and all pairs of one level g = i + j share the
 // weight 2^-7g: each level accumulates its (at most 8) slice GEMMs in one FP32 TMEM accumulator
 // exactly (sums below 2^23).  Levels g = 2..10 are kept (the dropped levels weigh below 2^-51 of
@@ -200,10 +200,10 @@ __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double
   }
 }
 
-// floor(v 2^(56 - ex)) of a non-negative double v < 2^ex, by its bits (0 for negative or non-finite v)
+// floor(|v| 2^(56 - ex)) of a finite double v, |v| < 2^ex, by its bits
 __host__ __device__ __forceinline__ unsigned long long fixed56(unsigned long long bits, int ex) {
-  const int be = (int)(bits >> 52);   // sign and exponent
-  if (be >= 0x7ff) return 0ull;
+  const int be = (int)(bits >> 52) & 0x7ff;
+  bits &= 0x7fffffffffffffffull;
   const unsigned long long m = be ? (bits & 0xfffffffffffffull) | (1ull << 52) : bits;
   const int sh = (be ? be : 1) - 1075 + 56 - ex;
   return sh >= 0 ? m << (sh & 63) : (sh > -64 ? m >> (-sh & 63) : 0ull);
@@ -275,6 +275,9 @@ __host__ __device__ __forceinline__ void split_pair(unsigned long long bits, flo
   lo = (d * 8.673617379884035e-19f) * s;   // 2^-60 2^(e + 8)
 }
 
+// sig[] of a row with a modulus that is not finite: all its entries are NaN, as the FP64 sums give them
+constexpr int kRowNaN = 1 << 20;
+
 // rows: element k of the class (first <= k < n) is output row slot[k], or row k - first without slots.
 // Kh null: FP64 rows only.
 __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
@@ -317,8 +320,8 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
   }
 
   // A slices: one element row per warp at a time, two subcells per lane (coalesced rho, packed
-  // 32-bit stores).  Moduli E_s scaled by sigma_e and cut into 8 x 7 bits by integer shifts; q = 3
-  // takes products instead of pow (both run on the FP64 pipes).
+  // 32-bit stores).  Moduli E_s scaled by sigma_e and cut into 8 x 7 bits and their sign by integer shifts;
+  // q = 3 takes products instead of pow (both run on the FP64 pipes).
   if (warp < kEpiWarps) {
     const bool cube = q == 3.0;
     const double dE = E0 - Emin;
@@ -336,12 +339,12 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
       }
       const unsigned long long e0 = v0 ? (unsigned long long)__double_as_longlong(modulus(r0)) : 0ull;
       const unsigned long long e1 = v1 ? (unsigned long long)__double_as_longlong(modulus(r1)) : 0ull;
-      // sigma_e = 2^ex > max E: from the largest exponent among the finite non-negative moduli
-      const int x0 = (int)(e0 >> 52), x1 = (int)(e1 >> 52);
-      const int xm = __reduce_max_sync(0xffffffffu, max(x0 < 0x7ff ? x0 : 0, x1 < 0x7ff ? x1 : 0));
+      // sigma_e = 2^ex > max |E|: from the largest exponent
+      const int xm = __reduce_max_sync(0xffffffffu, max((int)(e0 >> 52) & 0x7ff, (int)(e1 >> 52) & 0x7ff));
       const int ex = max(xm, 1) - 1022;
-      if (lane == 0) sig[r] = ex;
+      if (lane == 0) sig[r] = xm < 0x7ff ? ex : kRowNaN;
       if (s0 < kpad) {
+        const unsigned sgn = (unsigned)(e0 >> 63) << 15 | (unsigned)(e1 >> 63) << 31;
         const unsigned long long V0 = fixed56(e0, ex), V1 = fixed56(e1, ex);
         unsigned char* dst = As + core_off(r, s0, kpad);
 #pragma unroll
@@ -349,7 +352,7 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
           const int sh = kOpBits - kSliceBits * (i + 1);
           const unsigned a0 = __float_as_uint((float)(int)((V0 >> sh) & 127ull)) >> 16;
           const unsigned a1 = __float_as_uint((float)(int)((V1 >> sh) & 127ull)) & 0xffff0000u;
-          *reinterpret_cast<unsigned*>(dst + i * a_slice) = a0 | a1;   // BF16 of integers <= 127: exact
+          *reinterpret_cast<unsigned*>(dst + i * a_slice) = sgn | a0 | a1;   // BF16 of integers <= 127: exact
         }
       }
     }
@@ -440,7 +443,8 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
           const int p0 = I[0] * 128 + I[1], p1 = I[2] * 128 + I[3], p2 = I[5] * 128 + I[6], p3 = I[7] * 128 + I[8];
           const long long H = (long long)p0 * (1 << 21) + (long long)p1 * 128 + I[4];
           const long long Lw = (long long)p2 * (1 << 14) + p3;
-          const unsigned long long bits = levels_to_double(H, Lw, sexp + __ldg(tau + pos0 + c));
+          unsigned long long bits = levels_to_double(H, Lw, sexp + __ldg(tau + pos0 + c));
+          if (sexp == kRowNaN) bits = 0x7ff8000000000000ull;
           *reinterpret_cast<unsigned long long*>(st64 + lane * kStRow64 + c * 8) = bits;
           if (Kh) {
             float hi, lo;
