@@ -1,9 +1,12 @@
 // Step (d): the composite refinement indicator and the dp map update (Sec. 3.2, 3.3), and the
-// optimality-criteria design update.  All FP64: the integer maps must match the oracle exactly,
-// so every floating-point decision is taken in double with a fixed reduction order.
+// optimality-criteria design update.  All FP64 or its equal (the QR error's matrices from the sliced
+// tensor-core sums where those are no further off, see qr_kernel): the integer maps must match the oracle
+// exactly, so every floating-point decision is taken in double with a fixed reduction order.
 #include <algorithm>
 #include <cmath>
 #include <vector>
+
+#include <math_constants.h>
 
 #include "mto_internal.cuh"
 
@@ -277,14 +280,33 @@ __global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
 // One warp per element of a (p, d) class (Eq. 14).  Shared layout (doubles): A[L1] (the order p+1
 // matrix, lower triangle packed by rows, A_ij at i (i + 1) / 2 + j, factorised in place as
 // L D L^T), f[n0], f1[n1], u1[n1], ue[n0], rd[n1] (reciprocal pivots), cl[n1] (the pivot
-// column before scaling), pr[3 n1] (the pinned rows of the unmodified matrix) and, without rows, E[S],
-// with n0 = 2 (p+1)^2, n1 = 2 (p+2)^2, L1 = n1 (n1 + 1) / 2 rounded up.
+// column before scaling), pr[3 n1] (the pinned rows of the unmodified matrix); E[S], the moduli, in the
+// place of the last three until they are needed; with n0 = 2 (p+1)^2, n1 = 2 (p+2)^2,
+// L1 = n1 (n1 + 1) / 2 rounded up.
 // K^(p+1) = sum_s E_s K0_s comes as rows formed on the tensor cores (tc_rows, d <= 8), or is summed
-// here from the table (rows null).  The kernel is bound by the FP64 pipes (2 FMA per clock and SM),
-// where those sums were 81.6 k of 115 k FMAs of a Q3/d8 element (170.5 ms on the 1024 x 512 beam).
-// Indicators of a 320 x 160 adaptive mesh with the sums here 10.9 ms, with rows 6.9 ms.
+// here from the table (rows null, and the elements that `sliced_rows_hold` turns away).  The kernel is
+// bound by the FP64 pipes (2 FMA per clock and SM), where those sums were 81.6 k of 115 k FMAs of a Q3/d8
+// element (170.5 ms on the 1024 x 512 beam).
 // eps is invariant to rigid motions of u^(p), which are removed first (FP64) so that the element
 // energies carry no cancellation.
+//
+// The sliced rows are exact to about 2^-54 of the element's largest modulus times the column's largest
+// table entry, the FP64 sums to a few 2^-53 of the sum of each entry's own terms.  Those are alike while the
+// moduli are; beside void, entries that only soft subcells carry are far below the row's scale.
+// In extended precision (orders 1..5, d = 2..8, fields of solved shape) the error of eps with rows was, as
+// a geometric mean over the elements of a class, 0.8 to 1.1 times that with sums for fronts of a factor of
+// 16, up to 1.7 times for 125 and up to 4.5 times for 1e9: rows serve the elements within kQRContrast.
+constexpr double kQRContrast = 16.0;
+
+// whether the moduli's extremes over the element (lo, hi; ok: every one is a number of at least 0) let the rows be used
+__device__ __forceinline__ bool sliced_rows_hold(bool ok, double lo, double hi) {
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  return __all_sync(0xffffffffu, ok) && hi <= kQRContrast * lo;
+}
+
 __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, const int* __restrict__ elem,
                                                 const int* __restrict__ slot, int L, const int* __restrict__ gmap,
                                                 const Constraint* __restrict__ cons, const double* __restrict__ K64,
@@ -310,15 +332,21 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, 
   double* rd = ue + n0;
   double* cl = rd + n1;
   double* pr = cl + n1;
-  double* E = pr + 3 * n1;
-  if (rows) {
+  double* E = rd;   // S doubles (the launch's shared memory covers S > 5 n1)
+  bool ok = true;
+  double lo = CUDART_INF, hi = 0.0;
+  for (int s = lane; s < S; s += 32) {
+    const double r = rho[off[e] + s];
+    const double m = Emin + (q == 3.0 ? r * r * r : pow(r, q)) * (E0 - Emin);
+    E[s] = m;
+    ok = ok && m >= 0.0;
+    lo = fmin(lo, m);
+    hi = fmax(hi, m);
+  }
+  const bool sliced = rows && sliced_rows_hold(ok, lo, hi);
+  if (sliced) {
     const double2* src = reinterpret_cast<const double2*>(rows + (size_t)blockIdx.x * L1);
     for (int c = lane; c < L1 / 2; c += 32) reinterpret_cast<double2*>(A)[c] = src[c];
-  } else {
-    for (int s = lane; s < S; s += 32) {
-      double r = rho[off[e] + s];
-      E[s] = Emin + (q == 3.0 ? r * r * r : pow(r, q)) * (E0 - Emin);
-    }
   }
   // gather u_e (lanes over nodes), then remove its least-squares rigid motion about the element
   // centre (translations and rotation; node sums over the warp)
@@ -368,7 +396,7 @@ __global__ void __launch_bounds__(32) qr_kernel(int p, int d, int n, int first, 
     for (int kk = 0; kk < na; ++kk) s += R[jn * na + kk] * f[2 * kk + c];
     f1[i] = s;
   }
-  if (!rows) {
+  if (!sliced) {
     // K^(p+1) (table rows by upper packed index (i <= j)) into the lower triangle
     for (int c = lane; c < P1; c += 32) {
       double s = 0.0;
@@ -1173,7 +1201,7 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
     const PClass& c = h->pc[b.p];
     const int n0 = 2 * (b.p + 1) * (b.p + 1), n1 = 2 * (b.p + 2) * (b.p + 2), L1 = qr_row_len(b.p + 1);
     const bool tc = h->build_path == MTO_BUILD_TENSOR && b1.tcB;
-    const size_t smem = sizeof(double) * ((size_t)L1 + 2 * n0 + 7 * n1 + (tc ? 0 : b.S));
+    const size_t smem = sizeof(double) * ((size_t)L1 + 2 * n0 + 2 * n1 + std::max(5 * n1, b.S));
     if (smem > 48 * 1024) cudaFuncSetAttribute(qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int chunk = b.n;
     if (tc) {

@@ -92,3 +92,51 @@ def test_qr_error_of_nonfinite_and_negative_densities(mto, d, bad):
     if np.isfinite(bad):
         assert abs(got[e] - want[e]) <= 1e-9 * abs(want[e])
     h.close()
+
+
+@pytest.mark.parametrize("p,d", [(1, 8), (2, 4), (3, 8), (4, 3), (5, 8), (6, 2)])
+@pytest.mark.parametrize("design", ["binary", "graded", "void"])
+def test_qr_error_across_the_modulus_contrast(mto, p, d, design):
+    """Elements that mix solid with 1e-9 void, or grade from one to the other: the QR error comes from the
+    FP64 sums whatever the build path (equal bits), as the sliced rows keep only 2^-54 of the element's
+    largest modulus; elements of moduli within a factor of 16 may take the rows (kappa of the pinned problem
+    below 1e5 there, so 1e-9).  The maps of an adaptive step agree, and a sample agrees with the oracle to
+    2^-50 of the pinned problem's condition number."""
+    from oracle import indicators as oi
+    from oracle import mesh as om
+    from oracle.solve import K0_table
+    nx, ny = 17, 9
+    h = handle(mto, nx, ny, p, d)
+    m = om.DPMesh(nx, ny, np.full(nx * ny, p), np.full(nx * ny, d))
+    rng = np.random.default_rng(p + 10 * d)
+    e = np.arange(nx * ny)
+    c = (np.arange(d) + 0.5) / d
+    x = (e % nx)[:, None, None] + c[None, None, :]
+    y = (e // nx)[:, None, None] + c[None, :, None]
+    s = np.sin(0.9 * x + 0.3 * y) + np.sin(0.4 * x - 1.1 * y) + 0.2
+    rho = {"binary": (s > 0).astype(float), "graded": np.clip(1 / (1 + np.exp(-4 * s)), 1e-3, 1.0),
+           "void": np.zeros_like(s)}[design].reshape(nx * ny, d * d)
+    rho[5], rho[6] = 0.6, np.linspace(0.5, 0.9, d * d)
+    u = rng.standard_normal(h.ndof)
+    mat = mto.material()
+    h.set_supports(h.side_dofs(0))
+    h.build_elements(T(rho.ravel()), mat)
+    got = h.indicator(T(u), T(rho.ravel()), mat)
+    h.set_build_path(mto.BUILD_SIMT)
+    ref = h.indicator(T(u), T(rho.ravel()), mat)
+    a, b = got["eps_qr"].cpu().numpy(), ref["eps_qr"].cpu().numpy()
+    E = 1e-9 + rho ** 3 * (1.0 - 1e-9)
+    close = E.max(1) <= 15.9 * E.min(1)
+    far = E.max(1) >= 16.1 * E.min(1)
+    assert close.any() and (far.any() or design == "void")
+    np.testing.assert_array_equal(a[far], b[far])
+    assert np.abs(a - b)[close].max() <= 1e-9
+    for k in ("p_new", "d_new", "theta"):
+        np.testing.assert_array_equal(got[k].cpu().numpy(), ref[k].cpu().numpy())
+    K0 = K0_table(p + 1, d, 0.3, 1.0, 1.0)
+    fr = np.setdiff1d(np.arange(K0.shape[1]), oi.qr_fixed_local_dofs(p + 1))
+    for k in np.concatenate([np.flatnonzero(far)[::7], [5, 6]]):
+        kappa = np.linalg.cond(np.tensordot(E[k], K0, axes=(0, 0))[np.ix_(fr, fr)])
+        want = oi.qr_error_element(p, d, rho[k], m.gather(k, u), 1.0, 1e-9, 0.3, 3.0)
+        assert abs(a[k] - want) <= 2.0 ** -50 * kappa, (k, a[k], want, kappa)
+    h.close()
