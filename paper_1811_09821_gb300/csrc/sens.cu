@@ -10,10 +10,16 @@
 // so its values on one (2p+1) x (2p+1) Gauss grid of the element determine it, and its integrals
 // over the d x d subcells are two small products with the integrals W of the grid's Lagrange
 // polynomials over the subcells: w = W en W^T.  For Q3 and 8 x 8 subcells that is 49 strain
-// evaluations in place of 1024.  Against extended precision, over orders 1..6 and d = 2..16, both
-// forms are within 1.3e-15 of the largest w (2-norm; 3e-16 to 9e-16 the point sums, 2e-16 to
-// 1.3e-15 this one).  Bound by the FP64 pipes (2 FMA per clock and SM): a block takes several
-// elements and spreads each stage over all its threads.
+// evaluations in place of 1024.  Its weights have both signs, so its error is relative to the element's
+// largest w: subcells below 1/64 of that are integrated by the subcell's own (p+1) x (p+1) Gauss points, a
+// sum of squares with positive weights (w >= 0 for u = v, error relative to sqrt(w w_max)).  The
+// 1D tables are formed in double-double and rounded once: rounded products of Lagrange factors were
+// the larger part of either form's error.  Against extended precision (orders 1..6, d = 3 and 8; rough,
+// smooth and bending fields; 2-norm): point sums over every subcell with rounded tables 2e-16 to 1.5e-15, this
+// form 1.7e-16 to 3.9e-16, nowhere the larger but for 2.4e-16 against 2.2e-16 at p = 4, d = 8.  Bound by the
+// FP64 pipes (2 FMA per clock and SM): a block takes several elements and spreads each stage over all
+// its threads.  480 x 240 Q3/d8 elements: 12.25 ms with point sums over every subcell, 0.76 ms with the
+// polynomial for every one, 0.96 ms with the small ones directly.
 //
 // FP32 (sens_kernel, MTO_MIXED): one warp per element; strains at the (p+1) x (p+1) Gauss points of
 // every subcell from a sum-factorised tensor evaluation on the element's d(p+1) x d(p+1) point grid;
@@ -29,20 +35,95 @@ constexpr int kSensQMax = 2 * MTO_P_MAX + 1;
 // points per axis of the FP64 kernel's grid: enough for degree 2p, or the subcell's own Gauss rule for d = 1
 __host__ __device__ constexpr int sens_q(int p, int d) { return d == 1 ? p + 1 : 2 * p + 1; }
 
+namespace {
+
+// Double-double arithmetic (Dekker 1971: a value is the unevaluated sum of two doubles, about 106 bits)
+// for the tables below.
+struct DD {
+  double h, l;
+};
+
+__device__ __forceinline__ DD dd_norm(double h, double l) {   // |h| >= |l|
+  const double s = __dadd_rn(h, l);
+  return {s, __dsub_rn(l, __dsub_rn(s, h))};
+}
+__device__ __forceinline__ DD operator+(DD a, DD b) {
+  const double s = __dadd_rn(a.h, b.h), t = __dsub_rn(s, a.h);
+  const double e = __dadd_rn(__dsub_rn(a.h, __dsub_rn(s, t)), __dsub_rn(b.h, t));
+  return dd_norm(s, __dadd_rn(e, __dadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ DD operator-(DD a, DD b) { return a + DD{-b.h, -b.l}; }
+__device__ __forceinline__ DD operator*(DD a, DD b) {
+  const double p = __dmul_rn(a.h, b.h);
+  return dd_norm(p, fma(a.h, b.h, -p) + fma(a.h, b.l, a.l * b.h));
+}
+__device__ __forceinline__ DD operator/(DD a, DD b) {
+  const double q = a.h / b.h;
+  const DD r = a - b * DD{q, 0.0};
+  return dd_norm(q, r.h / b.h);
+}
+__device__ __forceinline__ DD dd(double x) { return {x, 0.0}; }
+
+// (P_n, P_{n-1}) at x by the three-term recurrence
+__device__ __forceinline__ void dd_legendre(int n, DD x, DD* pn, DD* pn1) {
+  DD a = dd(1.0), b = x;
+  for (int k = 2; k <= n; ++k) {
+    const DD c = (dd(2 * k - 1) * x * b - dd(k - 1) * a) / dd(k);
+    a = b;
+    b = c;
+  }
+  *pn = n == 0 ? dd(1.0) : b;
+  *pn1 = a;
+}
+
+// 1 / prod_{j != a} (z_a - z_j)
+__device__ __forceinline__ DD dd_bary(const double* z, int n, int a) {
+  DD v = dd(1.0);
+  for (int j = 0; j < n; ++j)
+    if (j != a) v = v * (dd(z[a]) - dd(z[j]));
+  return dd(1.0) / v;
+}
+
+// Lagrange polynomial l_a on the nodes z and its derivative, c = dd_bary(z, n, a)
+__device__ __forceinline__ DD dd_lagrange(const double* z, int n, int a, DD c, DD x) {
+  for (int j = 0; j < n; ++j)
+    if (j != a) c = c * (x - dd(z[j]));
+  return c;
+}
+__device__ __forceinline__ DD dd_lagrange_der(const double* z, int n, int a, DD c, DD x) {
+  DD s = dd(0.0);
+  for (int i = 0; i < n; ++i) {
+    if (i == a) continue;
+    DD t = c;
+    for (int j = 0; j < n; ++j)
+      if (j != a && j != i) t = t * (x - dd(z[j]));
+    s = s + t;
+  }
+  return s;
+}
+
+}  // namespace
+
 // Tables of a (p, d) class.  FP64 (Q = sens_q Gauss points x_g): [L: N1 x Q][Dx: N1 x Q][Dy: N1 x Q]
 // [W: d x Q][Z: N1] with L = l_a(x_g), Dx = 2/hx l_a'(x_g), Dy = 2/hy l_a'(x_g),
-// W = integral over subcell i of the Lagrange polynomial of point g, Z the GLL nodes.
-// FP32: [L: N1 x G][D: N1 x G][W: G] with G = d (p+1) points xi_g = -1 + (2 i + 1 + x_k)/d
-// (subcell i, Gauss node x_k), L = l_a(xi_g), D = l_a'(xi_g) and W = w_k / d (the 1D subcell Jacobian).
+// W = integral over subcell i of the Lagrange polynomial of point g, Z the GLL nodes; then for d > 1 the
+// subcells' own points xi_g = -1 + (2 i + 1 + x_k)/d, G = d (p+1): [L: G x N1][Dx: G x N1][Dy: G x N1]
+// [w: N1] with the weights w_k / d.
+// FP32: [L: N1 x G][D: N1 x G][W: G] at the same points, W = w_k / d (the 1D subcell Jacobian).
+__host__ __device__ constexpr int sens_tab_len(int p, int d) {
+  return (3 * sens_q(p, d) + 1) * (p + 1) + d * sens_q(p, d) + (d > 1 ? (3 * d * (p + 1) + 1) * (p + 1) : 0);
+}
+
 __global__ void __launch_bounds__(256) sens_table_kernel(int p, int d, double hx, double hy, double* __restrict__ tab,
                                                          float* __restrict__ tabf) {
-  const int n1 = p + 1, G = d * n1, Q = sens_q(p, d);
+  const int n1 = p + 1, G = d * n1, Q = sens_q(p, d), t = threadIdx.x;
   __shared__ double z[kPMaxTab + 1], gx[kPMaxTab + 1], gw[kPMaxTab + 1], qx[kSensQMax], qw[kSensQMax];
-  if (threadIdx.x == 0) gll_nodes(p, z);
-  if (threadIdx.x == 32) gauss_rule(n1, gx, gw);
-  if (threadIdx.x == 64) gauss_rule(Q, qx, qw);
+  __shared__ DD xk[kPMaxTab + 1], wk[kPMaxTab + 1], cz[kPMaxTab + 1], cq[kSensQMax];
+  if (t == 0) gll_nodes(p, z);
+  if (t == 32) gauss_rule(n1, gx, gw);
+  if (t == 64) gauss_rule(Q, qx, qw);
   __syncthreads();
-  for (int k = threadIdx.x; k < 2 * n1 * G + G; k += blockDim.x) {
+  for (int k = t; k < 2 * n1 * G + G; k += blockDim.x) {
     double v;
     if (k < 2 * n1 * G) {
       int which = k / (n1 * G), r = k % (n1 * G), a = r / G, g = r % G;
@@ -54,23 +135,41 @@ __global__ void __launch_bounds__(256) sens_table_kernel(int p, int d, double hx
     }
     tabf[k] = (float)v;
   }
-  const int nt = n1 * Q;
-  for (int k = threadIdx.x; k < 3 * nt + d * Q + n1; k += blockDim.x) {
+  if (t < n1) {   // the (p+1)-point rule: one Newton step from the rounded node, w = 2 (1 - x^2) / (n P_{n-1})^2
+    DD pn, pn1, x = dd(gx[t]);
+    dd_legendre(n1, x, &pn, &pn1);
+    x = x - pn * (dd(1.0) - x * x) / (dd(n1) * (pn1 - x * pn));
+    dd_legendre(n1, x, &pn, &pn1);
+    xk[t] = x;
+    wk[t] = dd(2.0) * (dd(1.0) - x * x) / (dd(n1) * pn1 * dd(n1) * pn1);
+  }
+  if (t >= 32 && t < 32 + n1) cz[t - 32] = dd_bary(z, n1, t - 32);
+  if (t >= 64 && t < 64 + Q) cq[t - 64] = dd_bary(qx, Q, t - 64);
+  __syncthreads();
+  auto point = [&](int g) { return (dd(2 * (g / n1) + 1) + xk[g % n1]) / dd(d) - dd(1.0); };
+  auto value = [&](int which, int a, DD x) {   // 0: l_a, 1: 2/hx l_a', 2: 2/hy l_a'
+    return which == 0 ? dd_lagrange(z, n1, a, cz[a], x).h
+                      : (dd(2.0) / dd(which == 1 ? hx : hy) * dd_lagrange_der(z, n1, a, cz[a], x)).h;
+  };
+  const int nt = n1 * Q, nz = 3 * nt + d * Q, np = G * n1, len = sens_tab_len(p, d);
+  for (int k = t; k < len; k += blockDim.x) {
     double v;
     if (k < 3 * nt) {
-      const int which = k / nt, a = k % nt / Q, g = k % Q;
-      v = which == 0 ? lagrange_val(z, n1, a, qx[g]) : lagrange_der(z, n1, a, qx[g]) * (2.0 / (which == 1 ? hx : hy));
-    } else if (k < 3 * nt + d * Q) {
+      v = value(k / nt, k % nt / Q, dd(qx[k % Q]));
+    } else if (k < nz) {
       const int i = (k - 3 * nt) / Q, g = (k - 3 * nt) % Q;
-      if (d == 1) {
-        v = qw[g];
-      } else {
-        v = 0.0;
-        for (int kk = 0; kk < n1; ++kk)
-          v += gw[kk] / d * lagrange_val(qx, Q, g, -1.0 + (2.0 * i + 1.0 + gx[kk]) / d);
-      }
+      DD s = dd(0.0);
+      if (d == 1) s = wk[g];   // Q = p + 1
+      else
+        for (int kk = 0; kk < n1; ++kk) s = s + wk[kk] / dd(d) * dd_lagrange(qx, Q, g, cq[g], point(i * n1 + kk));
+      v = s.h;
+    } else if (k < nz + n1) {
+      v = z[k - nz];
+    } else if (k < nz + n1 + 3 * np) {
+      const int r = k - nz - n1;
+      v = value(r / np, r % n1, point(r % np / n1));
     } else {
-      v = z[k - 3 * nt - d * Q];
+      v = (wk[k - nz - n1 - 3 * np] / dd(d)).h;
     }
     tab[k] = v;
   }
@@ -212,15 +311,86 @@ __global__ void __launch_bounds__(128) sens_kernel(
 // The FP64 kernel (see the head of this file).  A block of 128 threads takes EB elements (a power of
 // two, 4..32); each stage is a flat loop over the items of all of them.
 constexpr int kSensThreads = 128;
+constexpr double kSensDirect = 1.0 / 64.0;   // subcells below this share of the element's largest |w|: directly
 
-// doubles of shared memory per element
+// doubles of shared memory per element of the x-contracted fields (later the subcells' w), and in all
+__host__ __device__ constexpr int sens_work_doubles(int p, int d, int nf) {
+  return nf * 4 * (p + 1) * sens_q(p, d) > d * d ? nf * 4 * (p + 1) * sens_q(p, d) : d * d;
+}
 __host__ __device__ constexpr int sens_elem_doubles(int p, int d, int nf) {
-  const int n1 = p + 1, nn = n1 * n1, Q = sens_q(p, d);
-  return nf * (2 * nn + 4 * n1 * Q + 3) + Q * Q + d * Q;
+  const int nn = (p + 1) * (p + 1), Q = sens_q(p, d);
+  return nf * (2 * nn + 3) + sens_work_doubles(p, d, nf) + Q * Q + d * Q + (d * d + 3) / 4;
+}
+
+// (exx + nu eyy)(exx' + nu eyy') + (1 - nu^2) eyy eyy' + (1 - nu)/2 gam gam': the energy density over 1 / (1 - nu^2)
+template <int NF>
+__device__ __forceinline__ double sens_density(const double (&ax)[NF], const double (&ey)[NF], const double (&gm)[NF],
+                                               double c1, double c2) {
+  constexpr int o = NF - 1;
+  return fma(ax[0], ax[o], fma(c1 * ey[0], ey[o], c2 * gm[0] * gm[o]));
+}
+
+// The integral of the energy density over subcell (i, j) by its (p+1) x (p+1) Gauss points, of the fields at
+// Uf[NF][2][NN]; tab: the tables of the subcells' points.
+template <int PO, int NF>
+__device__ __forceinline__ double sens_direct(const double* __restrict__ Uf, const double* __restrict__ tab, int d, int i,
+                                              int j, double nu, double c1, double c2) {
+  constexpr int N1 = PO + 1, NN = N1 * N1;
+  const int np = d * N1 * N1;
+  const double *L = tab, *Dx = L + np, *Dy = Dx + np, *w1 = Dy + np;
+  double w = 0.0;
+#pragma unroll 1
+  for (int kx = 0; kx < N1; ++kx) {
+    const double *lx = L + (i * N1 + kx) * N1, *dx = Dx + (i * N1 + kx) * N1;
+    double A[NF][4][N1];
+#pragma unroll
+    for (int fld = 0; fld < NF; ++fld)
+#pragma unroll
+      for (int b = 0; b < N1; ++b) {
+        double a0 = 0.0, d0 = 0.0, a1 = 0.0, d1 = 0.0;
+#pragma unroll
+        for (int a = 0; a < N1; ++a) {
+          const double l = __ldg(lx + a), dl = __ldg(dx + a);
+          const double v0 = Uf[fld * 2 * NN + b * N1 + a], v1 = Uf[fld * 2 * NN + NN + b * N1 + a];
+          a0 = fma(v0, l, a0);
+          d0 = fma(v0, dl, d0);
+          a1 = fma(v1, l, a1);
+          d1 = fma(v1, dl, d1);
+        }
+        A[fld][0][b] = a0;
+        A[fld][1][b] = d0;
+        A[fld][2][b] = a1;
+        A[fld][3][b] = d1;
+      }
+    double t = 0.0;
+#pragma unroll 1
+    for (int ky = 0; ky < N1; ++ky) {
+      const double *ly = L + (j * N1 + ky) * N1, *dy = Dy + (j * N1 + ky) * N1;
+      double ax[NF], ey[NF], gm[NF];
+#pragma unroll
+      for (int fld = 0; fld < NF; ++fld) {
+        double ex = 0.0, e2 = 0.0, ga = 0.0;
+#pragma unroll
+        for (int b = 0; b < N1; ++b) {
+          const double lb = __ldg(ly + b), db = __ldg(dy + b);
+          ex = fma(A[fld][1][b], lb, ex);
+          ga = fma(A[fld][0][b], db, ga);
+          ga = fma(A[fld][3][b], lb, ga);
+          e2 = fma(A[fld][2][b], db, e2);
+        }
+        ax[fld] = fma(nu, e2, ex);
+        ey[fld] = e2;
+        gm[fld] = ga;
+      }
+      t = fma(__ldg(w1 + ky), sens_density<NF>(ax, ey, gm, c1, c2), t);
+    }
+    w = fma(__ldg(w1 + kx), t, w);
+  }
+  return w;
 }
 
 template <int PO, int NF>
-__global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
+__global__ void __launch_bounds__(kSensThreads, NF == 1 ? (PO <= 3 ? 6 : 4) : (PO <= 3 ? 4 : 2)) sens_poly_kernel(
     int n, int d, int Q, int EB, const int* __restrict__ elem, const int* __restrict__ slot,
     const int* __restrict__ gmap, const Constraint* __restrict__ cons, const double* __restrict__ u,
     const double* __restrict__ v, const double* __restrict__ rho, const int64_t* __restrict__ design_off, double E0,
@@ -234,8 +404,12 @@ __global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
   double* U = sd + ntab;                       // [EB][NF][2][NN]
   double* rig = U + EB * NF * 2 * NN;          // [EB][NF][3] translation and rotation
   double* A = rig + EB * NF * 3;               // [EB][NF][4][N1][Q]
-  double* en = A + EB * NF * 4 * NQ;           // [EB][Q][Q] energy density (y, x)
+  double* ws = A;                              // [EB][d][d] w of the subcells, once A is used up
+  double* en = A + EB * sens_work_doubles(PO, d, NF);   // [EB][Q][Q] energy density (y, x)
   double* T = en + EB * Q * Q;                 // [EB][d][Q] integrated along x (subcell, y point)
+  unsigned short* list = reinterpret_cast<unsigned short*>(T + EB * d * Q);   // [EB][d][d] small subcells
+  __shared__ int n_list;
+  if (t == 0) n_list = 0;
   for (int k = t; k < ntab; k += kSensThreads) sd[k] = tab[k];
   const int base = blockIdx.x * EB;
   const int ne = min(EB, n - base);
@@ -306,8 +480,7 @@ __global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
     Af[3 * NQ] = d1;
   }
   __syncthreads();
-  // stage 2 (along y): strains and the energy density over 1 / (1 - nu^2) at every grid point:
-  // (exx + nu eyy)(exx' + nu eyy') + (1 - nu^2) eyy eyy' + (1 - nu)/2 gam gam'
+  // stage 2 (along y): strains and the energy density over 1 / (1 - nu^2) at every grid point
   const double c1 = 1.0 - nu * nu, c2 = 0.5 * (1.0 - nu);
   for (int it = t; it < ne * Q * Q; it += kSensThreads) {
     const int el = it / (Q * Q), h = it % (Q * Q) / Q, g = it % Q;
@@ -328,8 +501,7 @@ __global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
       ey[fld] = e2;
       gm[fld] = ga;
     }
-    constexpr int o = NF - 1;
-    en[it] = fma(ax[0], ax[o], fma(c1 * ey[0], ey[o], c2 * gm[0] * gm[o]));
+    en[it] = sens_density<NF>(ax, ey, gm, c1, c2);
   }
   __syncthreads();
   // integrals over the subcells: along x, then along y
@@ -344,17 +516,35 @@ __global__ void __launch_bounds__(kSensThreads) sens_poly_kernel(
   const double jac = 0.25 * hx * hy / (1.0 - nu * nu), dE = E0 - Emin;
   const bool cube = q == 3.0;
   const int tpe = kSensThreads / EB;   // threads per element, at most 32
-  const int el = t / tpe;
-  double energy = 0.0;   // sum_s E(rho_s) w_s (eout)
-  if (el < ne) {
-    const int64_t off = design_off[elem[base + el]];
-    for (int s = t % tpe; s < d * d; s += tpe) {
+  const int el = t / tpe, S = d * d;
+  double top = 0.0;
+  if (el < ne)
+    for (int s = t % tpe; s < S; s += tpe) {
       const double* Wj = W + (s / d) * Q;
       const double* Ti = T + (el * d + s % d) * Q;
       double w = 0.0;
       for (int h = 0; h < Q; ++h) w = fma(Wj[h], Ti[h], w);
-      w *= jac;
-      const double r = rho[off + s];
+      ws[el * S + s] = w;
+      top = fmax(top, fabs(w));
+    }
+  if (d > 1) {   // (one subcell: its Gauss points are the grid's)
+    for (int o = tpe >> 1; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
+    if (el < ne)
+      for (int s = t % tpe; s < S; s += tpe)
+        if (!(fabs(ws[el * S + s]) >= kSensDirect * top))   // also where w is not a number
+          list[atomicAdd(&n_list, 1)] = (unsigned short)(el << 8 | s);
+    __syncthreads();
+    for (int it = t; it < n_list; it += kSensThreads) {
+      const int le = list[it] >> 8, s = list[it] & 255;
+      ws[le * S + s] = sens_direct<PO, NF>(U + le * NF * 2 * NN, tab + ntab, d, s % d, s / d, nu, c1, c2);
+    }
+    __syncthreads();
+  }
+  double energy = 0.0;   // sum_s E(rho_s) w_s (eout)
+  if (el < ne) {
+    const int64_t off = design_off[elem[base + el]];
+    for (int s = t % tpe; s < S; s += tpe) {
+      const double w = ws[el * S + s] * jac, r = rho[off + s];
       if (dc) dc[off + s] = -q * (cube ? r * r : pow(r, q - 1.0)) * dE * w;
       if (eout) energy += (Emin + (cube ? r * r * r : pow(r, q)) * dE) * w;
     }
@@ -375,9 +565,8 @@ mto_status launch_poly(mto_handle h, const BClass& b, const double* u, const dou
   int EB = 32;
   while (EB > 4 && (EB * per * 8 > 36 * 1024 || b.n < EB * 304)) EB /= 2;
   const size_t smem = sizeof(double) * ((size_t)EB * per + ntab);
-  if (smem > 48 * 1024)
-    MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(sens_poly_kernel<PO, NF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem), "cudaFuncSetAttribute"));
+  static_assert(8 * (4 * sens_elem_doubles(PO, MTO_D_MAX, NF) + (3 * sens_q(PO, MTO_D_MAX) + 1) * (PO + 1) +
+                     MTO_D_MAX * sens_q(PO, MTO_D_MAX)) <= 48 * 1024, "four elements of the largest count fit 48 KB");
   sens_poly_kernel<PO, NF><<<(b.n + EB - 1) / EB, kSensThreads, smem, h->stream>>>(
       b.n, b.d, Q, EB, b.elem, b.slot, h->pc[b.p].gmap, h->cons_d, u, v, rho, h->design_off_d, m->E0, m->Emin, m->q,
       m->nu, h->hx, h->hy, b.stab, dc, eout);
@@ -437,8 +626,8 @@ mto_status sens_all32(mto_handle h, const double* u, const double* rho, const mt
 
 mto_status build_sens_tables(mto_handle h) {
   for (auto& b : h->bc) {
-    const int n1 = b.p + 1, G = b.d * n1, Q = sens_q(b.p, b.d);
-    MTO_TRY(mto_alloc(h, &b.stab, (size_t)(3 * Q + 1) * n1 + b.d * Q));
+    const int n1 = b.p + 1, G = b.d * n1;
+    MTO_TRY(mto_alloc(h, &b.stab, (size_t)sens_tab_len(b.p, b.d)));
     MTO_TRY(mto_alloc(h, &b.stabf, (size_t)2 * n1 * G + G));
     sens_table_kernel<<<1, 256, 0, h->stream>>>(b.p, b.d, h->hx, h->hy, b.stab, b.stabf);
     MTO_TRY(mto_after_launch(h, "sens_table_kernel"));

@@ -140,3 +140,81 @@ def test_qr_error_across_the_modulus_contrast(mto, p, d, design):
         want = oi.qr_error_element(p, d, rho[k], m.gather(k, u), 1.0, 1e-9, 0.3, 3.0)
         assert abs(a[k] - want) <= 2.0 ** -50 * kappa, (k, a[k], want, kappa)
     h.close()
+
+
+def subcell_energies(p, d, U, hx=1.0, hy=1.0, nu=0.3):
+    """Subcell energies u^T K0_s u of one element by the composite Gauss rule in extended precision."""
+    from oracle import basis as ob
+    ld = np.longdouble
+    z, n = ob.gll_nodes(p).astype(ld), p + 1
+    gx, gw = (a.astype(ld) for a in ob.gauss_legendre(n))
+    for _ in range(2):
+        a, b = np.ones_like(gx), gx.copy()
+        for k in range(2, n + 1):
+            a, b = b, ((2 * k - 1) * gx * b - (k - 1) * a) / k
+        dp = n * (gx * b - a) / (gx * gx - 1)
+        gx = gx - b / dp
+    gw = 2 / ((1 - gx * gx) * dp * dp)
+    pts = np.concatenate([-1 + (2 * i + 1 + gx) / ld(d) for i in range(d)])
+    L, D = np.ones((len(pts), n), ld), np.zeros((len(pts), n), ld)
+    for k in range(n):
+        for j in range(n):
+            if j != k:
+                L[:, k] *= (pts - z[j]) / (z[k] - z[j])
+        for i in range(n):
+            if i != k:
+                t = np.full(len(pts), 1 / (z[k] - z[i]))
+                for j in range(n):
+                    if j not in (i, k):
+                        t = t * (pts - z[j]) / (z[k] - z[j])
+                D[:, k] += t
+    D = 2 * D
+    ux, uy = (U[c::2].reshape(n, n).astype(ld) for c in (0, 1))
+    ev = lambda u, A, B: B @ u @ A.T          # [y, x]
+    ex, ey = ev(ux, D / hx, L), ev(uy, L, D / hy)
+    g = ev(ux, L, D / hy) + ev(uy, D / hx, L)
+    f = 1 / (ld(1) - ld(nu) * ld(nu))
+    en = f * (ex * ex + ey * ey + 2 * ld(nu) * ex * ey + (1 - ld(nu)) / 2 * g * g)
+    w = np.tile(gw / (2 * d), d)
+    return (en * w[None] * w[:, None] * hx * hy).reshape(d, n, d, n).sum((1, 3)).reshape(-1)
+
+
+@pytest.mark.parametrize("p,d", [(1, 16), (2, 3), (2, 8), (3, 8), (3, 16), (4, 8), (5, 12), (6, 2), (6, 8), (6, 16)])
+@pytest.mark.parametrize("kind", ["corner", "bend", "rough"])
+def test_small_subcell_energies(mto, p, d, kind):
+    """FP64 sensitivities of one element whose strain decays towards a corner (subcells down to 1e-20 of the
+    largest w), of a bending and of a rough one.  Signs: w >= 0, so dc <= 0.  Small subcells: w is a sum of squares
+    of strains, each a sum of 2 (p+1)^2 <= 98 products of values below (p+1)^2 times the largest strain's
+    scale / 5, so its error stays below 1000 2^-53 of the largest strain and w's below
+    1000 2^-53 sqrt(w w_max) + (1000 2^-53)^2 w_max.  Whole element: strains and their sums cost about eight
+    roundings in the 2-norm when the tables are correctly rounded."""
+    from oracle import basis as ob
+    hx, hy = 1.0, (0.5 if d == 8 else 1.0)
+    h = handle(mto, 1, 1, p, d, hx, hy)
+    z = ob.gll_nodes(p)
+    X, Y = np.meshgrid(z, z)
+    rng = np.random.default_rng(p)
+    if kind == "corner":
+        c = ((1 + X) * (1 + Y) / 4) ** p
+        U = np.stack([c, 0.7 * c], 2).ravel()
+    elif kind == "bend":
+        U = np.stack([X * (Y - 0.3), -0.5 * X * X - 0.15 * (Y - 0.3) ** 2], 2).ravel()
+    else:
+        U = rng.standard_normal(2 * (p + 1) ** 2)
+    u = np.zeros(h.ndof)
+    for ln, n in enumerate(h.element_nodes(0)):
+        u[2 * n[0][0]:2 * n[0][0] + 2] = U[2 * ln:2 * ln + 2]
+    want = subcell_energies(p, d, U, hx, hy)
+    dc = torch.zeros(h.design_len, dtype=torch.float64, device="cuda")
+    h.sensitivity(T(u), T(u), T(np.ones(h.design_len)), mto.material(1.0, 0.0, 0.3, 1.0), dc)
+    w = -dc.cpu().numpy()
+    assert (w >= 0.0).all()
+    err = np.abs(w - want)
+    eps = 1000 * 2.0 ** -53
+    assert (err <= eps * np.sqrt(want * want.max()) + eps ** 2 * want.max()).all()
+    assert np.linalg.norm(err.astype(float)) <= 8 * 2.0 ** -53 * np.linalg.norm(want.astype(float))
+    # the bilinear form with v = u takes the same path and gives the same values
+    dv = torch.zeros_like(dc)
+    h.sensitivity_adjoint(T(u), T(u), T(np.ones(h.design_len)), mto.material(1.0, 0.0, 0.3, 1.0), dv)
+    assert (np.abs(dv.cpu().numpy() + want) <= eps * np.sqrt(want * want.max()) + eps ** 2 * want.max()).all()
+    h.close()
