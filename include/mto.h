@@ -268,7 +268,11 @@ mto_status mto_element_nodes(mto_handle h, int64_t e, int64_t* nodes, double* we
  * split-precision FP32 pair (hi = fl32(K_e), lo = fl32(K_e - hi), ~48 bits), applied on the FP32
  * pipes with error-free products and sums by the inner iterations of the mixed solves.  Matrices
  * stay in the handle, one row of the circulant-diagonal layout per element (D_k[i] = K[i][i+k mod
- * n_e], k = 0 .. n_e/2), element-major per order class.  Asynchronous. */
+ * n_e], k = 0 .. n_e/2), element-major per order class.  Asynchronous.  A density whose modulus is
+ * not finite gives a matrix of NaN (a solve then returns MTO_ENAN).  Where a bounded wait of the tensor-core
+ * kernel expires, the rows it did not finish are NaN, and the calls that read the matrices and synchronise
+ * (mto_solve, mto_solve_batched, mto_apply_operator with xKx, mto_element_matrix) return MTO_ETIMEOUT until
+ * the next build. */
 mto_status mto_build_elements(mto_handle h, const double* rho, const mto_material* mat, int32_t precision);
 
 /* Inspection (tests, tools): the current matrix of element e as its packed upper triangle
@@ -427,7 +431,9 @@ mto_status mto_sensitivity_adjoint(mto_handle h, const double* u, const double* 
  * Outputs (device, [nel]): gamma_a (Kelly, Eq. 9, no square root), gamma_d (density indicator),
  * eps_qr (Eq. 14), p_new, d_new (int32, per-axis design count), theta (int8 flag: -2, -1, 0, 1).
  * Any output pointer may be NULL except those the later stages need internally (all are
- * computed).  Asynchronous. */
+ * computed).  Asynchronous.  Where a bounded wait of the tensor-core kernel that forms the QR error's matrices
+ * expires, the elements' eps_qr are NaN and MTO_ETIMEOUT comes from this call if it synchronises (a fraction
+ * alpha_d below 1), else from the next mto_setup. */
 mto_status mto_indicator(mto_handle h, const double* u, const double* rho, const mto_material* mat,
                          const mto_indicator_opts* opts, double* gamma_a, double* gamma_d,
                          double* eps_qr, int32_t* p_new, int32_t* d_new, int8_t* theta);

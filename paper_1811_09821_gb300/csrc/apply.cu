@@ -1413,7 +1413,7 @@ mto_status apply_operator(mto_handle h, int op, const double* x, double* y, doub
   double s = 0.0;
   for (int i = 0; i < nres; ++i) s += h->host_pinned[i];
   *xKx = s;
-  return MTO_OK;
+  return tc_check(h, TC_BUILD);
 }
 
 // Autotuner of the split operator's kernel per order class (n_e <= 32: register pipeline, bulk-copy
@@ -1573,6 +1573,7 @@ mto_status solve(mto_handle h, const double* f, double* u, const mto_solve_opts*
     // FP64 residual with the FP64 element matrices
     h->inner_split = false;
     MTO_TRY(true_residual(h, f, u, nrm, &rr, &ff));
+    MTO_TRY(tc_check(h, TC_BUILD));
     MTO_TRY(mg_build_check(h));
     if (h->solve_log)
       std::fprintf(stderr, "mto_solve: step %d inner_iters %d relres %.3e split %d wall_ms %.1f\n", outer, last_it,
@@ -1694,7 +1695,8 @@ mto_status job_on_residual(BatchJob& j) {
   const mto_solve_opts* o = j.o;
   residual_take(h, j.nrm, &j.rr, &j.ff);
   {
-    const mto_status sb = mg_build_check(h);
+    const mto_status st = tc_check(h, TC_BUILD);
+    const mto_status sb = st != MTO_OK ? st : mg_build_check(h);
     if (sb != MTO_OK) {
       job_finish(j, sb);
       return MTO_OK;

@@ -417,7 +417,7 @@ mto_status element_matrix(mto_handle h, int64_t e, double* host_out) {
     st = mto_cuda_check(h, cudaMemcpyAsync(host_out, tmp, sizeof(double) * c.P, cudaMemcpyDeviceToHost, h->stream), "copy");
   if (st == MTO_OK) st = mto_cuda_check(h, cudaStreamSynchronize(h->stream), "sync");
   cudaFree(tmp);
-  return st;
+  return st != MTO_OK ? st : tc_check(h, TC_BUILD);
 }
 
 __global__ void gather_element_split_kernel(int P, int L, const int2* __restrict__ dpos, int slot,
@@ -448,7 +448,7 @@ mto_status element_matrix_split(mto_handle h, int64_t e, float* hi, float* lo) {
                         "copy");
   if (st == MTO_OK) st = mto_cuda_check(h, cudaStreamSynchronize(h->stream), "sync");
   cudaFree(tmp);
-  return st;
+  return st != MTO_OK ? st : tc_check(h, TC_BUILD);
 }
 
 mto_status build_tables(mto_handle h) {
@@ -477,6 +477,7 @@ mto_status build_tables(mto_handle h) {
 
 mto_status build_elements(mto_handle h, const double* rho, const mto_material* m, int precision) {
   TimedScope ts(h, F_BUILD);
+  ++h->tc_tag[TC_BUILD];
   // the subcell tables depend only on nu (and the mesh): computed on the first build and again
   // whenever nu changes
   if (!(h->k0_nu == m->nu)) {

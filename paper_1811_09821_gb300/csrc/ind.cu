@@ -1131,6 +1131,7 @@ mto_status map_update(mto_handle h, const double* ga, const double* gd, const do
     unsigned long long hc[2];
     MTO_TRY(mto_cuda_check(h, cudaMemcpyAsync(hc, cnt, sizeof(hc), cudaMemcpyDeviceToHost, h->stream), "copy"));
     MTO_TRY(mto_cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
+    MTO_TRY(tc_check(h, TC_INDICATOR));
     const int64_t nneg = (int64_t)hc[0], npos = (int64_t)hc[1];
     if (T.dc_mode == 0) {
       const int64_t kc = (int64_t)std::floor(o->alpha_d_coarsen * (double)nneg);
@@ -1193,6 +1194,7 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
   gamma_d_kernel<<<grid_for(nel, 32 * kGdWarps, 152 * 6), 32 * kGdWarps, 0, h->stream>>>(
       nel, h->design_off_d, rho, mm, o->cycle, o->alpha, o->beta, gd_);
   MTO_TRY(mto_after_launch(h, "gamma_d_kernel"));
+  ++h->tc_tag[TC_INDICATOR];
   // QR error per (p, d) class, in chunks of elements whose rows fit 448 MB, full waves of the row
   // kernel (128 elements per SM) where a chunk is that large (38,912 elements of Q3)
   for (size_t ci = 0; ci < h->bc.size(); ++ci) {
@@ -1221,7 +1223,8 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
     }
     for (int first = 0; first < b.n; first += chunk) {
       const int cn = std::min(chunk, b.n - first);
-      if (tc) MTO_TRY(tc_rows(h, b, b1, L1, first, cn, nullptr, rho, m, h->qr_rows, nullptr, nullptr));
+      if (tc) MTO_TRY(tc_rows(h, b, b1, L1, first, cn, nullptr, rho, m, h->qr_rows, nullptr, nullptr,
+                              TC_INDICATOR));
       qr_kernel<<<cn, 32, smem, h->stream>>>(b.p, b.d, b.n, first, b.elem, b.slot, c.L, c.gmap, h->cons_d, c.K64,
                                              tc ? h->qr_rows : nullptr, b1.K0T, h->qr[b.p].R, u, rho,
                                              h->design_off_d, m->E0, m->Emin, m->q, B, h->hx, h->hy, eq_);

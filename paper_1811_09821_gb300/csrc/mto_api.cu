@@ -329,6 +329,8 @@ mto_status mto_create(mto_handle* out, int device, void* stream) {
   // mto_set_operator_kernel does (register pipeline / bulk-copy staging / generic)
   if (const char* ok = std::getenv("MTO_OP_KERNEL"))
     h->op_kernel = (ok[0] >= '0' && ok[0] <= '2') ? ok[0] - '0' : -1;
+  // MTO_TC_POLLS=n: polls before a wait of the tensor-core build expires (0: at once, to test the error path)
+  if (const char* tp = std::getenv("MTO_TC_POLLS")) h->tc_polls = (unsigned)std::strtoul(tp, nullptr, 10);
   cudaSetDevice(device);
   if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
@@ -351,6 +353,7 @@ mto_status mto_create(mto_handle* out, int device, void* stream) {
     delete h;
     return MTO_ENOMEM;
   }
+  std::memset(h->host_flags, 0, 16 * sizeof(int));
   *out = h;
   return MTO_OK;
 }
@@ -401,6 +404,12 @@ mto_status mto_setup(mto_handle h, int32_t nelx, int32_t nely, double hx, double
       return mto_fail(h, MTO_EINVAL, "mto_setup: d outside 1..MTO_D_MAX at element " + std::to_string(e));
   }
   cudaSetDevice(h->device);
+  if (h->tc_tag[TC_INDICATOR]) {   // the maps may come from an indicator whose wait expired: reported once
+    MTO_TRY(mto_cuda_check(h, cudaStreamSynchronize(h->stream), "mto_setup"));
+    const mto_status st = tc_check(h, TC_INDICATOR);
+    h->host_flags[9 + TC_INDICATOR] = 0;
+    MTO_TRY(st);
+  }
   release_mesh(h);
   h->nelx = nelx;
   h->nely = nely;

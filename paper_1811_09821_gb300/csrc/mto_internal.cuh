@@ -79,6 +79,11 @@ struct QRTab {
 // Row length of the QR indicator's order-p matrices: the packed lower triangle, padded to whole 32 bytes.
 __host__ __device__ constexpr int qr_row_len(int p) { return round_up(packed_size(2 * (p + 1) * (p + 1)), 4); }
 
+// The uses of the tensor-core rows (tc.cu), each with its own error word: host_flags[9 + use] holds the tag
+// of the launch whose wait expired, tc_tag[use] that of the current one.
+enum TcUse { TC_BUILD = 0, TC_INDICATOR = 1 };
+constexpr unsigned kTcPolls = 1u << 26;   // polls of a barrier before its wait expires
+
 // Kernel families timed with CUDA events when timing is enabled (see mto_timing_enable).
 enum Family { F_APPLY32 = 0, F_APPLY64 = 1, F_BUILD = 2, F_SENS = 3, F_INDICATOR = 4, F_VECTOR = 5,
               F_APPLYDF64 = 6, F_PRECOND = 7, F_OC = 8, F_APPLYLEAD = 9, F_COUNT = 10 };
@@ -248,7 +253,9 @@ struct mto_handle_s {
   double* red = nullptr;                       // misc reduction scratch [64]
   double* eng = nullptr;                       // CG energy log of the compliance-accuracy test [128]
   int* flags = nullptr;                        // [0] iterations when done, [1] error code, [2..] misc
-  int* host_flags = nullptr;                   // pinned host mirror of flags[0..1]
+  int* host_flags = nullptr;                   // pinned: mirror of flags[0..1], [8] of flags[6], [9..] expired waits
+  int tc_tag[2] = {0, 0};                      // see TcUse
+  unsigned tc_polls = mto::kTcPolls;
   double* host_pinned = nullptr;               // pinned host mirror for small read-backs [64]
   unsigned long long* sel = nullptr;           // selection / small integer scratch [1024]
   void* basis_tab = nullptr;                   // GLL / Gauss tables for the indicator kernels
@@ -473,7 +480,8 @@ void mg_release(mto_handle h);
 mto_status tc_tables(mto_handle h);
 mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision);
 mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int first, int n, const int* slot,
-                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl);
+                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl, TcUse use);
+mto_status tc_check(mto_handle h, TcUse use);                            // expired waits, after a synchronisation
 int ebe_blocks(int p, int n);                                           // grid of one operator launch
 // apply.cu
 mto_status apply64(mto_handle h, const double* x, double* y);        // y += K x (FP64 vectors)

@@ -30,7 +30,8 @@
 // tile before.  Warps 0-7 read their row's 8 positions with tcgen05.ld and write whole sectors of
 // their rows through a small shared staging.
 // Operands use the no-swizzle K-major core-matrix layout (8 rows x 16 bytes per core matrix).
-// Every wait is bounded: on expiry the kernel records an error word and stops this CTA.
+// Every wait is bounded: on expiry the CTA records an error word that the host reads (tc_check), waits for
+// its own copies and MMAs in flight, and its rows are NaN from there on.
 //
 // Measured (build and one operator product together): 480 x 240 Q3/d8, mixed: 5.32 ms with an FP64
 // epilogue of 24 FP64 instructions per entry and 43 single-slice MMAs per K step, 1.10 ms now;
@@ -39,6 +40,8 @@
 #include <cstdio>
 #include <cstring>
 #include <vector>
+
+#include <math_constants.h>
 
 #include "mto_internal.cuh"
 
@@ -59,7 +62,6 @@ constexpr int kTmemStage = 256;
 // 16-byte stores by 32 lanes)
 constexpr int kStRow64 = 80, kStRow32 = 48;
 constexpr int kStWarp = 32 * (kStRow64 + 2 * kStRow32);
-constexpr unsigned kSpinLimit = 1u << 26;
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -150,8 +152,8 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 }
 
 // bounded wait for the phase of parity `parity`; false when the limit expires
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
-  for (unsigned n = 0; n < kSpinLimit; ++n)
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned limit) {
+  for (unsigned n = 0; n < limit; ++n)
     if (mbar_try_wait(bar, parity)) return true;
   return false;
 }
@@ -279,12 +281,12 @@ __host__ __device__ __forceinline__ void split_pair(unsigned long long bits, flo
 constexpr int kRowNaN = 1 << 20;
 
 // rows: element k of the class (first <= k < n) is output row slot[k], or row k - first without slots.
-// Kh null: FP64 rows only.
+// Kh null: FP64 rows only.  err: the host's error word (pinned), which receives `tag` when a wait expires.
 __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
     int n, int first, int S, int kpad, int L, int ntile, int tiles_per_cta, const int* __restrict__ elem,
     const int* __restrict__ slot, const int64_t* __restrict__ design_off, const double* __restrict__ rho, double E0,
     double Emin, double q, const unsigned short* __restrict__ Bt, const int* __restrict__ tau,
-    double* __restrict__ K64, float* __restrict__ Kh, float* __restrict__ Kl, int* __restrict__ err) {
+    double* __restrict__ K64, float* __restrict__ Kh, float* __restrict__ Kl, unsigned limit, volatile int* err, int tag) {
   extern __shared__ __align__(1024) unsigned char smem[];
   const uint32_t a_slice = (uint32_t)kTM * kpad * 2, b_slice = (uint32_t)kTN * kpad * 2;
   const uint32_t b_tile = kSlices * b_slice;
@@ -369,10 +371,11 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
       const uint32_t sbo = (uint32_t)(kpad >> 3) * 128u;
       const int kst = kpad / 16;
       const uint32_t a0 = smem_u32(As);
+      int issued = min(kBRing, nt), committed = 0;
       for (int it = 0; it < nt && ok; ++it) {
         const int st = it & 1;
-        ok = mbar_wait(bfull + it % kBRing, (uint32_t)((it / kBRing) & 1));
-        if (ok && it >= 2) ok = mbar_wait(empty + st, (uint32_t)(((it >> 1) - 1) & 1));
+        ok = mbar_wait(bfull + it % kBRing, (uint32_t)((it / kBRing) & 1), limit);
+        if (ok && it >= 2) ok = mbar_wait(empty + st, (uint32_t)(((it >> 1) - 1) & 1), limit);
         if (!ok) break;
         tc_fence_after();
         const uint32_t b0 = smem_u32(Bs + (it % kBRing) * b_tile);
@@ -389,22 +392,24 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
         for (int i = 3; i <= kSlices; ++i)
           for (int ks = 0; ks < kst; ++ks) mma(i, 1, kLevels + 1 - i, ks, 1);
         umma_commit(full + st);
+        committed = it + 1;
         // refill the ring slot of the tile before, whose MMAs are done once its stage is committed
         if (it >= 1 && it - 1 + kBRing < nt) {
           const int nx = it - 1 + kBRing;
-          ok = mbar_wait(full + (st ^ 1), (uint32_t)(((it - 1) >> 1) & 1));
+          ok = mbar_wait(full + (st ^ 1), (uint32_t)(((it - 1) >> 1) & 1), limit);
           if (!ok) break;
           mbar_expect(bfull + nx % kBRing, b_tile);
           tc_bulk_g2s(Bs + (nx % kBRing) * b_tile, reinterpret_cast<const unsigned char*>(Bt) + (size_t)(tile0 + nx) * b_tile,
                       b_tile, bfull + nx % kBRing);
+          issued = nx + 1;
         }
       }
       if (!ok) {
-        // a wait expired: let every copy that was issued land before the CTA gives up its memory
-        for (int b = 0; b < kBRing; ++b) {
-          mbar_wait(bfull + b, 0);
-          mbar_wait(bfull + b, 1);
-        }
+        // a wait expired: every copy that was issued lands, and every MMA ends, before the CTA gives up its memory
+        for (int i = max(0, issued - kBRing); i < issued; ++i)
+          mbar_wait(bfull + i % kBRing, (uint32_t)((i / kBRing) & 1), kTcPolls);
+        if (committed > 0)
+          mbar_wait(full + ((committed - 1) & 1), (uint32_t)(((committed - 1) >> 1) & 1), kTcPolls);
       }
     }
     __syncwarp();
@@ -416,9 +421,10 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
     unsigned char* st64 = stage + warp * kStWarp;
     unsigned char* sth = st64 + 32 * kStRow64;
     unsigned char* stl = sth + 32 * kStRow32;
-    for (int it = 0; it < nt; ++it) {
+    int it = 0;
+    for (; it < nt; ++it) {
       const int st = it & 1;
-      ok = mbar_wait(full + st, (uint32_t)((it >> 1) & 1));
+      ok = mbar_wait(full + st, (uint32_t)((it >> 1) & 1), limit);
       if (!__all_sync(0xffffffffu, ok)) {
         ok = false;
         break;
@@ -478,9 +484,15 @@ __global__ void __launch_bounds__(32 * (kEpiWarps + 1), 1) tc_build_kernel(
         __syncwarp();
       }
     }
+    for (; it < nt && sl >= 0; ++it)   // after an expired wait
+      for (int pos = (tile0 + it) * kTN + c0; pos < min((tile0 + it) * kTN + c0 + 8, L); ++pos) {
+        const size_t at = (size_t)sl * L + pos;
+        K64[at] = CUDART_NAN;
+        if (Kh) Kh[at] = Kl[at] = CUDART_NAN_F;
+      }
   }
   tc_fence_before();
-  if (__syncthreads_or(!ok) && t == 0) atomicExch(err, 1);   // the rows are not trustworthy
+  if (__syncthreads_or(!ok) && t == 0) *err = tag;
   tc_fence_after();
   if (warp == 0) tmem_dealloc(tmem, kTmemCols);
 }
@@ -523,7 +535,7 @@ size_t tc_smem_bytes(int kpad) {
 // The N tiles of few elements are split over CTAs (each forms its elements' A slices again, about the
 // cost of three tiles) until the launch has about one CTA per SM.
 mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int first, int n, const int* slot,
-                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl) {
+                   const double* rho, const mto_material* m, double* K64, float* Kh, float* Kl, TcUse use) {
   const int kpad = (b.S + 15) / 16 * 16;
   const int ntile = (L + kTN - 1) / kTN;
   const size_t smem = tc_smem_bytes(kpad);
@@ -534,7 +546,7 @@ mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int 
   const int per = (ntile + gy - 1) / gy;
   tc_build_kernel<<<dim3(gx, (ntile + per - 1) / per), 32 * (kEpiWarps + 1), smem, h->stream>>>(
       first + n, first, b.S, kpad, L, ntile, per, b.elem, slot, h->design_off_d, rho, m->E0, m->Emin, m->q, tab.tcB,
-      tab.tcTau, K64, Kh, Kl, h->flags + 4);
+      tab.tcTau, K64, Kh, Kl, h->tc_polls, h->host_flags + 9 + use, h->tc_tag[use]);
   return mto_after_launch(h, "tc_build_kernel");
 }
 
@@ -542,7 +554,16 @@ mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int 
 mto_status tc_build_class(mto_handle h, const BClass& b, const double* rho, const mto_material* m, int precision) {
   const PClass& c = h->pc[b.p];
   const bool mixed = precision == MTO_MIXED;
-  return tc_rows(h, b, b, c.L, 0, b.n, b.slot, rho, m, c.K64, mixed ? c.K32 : nullptr, mixed ? c.K32lo : nullptr);
+  return tc_rows(h, b, b, c.L, 0, b.n, b.slot, rho, m, c.K64, mixed ? c.K32 : nullptr, mixed ? c.K32lo : nullptr,
+                 TC_BUILD);
+}
+
+// After a synchronisation of the stream: whether a wait of the current build (or the last indicator's
+// rows) expired.
+mto_status tc_check(mto_handle h, TcUse use) {
+  if (h->host_flags[9 + use] != h->tc_tag[use] || h->tc_tag[use] == 0) return MTO_OK;
+  return mto_fail(h, MTO_ETIMEOUT, use == TC_BUILD ? "element build: a bounded device wait expired"
+                                                   : "QR indicator: a bounded device wait expired");
 }
 
 }  // namespace mto

@@ -218,3 +218,53 @@ def test_small_subcell_energies(mto, p, d, kind):
     h.sensitivity_adjoint(T(u), T(u), T(np.ones(h.design_len)), mto.material(1.0, 0.0, 0.3, 1.0), dv)
     assert (np.abs(dv.cpu().numpy() + want) <= eps * np.sqrt(want * want.max()) + eps ** 2 * want.max()).all()
     h.close()
+
+
+def test_expired_waits_are_reported(mto, monkeypatch):
+    """With a limit of no polls every wait of the tensor-core build expires: its rows are NaN, every call that
+    reads them and synchronises returns MTO_ETIMEOUT (6), the indicator's own rows likewise (eps_qr NaN, the map
+    update's read-back and the next mto_setup report it), and the CUDA-core build that follows is sound."""
+    monkeypatch.setenv("MTO_TC_POLLS", "0")
+    nx, ny, p, d = 43, 3, 2, 4
+    h = handle(mto, nx, ny, p, d)
+    fixed, f = mto.load_case(h, "cantilever")
+    h.set_supports(fixed)
+    mat = mto.material()
+    rho = torch.full((h.design_len,), 0.6, dtype=torch.float64, device="cuda")
+    u = torch.zeros(h.ndof, dtype=torch.float64, device="cuda")
+
+    def timeout(fn, *a, **k):
+        with pytest.raises(mto.MTOError) as ei:
+            fn(*a, **k)
+        assert ei.value.status == 6
+
+    h.build_elements(rho, mat, mto.MTO_MIXED)
+    timeout(h.element_matrix, 5, p)
+    timeout(h.element_matrix_split, 128, p)
+    timeout(h.apply_operator, torch.ones_like(u), torch.empty_like(u), mto.OP_SPLIT)
+    for pc in (mto.PREC_JACOBI, mto.PREC_SCHWARZ, mto.PREC_MG):
+        timeout(h.solve, f, u, precision=mto.MTO_MIXED, precond=pc)
+    timeout(mto.solve_batched, [h], [f], [u])
+    y = torch.zeros_like(u)
+    h.apply(torch.ones_like(u), y)
+    assert torch.isnan(y).all()
+    h.set_build_path(mto.BUILD_SIMT)
+    h.build_elements(rho, mat, mto.MTO_MIXED)
+    assert np.isfinite(h.element_matrix(5, p)).all()
+    it, rr = h.solve(f, u, precision=mto.MTO_MIXED, precond=mto.PREC_MG, rtol=1e-9)
+    assert rr <= 1e-9
+    want = h.indicator(u, rho, mat)["eps_qr"]
+    h.set_build_path(mto.BUILD_TENSOR)
+    assert torch.isnan(h.indicator(u, rho, mat, maps=False)["eps_qr"]).all()
+    o = mto.IndicatorOpts.paper(1)
+    o.alpha_d_refine = 0.5
+    timeout(h.indicator, u, rho, mat, o)
+    args = (nx, ny, np.full(nx * ny, p, np.int32), np.full(nx * ny, d, np.int32))
+    h.indicator(u, rho, mat)
+    timeout(h.setup, *args)
+    h.setup(*args)
+    h.set_supports(fixed)
+    h.set_build_path(mto.BUILD_SIMT)
+    h.build_elements(rho, mat, mto.MTO_MIXED)
+    assert torch.equal(h.indicator(u, rho, mat)["eps_qr"], want)
+    h.close()
