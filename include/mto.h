@@ -431,7 +431,10 @@ mto_status mto_sensitivity_adjoint(mto_handle h, const double* u, const double* 
  * Outputs (device, [nel]): gamma_a (Kelly, Eq. 9, no square root), gamma_d (density indicator),
  * eps_qr (Eq. 14), p_new, d_new (int32, per-axis design count), theta (int8 flag: -2, -1, 0, 1).
  * Any output pointer may be NULL except those the later stages need internally (all are
- * computed).  Asynchronous.  Where a bounded wait of the tensor-core kernel that forms the QR error's matrices
+ * computed).  Asynchronous.  With MTO_BUILD_TENSOR the QR error's matrices of classes with d <= 8 pass
+ * through device memory of the handle, up to 448 MB in chunks (smaller ones where less is left, else the
+ * matrices are summed where they are used), kept until the next mto_setup.  Where a bounded wait of the
+ * tensor-core kernel that forms the QR error's matrices
  * expires, the elements' eps_qr are NaN and MTO_ETIMEOUT comes from this call if it synchronises (a fraction
  * alpha_d below 1), else from the next mto_setup. */
 mto_status mto_indicator(mto_handle h, const double* u, const double* rho, const mto_material* mat,

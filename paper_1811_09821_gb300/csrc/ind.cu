@@ -1202,7 +1202,7 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
     const BClass& b1 = h->bc_qr[ci];
     const PClass& c = h->pc[b.p];
     const int n0 = 2 * (b.p + 1) * (b.p + 1), n1 = 2 * (b.p + 2) * (b.p + 2), L1 = qr_row_len(b.p + 1);
-    const bool tc = h->build_path == MTO_BUILD_TENSOR && b1.tcB;
+    bool tc = h->build_path == MTO_BUILD_TENSOR && b1.tcB;
     const size_t smem = sizeof(double) * ((size_t)L1 + 2 * n0 + 2 * n1 + std::max(5 * n1, b.S));
     if (smem > 48 * 1024) cudaFuncSetAttribute(qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int chunk = b.n;
@@ -1214,11 +1214,20 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
         if (h->qr_rows) {
           MTO_TRY(mto_cuda_check(h, cudaStreamSynchronize(h->stream), "sync"));
           cudaFree(h->qr_rows);
+          h->qr_rows = nullptr;
           h->bytes -= (int64_t)(h->qr_cap * sizeof(double));
           h->qr_cap = 0;
         }
-        MTO_TRY(mto_alloc(h, &h->qr_rows, (size_t)chunk * L1));
-        h->qr_cap = (size_t)chunk * L1;
+        // where the device has not that much left: smaller chunks, or the sums in the kernel
+        while (mto_alloc(h, &h->qr_rows, (size_t)chunk * L1) != MTO_OK && chunk > 128)
+          chunk = (chunk / 2 + 127) / 128 * 128;
+        if (h->qr_rows) h->qr_cap = (size_t)chunk * L1;
+        else {
+          tc = false;
+          chunk = b.n;
+        }
+        cudaGetLastError();
+        h->err.clear();
       }
     }
     for (int first = 0; first < b.n; first += chunk) {

@@ -268,3 +268,49 @@ def test_expired_waits_are_reported(mto, monkeypatch):
     h.build_elements(rho, mat, mto.MTO_MIXED)
     assert torch.equal(h.indicator(u, rho, mat)["eps_qr"], want)
     h.close()
+
+
+@pytest.mark.parametrize("left", [24 << 20, 0])
+def test_indicator_with_little_memory_left(mto, left):
+    """The QR indicator wants 61 MB for its matrices here; with 24 MB of device memory left it takes smaller
+    chunks (equal bits), with none it sums in the kernel (equal bits with the CUDA-core path)."""
+    nx, ny, p, d = 100, 60, 3, 8
+    h = handle(mto, nx, ny, p, d)
+    h.set_supports(h.side_dofs(0))
+    mat = mto.material()
+    rng = np.random.default_rng(0)
+    rho = T(rng.uniform(0.5, 1.0, h.design_len))
+    u = T(rng.standard_normal(h.ndof))
+    h.build_elements(rho, mat)
+    h.set_build_path(mto.BUILD_SIMT)
+    sums = h.indicator(u, rho, mat)
+    g = handle(mto, nx, ny, p, d)
+    g.set_supports(g.side_dofs(0))
+    g.build_elements(rho, mat)
+    rows = g.indicator(u, rho, mat)["eps_qr"]
+    want = rows if left else sums["eps_qr"]
+    g.close()
+    assert not torch.equal(rows, sums["eps_qr"])   # the two paths differ in their last bits
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    hold = [torch.empty(max(0, torch.cuda.mem_get_info()[0] - left - (64 << 20)) >> 21 << 21, dtype=torch.uint8, device="cuda")]
+    spare = torch.empty(1 << 20, dtype=torch.uint8, device="cuda")
+    try:
+        while torch.cuda.mem_get_info()[0] > left + (2 << 20):
+            hold.append(torch.empty(1 << 20, dtype=torch.uint8, device="cuda"))
+    except torch.cuda.OutOfMemoryError:
+        pass
+    del spare   # the outputs' memory
+    try:
+        h.set_build_path(mto.BUILD_TENSOR)
+        for _ in range(2):
+            got = h.indicator(u, rho, mat)
+            assert torch.equal(got["eps_qr"], want)
+            for k in ("p_new", "d_new", "theta"):
+                assert torch.equal(got[k], sums[k])
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+    got = h.indicator(u, rho, mat)
+    assert torch.equal(got["eps_qr"], rows)
+    h.close()
