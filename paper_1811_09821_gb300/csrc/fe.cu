@@ -367,9 +367,7 @@ mto_status launch_schwarz(mto_handle h, PClass& c) {
   constexpr int NE = 2 * (PO + 1) * (PO + 1), P = NE * (NE + 1) / 2;
   const int wpb = NE <= 32 ? 8 : (NE <= 50 ? 4 : 2);
   const size_t smem = (size_t)wpb * (P + 2 * NE) * sizeof(double) + (size_t)wpb * NE * sizeof(int) + 2 * P + 16;
-  if (smem > 48 * 1024)
-    MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(schwarz_kernel<PO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   (int)smem), "cudaFuncSetAttribute"));
+  MTO_TRY(allow_smem(h, schwarz_kernel<PO>, smem));   // one size per order
   const bool df = h->built_precision == MTO_MIXED;
   const int blocks = grid_for(c.n, wpb, 152 * 8);
   schwarz_kernel<PO><<<blocks, 32 * wpb, smem, h->stream>>>(c.n, c.L, c.gmap, h->cons_d, c.K64, h->diag64, h->invd64,
@@ -509,9 +507,8 @@ mto_status build_elements(mto_handle h, const double* rho, const mto_material* m
       MTO_TRY(tc_build_class(h, b, rho, m, precision));
       continue;
     }
-    size_t smem = sizeof(double) * 32 * (b.S | 1);
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(build_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(double) * 32 * (b.S | 1);
+    MTO_TRY(allow_smem(h, build_simt_kernel, sizeof(double) * 32 * (MTO_D_MAX * MTO_D_MAX + 1)));
     build_simt_kernel<<<(b.n + 31) / 32, 256, smem, h->stream>>>(
         b.n, b.S, b.P, b.elem, b.slot, h->design_off_d, rho, m->E0, m->Emin, m->q, b.K0T, c.L, c.dpos,
         c.K64, precision == MTO_MIXED ? c.K32 : nullptr, precision == MTO_MIXED ? c.K32lo : nullptr);

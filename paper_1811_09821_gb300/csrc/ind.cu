@@ -298,6 +298,12 @@ __global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
 // 16, up to 1.7 times for 125 and up to 4.5 times for 1e9: rows serve the elements within kQRContrast.
 constexpr double kQRContrast = 16.0;
 
+// dynamic shared memory of qr_kernel (its layout above)
+size_t qr_smem_bytes(int p, int S) {
+  const int n0 = 2 * (p + 1) * (p + 1), n1 = 2 * (p + 2) * (p + 2);
+  return sizeof(double) * ((size_t)qr_row_len(p + 1) + 2 * n0 + 2 * n1 + std::max(5 * n1, S));
+}
+
 // whether the moduli's extremes over the element (lo, hi; ok: every one is a number of at least 0) let the rows be used
 __device__ __forceinline__ bool sliced_rows_hold(bool ok, double lo, double hi) {
   for (int o = 16; o > 0; o >>= 1) {
@@ -1201,10 +1207,10 @@ mto_status indicators(mto_handle h, const double* u, const double* rho, const mt
     const BClass& b = h->bc[ci];
     const BClass& b1 = h->bc_qr[ci];
     const PClass& c = h->pc[b.p];
-    const int n0 = 2 * (b.p + 1) * (b.p + 1), n1 = 2 * (b.p + 2) * (b.p + 2), L1 = qr_row_len(b.p + 1);
+    const int L1 = qr_row_len(b.p + 1);
     bool tc = h->build_path == MTO_BUILD_TENSOR && b1.tcB;
-    const size_t smem = sizeof(double) * ((size_t)L1 + 2 * n0 + 2 * n1 + std::max(5 * n1, b.S));
-    if (smem > 48 * 1024) cudaFuncSetAttribute(qr_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = qr_smem_bytes(b.p, b.S);
+    MTO_TRY(allow_smem(h, qr_kernel, qr_smem_bytes(MTO_P_MAX, MTO_D_MAX * MTO_D_MAX)));
     int chunk = b.n;
     if (tc) {
       const int wave = 152 * 128;
@@ -1270,9 +1276,7 @@ mto_status oc_update(mto_handle h, const double* rho, const double* dc, double v
   MTO_TRY(mto_after_launch(h, "oc_prep_kernel"));
   if (n <= kOCSmall) {
     const size_t smem = 3 * sizeof(double) * (size_t)n;
-    if (smem > 48 * 1024)
-      MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(oc_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                     3 * (int)sizeof(double) * kOCSmall), "cudaFuncSetAttribute"));
+    MTO_TRY(allow_smem(h, oc_small_kernel, 3 * sizeof(double) * kOCSmall));
     oc_small_kernel<<<1, 1024, smem, h->stream>>>((int)n, T, Lo, Hi, eta, target, tol, st);
     MTO_TRY(mto_after_launch(h, "oc_small_kernel"));
   } else {

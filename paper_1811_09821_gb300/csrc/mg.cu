@@ -990,6 +990,9 @@ __global__ void mg_cheb_coef_kernel(int nlev, const double* __restrict__ lmax, d
 
 int vec_grid(int64_t n) { return grid_for(n, 256, kMGBlocks); }
 
+// dynamic shared memory of mg_strip_chain_kernel for m DOFs a line
+size_t strip_smem_bytes(int m) { return sizeof(double) * (2 * m * (m + 1) + 6 * m); }
+
 StripGeom strip_geom(const MGLevel& L) {
   StripGeom g;
   g.nx = L.nx;
@@ -1332,11 +1335,9 @@ mto_status mg_build(mto_handle h) {
     const StripGeom g = strip_geom(C);
     double* Gc = h->mg_Awork;
     MTO_TRY(mto_cuda_check(h, cudaMemsetAsync(h->flags + 6, 0, sizeof(int), h->stream), "memset"));
-    const size_t smem = sizeof(double) * (2 * g.m * (g.m + 1) + 6 * g.m);
+    const size_t smem = strip_smem_bytes(g.m);
     auto chain = [&](auto kernel) -> mto_status {
-      if (smem > 48 * 1024)
-        MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
-                               "cudaFuncSetAttribute"));
+      MTO_TRY(allow_smem(h, kernel, strip_smem_bytes(kLineMax)));
       for (int middle = 0; middle < 2; ++middle) {
         kernel<<<middle ? 1 : 2, kInvThreads, smem, h->stream>>>(g, middle, C.S, C.mask, Gc, h->flags + 6);
         MTO_TRY(mto_after_launch(h, "mg_strip_chain_kernel"));

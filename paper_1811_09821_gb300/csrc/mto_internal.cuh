@@ -313,6 +313,15 @@ mto_status mto_alloc(mto_handle h, T** ptr, size_t count) {
   return MTO_OK;
 }
 
+// Allows `most` bytes of dynamic shared memory to a kernel: the largest size of any call and not the
+// coming launch's, since the limit is the process's and another thread may be about to launch too.
+template <typename K>
+mto_status allow_smem(mto_handle h, K* kernel, size_t most) {
+  if (most <= 48 * 1024) return MTO_OK;
+  return mto_cuda_check(h, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most),
+                        "cudaFuncSetAttribute");
+}
+
 inline int grid_for(int64_t n, int block, int cap = 152 * 16) {
   int64_t g = (n + block - 1) / block;
   if (g < 1) g = 1;

@@ -577,13 +577,10 @@ mto_status launch_poly(mto_handle h, const BClass& b, const double* u, const dou
 template <int PO>
 mto_status launch_sens(mto_handle h, const BClass& b, const double* u, const double* rho, const mto_material* m,
                        double* dc) {
-  const int N1 = PO + 1, G = b.d * N1;
-  const size_t per_warp = (size_t)(4 * N1 * G + G + 2 * N1 * N1) * sizeof(float);
-  const int warps = 4;
-  const size_t smem = per_warp * warps;
-  if (smem > 227 * 1024) return mto_fail(h, MTO_EINVAL, "sensitivity: element class too large for shared memory");
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(sens_kernel<PO>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int N1 = PO + 1, warps = 4;
+  auto smem_bytes = [](int d) { return sizeof(float) * warps * (size_t)(4 * N1 * d * N1 + d * N1 + 2 * N1 * N1); };
+  const size_t smem = smem_bytes(b.d);
+  MTO_TRY(allow_smem(h, sens_kernel<PO>, smem_bytes(MTO_D_MAX)));
   const PClass& c = h->pc[b.p];
   const int Q = sens_q(PO, b.d);
   sens_kernel<PO><<<(b.n + warps - 1) / warps, 32 * warps, smem, h->stream>>>(

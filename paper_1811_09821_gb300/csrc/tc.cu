@@ -539,8 +539,7 @@ mto_status tc_rows(mto_handle h, const BClass& b, const BClass& tab, int L, int 
   const int kpad = (b.S + 15) / 16 * 16;
   const int ntile = (L + kTN - 1) / kTN;
   const size_t smem = tc_smem_bytes(kpad);
-  MTO_TRY(mto_cuda_check(h, cudaFuncSetAttribute(tc_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)smem), "cudaFuncSetAttribute"));
+  MTO_TRY(allow_smem(h, tc_build_kernel, tc_smem_bytes(64)));
   const int gx = (n + kTM - 1) / kTM;
   const int gy = std::max(1, std::min(ntile, 152 / gx));
   const int per = (ntile + gy - 1) / gy;

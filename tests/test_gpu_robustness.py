@@ -314,3 +314,44 @@ def test_indicator_with_little_memory_left(mto, left):
     got = h.indicator(u, rho, mat)
     assert torch.equal(got["eps_qr"], rows)
     h.close()
+
+
+def test_threads_with_different_sizes(mto):
+    """Three threads on three handles whose kernels ask for different amounts of shared memory (design counts 8, 3 and
+    16, orders 6, 4 and 2, coarsest lines of 64 and 56 DOFs): builds, FP32 sensitivities, indicators and
+    multigrid set-ups side by side.  The limit of a kernel is the process's: none may lower another's."""
+    import threading
+    err = []
+    go = threading.Barrier(3)
+
+    def work(nx, ny, p, d):
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()):
+                h = handle(mto, nx, ny, p, d)
+                fixed, f = mto.load_case(h, "cantilever")
+                h.set_supports(fixed)
+                rho = torch.full((h.design_len,), 0.5, dtype=torch.float64, device="cuda")
+                dc = torch.empty_like(rho)
+                u = torch.zeros(h.ndof, dtype=torch.float64, device="cuda")
+                mat = mto.material()
+                go.wait()
+                for k in range(400):
+                    for path in (mto.BUILD_TENSOR, mto.BUILD_SIMT):
+                        h.set_build_path(path)
+                        h.build_elements(rho, mat, mto.MTO_FP64)
+                    for _ in range(4):
+                        h.sensitivity(u, f, rho, mat, dc, precision=mto.MTO_MIXED, want_C=False)
+                    if k % 20 == 0:
+                        h.indicator(u, rho, mat, maps=False)
+                        h.solve(f, u, precision=mto.MTO_FP64, rtol=0.5, precond=mto.PREC_MG, check_every=2, max_iter=4,
+                                raise_on_noconv=False)
+                h.close()
+        except Exception as e:
+            err.append(repr(e))
+
+    ts = [threading.Thread(target=work, args=a) for a in ((31, 31, 6, 8), (27, 27, 4, 3), (31, 31, 2, 16))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not err, err
