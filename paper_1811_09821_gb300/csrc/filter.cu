@@ -49,7 +49,6 @@ __global__ void __launch_bounds__(256) filter_table_kernel(FilterTab ft, unsigne
   for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
   if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = sum;
   __syncthreads();
-  __syncthreads();
   if (threadIdx.x == 0) {
     for (int w = 1; w < 8; ++w) sum += ws[w];
     // the usual small stencils: in the order of the cells' own sums, whose rounding it then shares
@@ -140,6 +139,7 @@ constexpr int kFEl = 32;
 template <int MODE>
 __global__ void __launch_bounds__(128) filter_mixed_kernel(int nelx, int nely, double hx, double hy, double R,
                                                            int reach, FilterTab ft, const double* __restrict__ H,
+                                                           const int* __restrict__ ext,
                                                            const int* __restrict__ dmap,
                                                            const int64_t* __restrict__ off,
                                                            const double* __restrict__ x, double* __restrict__ out) {
@@ -162,6 +162,7 @@ __global__ void __launch_bounds__(128) filter_mixed_kernel(int nelx, int nely, d
     const double cx = (ex + cen[d][i]) * hx, cy = (ey + cen[d][j]) * hy;
     const int kx = ft.kx[d], ky = ft.ky[d];
     const double* Hd = H + ft.h0[d];
+    const int* ed = ext + ft.e0[d];
     double wsum = 0.0, acc = 0.0;
     for (int ny = max(ey - reach, 0); ny <= min(ey + reach, nely - 1); ++ny) {
       // distance from the centre to the neighbour row's y-range
@@ -172,12 +173,12 @@ __global__ void __launch_bounds__(128) filter_mixed_kernel(int nelx, int nely, d
         if (dx0 * dx0 + dy0 * dy0 >= R * R) continue;
         const int n = ny * nelx + nx, dn = dmap[n];
         const double* xn = x + off[n];
-        if (dn == d) {   // offsets on the common fine grid
+        if (dn == d) {   // offsets on the common fine grid; a value out of reach is not touched (it may be no number)
           const int bi = (nx - ex) * d - i, bj = (ny - ey) * d - j;
-          const int i0 = max(0, -kx - bi), i1 = min(d - 1, kx - bi);
           const int j0 = max(0, -ky - bj), j1 = min(d - 1, ky - bj);
           for (int jj = j0; jj <= j1; ++jj) {
-            const double* Hr = Hd + abs(bj + jj) * (kx + 1);
+            const int aj = abs(bj + jj), i0 = max(0, -ed[aj] - bi), i1 = min(d - 1, ed[aj] - bi);
+            const double* Hr = Hd + aj * (kx + 1);
             for (int ii = i0; ii <= i1; ++ii) {
               const double w = Hr[abs(bi + ii)];
               if (MODE != kSum) wsum += w;
@@ -192,7 +193,8 @@ __global__ void __launch_bounds__(128) filter_mixed_kernel(int nelx, int nely, d
               const double tx = (nx + cen[dn][ii]) * hx - cx;
               const double d2 = fma(tx, tx, ty2);
               if (d2 >= R * R) continue;
-              const double w = fmax(R - sqrt(d2), 0.0);
+              const double w = R - sqrt(d2);
+              if (!(w > 0.0)) continue;
               if (MODE != kSum) wsum += w;
               if (MODE != kScale) acc = fma(w, xn[jj * dn + ii], acc);
             }
@@ -313,7 +315,7 @@ mto_status density_filter(mto_handle h, double R, const double* x, double* out, 
   }
   auto go = [&](auto kernel, const double* in, double* o) -> mto_status {
     kernel<<<(nel + kFEl - 1) / kFEl, 128, 0, h->stream>>>(h->nelx, h->nely, h->hx, h->hy, R, reach, ft, h->filt_H,
-                                                           h->d_d, h->design_off_d, in, o);
+                                                           h->filt_ext, h->d_d, h->design_off_d, in, o);
     return mto_after_launch(h, "filter_mixed_kernel");
   };
   if (!adjoint) return go(filter_mixed_kernel<kForward>, x, out);

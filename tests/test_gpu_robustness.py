@@ -355,3 +355,28 @@ def test_threads_with_different_sizes(mto):
     for t in ts:
         t.join()
     assert not err, err
+
+
+@pytest.mark.parametrize("counts", [(3, 4), (4, 8), (5,)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_filter_reach_of_nonfinite_values(mto, bad, counts):
+    """A value that is not finite reaches exactly the subcells within the radius (0.873 is no distance of two
+    subcell centres here), in the filter and its adjoint, on meshes of one and of two design counts."""
+    nx, ny, R = 9, 7, 0.873
+    rng = np.random.default_rng(1)
+    dm = rng.choice(counts, nx * ny)
+    h = handle(mto, nx, ny, 1, dm)
+    off = np.concatenate([[0], np.cumsum(dm.astype(int) ** 2)])
+    xy = np.concatenate([np.stack([(np.arange(d * d) % d + 0.5) / d + e % nx, (np.arange(d * d) // d + 0.5) / d + e // nx], 1)
+                         for e, d in enumerate(dm)])
+    x = rng.uniform(size=h.design_len)
+    t = [off[10], off[40] + 4]
+    x[t] = bad
+    out = torch.empty(h.design_len, dtype=torch.float64, device="cuda")
+    hit = np.zeros(len(x), bool)
+    for k in t:
+        hit |= np.hypot(*(xy - xy[k]).T) < R
+    for fn in (h.filter, h.filter_adjoint):
+        fn(T(x), out, R)
+        np.testing.assert_array_equal(np.isfinite(out.cpu().numpy()), ~hit)
+    h.close()
