@@ -10,6 +10,7 @@
 #include <vector>
 
 #include "../../include/mto.h"
+#include "bits.cuh"
 
 namespace mto {
 
@@ -436,19 +437,6 @@ __device__ __forceinline__ double k_entry(const double* __restrict__ K64, const 
   const size_t o = (size_t)slot * L + pos;
   if (K64) return K64[o];
   return (double)Kh[o] + (double)Kl[o];
-}
-
-// 1 / d: Newton's iteration x <- x + x (1 - d x) on the mantissa, from its FP32 reciprocal (2^-23, squared
-// twice); plain division at the ends of the exponent range, for negative values, infinities and NaN
-__device__ __forceinline__ double newton_rcp(double d) {
-  const long long b = __double_as_longlong(d);
-  const int be = (int)(b >> 52);
-  if (be < 8 || be > 2038) return 1.0 / d;
-  const double md = __longlong_as_double((b & 0xfffffffffffffll) | (1023ll << 52));
-  double r = (double)(1.0f / __int_as_float(0x3f800000 | (int)((b >> 29) & 0x7fffff)));
-  r = fma(r, fma(-md, r, 1.0), r);
-  r = fma(r, fma(-md, r, 1.0), r);
-  return __longlong_as_double(__double_as_longlong(r) - ((long long)(be - 1023) << 52));
 }
 
 // Order-preserving map of a double to an unsigned 64-bit key (for radix selection).
