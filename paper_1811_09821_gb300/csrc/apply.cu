@@ -1144,8 +1144,8 @@ CGVecs<float> cg_vecs<float>(mto_handle h, float* x, float* r) {
 // result j of reduction slot k
 inline const double* res_slot(mto_handle h, int k) { return h->cg_res + 8 * k; }
 
-// The preconditioner step (rounded: the FP32 cycle finds r already rounded) z = M^-1 r with r^T z into reduction slot `slot` (element-block Schwarz:
-// one result per class launch; multigrid: one).
+// The preconditioner step z = M^-1 r with r^T z into reduction slot `slot` (element-block Schwarz: one result
+// per class launch; multigrid: one).  rounded: the FP32 cycle finds r in its own b already.
 template <typename T>
 mto_status precond_step(mto_handle h, const CGVecs<T>& v, int pc, int deg, int slot, const int* done,
                         bool rounded = false);

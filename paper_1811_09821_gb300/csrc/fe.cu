@@ -249,11 +249,9 @@ __global__ void zero_fixed_kernel(int64_t n, const int64_t* __restrict__ fixed, 
   }
 }
 
-__global__ void gather_element_matrix_kernel(int P, int L, const int2* __restrict__ dpos, int slot,
-                                             const double* __restrict__ K64, const float* __restrict__ Kh,
-                                             const float* __restrict__ Kl, double* __restrict__ out) {
-  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < P; c += gridDim.x * blockDim.x)
-    out[c] = k_entry(K64, Kh, Kl, L, slot, dpos[c].x);
+__global__ void gather_element_matrix_kernel(int P, const int2* __restrict__ dpos, const double* __restrict__ row,
+                                             double* __restrict__ out) {
+  for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < P; c += gridDim.x * blockDim.x) out[c] = row[dpos[c].x];
 }
 
 template <int PO>
@@ -408,8 +406,7 @@ mto_status element_matrix(mto_handle h, int64_t e, double* host_out) {
   MTO_TRY(mto_cuda_check(h, cudaMemcpy(&slot, h->slot_d + e, sizeof(int), cudaMemcpyDeviceToHost), "copy"));
   double* tmp = nullptr;
   MTO_TRY(mto_cuda_check(h, cudaMalloc(&tmp, sizeof(double) * c.P), "cudaMalloc"));
-  gather_element_matrix_kernel<<<(c.P + 255) / 256, 256, 0, h->stream>>>(c.P, c.L, c.dpos, slot, c.K64, c.K32,
-                                                                         c.K32lo, tmp);
+  gather_element_matrix_kernel<<<(c.P + 255) / 256, 256, 0, h->stream>>>(c.P, c.dpos, c.K64 + (size_t)slot * c.L, tmp);
   mto_status st = mto_after_launch(h, "gather_element_matrix_kernel");
   if (st == MTO_OK)
     st = mto_cuda_check(h, cudaMemcpyAsync(host_out, tmp, sizeof(double) * c.P, cudaMemcpyDeviceToHost, h->stream), "copy");

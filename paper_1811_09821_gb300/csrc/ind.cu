@@ -42,8 +42,7 @@ __global__ void __launch_bounds__(256) basis_table_kernel(BasisTab* t) {
   }
 }
 
-// Local displacement of element e (order p): 2 (p+1)^2 values, minimum-rule constraints applied.
-// both components of local node ln of the element in slot `slot` (through its constraint if hanging)
+// Both components of local node ln of the element in slot `slot` (through its constraint if hanging)
 __device__ __forceinline__ void gather_node(int nn, int slot, int ln, const int* __restrict__ gmap,
                                             const Constraint* __restrict__ cons, const double* __restrict__ u,
                                             double* ue) {
@@ -944,7 +943,7 @@ __global__ void __launch_bounds__(kOCBlock) oc_locate_kernel(int64_t n, const do
 
 // One bisection step from [l1, l2], l1 > 0.  Block b holds seg consecutive places of T, Lo, Hi; the first
 // cnt_b of them are its unsettled values (first: all of them), with acc[b], acc[G + b] the constant and the
-// slope of the settled ones.  part: [3][gridDim.x].
+// slope of the settled ones.  part: [2][gridDim.x].
 __global__ void __launch_bounds__(kOCBlock) oc_pass_kernel(int64_t n, int seg, int first, double* __restrict__ T,
                                                            double* __restrict__ Lo, double* __restrict__ Hi,
                                                            double eta, double target, double tol,

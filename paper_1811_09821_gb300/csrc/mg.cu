@@ -83,8 +83,6 @@ __device__ __forceinline__ int circ_pos(int i, int j, int ne) {
 template <int PO>
 __global__ void __launch_bounds__(128) mg_galerkin_p_kernel(int n, const int* __restrict__ elem, int L,
                                                             const double* __restrict__ K64,
-                                                            const float* __restrict__ Kh,
-                                                            const float* __restrict__ Kl,
                                                             const double* __restrict__ B,
                                                             double* __restrict__ K1) {
   constexpr int NN = (PO + 1) * (PO + 1), NE = 2 * NN;
@@ -112,7 +110,7 @@ __global__ void __launch_bounds__(128) mg_galerkin_p_kernel(int n, const int* __
 #pragma unroll
         for (int c2 = 0; c2 < 2; ++c2) {
           const int pos = circ_pos(i, 2 * b + c2, NE);
-          const double kij = K64 ? K64[row + pos] : (double)Kh[row + pos] + (double)Kl[row + pos];
+          const double kij = K64[row + pos];
 #pragma unroll
           for (int v = 0; v < 4; ++v) t[c2][v] = fma(kij, B[b * 4 + v], t[c2][v]);
         }
@@ -360,8 +358,9 @@ struct FirstStep {
 // level l -> l+1: the residual b - A x by the stencil on a tile of fine vertices in shared memory, full
 // weighting (the transpose of bilinear interpolation) on the free DOFs, and the coarse level's first step.
 // One launch of the four that the residual, the restriction, the first step and (above) the correction
-// took: 160 x 80 solve 74.3 -> 71.1 ms.  Tiles of 8 x 4: with 16 x 8 the middle levels have too few blocks
-// (the same solve 6 % slower than unfused).
+// took: a 160 x 80 solve 4 % faster (74.3 -> 71.1 ms, the same inputs in turn; a design of another seed takes
+// up to 87 ms, by its iterations).  Tiles of 8 x 4: with 16 x 8 the middle levels have too few blocks (6 %
+// slower than unfused).
 constexpr int kRX = 8, kRY = 4;   // coarse vertices per block
 constexpr int kRThreads = 160;    // 17 x 9 fine vertices
 template <typename TS, typename V>
@@ -1301,15 +1300,14 @@ mto_status mg_build(mto_handle h) {
     const PClass& c = h->pc[p];
     if (c.n == 0) continue;
     const double* B = h->mg_btab + h->mg_boff[p];
-    const double* K64 = c.K64;   // both builds keep the FP64 matrices
     const int grd = (c.n + 127) / 128;
     switch (p) {
-      case 1: mg_galerkin_p_kernel<1><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
-      case 2: mg_galerkin_p_kernel<2><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
-      case 3: mg_galerkin_p_kernel<3><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
-      case 4: mg_galerkin_p_kernel<4><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
-      case 5: mg_galerkin_p_kernel<5><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
-      case 6: mg_galerkin_p_kernel<6><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, K64, c.K32, c.K32lo, B, L1.K); break;
+      case 1: mg_galerkin_p_kernel<1><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
+      case 2: mg_galerkin_p_kernel<2><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
+      case 3: mg_galerkin_p_kernel<3><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
+      case 4: mg_galerkin_p_kernel<4><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
+      case 5: mg_galerkin_p_kernel<5><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
+      case 6: mg_galerkin_p_kernel<6><<<grd, 128, 0, h->stream>>>(c.n, c.elem, c.L, c.K64, B, L1.K); break;
     }
     MTO_TRY(mto_after_launch(h, "mg_galerkin_p_kernel"));
   }
@@ -1533,8 +1531,8 @@ mto_status mg_cycle(mto_handle h, const V* b0, V* x0, V* q0, V* d0, V* v0, V* w0
 // the FP32 cycle's rounded residual, for the PCG kernel that updates r (null when the cycle is in FP64)
 float* mg_residual32(mto_handle h) { return mg_fp32_cycle(h) ? h->mg_f32 : nullptr; }
 
-// z = M^-1 r (rounded: r is already rounded into the FP32 cycle's b): one V-cycle, with r^T z into *dot_res when dot_part is set (block partials in
-// dot_part, counter dot_cnt).  FP64 cycle: level-0 vectors b = r, x = z, q = mg_q0, d = mg_d0,
+// z = M^-1 r: one V-cycle, with r^T z into *dot_res when dot_part is set (block partials in dot_part, counter
+// dot_cnt).  rounded: r is in the FP32 cycle's b already.  FP64 cycle: level-0 vectors b = r, x = z, q = mg_q0, d = mg_d0,
 // v = mg_v0.  FP32 cycle (the cycle on FP32 copies of a mixed build): r rounded into its own FP32
 // level-0 vectors, z and r^T z written in FP64 by the last smoothing step.
 mto_status mg_vcycle(mto_handle h, const double* r, double* z, int degree, const int* done, double* dot_part,

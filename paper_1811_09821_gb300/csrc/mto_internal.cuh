@@ -430,15 +430,6 @@ __host__ __device__ inline int packed_index(int n, int i, int j) {
   return i * n - i * (i - 1) / 2 + (j - i);
 }
 
-// Entry at row position `pos` (see PClass::dpos) of the element matrix in slot `slot`, as a double:
-// from the FP64 matrices when present, else from the split-precision pair (hi + lo).
-__device__ __forceinline__ double k_entry(const double* __restrict__ K64, const float* __restrict__ Kh,
-                                          const float* __restrict__ Kl, int L, int slot, int pos) {
-  const size_t o = (size_t)slot * L + pos;
-  if (K64) return K64[o];
-  return (double)Kh[o] + (double)Kl[o];
-}
-
 // Order-preserving map of a double to an unsigned 64-bit key (for radix selection).
 __host__ __device__ inline unsigned long long order_key(double v) {
   unsigned long long u;

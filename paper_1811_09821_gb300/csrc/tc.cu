@@ -35,7 +35,8 @@
 //
 // Measured (build and one operator product together): 480 x 240 Q3/d8, mixed: 5.32 ms with an FP64
 // epilogue of 24 FP64 instructions per entry and 43 single-slice MMAs per K step, 1.10 ms now;
-// 320 x 160 adaptive maps (16 classes), FP64: 11.8 ms and 1.62 ms.
+// 320 x 160 adaptive maps (16 classes), FP64: 11.8 ms, 1.62 ms with this epilogue, 1.02 ms with the diagonal
+// spread over the local nodes as well.
 #include <algorithm>
 #include <cstdio>
 #include <cstring>
@@ -166,7 +167,8 @@ __device__ __forceinline__ void tc_bulk_g2s(void* dst, const void* src, uint32_t
 }
 
 // B operand tables of a class: per N tile, 8 slices of kTN x kpad BF16 in the core layout (so the
-// slices of a tile stack along N), and per position the exponent of its power-of-two scale tau.  One thread per (position, subcell).
+// slices of a tile stack along N), and per position the exponent of its power-of-two scale tau.  One
+// thread per (position, subcell).
 __global__ void tc_btable_kernel(int S, int kpad, int L, int ntile, const double* __restrict__ K0T,
                                  const int* __restrict__ posc, unsigned short* __restrict__ Bt,
                                  int* __restrict__ tau) {
