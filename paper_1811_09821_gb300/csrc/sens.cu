@@ -11,7 +11,7 @@
 // over the d x d subcells are two small products with the integrals W of the grid's Lagrange
 // polynomials over the subcells: w = W en W^T.  For Q3 and 8 x 8 subcells that is 49 strain
 // evaluations in place of 1024.  Its weights have both signs, so its error is relative to the element's
-// largest w: subcells below 1/64 of that are integrated by the subcell's own (p+1) x (p+1) Gauss points, a
+// largest w: subcells below 1/64 of that (Q1: 1/16) are integrated by the subcell's own (p+1) x (p+1) Gauss points, a
 // sum of squares with positive weights (w >= 0 for u = v, error relative to sqrt(w w_max)).  The
 // 1D tables are formed in double-double and rounded once: rounded products of Lagrange factors were
 // the larger part of either form's error.  Against extended precision (orders 1..6, d = 3 and 8; rough,
@@ -311,7 +311,11 @@ __global__ void __launch_bounds__(128) sens_kernel(
 // The FP64 kernel (see the head of this file).  A block of 128 threads takes EB elements (a power of
 // two, 4..32); each stage is a flat loop over the items of all of them.
 constexpr int kSensThreads = 128;
-constexpr double kSensDirect = 1.0 / 64.0;   // subcells below this share of the element's largest |w|: directly
+// Subcells below this share of the element's largest |w| are integrated directly.  Down to it the polynomial's
+// error, relative to the subcell's own w, was 0.3 to 1.1 times that of point sums with rounded tables in most
+// classes of the study (1.7 times in the worst, bending Q4 elements with 8 x 8 subcells); it grows with the
+// inverse of the share.
+__host__ __device__ constexpr double sens_direct_share(int p) { return p == 1 ? 1.0 / 16.0 : 1.0 / 64.0; }
 
 // doubles of shared memory per element of the x-contracted fields (later the subcells' w), and in all
 __host__ __device__ constexpr int sens_work_doubles(int p, int d, int nf) {
@@ -531,7 +535,7 @@ __global__ void __launch_bounds__(kSensThreads, NF == 1 ? (PO <= 3 ? 6 : 4) : (P
     for (int o = tpe >> 1; o > 0; o >>= 1) top = fmax(top, __shfl_xor_sync(0xffffffffu, top, o));
     if (el < ne)
       for (int s = t % tpe; s < S; s += tpe)
-        if (!(fabs(ws[el * S + s]) >= kSensDirect * top))   // also where w is not a number
+        if (!(fabs(ws[el * S + s]) >= sens_direct_share(PO) * top))   // also where w is not a number
           list[atomicAdd(&n_list, 1)] = (unsigned short)(el << 8 | s);
     __syncthreads();
     for (int it = t; it < n_list; it += kSensThreads) {
