@@ -334,63 +334,58 @@ __device__ __forceinline__ double sens_density(const double (&ax)[NF], const dou
   return fma(ax[0], ax[o], fma(c1 * ey[0], ey[o], c2 * gm[0] * gm[o]));
 }
 
-// The integral of the energy density over subcell (i, j) by its (p+1) x (p+1) Gauss points, of the fields at
-// Uf[NF][2][NN]; tab: the tables of the subcells' points.
+// Column kx of the (p+1) x (p+1) Gauss points of subcell (i, j): the energy density integrated along y, of the
+// fields at Uf[NF][2][NN]; tab: the tables of the subcells' points.
 template <int PO, int NF>
 __device__ __forceinline__ double sens_direct(const double* __restrict__ Uf, const double* __restrict__ tab, int d, int i,
-                                              int j, double nu, double c1, double c2) {
+                                              int j, int kx, double nu, double c1, double c2) {
   constexpr int N1 = PO + 1, NN = N1 * N1;
   const int np = d * N1 * N1;
   const double *L = tab, *Dx = L + np, *Dy = Dx + np, *w1 = Dy + np;
-  double w = 0.0;
-#pragma unroll 1
-  for (int kx = 0; kx < N1; ++kx) {
-    const double *lx = L + (i * N1 + kx) * N1, *dx = Dx + (i * N1 + kx) * N1;
-    double A[NF][4][N1];
+  const double *lx = L + (i * N1 + kx) * N1, *dx = Dx + (i * N1 + kx) * N1;
+  double A[NF][4][N1];
 #pragma unroll
-    for (int fld = 0; fld < NF; ++fld)
+  for (int fld = 0; fld < NF; ++fld)
+#pragma unroll
+    for (int b = 0; b < N1; ++b) {
+      double a0 = 0.0, d0 = 0.0, a1 = 0.0, d1 = 0.0;
+#pragma unroll
+      for (int a = 0; a < N1; ++a) {
+        const double l = __ldg(lx + a), dl = __ldg(dx + a);
+        const double v0 = Uf[fld * 2 * NN + b * N1 + a], v1 = Uf[fld * 2 * NN + NN + b * N1 + a];
+        a0 = fma(v0, l, a0);
+        d0 = fma(v0, dl, d0);
+        a1 = fma(v1, l, a1);
+        d1 = fma(v1, dl, d1);
+      }
+      A[fld][0][b] = a0;
+      A[fld][1][b] = d0;
+      A[fld][2][b] = a1;
+      A[fld][3][b] = d1;
+    }
+  double t = 0.0;
+#pragma unroll 1
+  for (int ky = 0; ky < N1; ++ky) {
+    const double *ly = L + (j * N1 + ky) * N1, *dy = Dy + (j * N1 + ky) * N1;
+    double ax[NF], ey[NF], gm[NF];
+#pragma unroll
+    for (int fld = 0; fld < NF; ++fld) {
+      double ex = 0.0, e2 = 0.0, ga = 0.0;
 #pragma unroll
       for (int b = 0; b < N1; ++b) {
-        double a0 = 0.0, d0 = 0.0, a1 = 0.0, d1 = 0.0;
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-          const double l = __ldg(lx + a), dl = __ldg(dx + a);
-          const double v0 = Uf[fld * 2 * NN + b * N1 + a], v1 = Uf[fld * 2 * NN + NN + b * N1 + a];
-          a0 = fma(v0, l, a0);
-          d0 = fma(v0, dl, d0);
-          a1 = fma(v1, l, a1);
-          d1 = fma(v1, dl, d1);
-        }
-        A[fld][0][b] = a0;
-        A[fld][1][b] = d0;
-        A[fld][2][b] = a1;
-        A[fld][3][b] = d1;
+        const double lb = __ldg(ly + b), db = __ldg(dy + b);
+        ex = fma(A[fld][1][b], lb, ex);
+        ga = fma(A[fld][0][b], db, ga);
+        ga = fma(A[fld][3][b], lb, ga);
+        e2 = fma(A[fld][2][b], db, e2);
       }
-    double t = 0.0;
-#pragma unroll 1
-    for (int ky = 0; ky < N1; ++ky) {
-      const double *ly = L + (j * N1 + ky) * N1, *dy = Dy + (j * N1 + ky) * N1;
-      double ax[NF], ey[NF], gm[NF];
-#pragma unroll
-      for (int fld = 0; fld < NF; ++fld) {
-        double ex = 0.0, e2 = 0.0, ga = 0.0;
-#pragma unroll
-        for (int b = 0; b < N1; ++b) {
-          const double lb = __ldg(ly + b), db = __ldg(dy + b);
-          ex = fma(A[fld][1][b], lb, ex);
-          ga = fma(A[fld][0][b], db, ga);
-          ga = fma(A[fld][3][b], lb, ga);
-          e2 = fma(A[fld][2][b], db, e2);
-        }
-        ax[fld] = fma(nu, e2, ex);
-        ey[fld] = e2;
-        gm[fld] = ga;
-      }
-      t = fma(__ldg(w1 + ky), sens_density<NF>(ax, ey, gm, c1, c2), t);
+      ax[fld] = fma(nu, e2, ex);
+      ey[fld] = e2;
+      gm[fld] = ga;
     }
-    w = fma(__ldg(w1 + kx), t, w);
+    t = fma(__ldg(w1 + ky), sens_density<NF>(ax, ey, gm, c1, c2), t);
   }
-  return w;
+  return t;
 }
 
 template <int PO, int NF>
@@ -413,6 +408,7 @@ __global__ void __launch_bounds__(kSensThreads, NF == 1 ? (PO <= 3 ? 6 : 4) : (P
   double* T = en + EB * Q * Q;                 // [EB][d][Q] integrated along x (subcell, y point)
   unsigned short* list = reinterpret_cast<unsigned short*>(T + EB * d * Q);   // [EB][d][d] small subcells
   __shared__ int n_list;
+  __shared__ double part[kSensThreads];
   if (t == 0) n_list = 0;
   for (int k = t; k < ntab; k += kSensThreads) sd[k] = tab[k];
   const int base = blockIdx.x * EB;
@@ -538,11 +534,26 @@ __global__ void __launch_bounds__(kSensThreads, NF == 1 ? (PO <= 3 ? 6 : 4) : (P
         if (!(fabs(ws[el * S + s]) >= sens_direct_share(PO) * top))   // also where w is not a number
           list[atomicAdd(&n_list, 1)] = (unsigned short)(el << 8 | s);
     __syncthreads();
-    for (int it = t; it < n_list; it += kSensThreads) {
-      const int le = list[it] >> 8, s = list[it] & 255;
-      ws[le * S + s] = sens_direct<PO, NF>(U + le * NF * 2 * NN, tab + ntab, d, s % d, s / d, nu, c1, c2);
+    // a thread per column of points (one per subcell left small meshes waiting for its chain)
+    constexpr int kItems = kSensThreads / N1;
+    const int small = n_list;
+    const double* w1 = tab + ntab + 3 * d * N1 * N1;
+    for (int first = 0; first < small; first += kItems) {
+      const int it = first + t / N1;
+      if (t < kItems * N1 && it < small) {
+        const int le = list[it] >> 8, s = list[it] & 255;
+        part[t] = sens_direct<PO, NF>(U + le * NF * 2 * NN, tab + ntab, d, s % d, s / d, t % N1, nu, c1, c2);
+      }
+      __syncthreads();
+      if (t < min(kItems, small - first)) {
+        const int e = list[first + t];
+        double w = 0.0;
+#pragma unroll
+        for (int kx = 0; kx < N1; ++kx) w = fma(__ldg(w1 + kx), part[t * N1 + kx], w);
+        ws[(e >> 8) * S + (e & 255)] = w;
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
   double energy = 0.0;   // sum_s E(rho_s) w_s (eout)
   if (el < ne) {
@@ -570,7 +581,7 @@ mto_status launch_poly(mto_handle h, const BClass& b, const double* u, const dou
   while (EB > 4 && (EB * per * 8 > 36 * 1024 || b.n < EB * 304)) EB /= 2;
   const size_t smem = sizeof(double) * ((size_t)EB * per + ntab);
   static_assert(8 * (4 * sens_elem_doubles(PO, MTO_D_MAX, NF) + (3 * sens_q(PO, MTO_D_MAX) + 1) * (PO + 1) +
-                     MTO_D_MAX * sens_q(PO, MTO_D_MAX)) <= 48 * 1024, "four elements of the largest count fit 48 KB");
+                     MTO_D_MAX * sens_q(PO, MTO_D_MAX)) + 8 * kSensThreads + 16 <= 48 * 1024, "four elements of the largest count fit 48 KB");
   sens_poly_kernel<PO, NF><<<(b.n + EB - 1) / EB, kSensThreads, smem, h->stream>>>(
       b.n, b.d, Q, EB, b.elem, b.slot, h->pc[b.p].gmap, h->cons_d, u, v, rho, h->design_off_d, m->E0, m->Emin, m->q,
       m->nu, h->hx, h->hy, b.stab, dc, eout);
