@@ -650,9 +650,11 @@ size_t tma_smem_bytes(int L, int G, int nm, int stages) {
 
 }  // namespace
 
-// Threads per block of an element-operator launch of `warps` warps: two warps while that leaves at most
-// one wave of blocks, so that the warps of small classes spread over the SMs, else eight.
-static int ebe_threads(int warps) { return warps <= 2 * 152 * 8 ? 64 : 256; }
+// Threads per block of an element-operator launch of `warps` warps: four warps up to four per SM, so that
+// small classes spread over the SMs, else eight (more blocks cost the launch's reduction one more atomic on
+// one address each).  Measured in us at 64 / 128 / 256 threads: 300 Q4 elements, FP64 19.0 / 18.9 / 20.7;
+// 600 Q6, FP64 51.1 / 49.3 / 52.2; 1200 Q3, FP64 17.5 / 15.7 / 14.5; 2400 Q3, split 20.1 / 16.1 / 15.1.
+static int ebe_threads(int warps) { return warps <= 4 * 152 ? 128 : 256; }
 
 // Blocks of one element-operator launch for an order class (fixed per class size).
 template <int PO>
@@ -757,9 +759,8 @@ void launch_ebe(mto_handle h, const PClass& c, const double* M64, const float* M
         }
         return;
       }
-      // persistent: two blocks of 8 warps per SM (the register budget of the pipelined rows); small
-      // classes in blocks of two warps, spread over the SMs
-      const int th = warps <= 152 * 8 ? 64 : 256;
+      // persistent: two blocks of 8 warps per SM (the register budget of the pipelined rows)
+      const int th = ebe_threads(warps);
       int blocks = (warps + th / 32 - 1) / (th / 32);
       if (th == 256 && blocks > 152 * 2) blocks = 152 * 2;
       if (lo)
