@@ -392,7 +392,8 @@ mto_status mto_element_matrix_split(mto_handle h, int64_t e, float* hi, float* l
  * self-adjoint compliance problem is -u.  u, f: device double[ndof]; rho, dc: device
  * double[design_len]; C: host double (may be NULL: then no synchronisation).  precision as for
  * the build: MTO_MIXED evaluates the quadratic forms in FP32 after an FP64 removal of the
- * element's rigid-body motion. */
+ * element's rigid-body motion.  u_e^T K0_s u_e is never negative, so dc <= 0; its rounding error is
+ * relative to the square root of the subcell's value times the element's largest. */
 mto_status mto_sensitivity(mto_handle h, const double* u, const double* f, const double* rho,
                            const mto_material* mat, int32_t precision, double* dc, double* C);
 

@@ -330,7 +330,8 @@ mto_status mto_create(mto_handle* out, int device, void* stream) {
   if (const char* ok = std::getenv("MTO_OP_KERNEL"))
     h->op_kernel = (ok[0] >= '0' && ok[0] <= '2') ? ok[0] - '0' : -1;
   // MTO_TC_POLLS=n: polls before a wait of the tensor-core build expires (0: at once, to test the error path)
-  if (const char* tp = std::getenv("MTO_TC_POLLS")) h->tc_polls = (unsigned)std::strtoul(tp, nullptr, 10);
+  if (const char* tp = std::getenv("MTO_TC_POLLS"))
+    if (tp[0] >= '0' && tp[0] <= '9') h->tc_polls = (unsigned)std::strtoul(tp, nullptr, 10);
   cudaSetDevice(device);
   if (cudaStreamCreateWithFlags(&h->stream, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&h->ev_in, cudaEventDisableTiming) != cudaSuccess ||
