@@ -283,9 +283,11 @@ __global__ void __launch_bounds__(32 * kGdWarps) gamma_d_kernel(
 // place of the last three until they are needed; with n0 = 2 (p+1)^2, n1 = 2 (p+2)^2,
 // L1 = n1 (n1 + 1) / 2 rounded up.
 // K^(p+1) = sum_s E_s K0_s comes as rows formed on the tensor cores (tc_rows, d <= 8), or is summed
-// here from the table (rows null, and the elements that `sliced_rows_hold` turns away).  The kernel is
-// bound by the FP64 pipes (2 FMA per clock and SM), where those sums were 81.6 k of 115 k FMAs of a Q3/d8
-// element (170.5 ms on the 1024 x 512 beam).
+// here from the table (rows null, and the elements that `sliced_rows_hold` turns away: 81.6 k of 115 k FMAs
+// of a Q3/d8 element).  With rows the FP64 pipes (2 FMA per clock and SM) are 75 % busy, the rest is the
+// L D L^T's shared-memory round trips: 12,800 Q3/d8 elements 1.2 ms.  A graded design, most of whose
+// elements sum, takes 3.2 ms and is bound by L1 (a lane's table row lies S doubles from the next lane's).
+// Indicators of a 320 x 160 adaptive mesh, graded: 10.9 ms with sums, 6.9 with rows, 9.7 with both by this rule.
 // eps is invariant to rigid motions of u^(p), which are removed first (FP64) so that the element
 // energies carry no cancellation.
 //

@@ -19,7 +19,7 @@
 // form 1.7e-16 to 3.9e-16, nowhere the larger but for 2.4e-16 against 2.2e-16 at p = 4, d = 8.  Bound by the
 // FP64 pipes (2 FMA per clock and SM): a block takes several elements and spreads each stage over all
 // its threads.  480 x 240 Q3/d8 elements: 12.25 ms with point sums over every subcell, 0.76 ms with the
-// polynomial for every one, 0.96 ms with the small ones directly.
+// polynomial for every one, 0.87 ms with the small ones directly.
 //
 // FP32 (sens_kernel, MTO_MIXED): one warp per element; strains at the (p+1) x (p+1) Gauss points of
 // every subcell from a sum-factorised tensor evaluation on the element's d(p+1) x d(p+1) point grid;
